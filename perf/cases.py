@@ -330,8 +330,13 @@ def run(state):
             order = order[torch.argsort(keys[order, 1], stable=True)]
         else:
             order = torch.argsort(keys[:, 0])
+        n = len(order)
         for whole, rows in zip(state["out"], (keys, counts, ext, codes)):
-            torch.index_select(rows, 0, order, out=whole[:len(order)])
+            if rows.dim() == 1 or rows.shape[1] * rows.element_size() < 16:
+                torch.index_select(rows, 0, order, out=whole[:n])
+            else:  # 16 bytes at a time
+                for to, column in zip(whole.view(torch.complex128).unbind(1), rows.view(torch.complex128).unbind(1)):
+                    to[:n] = column[order]
         return {"n": int(info.n), "n_uu": int(info.n_uu), "windows": int(info.valid_windows), "records": state["out"]}
     if kind == "batch":
         graph = state["graph"]
