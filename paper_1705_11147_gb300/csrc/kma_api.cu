@@ -94,18 +94,21 @@ struct Derived {
   u64 codes_words, bit_words, mark_words;
   u64 staging;
   unsigned P;      // on-chip partitions (1: one table)
-  u64 Wp, Sp;      // Bloom words / table slots per partition
-  u64 Wt;          // key filter words per partition (partitioned Bloom mode, else 0)
+  u64 Sp;          // table slots per partition
   u64 rec_bytes;   // bytes per record in partitioned mode
+  unsigned log_b, sub_max, avg;  // partitioned mode: buckets, sub-buckets per bucket, records per sub-bucket
 };
 
-// Key filter of the partitioned recount: a second blocked Bloom filter that records the keys
-// inserted into the table, sized at this many bits per key the table is built for.
-constexpr double kKeyFilterBitsPerKey = 12.0;
+// Partitioned mode sorts records into buckets, then sub-buckets of about this part of what the
+// count kernel stages, and does both sorts with about as many bins. The rest is for the spread of
+// their sizes: at 30x coverage one in a thousand overflows.
+constexpr double kSubBucketFill = 0.72;
+// The sorted copy of the records made by the split: as large as all of them below this size, one
+// launch; above it the buckets are split and counted in groups that share a smaller copy.
+constexpr u64 kSplitAtOnce = 2ull << 30;
+constexpr u64 kSplitGroups = 12;
 
-// Partitioned above 32 MB of filter + table: from 45 MB (7.5 Mbases, k = 31) up, two L2-sized
-// partitions beat one table (0.62 -> 0.57 ms; 1.87 -> 1.41 ms at 30 Mbases).
-constexpr u64 kAutoPartitionAbove = 32ull << 20;   // filter + table bytes
+constexpr u64 kAutoPartitionAbove = 32ull << 20;   // partitioned above: filter + table bytes
 constexpr u64 kPartitionTarget = 64ull << 20;      // filter + table bytes per partition
 
 int check_params(const kma_params* p) {
@@ -148,7 +151,7 @@ int derive(const kma_params* p, Derived& d) {
     const double lf = p->load_factor > 0 ? p->load_factor : 0.5;
     d.plan.table_slots = (u64)std::ceil(keys / lf) + 64;
   }
-  // on-chip partitions: each part's Bloom sub-filter and sub-table sized for L2
+  // on-chip partitions of the table
   {
     const u64 W = d.plan.bloom_words, S = d.plan.table_slots;
     const u64 bytes = W * 8 + S * sizeof(Slot);
@@ -158,23 +161,22 @@ int derive(const kma_params* p, Derived& d) {
     if (P > max_parts) P = max_parts;
     if (P < 1) P = 1;
     d.P = (unsigned)P;
-    d.Wp = (W + P - 1) / P;
     d.Sp = (S + P - 1) / P;
     if (P > 1) {
       if (d.Sp < 64) d.Sp = 64;
-      d.plan.bloom_words = W ? d.Wp * P : 0;
+      d.plan.bloom_words = W ? (W + P - 1) / P * P : 0;
       d.plan.table_slots = d.Sp * P;
     } else {
-      d.Wp = W;
       d.Sp = S;
     }
     d.plan.partitions = d.P;
-    d.rec_bytes = (p->k > 32 ? 16 : 8) + 1;
-    if (P > 1 && p->use_bloom) {
-      const double lf = p->load_factor > 0 ? p->load_factor : 0.5;
-      const double keys = (double)d.plan.table_slots * lf;
-      d.Wt = std::max<u64>((u64)std::ceil(keys * kKeyFilterBitsPerKey / 64.0 / (double)P), 64);
-    }
+    d.rec_bytes = p->k > 32 ? 16 : 8;
+    const double parts = p->n_parts > 1 ? p->n_parts : 1;
+    d.avg = (unsigned)((p->k > 32 ? kCountCap2 : kCountCap1) * kSubBucketFill);
+    const double subs = (double)p->max_bases / parts / d.avg;
+    const long lb = std::lround(0.5 * std::log2(std::max(subs, 1.0)));
+    d.log_b = (unsigned)std::min<long>(std::max<long>(lb, kMinLogBuckets), kMaxLogBuckets);
+    d.sub_max = (unsigned)std::min<double>(std::ceil(subs / (double)(1u << d.log_b)) + 1.0, kMaxSubBuckets);
   }
   // bit slices of the key hash address at most 2^32 Bloom words and 2^32 slots per partition
   if (d.plan.bloom_words >= (1ull << 32) || d.Sp >= (1ull << 32)) return KMA_EINVAL;
@@ -186,10 +188,13 @@ int derive(const kma_params* p, Derived& d) {
   d.mark_words = pos / 32 + 4;
   d.staging = p->staging_bytes ? p->staging_bytes : kDefaultStaging;
   d.plan.device_bytes = 2 * d.codes_words * 8 + 2 * d.bit_words * 8 + d.mark_words * 4 +
-                        d.plan.bloom_words * 8 + d.plan.table_slots * sizeof(Slot) +
+                        (d.P > 1 ? 0 : d.plan.bloom_words * 8) + d.plan.table_slots * sizeof(Slot) +
                         sizeof(DevStatus) + 2 * (2 * d.staging + (d.staging / 16 + 2) * 8);
-  if (d.P > 1)  // record buckets and the key filter
-    d.plan.device_bytes += (p->max_bases + p->max_bases / 16) * d.rec_bytes + d.Wt * d.P * 8;
+  if (d.P > 1) {  // scatter tiles with their offset rows, and the split's sorted copy
+    const u64 tiles = pos / kPartTile + 1, recs = tiles * kPartTile * d.rec_bytes;
+    const u64 copy = recs <= kSplitAtOnce ? recs : std::max(kSplitAtOnce, recs / kSplitGroups);
+    d.plan.device_bytes += recs + tiles * (((u64)1 << d.log_b) + 8) * 2 + 4 * copy;
+  }
   return KMA_OK;
 }
 
@@ -287,9 +292,9 @@ void pinned_give(void* b) {
 
 }  // namespace
 
-// finalize_to_host splits the recount and classification into this many groups of
+// finalize_to_host splits the counting and classification into this many groups of
 // partitions (of table slots with one table), so that each group's records are copied to the
-// host while the next group is still being recounted.
+// host while the next group is still being counted.
 constexpr unsigned kFinalizeGroups = 8;
 
 struct kma_handle {
@@ -311,8 +316,7 @@ struct kma_handle {
   u64* inv = nullptr;
   u64* hq = nullptr;
   unsigned* marks = nullptr;
-  u64* bloom = nullptr;
-  u64* keyfilter = nullptr;  // partitioned Bloom mode: keys inserted into the table
+  u64* bloom = nullptr;      // one-table mode
   Slot* table = nullptr;
   DevStatus* status = nullptr;
   DevStatus* host_status = nullptr;  // pinned
@@ -323,18 +327,18 @@ struct kma_handle {
   int stage_next = 0;
 
   u64 q_used = 0, reads_used = 0, bases_used = 0;
-  // Upper bound on the occurrences any one key can have collected since the last reset
-  // (windows counted in one table; bucket + overflow records per batch in partitioned
-  // mode). Below 2^32 no counter can wrap and the passes count with plain reductions.
+  // One table: windows counted since the last reset, an upper bound on the occurrences of any
+  // one key. Below 2^32 no counter can wrap and the passes count with plain reductions.
   u64 count_bound = 0;
   bool finalized = false;
   bool failed = false;
   bool pack_only = false;  // estimation handles: count() packs the reads, no counting pass
 
-  // partitioned mode: per-partition histogram / cursors and the record buckets of each
-  // count() batch (kept until finalize has recounted them)
-  struct RecBatch { void* keys; unsigned char* info; u64* fill; u64 cap, ocap; };
-  std::vector<RecBatch> rec_batches;
+  // partitioned mode: the scatter tiles of the count() calls, in slabs kept until finalize has
+  // counted them, and the records per bucket
+  struct Slab { u64* recs; unsigned short* offs; u64 cap, used; double windows, positions; };
+  std::vector<Slab> slabs;
+  u64* totals = nullptr;
 
   // contigs of the finalized result (kmer_analysis_contigs), freed by reset / destroy
   char* contig_seq = nullptr;
@@ -413,12 +417,11 @@ int timed_launch(kma_handle* h, int kind, cudaStream_t stream, bool has_work, F&
 }
 
 void free_records(kma_handle* h) {
-  for (auto& b : h->rec_batches) {
-    if (b.keys) cudaFreeAsync(b.keys, h->stream);
-    if (b.info) cudaFreeAsync(b.info, h->stream);
-    if (b.fill) cudaFreeAsync(b.fill, h->stream);
+  for (auto& b : h->slabs) {
+    if (b.recs) cudaFreeAsync(b.recs, h->stream);
+    if (b.offs) cudaFreeAsync(b.offs, h->stream);
   }
-  h->rec_batches.clear();
+  h->slabs.clear();
 }
 
 void free_contigs(kma_handle* h) {
@@ -432,7 +435,7 @@ void free_contigs(kma_handle* h) {
 void free_all(kma_handle* h) {
   free_records(h);
   dfree(h, h->codes); dfree(h, h->rcodes); dfree(h, h->inv); dfree(h, h->hq); dfree(h, h->marks);
-  dfree(h, h->bloom); dfree(h, h->keyfilter); dfree(h, h->table); dfree(h, h->status);
+  dfree(h, h->bloom); dfree(h, h->totals); dfree(h, h->table); dfree(h, h->status);
   for (int i = 0; i < 2; ++i) { dfree(h, h->stage_seq[i]); dfree(h, h->stage_qual[i]); dfree(h, h->stage_offs[i]); }
   dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
   free_contigs(h);
@@ -458,7 +461,7 @@ void free_all(kma_handle* h) {
   h->event_pool.clear();
 }
 
-// Back to the empty state: status, Bloom filter, key filter and table cleared on the handle's
+// Back to the empty state: status, Bloom filter, bucket totals and table cleared on the handle's
 // stream. The arena is not cleared: every count() rewrites the words of its batch and sets the
 // slack words behind it invalid (reserve_batch).
 int clear_state(kma_handle* h) {
@@ -466,7 +469,7 @@ int clear_state(kma_handle* h) {
   free_contigs(h);
   KMA_CUDA(cudaMemsetAsync(h->status, 0, sizeof(DevStatus), h->stream));
   if (h->bloom) KMA_CUDA(cudaMemsetAsync(h->bloom, 0, h->d.plan.bloom_words * 8, h->stream));
-  if (h->keyfilter) KMA_CUDA(cudaMemsetAsync(h->keyfilter, 0, h->d.Wt * h->d.P * 8, h->stream));
+  if (h->totals) KMA_CUDA(cudaMemsetAsync(h->totals, 0, sizeof(u64) << h->d.log_b, h->stream));
   int rc = timed_launch(h, KMA_KERNEL_INIT, h->stream, h->d.plan.table_slots > 0,
                         [&] { return launch_table_init(h->table, h->d.plan.table_slots, h->stream); });
   if (rc) return rc;
@@ -492,7 +495,7 @@ void choose_shape(kma_handle* h) {
 int flags_to_code(unsigned flags) {
   if (flags & kFlagTimeout) return KMA_ETIMEOUT;
   if (flags & kFlagBadOffsets) return KMA_EINVAL;
-  if (flags & kFlagFull) return KMA_EFULL;
+  if (flags & (kFlagFull | kFlagOutput)) return KMA_EFULL;
   if (flags & kFlagOverflow) return KMA_EOVERFLOW;
   return KMA_OK;
 }
@@ -555,101 +558,196 @@ int reserve_batch(kma_handle* h, u64 n_reads, u64 n_bases, PackDesc& pd, u64& q0
 PartGeom part_geom(kma_handle* h) {
   PartGeom g;
   std::memset(&g, 0, sizeof(g));
-  g.bloom = h->bloom;
-  g.keyfilter = h->keyfilter;
-  g.Wk = h->d.Wt;
   g.table = h->table;
   g.status = h->status;
-  g.Wp = h->d.Wp;
   g.Sp = h->d.Sp;
   g.P = h->d.P;
-  g.bloom_h = h->d.plan.bloom_hashes;
   g.k = h->p.k;
   g.canonical = h->p.canonical;
   g.n_parts = h->p.n_parts > 1 ? h->p.n_parts : 1;
   g.part = h->p.n_parts > 1 ? h->p.part : 0;
-  g.rpt = h->p.windows_per_thread >= 4 ? 4 : 2;
-  g.wait_limit = kWaitPolls;
-  g.no_overflow = h->count_bound < (1ull << 32) ? 1u : 0u;
-  g.group = h->p.heavy_hitters ? 1u : 0u;
+  g.log_b = h->d.log_b;
+  g.sub_max = h->d.sub_max;
+  g.avg = h->d.avg;
+  g.cap = h->p.k > 32 ? kCountCap2 : kCountCap1;
+  g.min_count = h->p.use_bloom ? 2 : 1;
   return g;
 }
 
-// First pass over the windows [q0, q0 + n_pos) of one packed batch (n_reads reads, n_bases
-// bases) on stream `st`. One table: Bloom test-and-set (or counting) in place. Partitions:
-// scatter into per-partition record buckets, then the record pass part by part; the buckets
-// are kept for the recount in finalize. Nothing here waits for the GPU.
-// Partitioned mode: record buckets for a count() call of n_pos arena positions (n_reads reads,
-// n_bases bases), appended to the handle's record batches (kept for the recount).
-int prepare_records(kma_handle* h, u64 n_pos, u64 n_reads, u64 n_bases, cudaStream_t st, size_t& index) {
-  const u64 P = h->d.P, k = h->p.k;
-  // Bucket capacity from the window count of reads of length >= k (exact for such reads);
-  // shorter reads, hash imbalance and repeated k-mers spill into the overflow area. Both are
-  // multiples of 16 records (the record passes stage 16-byte aligned tiles).
-  const u64 w_est = n_bases > (k - 1) * n_reads ? n_bases - (k - 1) * n_reads : 0;
-  u64 cap = ((u64)((double)w_est / (double)P * 1.05) + 64 + 15) & ~15ull;
-  u64 ocap = n_pos / 16 + 65536;
-  if (P * cap < n_bases) ocap = std::max(ocap, n_bases - P * cap + n_pos / 64);
-  ocap = (ocap + 15) & ~15ull;
-  // the kernels hold in-bucket and overflow positions, and tile numbers, in 32 bits
-  const u64 tile_recs = 32ull * part_geom(h).rpt;
-  if (cap >= (1ull << 32) || ocap >= (1ull << 32) ||
-      P * ((cap + tile_recs - 1) / tile_recs) + (ocap + tile_recs - 1) / tile_recs >= (1ull << 31))
-    return KMA_EINVAL;  // more partitions, or smaller count() batches, are needed
-  h->count_bound += cap + ocap;
-  const u64 total = P * cap + ocap;
-  kma_handle::RecBatch rb{nullptr, nullptr, nullptr, cap, ocap};
-  const size_t kb = (size_t)total * (k > 32 ? 16 : 8);
-  cudaError_t e = cudaMallocFromPoolAsync(&rb.keys, kb, h->pool, st);
-  if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&rb.info, (size_t)total, h->pool, st);
-  // fill[0..P], then one word for the record passes' tile queue
-  if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)&rb.fill, (size_t)(P + 2) * 8, h->pool, st);
+// Scatter tiles of slab `sl` (tile0: where the next scatter launch writes).
+PartTiles tiles_of(kma_handle* h, const kma_handle::Slab& sl, u64 tile0) {
+  PartTiles t;
+  t.recs = sl.recs;
+  t.offs = sl.offs;
+  t.totals = h->totals;
+  t.tile0 = tile0;
+  t.n_tiles = (unsigned)sl.used;
+  t.stride = (1u << h->d.log_b) + 8;
+  return t;
+}
+
+u64 tiles_for(u64 n_pos) { return (n_pos + kPartTile - 1) / kPartTile; }
+
+// Partitioned mode: room for `tiles` more scatter tiles in the handle's last slab, or a new slab
+// that also has room for later calls (up to what max_bases allows, 2048 tiles at most), so that
+// many small count() calls fill common chunks.
+int prepare_tiles(kma_handle* h, u64 tiles, cudaStream_t st) {
+  if (!h->slabs.empty() && h->slabs.back().used + tiles <= h->slabs.back().cap) return KMA_OK;
+  const u64 left = tiles_for(h->d.plan.arena_positions - std::min<u64>(h->q_used, h->d.plan.arena_positions)) + 1;
+  const u64 cap = std::max<u64>(tiles, std::min<u64>(left, 2048));
+  if (cap >= (1ull << 31)) return KMA_EINVAL;  // tile numbers are 32-bit
+  kma_handle::Slab sl{nullptr, nullptr, cap, 0, 0.0, 0.0};
+  cudaError_t e = cudaMallocFromPoolAsync((void**)&sl.recs, (size_t)cap * kPartTile * h->d.rec_bytes, h->pool, st);
+  if (e == cudaSuccess)
+    e = cudaMallocFromPoolAsync((void**)&sl.offs, (size_t)cap * (((u64)1 << h->d.log_b) + 8) * 2, h->pool, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
-    if (rb.keys) cudaFreeAsync(rb.keys, st);
-    if (rb.info) cudaFreeAsync(rb.info, st);
-    if (rb.fill) cudaFreeAsync(rb.fill, st);
-    return e == cudaErrorMemoryAllocation ? KMA_ENOMEM : cuda_fail(e, "record buckets");
+    if (sl.recs) cudaFreeAsync(sl.recs, st);
+    return e == cudaErrorMemoryAllocation ? KMA_ENOMEM : cuda_fail(e, "scatter tiles");
   }
-  h->rec_batches.push_back(rb);
-  index = h->rec_batches.size() - 1;
-  KMA_CUDA(cudaMemsetAsync(rb.fill, 0, (size_t)(P + 2) * 8, st));
+  h->slabs.push_back(sl);
   return KMA_OK;
 }
 
-// Record batch `rb` of a handle with P partitions, all of it (every bucket, then the
-// overflow area).
-PartRecords records_of(const kma_handle::RecBatch& rb, u64 P) {
-  PartRecords r;
-  r.keys = rb.keys; r.info = rb.info; r.cap = rb.cap; r.ocap = rb.ocap; r.fill = rb.fill;
-  r.queue = reinterpret_cast<unsigned*>(rb.fill + P + 1);
-  r.p_begin = 0; r.p_end = (unsigned)P; r.overflow = 1; r.pad = 0;
-  return r;
-}
-
-// Partitioned mode: the windows [q0, q0 + n_pos) into record batch `index`.
-int scatter_windows(kma_handle* h, size_t index, u64 q0, u64 n_pos, cudaStream_t st) {
+// Partitioned mode: the windows [q0, q0 + n_pos) (n_reads reads, n_bases bases) into the last
+// slab, which has room for them.
+int scatter_windows(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, cudaStream_t st) {
   const PartGeom g = part_geom(h);
   PartWindows w;
   w.codes = h->codes; w.rcodes = h->rcodes; w.inv = h->inv; w.hq = h->hq;
   w.q0 = q0; w.q1 = q0 + n_pos;
-  const PartRecords r = records_of(h->rec_batches[index], h->d.P);
+  kma_handle::Slab& sl = h->slabs.back();
+  const PartTiles t = tiles_of(h, sl, sl.used);
+  sl.used += tiles_for(n_pos);
+  sl.positions += (double)n_pos;
+  const u64 k1 = h->p.k - 1;
+  sl.windows += (n_bases > k1 * n_reads ? (double)(n_bases - k1 * n_reads) : 0.0) / std::max(1u, h->p.n_parts);
   return timed_launch(h, KMA_KERNEL_SCATTER, st, n_pos > 0,
-                      [&] { return launch_part_scatter(g, w, r, st, h->num_sms); });
+                      [&] { return launch_part_scatter(g, w, t, st, h->num_sms); });
 }
 
-// Partitioned mode: the record pass (Bloom test-and-set, or counting) over batch `index`.
-int record_pass(kma_handle* h, size_t index, cudaStream_t st) {
-  const unsigned mode = h->p.use_bloom ? kModeBloom : kModeCount;
-  const PartGeom g = part_geom(h);
-  const PartRecords r = records_of(h->rec_batches[index], h->d.P);
-  return timed_launch(h, KMA_KERNEL_PASS, st, true, [&] { return launch_part_pass(g, r, mode, st, h->num_sms); });
+// Lanes (log2) that copy one run of `len` records on average.
+unsigned lanes_for(double len) {
+  const double l = std::floor(std::log2(std::max(len, 1.0)) + 0.3);
+  return (unsigned)std::min(5.0, l);
+}
+
+// Partitioned mode: counts the handle's records into its table on stream `st`, the buckets in
+// order, `parts` groups of them or more, and calls after(end) when the buckets below `end` have
+// been enqueued. The sorted copy of the split is sized for all records when they are few or
+// when the call may not wait for the GPU (may_sync = false, capture); otherwise from the bucket
+// totals, a twelfth of the records or the largest bucket.
+template <typename F>
+int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sync, unsigned parts, F&& after) {
+  const unsigned B = 1u << h->d.log_b;
+  u64 bound = 0, n_chunks = 0;
+  double windows = 0, positions = 0;
+  std::vector<unsigned> chunk_tiles;
+  for (auto& sl : h->slabs) {
+    const double least = 0.5 / std::max(1u, h->p.n_parts);  // against many reads shorter than k
+    const double occ = std::min(1.0, std::max(least, sl.positions > 0 ? sl.windows / sl.positions : 1.0));
+    // a bucket's records from one chunk fill 85 % of a sub-tile
+    const double c = 0.85 * kPartSubTile * B / (kPartTile * occ);
+    chunk_tiles.push_back((unsigned)std::min<double>(std::max(1.0, std::floor(c)), kMaxChunkTiles));
+    n_chunks += (sl.used + chunk_tiles.back() - 1) / chunk_tiles.back();
+    bound += sl.used * kPartTile;
+    windows += sl.windows;
+    positions += sl.positions;
+  }
+  if (n_chunks == 0) return after(B);
+  if (parts > B) parts = B;
+  std::vector<unsigned> ends;
+  u64 most = bound;        // records of a group
+  unsigned most_buckets = 0;
+  if (!may_sync || bound * h->d.rec_bytes <= kSplitAtOnce) {
+    for (unsigned i = 0; i < parts; ++i) ends.push_back((unsigned)((u64)B * (i + 1) / parts));
+  } else {
+    std::vector<u64> totals(B);
+    KMA_CUDA(cudaMemcpyAsync(totals.data(), h->totals, B * sizeof(u64), cudaMemcpyDeviceToHost, st));
+    KMA_CUDA(cudaStreamSynchronize(st));
+    u64 all = 0;
+    for (u64 t : totals) all += t;
+    const u64 aim = std::max(kSplitAtOnce / h->d.rec_bytes, all / kSplitGroups);
+    const unsigned widest = (B + parts - 1) / parts;
+    most = 0;
+    for (unsigned b = 0; b < B;) {
+      unsigned e = b;
+      u64 sum = 0;
+      do sum += totals[e++];
+      while (e < B && e - b < widest && sum + totals[e] <= aim);
+      ends.push_back(e);
+      most = std::max(most, sum);
+      b = e;
+    }
+  }
+  for (size_t i = 0; i < ends.size(); ++i) most_buckets = std::max(most_buckets, ends[i] - (i ? ends[i - 1] : 0));
+  PartSplit s;
+  std::memset(&s, 0, sizeof(s));
+  PartGeom g = part_geom(h);
+  // sub-buckets for the windows expected (one more than that for reads shorter than k)
+  g.sub_max = (unsigned)std::min<double>(g.sub_max, std::ceil(1.05 * windows / ((double)g.avg * B)) + 1.0);
+  const u64 n_subs = (u64)most_buckets * g.sub_max;
+  const u64 n_segs = most / kPartSubTile + (u64)most_buckets * n_chunks + 1;
+  if (n_chunks >= (1ull << 31) || n_segs >= (1ull << 32)) return KMA_EINVAL;
+  std::vector<void*> temps;
+  auto temp = [&](void** ptr, u64 bytes) -> int {
+    cudaError_t e = cudaMallocFromPoolAsync(ptr, bytes, h->pool, st);
+    if (e == cudaSuccess) {
+      temps.push_back(*ptr);
+      return KMA_OK;
+    }
+    cudaGetLastError();
+    return e == cudaErrorMemoryAllocation ? KMA_ENOMEM : cuda_fail(e, "split output");
+  };
+  auto run = [&]() -> int {
+    int rc;
+    u64* zero = nullptr;  // [sub-buckets], overflow records, list entries, then segments per bucket (32 bits)
+    const u64 n_zero = n_subs + 2 + (most_buckets + 1) / 2;
+    const unsigned key_words = kMaxKeyWords - (h->d.rec_bytes == 8 ? 2 : 0);
+    const u64 keys = most / (h->p.use_bloom ? 2 : 1) + 1;
+    if ((rc = temp((void**)&s.recs, n_subs * g.cap * h->d.rec_bytes)) || (rc = temp((void**)&s.over, most * h->d.rec_bytes)) ||
+        (rc = temp((void**)&s.keys, keys * key_words * 4)) || (rc = temp((void**)&zero, n_zero * 8)) ||
+        (rc = temp((void**)&s.segs, n_segs * sizeof(PartSegment))) ||
+        (rc = temp((void**)&s.seg_base, most_buckets * sizeof(unsigned))))
+      return rc;
+    s.fill = zero;
+    s.over_n = zero + n_subs;
+    s.n_keys = zero + n_subs + 1;
+    s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 2);
+    s.n_chunks = (unsigned)n_chunks;
+    const double occ = std::min(1.0, std::max(0.3, positions > 0 ? windows / positions : 1.0));
+    s.log_lanes = lanes_for(kPartTile * occ / B);
+    for (size_t i = 0; i < ends.size(); ++i) {
+      s.b0 = i ? ends[i - 1] : 0;
+      s.b1 = ends[i];
+      KMA_CUDA(cudaMemsetAsync(zero, 0, n_zero * 8, st));
+      if ((rc = timed_launch(timed, KMA_KERNEL_SCATTER, st, true,
+                             [&] { return launch_part_base(h->totals, s, st); })))
+        return rc;
+      for (size_t j = 0; j < h->slabs.size(); ++j) {
+        const PartTiles t = tiles_of(h, h->slabs[j], 0);
+        s.chunk_tiles = chunk_tiles[j];
+        if ((rc = timed_launch(timed, KMA_KERNEL_SCATTER, st, t.n_tiles > 0,
+                               [&] { return launch_part_split(g, t, s, st, h->num_sms); })))
+          return rc;
+      }
+      if ((rc = timed_launch(timed, KMA_KERNEL_PASS, st, true,
+                             [&] { return launch_part_count(g, s, st, h->num_sms); })) ||
+          (rc = timed_launch(timed, KMA_KERNEL_RECOUNT, st, true,
+                             [&] { return launch_part_insert(g, s, st, h->num_sms); })))
+        return rc;
+      if ((rc = after(s.b1))) return rc;
+    }
+    return KMA_OK;
+  };
+  const int rc = run();
+  for (void* t : temps) cudaFreeAsync(t, st);
+  return rc;
 }
 
 // First pass over the windows [q0, q0 + n_pos) of one packed batch (n_reads reads, n_bases
 // bases) on stream `st`. One table: Bloom test-and-set (or counting) in place. Partitions:
-// scatter into per-partition record buckets, then the record pass part by part; the buckets
-// are kept for the recount in finalize. Nothing here waits for the GPU.
+// scatter into tiles, which finalize counts. Nothing here waits for the GPU.
 int first_pass(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, cudaStream_t st) {
   const unsigned mode = h->p.use_bloom ? kModeBloom : kModeCount;
   if (h->d.P <= 1) {
@@ -665,10 +763,8 @@ int first_pass(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, cudaS
     return timed_launch(h, KMA_KERNEL_PASS, st, b.total_tiles > 0,
                         [&] { return launch_pass(b, h->shape, h->agg, st); });
   }
-  size_t index = 0;
-  int rc = prepare_records(h, n_pos, n_reads, n_bases, st, index);
-  if (rc || (rc = scatter_windows(h, index, q0, n_pos, st))) return rc;
-  return n_pos ? record_pass(h, index, st) : KMA_OK;
+  int rc = prepare_tiles(h, tiles_for(n_pos), st);
+  return rc ? rc : scatter_windows(h, q0, n_pos, n_reads, n_bases, st);
 }
 
 int run_pack_and_pass(kma_handle* h, const PackDesc& pd) {
@@ -775,7 +871,8 @@ int kmer_analysis_create(const kma_params* params, void* cuda_stream, kma_handle
   if ((rc = dalloc(h, &h->codes, d.codes_words)) || (rc = dalloc(h, &h->rcodes, d.codes_words)) ||
       (rc = dalloc(h, &h->inv, d.bit_words)) ||
       (rc = dalloc(h, &h->hq, d.bit_words)) || (rc = dalloc(h, &h->marks, d.mark_words)) ||
-      (rc = dalloc(h, &h->bloom, d.plan.bloom_words)) || (rc = dalloc(h, &h->keyfilter, d.Wt * d.P)) ||
+      (rc = dalloc(h, &h->bloom, d.P > 1 ? 0 : d.plan.bloom_words)) ||
+      (rc = dalloc(h, &h->totals, d.P > 1 ? 1ull << d.log_b : 0)) ||
       (rc = dalloc(h, &h->table, d.plan.table_slots)) || (rc = dalloc(h, &h->status, 1))) {
     free_all(h);
     delete h;
@@ -856,18 +953,15 @@ int kmer_analysis_count(kma_handle* h, const char* seq, const char* qual, const 
   if (!offsets_nondecreasing(offsets, n_reads)) return KMA_EINVAL;
   if (offsets[n_reads] - offsets[0] + h->bases_used > h->p.max_bases) return KMA_EFULL;
   if ((rc = setup_staging(h))) return rc;
-  // With partitions, every staged chunk is packed and scattered into one set of record buckets
-  // (so the copy of the next chunk overlaps both), and the record pass runs once over all of
-  // them: a pass per chunk would bring every partition's filter and table back into L2 once
-  // per chunk.
+  // With partitions, every staged chunk is packed and scattered, so the copy of the next chunk
+  // overlaps both.
   const bool parts = h->d.P > 1 && !h->pack_only;
-  size_t rec_index = 0;
   if (parts) {
-    // positions of the whole call: every chunk is rounded up to 64 positions, and a chunk
-    // ends only when the next read would overflow the staged bases or read offsets
+    // tiles of the whole call: every chunk starts a tile, and a chunk ends only when the next
+    // read would overflow the staged bases or read offsets
     const u64 nb_all = offsets[n_reads] - offsets[0];
     const u64 chunks = 2 * (nb_all / h->d.staging + n_reads / (h->stage_offs_cap - 1) + 1);
-    if ((rc = prepare_records(h, nb_all + n_reads + 64 * chunks, n_reads, nb_all, h->stream, rec_index))) return rc;
+    if ((rc = prepare_tiles(h, tiles_for(nb_all + n_reads + 64 * chunks) + chunks, h->stream))) return rc;
   }
   u64 r0 = 0;
   while (r0 < n_reads) {
@@ -901,21 +995,21 @@ int kmer_analysis_count(kma_handle* h, const char* seq, const char* qual, const 
       return rc;
     KMA_CUDA(cudaEventRecord(h->consumed[b], h->stream));
     if (parts) {
-      if ((rc = scatter_windows(h, rec_index, q0, n_pos, h->stream))) return rc;
+      if ((rc = scatter_windows(h, q0, n_pos, r1 - r0, nb, h->stream))) return rc;
     } else if (!h->pack_only && (rc = first_pass(h, q0, n_pos, r1 - r0, nb, h->stream))) {
       return rc;
     }
     r0 = r1;
   }
-  if (parts && (rc = record_pass(h, rec_index, h->stream))) return rc;
   // Host buffers may be reused once the call returns: wait for the copies.
   KMA_CUDA(cudaStreamSynchronize(h->copy_stream));
   return KMA_OK;
 }
 
-// Recount pass (first sightings) of the Bloom handles: one launch for all one-table handles,
-// one per record batch of the partitioned ones. Enqueued on h0's stream.
-static int enqueue_recount(kma_handle* const* hs, uint32_t n) {
+// What is left of the counting: one launch of the recount (first sightings) for all one-table
+// Bloom handles, and the records of the partitioned ones. Enqueued on h0's stream; may_sync:
+// see count_records.
+static int enqueue_recount(kma_handle* const* hs, uint32_t n, bool may_sync) {
   kma_handle* h0 = hs[0];
   PassBatch pb;
   std::memset(&pb, 0, sizeof(pb));
@@ -934,25 +1028,16 @@ static int enqueue_recount(kma_handle* const* hs, uint32_t n) {
   int rc = timed_launch(h0, KMA_KERNEL_RECOUNT, h0->stream, pb.n > 0 && tiles > 0,
                         [&] { return launch_pass(pb, h0->shape, h0->agg, h0->stream); });
   if (rc) return rc;
-  for (uint32_t i = 0; i < n; ++i) {  // partitioned handles: recount their record buckets
+  for (uint32_t i = 0; i < n; ++i) {
     kma_handle* h = hs[i];
-    if (!h->p.use_bloom || h->d.P <= 1) continue;
-    const PartGeom g = part_geom(h);
-    rc = timed_launch(h0, KMA_KERNEL_RECOUNT, h0->stream, g.Wk > 0,
-                      [&] { return launch_keyfilter_build(g, h0->stream, h0->num_sms); });
-    if (rc) return rc;
-    for (auto& rb : h->rec_batches) {
-      const PartRecords r = records_of(rb, h->d.P);
-      rc = timed_launch(h0, KMA_KERNEL_RECOUNT, h0->stream, true,
-                        [&] { return launch_part_pass(g, r, kModeRecount, h0->stream, h0->num_sms); });
-      if (rc) return rc;
-    }
+    if (h->d.P <= 1) continue;
+    if ((rc = count_records(h, h0, h0->stream, may_sync, 1, [](unsigned) { return (int)KMA_OK; }))) return rc;
   }
   return KMA_OK;
 }
 
 // Classification + compaction of the handles with ok[i] into their current output buffers,
-// one launch; then their record buckets are released. Enqueued on h0's stream.
+// one launch; then their records are released. Enqueued on h0's stream.
 static int enqueue_classify(kma_handle* const* hs, uint32_t n, const std::vector<int>& ok) {
   kma_handle* h0 = hs[0];
   for (uint32_t i = 0; i < n; ++i)
@@ -972,7 +1057,7 @@ static int enqueue_classify(kma_handle* const* hs, uint32_t n, const std::vector
   int rc = timed_launch(h0, KMA_KERNEL_CLASSIFY, h0->stream, cb.n > 0 && blocks > 0,
                         [&] { return launch_classify(cb, h0->stream, h0->num_sms); });
   if (rc) return rc;
-  for (uint32_t i = 0; i < n; ++i) {  // the record buckets are not needed after the recount
+  for (uint32_t i = 0; i < n; ++i) {  // the records are not needed any more
     cudaStream_t saved = hs[i]->stream;
     hs[i]->stream = h0->stream;
     free_records(hs[i]);
@@ -1007,7 +1092,7 @@ static int finalize_many(kma_handle* const* hs, uint32_t n, kma_result* out) {
       if (e != cudaSuccess) return cuda_fail(e, "stream ordering");
     }
   }
-  if ((rc = enqueue_recount(hs, n))) return rc;
+  if ((rc = enqueue_recount(hs, n, true))) return rc;
   // statuses -> output capacities (table_keys bounds the records)
   for (uint32_t i = 0; i < n; ++i)
     KMA_CUDA(cudaMemcpyAsync(hs[i]->host_status, hs[i]->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, h0->stream));
@@ -1061,7 +1146,7 @@ int kmer_analysis_finalize_batch_async(kma_handle* const* hs, uint32_t n) {
   if (rc) return rc;
   for (uint32_t i = 0; i < n; ++i)
     if (!hs[i]->out_keys) return KMA_ESTATE;  // kmer_analysis_reserve_output first
-  if ((rc = enqueue_recount(hs, n))) return rc;
+  if ((rc = enqueue_recount(hs, n, false))) return rc;
   std::vector<int> ok(n, 1);
   if ((rc = enqueue_classify(hs, n, ok))) return rc;
   for (uint32_t i = 0; i < n; ++i) hs[i]->finalized = true;
@@ -1115,7 +1200,7 @@ int kmer_analysis_count_batch(kma_handle* const* hs, const kma_reads* reads, uin
     pd.chunk_begin = words;
     words += (n_pos / 64 + kPackChunkWords - 1) / kPackChunkWords;
     pk.d[pk.n++] = pd;
-    if (h->d.P > 1) {  // partitioned: its own histogram/scatter/record pass after the packing
+    if (h->d.P > 1) {  // partitioned: its own scatter after the packing
       part_later.push_back({h, q0, n_pos, reads[i].n_reads, reads[i].n_bases});
       continue;
     }
@@ -1165,58 +1250,20 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
     for (auto& e : h->group_ev) KMA_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   }
   if (!h->copy_stream) KMA_CUDA(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
-  // Everything counted so far: the keys in the table bound the records.
+  const bool parts = h->d.P > 1;
+  const u64 S = h->d.plan.table_slots;
+  // One table: the keys counted so far bound the records. Partitions: nothing is in the table
+  // yet; room for as many records as the caller has room for (more of them: classified again
+  // below).
   int rc = read_status(h);
   if (rc) return rc;
   if ((rc = flags_to_code(h->host_status->flags))) { h->failed = true; return rc; }
-  if ((rc = ensure_output(h, h->host_status->table_keys))) { h->failed = true; return rc; }
+  if ((rc = ensure_output(h, parts ? std::min<u64>(capacity, S) : h->host_status->table_keys))) { h->failed = true; return rc; }
   KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
-  const bool parts = h->d.P > 1;
-  const bool recount_parts = parts && h->p.use_bloom;
-  const u64 S = h->d.plan.table_slots;
   const unsigned G = (unsigned)std::max<u64>(1, std::min<u64>(kFinalizeGroups, parts ? h->d.P : S / kClassTile));
-  const PartGeom g = part_geom(h);
-  // What the groups do not split: the one-table recount (a pass over the windows), or the
-  // overflow records of every partition.
-  if (h->p.use_bloom && !parts) {
-    kma_handle* hs[1] = {h};
-    if ((rc = enqueue_recount(hs, 1))) return rc;
-  }
-  if (recount_parts) {
-    if ((rc = timed_launch(h, KMA_KERNEL_RECOUNT, h->stream, g.Wk > 0,
-                           [&] { return launch_keyfilter_build(g, h->stream, h->num_sms); })))
-      return rc;
-    for (auto& rb : h->rec_batches) {
-      PartRecords r = records_of(rb, h->d.P);
-      r.p_end = 0;  // overflow area only
-      if ((rc = timed_launch(h, KMA_KERNEL_RECOUNT, h->stream, true,
-                             [&] { return launch_part_pass(g, r, kModeRecount, h->stream, h->num_sms); })))
-        return rc;
-    }
-  }
-  // Per group: recount its partitions, classify its slots (the records append to the output),
-  // publish the record count so far.
-  for (unsigned i = 0; i < G; ++i) {
-    u64 s0, s1;
-    if (parts) {
-      const u64 p0 = h->d.P * i / G, p1 = h->d.P * (i + 1) / G;
-      s0 = p0 * h->d.Sp;
-      s1 = p1 * h->d.Sp;
-      if (recount_parts) {
-        for (auto& rb : h->rec_batches) {
-          PartRecords r = records_of(rb, h->d.P);
-          r.p_begin = (unsigned)p0;
-          r.p_end = (unsigned)p1;
-          r.overflow = 0;
-          if ((rc = timed_launch(h, KMA_KERNEL_RECOUNT, h->stream, p1 > p0,
-                                 [&] { return launch_part_pass(g, r, kModeRecount, h->stream, h->num_sms); })))
-            return rc;
-        }
-      }
-    } else {
-      s0 = S * i / G;
-      s1 = S * (i + 1) / G;
-    }
+  unsigned published = 0;  // groups whose records have been appended to the output
+  // Classify the table slots [s0, s1) and publish the record count so far.
+  auto publish = [&](u64 s0, u64 s1) -> int {
     ClassBatch cb;
     std::memset(&cb, 0, sizeof(cb));
     cb.write = 1;
@@ -1225,18 +1272,42 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
     cb.d[0].table = h->table + s0;
     cb.d[0].slots = s1 - s0;
     cb.total_blocks = (s1 - s0 + kClassTile - 1) / kClassTile;
-    if ((rc = timed_launch(h, KMA_KERNEL_CLASSIFY, h->stream, cb.total_blocks > 0,
-                           [&] { return launch_classify(cb, h->stream, h->num_sms); })))
-      return rc;
-    KMA_CUDA(cudaMemcpyAsync(&h->host_groups[i], &h->status->n_out, sizeof(u64), cudaMemcpyDeviceToHost, h->stream));
-    KMA_CUDA(cudaEventRecord(h->group_ev[i], h->stream));
+    int rc2 = timed_launch(h, KMA_KERNEL_CLASSIFY, h->stream, cb.total_blocks > 0,
+                           [&] { return launch_classify(cb, h->stream, h->num_sms); });
+    if (rc2) return rc2;
+    KMA_CUDA(cudaMemcpyAsync(&h->host_groups[published], &h->status->n_out, sizeof(u64), cudaMemcpyDeviceToHost, h->stream));
+    KMA_CUDA(cudaEventRecord(h->group_ev[published], h->stream));
+    ++published;
+    return KMA_OK;
+  };
+  if (!parts) {
+    // the recount is a pass over the windows: the groups only split the classification
+    if (h->p.use_bloom) {
+      kma_handle* hs[1] = {h};
+      if ((rc = enqueue_recount(hs, 1, true))) return rc;
+    }
+    for (unsigned i = 0; i < G; ++i)
+      if ((rc = publish(S * i / G, S * (i + 1) / G))) return rc;
+  } else {
+    // Buckets and partitions are ranges of the same hash: with the buckets below `end` counted,
+    // the partitions below end * P / B are complete.
+    const unsigned B = 1u << h->d.log_b;
+    u64 p0 = 0;
+    rc = count_records(h, h, h->stream, true, G, [&](unsigned end) -> int {
+      const u64 p1 = (u64)end * h->d.P / B;
+      if (end != B && (p1 == p0 || (u64)end * G / B <= published)) return KMA_OK;
+      const u64 from = p0;
+      p0 = p1;
+      return publish(from * h->d.Sp, p1 * h->d.Sp);
+    });
+    if (rc) return rc;
   }
   KMA_CUDA(cudaMemcpyAsync(h->host_status, h->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, h->stream));
   // As each group completes, its records go to the host on the copy stream while the GPU
-  // recounts the next group.
+  // counts the next group.
   const u64 cap = std::min<u64>(capacity, h->out_cap);
   u64 done = 0;
-  for (unsigned i = 0; i < G; ++i) {
+  for (unsigned i = 0; i < published; ++i) {
     KMA_CUDA(cudaEventSynchronize(h->group_ev[i]));
     const u64 upto = std::min<u64>(h->host_groups[i], cap);
     if (upto <= done) continue;
@@ -1251,6 +1322,15 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
   free_records(h);
   KMA_CUDA(cudaStreamSynchronize(h->stream));
   KMA_CUDA(cudaStreamSynchronize(h->copy_stream));
+  if (h->host_status->n_out > h->out_cap && !(h->host_status->flags & ~kFlagOutput)) {
+    // more records than the caller (and so the device output) has room for: all of them into a
+    // larger device output; the host has the first `capacity` of the same set
+    if ((rc = ensure_output(h, h->host_status->n_out))) { h->failed = true; return rc; }
+    KMA_CUDA(cudaMemsetAsync(&h->status->flags, 0, sizeof(h->status->flags), h->stream));
+    KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
+    published = 0;
+    if ((rc = publish(0, S)) || (rc = read_status(h))) { h->failed = true; return rc; }
+  }
   if ((rc = flags_to_code(h->host_status->flags))) {
     h->failed = true;
     if (out) std::memset(out, 0, sizeof(kma_result));
@@ -1368,7 +1448,7 @@ int kmer_analysis_contigs(kma_handle* h, kma_contigs* out) {
   if (rc) return rc;
   int st = read_status(h);
   if (st) return st;
-  if (h->host_status->flags & kFlagFull) return KMA_EFULL;
+  if (h->host_status->flags & (kFlagFull | kFlagOutput)) return KMA_EFULL;
   out->n_contigs = h->contig_n;
   out->n_bases = h->contig_bases;
   out->n_vertices = h->contig_vertices;

@@ -75,51 +75,6 @@ __device__ __forceinline__ u64 bloom_mask(u64 h, unsigned nbits) {
   return mask_from_fields((h ^ (h >> 32)) * 0xd6e8feb86659fd93ull, nbits);
 }
 
-// Key filter (partitioned recount): one 64-bit word per key, chosen by the low half of
-// h * phi (the table slot uses its high half), bits from the top of (h ^ h >> 32) * c' with a
-// multiplier of its own.
-__device__ __forceinline__ u64 keyfilter_index(u64 h, u64 words) {
-  return __umulhi((unsigned)scramble(h), (unsigned)words);
-}
-__device__ __forceinline__ u64 keyfilter_mask(u64 h, unsigned nbits) {
-  return mask_from_fields((h ^ (h >> 32)) * 0x94d049bb133111ebull, nbits);
-}
-
-// L2 cache policy for data read or written once (record streams): evict first, so the
-// partition's Bloom sub-filter and sub-table stay resident.
-__device__ __forceinline__ u64 policy_evict_first() {
-  u64 pol;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-  return pol;
-}
-__device__ __forceinline__ ulonglong2 ld_stream(const ulonglong2* p, u64 pol) {
-  ulonglong2 v;
-  asm volatile("ld.global.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
-               : "=l"(v.x), "=l"(v.y) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ u64 ld_stream(const u64* p, u64 pol) {
-  u64 v;
-  asm volatile("ld.global.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ unsigned ld_stream(const unsigned char* p, u64 pol) {
-  unsigned v;
-  asm volatile("ld.global.L2::cache_hint.u8 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ void st_stream(ulonglong2* p, ulonglong2 v, u64 pol) {
-  asm volatile("st.global.L2::cache_hint.v2.u64 [%0], {%1, %2}, %3;" ::"l"(p), "l"(v.x), "l"(v.y), "l"(pol)
-               : "memory");
-}
-__device__ __forceinline__ void st_stream(u64* p, u64 v, u64 pol) {
-  asm volatile("st.global.L2::cache_hint.u64 [%0], %1, %2;" ::"l"(p), "l"(v), "l"(pol) : "memory");
-}
-__device__ __forceinline__ void st_stream(unsigned char* p, unsigned v, u64 pol) {
-  asm volatile("st.global.L2::cache_hint.u8 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(pol) : "memory");
-}
-
-
 // ------------------------------------------------------------------ bulk copies (TMA)
 
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
@@ -140,14 +95,6 @@ __device__ __forceinline__ void mbar_expect_tx(unsigned bar, unsigned bytes) {
 __device__ __forceinline__ void tma_load_1d(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
-// The same copy with an L2 cache policy (evict-first for streams read once).
-__device__ __forceinline__ void tma_load_1d_hint(unsigned dst, const void* src, unsigned bytes, unsigned bar,
-                                                 u64 pol) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-      ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(pol) : "memory");
 }
 
 // Orders this thread's earlier generic-proxy accesses to shared memory before later bulk

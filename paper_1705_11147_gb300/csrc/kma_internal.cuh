@@ -37,6 +37,7 @@ constexpr uint32_t kFlagFull = 1u;
 constexpr uint32_t kFlagOverflow = 2u;
 constexpr uint32_t kFlagBadOffsets = 4u;
 constexpr uint32_t kFlagTimeout = 8u;     // a bounded device wait gave up
+constexpr uint32_t kFlagOutput = 16u;     // more records than the output arrays hold
 
 // One hash-table slot. Every occurrence has exactly one left outcome (a usable base A/C/G/T
 // or none) and one right outcome, so the slot keeps five counters per side and no separate
@@ -151,35 +152,37 @@ struct ClassBatch {
 };
 
 // ---- Partitioned mode ("owner-computes on chip", Section 5.1's k-mer -> owner map) -------
-// The k-mer space is split by a hash into P partitions; partition p owns Bloom words
-// [p*Wp, (p+1)*Wp) and table slots [p*Sp, (p+1)*Sp). Windows are first scattered into
-// per-partition record buckets (streaming writes), then the buckets are processed in order,
-// so the random Bloom/table traffic of one partition stays in L2.
+// The k-mer space is split by the key hash twice: 2^log_b buckets (its top bits), then up to
+// sub_max sub-buckets of each, small enough to be counted in one SM's shared memory
+// (kma_partition.cu). The table is laid out in P partitions by the same hash: partition p owns
+// slots [p*Sp, (p+1)*Sp), so the keys of one bucket go to one or two partitions.
 constexpr unsigned kMaxPartitions = 4096;      // k <= 32 (one-word keys)
-constexpr unsigned kMaxPartitionsWide = 2048;  // k > 32: the scatter's staged tile is larger
+constexpr unsigned kMaxPartitionsWide = 2048;  // k > 32
 
-// Record info byte: bits 0-1 left base, bit 2 left usable, bits 3-4 right base,
-// bit 5 right usable, bit 7 first sighting (set by the Bloom pass).
-constexpr unsigned char kInfoFirst = 0x80;
+constexpr unsigned kMinLogBuckets = 6;         // the record's outcome bits take the place of 6 hash bits
+constexpr unsigned kMaxLogBuckets = 11;
+constexpr unsigned kMaxSubBuckets = 2048;
+constexpr unsigned kPartTile = 8192;           // window starts (and records, at most) per scatter tile
+constexpr unsigned kPartSubTile = 4096;        // records per sub-tile of the split
+constexpr unsigned kMaxChunkTiles = 1024;      // scatter tiles gathered together by the split
+constexpr unsigned kSplitBuckets = 8;          // adjacent buckets per work item of the split
+constexpr unsigned kCountCap1 = 3072;          // records of a sub-bucket counted in one go (k <= 32)
+constexpr unsigned kCountCap2 = 2304;          // (k > 32)
 
 struct PartGeom {
-  unsigned long long* bloom;
   Slot* table;
   DevStatus* status;
-  unsigned long long* keyfilter;  // Bloom mode: blocked Bloom filter of the keys in the table
-  unsigned long long Wp;        // Bloom words per partition
   unsigned long long Sp;        // table slots per partition
-  unsigned long long Wk;        // key-filter words per partition (0: no key filter)
   unsigned int P;
-  unsigned int bloom_h;
   unsigned int k;
   unsigned int canonical;
   unsigned int n_parts;         // multi-GPU owner filter (as PassDesc)
   unsigned int part;
-  unsigned int rpt;             // records per thread in flight in the record passes (2 or 4)
-  unsigned int wait_limit;      // polls of the bounded wait for a staged record tile
-  unsigned int no_overflow;     // 1: no count can reach 2^32 (host bound), counts use red.add
-  unsigned int group;           // 1: group equal keys within a warp (heavy hitters)
+  unsigned int log_b;           // log2 of the buckets
+  unsigned int sub_max;         // most sub-buckets per bucket
+  unsigned int avg;             // records per sub-bucket aimed at
+  unsigned int cap;             // records a sub-bucket has room for
+  unsigned int min_count;       // a key reaches the table with at least this many occurrences (1 or 2)
 };
 
 struct PartWindows {
@@ -190,34 +193,49 @@ struct PartWindows {
   unsigned long long q0, q1;    // window starts of one count() batch (multiples of 64)
 };
 
-// Record buckets of one count() batch: P buckets of `cap` records (bucket p starts at p*cap),
-// then an overflow area of `ocap` records for partitions whose bucket filled up. cap and ocap
-// are multiples of 16 and both arrays 16-byte aligned, so every tile of the record passes
-// starts on a 16-byte boundary and may be staged with 1-D bulk copies rounded up to 16
-// records without leaving its bucket (or the overflow area). fill[p]
-// counts the records that were assigned to bucket p (those beyond cap went to the overflow
-// area); fill[P] counts the overflow records.
-// The record passes hand out their tiles (32 * rpt records, in bucket order) from a queue:
-// `queue` counts the chunks of tiles taken so far and is zeroed before every launch.
-struct PartRecords {
-  void* keys;                   // unsigned long long[] (k <= 32) or ulonglong2[]
-  unsigned char* info;
-  unsigned long long cap;       // records per bucket
-  unsigned long long ocap;      // overflow records
-  unsigned long long* fill;     // [P + 1]
-  unsigned* queue;              // record passes: chunks of tiles handed out so far
-  // record passes: the buckets of partitions [p_begin, p_end), then the overflow area if
-  // `overflow` (the whole batch: 0, P, 1); the scatter ignores these
-  unsigned int p_begin, p_end;
-  unsigned int overflow, pad;
+// Scatter tiles: tile i holds its records, sorted by bucket, from recs + i * kPartTile records on;
+// row i of offs (stride entries) holds the buckets' first records and, at [2^log_b], their number.
+struct PartTiles {
+  unsigned long long* recs;     // one word per record (k <= 32) or two
+  unsigned short* offs;
+  unsigned long long* totals;   // [2^log_b] records per bucket (added to by the scatter)
+  unsigned long long tile0;     // scatter: first tile of this launch
+  unsigned int n_tiles;         // split: tiles to gather from
+  unsigned int stride;
 };
 
-cudaError_t launch_part_scatter(const PartGeom& g, const PartWindows& w, const PartRecords& r,
-                                cudaStream_t stream, int num_sms);
-cudaError_t launch_part_pass(const PartGeom& g, const PartRecords& r, unsigned mode,
-                             cudaStream_t stream, int num_sms);
-// Key filter of the recount: set by every key in the table (after the Bloom pass).
-cudaError_t launch_keyfilter_build(const PartGeom& g, cudaStream_t stream, int num_sms);
+// Split output for the buckets [b0, b1): sub-bucket s of bucket b has the G.cap places from
+// recs[((b - b0) * n_sub + s) * cap] on, and fill[(b - b0) * n_sub + s] records; those beyond cap
+// lie in the bucket's overflow segments, over[pos .. pos + n) each.
+struct PartSegment {
+  unsigned long long pos;
+  unsigned int n, pad;
+};
+struct PartSplit {
+  unsigned long long* recs;
+  unsigned long long* fill;     // starts at 0
+  unsigned long long* over;     // room for all records of the buckets
+  unsigned long long* over_n;   // records in it; starts at 0
+  PartSegment* segs;            // the buckets' segments, bucket b's from seg_base[b - b0] on
+  unsigned int* seg_base;       // [b1 - b0]
+  unsigned int* n_segs;         // [b1 - b0], starts at 0
+  unsigned int b0, b1;
+  unsigned int n_chunks;        // chunks of all record slabs
+  unsigned int chunk_tiles;     // tiles per chunk
+  unsigned int log_lanes;       // lanes per gathered run (log2)
+  unsigned int pad;
+  unsigned int* keys;           // count: the counted keys for the table (kma_partition.cu)
+  unsigned long long* n_keys;   // their number; starts at 0
+};
+
+cudaError_t launch_part_scatter(const PartGeom& g, const PartWindows& w, const PartTiles& t, cudaStream_t stream,
+                                int num_sms);
+cudaError_t launch_part_base(const unsigned long long* totals, const PartSplit& s, cudaStream_t stream);
+cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartSplit& s, cudaStream_t stream,
+                              int num_sms);
+cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
+cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
+constexpr unsigned kMaxKeyWords = 9;           // words of one counted key in the list
 
 // FASTQ parsing (kma_fastq.cu) and the device-wide exclusive scan it uses.
 unsigned long long scan_scratch_items(unsigned long long n);

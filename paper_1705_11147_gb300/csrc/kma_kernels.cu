@@ -565,7 +565,7 @@ __global__ void __launch_bounds__(kClassThreads) classify_kernel(const __grid_co
         reinterpret_cast<uint4*>(D.out_ext)[2 * pos + 1] = e1;
         reinterpret_cast<uchar2*>(D.out_codes)[pos] = make_uchar2((unsigned char)lc, (unsigned char)rc);
       } else {
-        atomicOr(&D.status->flags, kFlagFull);
+        atomicOr(&D.status->flags, kFlagOutput);
       }
       ++pos;
     }

@@ -1,16 +1,23 @@
-// Partitioned mode of the counting passes: the paper's owner-computes scheme (Section 5.1:
-// a deterministic k-mer -> owner map, every owner counting in a local table behind its own
-// Bloom filter) applied on one GPU, with L2-sized partitions as the owners.
+// Partitioned mode of the counting passes: the paper's owner-computes scheme (Section 5.1: a
+// deterministic k-mer -> owner map, every owner counting in a table of its own) applied on one
+// GPU, with owners small enough to count in one SM's shared memory.
 //
-//   part_scatter_kernel  each window becomes a record {canonical key, extension info byte},
-//                        appended to its partition's bucket (streaming writes); buckets
-//                        have a fixed capacity and spill into a shared overflow area
-//   part_pass_kernel     buckets processed in order: Bloom test-and-set in the partition's
-//                        sub-filter, insert/count in its sub-table, or (recount) the first
-//                        sightings added to k-mers that reached the table
+//   part_scatter_kernel  every window becomes a record (key hash, rest of the key, extension
+//                        outcomes); each tile of 8192 window starts is sorted by bucket (the top
+//                        bits of the key hash) in shared memory and written out as it lies, with
+//                        a row of bucket offsets
+//   part_split_kernel    gathers a bucket's runs from many scatter tiles, sorts them by sub-bucket
+//                        (the next part of the hash) and writes them the same way
+//   part_count_kernel    gathers a sub-bucket's runs into shared memory: all occurrences of a few
+//                        hundred to a few thousand k-mers, counted there; only k-mers seen at
+//                        least twice (every k-mer without the singleton filter) go to the table
+//                        in HBM, each inserted once with its final counters
 //
-// The random atomics of one partition touch only its sub-filter and sub-table, sized to stay
-// resident in L2, instead of the whole multi-GB filter and table in HBM.
+// Why two sorts and no filter in front of the table: a Bloom test-and-set plus table atomics in
+// L2 took 4.6 L2 requests per window, 21 ns per 1000 windows, and a second pass over the first
+// sightings another 8 ns. A sort pass reads and writes 16 bytes per window in whole lines, and
+// with all occurrences of a k-mer in one shared memory the singletons (error k-mers) are known
+// exactly, so they cost no memory traffic outside the SM.
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -19,83 +26,130 @@
 
 namespace kma {
 
+// ------------------------------------------------------------------ records
+//
+// A record keeps the key in hashed form: h = key_hash(lo, hi) is a bijection of lo for a given
+// hi, so (h, hi) identifies the key and lo is recomputed only for the k-mers that reach the
+// table. The top kInfoBits of h are implied by the bucket (at least 2^6 buckets) and make room
+// for the two extension outcomes. 8 bytes for k <= 32 (hi = 0), 16 above.
+//   word 0   left outcome (bits 58..60: 0-3 base, 4 none) | right outcome (61..63) | h bits 0..57
+//   word 1   hi (k > 32)
 
-__device__ __forceinline__ unsigned char info_of(const Window& w) {
-  return (unsigned char)(w.lb | ((unsigned)w.lu << 2) | (w.rb << 3) | ((unsigned)w.ru << 5));
+constexpr unsigned kInfoBits = 6;
+constexpr u64 kHashMask = (1ull << (64 - kInfoBits)) - 1;
+
+__device__ __forceinline__ unsigned left_outcome(u64 r) { return (unsigned)(r >> 58) & 7u; }
+__device__ __forceinline__ unsigned right_outcome(u64 r) { return (unsigned)(r >> 61); }
+
+__device__ __forceinline__ u64 unxorshift33(u64 x) { return x ^ (x >> 33); }
+// Inverse of key_hash in lo: fmix64 backwards (its shifts are involutions, its multipliers odd,
+// the constants are their inverses modulo 2^64).
+__device__ __forceinline__ u64 key_lo(u64 h, u64 hi) {
+  u64 x = unxorshift33(h) * 0x9cb4b2f8129337dbull;
+  x = unxorshift33(x) * 0x4f74430c22a54005ull;
+  return unxorshift33(x) ^ (hi * 0x9e3779b97f4a7c15ull + 0x632be59bd9b4e019ull);
 }
 
-__device__ __forceinline__ void window_of(unsigned char inf, Window& w) {
-  w.lb = inf & 3u;
-  w.lu = (inf >> 2) & 1u;
-  w.rb = (inf >> 3) & 3u;
-  w.ru = (inf >> 5) & 1u;
+// Sub-bucket of a record inside its bucket: the 32 hash bits after the bucket's, scaled to n.
+__device__ __forceinline__ unsigned sub_of(u64 r, unsigned log_b, unsigned n) {
+  return __umulhi((unsigned)((r << log_b) >> 32), n);
 }
 
-constexpr int kPartThreads = 256;
+// Sub-buckets per bucket, from the windows counted so far (the same value in every kernel of
+// one finalize): `avg` records each on average.
+__device__ __forceinline__ unsigned sub_buckets(const PartGeom& G) {
+  const u64 per = (u64)G.avg << G.log_b;
+  const u64 n = (__ldcg(&G.status->valid_windows) + per - 1) / per;
+  return n < 1 ? 1u : n > G.sub_max ? G.sub_max : (unsigned)n;
+}
+
+// ------------------------------------------------------------------ small block helpers
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(unsigned dst, const void* src) {
+  if (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// 1-D bulk copy shared -> global (16-byte aligned, a multiple of 16 bytes).
+__device__ __forceinline__ void tma_store_1d(void* dst, unsigned src, unsigned bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// Until the committed stores have read their shared memory / are complete.
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void tma_store_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// Exclusive scan of one value per thread over the block; `total` is the block's sum. wsum: one
+// word per warp (32). One block barrier inside, after which wsum may be read by other warps: a
+// second call needs a barrier in between.
+template <int THREADS>
+__device__ __forceinline__ unsigned block_scan(unsigned v, unsigned* wsum, unsigned& total) {
+  constexpr int kWarps = THREADS / 32;
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned incl = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= (unsigned)o) incl += x;
+  }
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  const unsigned ws = lane < kWarps ? wsum[lane] : 0u;
+  unsigned wi = ws;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned x = __shfl_up_sync(0xffffffffu, wi, o);
+    if (lane >= (unsigned)o) wi += x;
+  }
+  total = __shfl_sync(0xffffffffu, wi, 31);
+  return __shfl_sync(0xffffffffu, wi - ws, warp) + incl - v;
+}
 
 // ------------------------------------------------------------------ scatter
 //
-// One tile = kScatterThreads * kScatterWpt consecutive window starts; thread t takes the
-// kScatterWpt consecutive starts t * kScatterWpt + j.
+// One tile = 8192 consecutive window starts; thread t takes the kScatterWpt consecutive starts
+// t * kScatterWpt + j.
 //  1. extract the windows (one set of word loads per thread, then the forward k-mer and its
-//     reverse complement are rolled one base at a time), stage key + info in shared memory,
-//     rank each window inside its partition for this tile (shared-memory atomics);
-//  2. thread t owns a contiguous chunk of partitions: it reserves each present partition's
-//     run in the bucket (one global atomic, bucket first, the rest in the overflow area) and,
-//     while those atomics are in flight, takes part in the exclusive scan of the counts that
-//     sorts the tile's records by partition;
-//  3. permute the staged records into partition order and write them out: consecutive
-//     threads write consecutive records of the same bucket, so the stores coalesce.
-// A CTA of 512 threads with its 4096-window tile leaves room for two CTAs per SM (with up to
-// about a thousand partitions), so one CTA's block barriers and reservation round trips
-// overlap the other's extraction and stores.
+//     reverse complement are rolled one base at a time), stage the records in shared memory,
+//     rank each inside its bucket for this tile (shared-memory atomics);
+//  2. exclusive scan of the bucket counts: the tile's offset row;
+//  3. the staged records into bucket order (through registers, in place), and the sorted tile to
+//     HBM with bulk copies.
+// The tile keeps a fixed place (tile number * 8192 records), so nothing is reserved: no global
+// atomics, no bucket capacities and no overflow, whatever the skew of the keys.
 
 constexpr int kScatterThreads = 1024;
 constexpr int kScatterWpt = 8;
-constexpr int kScatterTile = kScatterThreads * kScatterWpt;  // 4096: ranks and slots < 2^12
-constexpr int kScatterMaxChunk = 4;                          // partitions per thread (4096 / 512)
+constexpr int kScatterTile = kScatterThreads * kScatterWpt;
+static_assert(kScatterTile == kPartTile && kScatterTile <= 8192, "ranks are 13 bits");
+constexpr int kScatterMaxPer = (1 << kMaxLogBuckets) / kScatterThreads;  // buckets per thread
 
-__host__ __device__ constexpr size_t scatter_smem(unsigned P, int kw) {
-  return (size_t)kScatterTile * (kw * 8) +   // staged keys
-         (size_t)kScatterTile * 4 +          // sorted order: slot | partition << 12
-         (size_t)P * 20 +                    // cnt, off, gbase, n1, obase (32-bit each)
-         (size_t)32 * 4 +                    // warp sums
-         (size_t)kScatterTile;               // staged info
+__host__ __device__ constexpr size_t scatter_smem(unsigned log_b, int kw) {
+  return (size_t)kScatterTile * kw * 8 + ((size_t)4 << log_b) + 32 * 4;
 }
-
-static_assert(scatter_smem(kMaxPartitions, 1) <= 227 * 1024 && scatter_smem(kMaxPartitionsWide, 2) <= 227 * 1024,
-              "the scatter's shared memory must fit one CTA for every allowed partition count");
-static_assert(kMaxPartitions <= kScatterThreads * kScatterMaxChunk,
-              "partition numbers must fit the sorted order's 12 bits and the threads' chunks");
 
 template <int KW>
 __global__ void __launch_bounds__(kScatterThreads, 1) part_scatter_kernel(const __grid_constant__ PartGeom G,
                                                                           const __grid_constant__ PartWindows W,
-                                                                          const __grid_constant__ PartRecords R) {
-  constexpr int kWarps = kScatterThreads / 32;
-  extern __shared__ __align__(16) unsigned char s_raw[];
-  const unsigned P = G.P;
-  u64* s_keys = reinterpret_cast<u64*>(s_raw);                              // [tile * KW]
-  unsigned* s_order = reinterpret_cast<unsigned*>(s_keys + kScatterTile * KW);  // [tile]
-  unsigned* s_cnt = s_order + kScatterTile;                                 // [P] records in this tile
-  unsigned* s_off = s_cnt + P;                                              // [P] first sorted position
-  unsigned* s_gbase = s_off + P;                                            // [P] run start in the bucket
-  unsigned* s_n1 = s_gbase + P;                                             // [P] records of the run in the bucket
-  unsigned* s_obase = s_n1 + P;                                             // [P] rest: overflow area position
-  unsigned* s_wsum = s_obase + P;                                           // [32]
-  unsigned char* s_info = reinterpret_cast<unsigned char*>(s_wsum + 32);    // [tile]
-  const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+                                                                          const __grid_constant__ PartTiles T) {
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  const unsigned B = 1u << G.log_b;
+  u64* s_rec = reinterpret_cast<u64*>(s_raw);                                  // [tile * KW]
+  unsigned* s_bin = reinterpret_cast<unsigned*>(s_rec + kScatterTile * KW);    // [B] counts, then offsets
+  unsigned* s_wsum = s_bin + B;                                                // [32]
+  const unsigned tid = threadIdx.x, lane = tid & 31;
   const unsigned n_tiles = (unsigned)((W.q1 - W.q0 + kScatterTile - 1) / kScatterTile);
-  const u64 pol = policy_evict_first();
-  const unsigned per = (P + kScatterThreads - 1) / kScatterThreads;  // partitions per thread (<= 8)
-  const unsigned p0 = min(P, tid * per), p1 = min(P, p0 + per);
-  const u64 cap = R.cap, ocap = R.ocap;
+  const unsigned per = (B + kScatterThreads - 1) / kScatterThreads;
   unsigned acc_valid = 0;
-  for (unsigned p = tid; p < P; p += kScatterThreads) s_cnt[p] = 0;
-  __syncthreads();
+  unsigned acc_bucket[kScatterMaxPer] = {};  // records of this thread's buckets, over the CTA's tiles
   for (unsigned t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    // 1: windows -> staged records, rank inside the partition
-    unsigned pr[kScatterWpt];  // partition << 13 | rank, or ~0u
+    if (tid == 0) tma_store_wait_read();  // the previous tile has left shared memory
+    for (unsigned p = tid; p < B; p += kScatterThreads) s_bin[p] = 0;
+    __syncthreads();
+    unsigned pr[kScatterWpt];  // bucket << 13 | rank, or ~0u
 #pragma unroll
     for (int j = 0; j < kScatterWpt; ++j) pr[j] = 0xFFFFFFFFu;
     const u64 q = W.q0 + (u64)t * kScatterTile + (u64)tid * kScatterWpt;
@@ -110,608 +164,784 @@ __global__ void __launch_bounds__(kScatterThreads, 1) part_scatter_kernel(const 
           if (G.n_parts <= 1 || owner_of(h, G.n_parts) == G.part) {
             ++acc_valid;
             const unsigned slot = j * kScatterThreads + tid;
-            const unsigned p = part_of(h, P);
-            pr[j] = (p << 13) | atomicAdd(&s_cnt[p], 1u);
-            if (KW == 1) s_keys[slot] = w.lo;
-            else reinterpret_cast<ulonglong2*>(s_keys)[slot] = make_ulonglong2(w.lo, w.hi);
-            s_info[slot] = info_of(w);
+            const unsigned p = (unsigned)(h >> (64 - G.log_b));
+            pr[j] = (p << 13) | atomicAdd(&s_bin[p], 1u);
+            const unsigned info = (w.lu ? w.lb : 4u) | ((w.ru ? w.rb : 4u) << 3);
+            const u64 r = (h & kHashMask) | ((u64)info << (64 - kInfoBits));
+            if (KW == 1) s_rec[slot] = r;
+            else reinterpret_cast<ulonglong2*>(s_rec)[slot] = make_ulonglong2(r, w.hi);
           }
         }
         if (j + 1 < kScatterWpt) rw.roll();
       }
     }
     __syncthreads();
-    // 2: reservations of this thread's partitions (in flight during the scan), then the
-    // exclusive scan of the counts
-    unsigned long long res[kScatterMaxChunk];
+    // bucket offsets (thread t: buckets t * per ..), written as the tile's row
+    unsigned c[kScatterMaxPer];
     unsigned local = 0;
 #pragma unroll
-    for (unsigned x = 0; x < kScatterMaxChunk; ++x) {
-      const unsigned p = p0 + x;
-      res[x] = 0;
-      if (p < p1) {
-        const unsigned c = s_cnt[p];
-        local += c;
-        if (c) res[x] = atomicAdd(&R.fill[p], (u64)c);
+    for (unsigned x = 0; x < kScatterMaxPer; ++x) {
+      const unsigned p = tid * per + x;
+      c[x] = x < per && p < B ? s_bin[p] : 0u;
+      local += c[x];
+      acc_bucket[x] += c[x];
+    }
+    unsigned total;
+    unsigned run = block_scan<kScatterThreads>(local, s_wsum, total);
+    unsigned short* row = T.offs + (T.tile0 + t) * T.stride;
+#pragma unroll
+    for (unsigned x = 0; x < kScatterMaxPer; ++x) {
+      const unsigned p = tid * per + x;
+      if (x < per && p < B) {
+        s_bin[p] = run;
+        row[p] = (unsigned short)run;
+        run += c[x];
       }
     }
-    unsigned incl = local;
+    if (tid == 0) row[B] = (unsigned short)total;
+    // own records back into registers, then to their sorted places
+    u64 r0[kScatterWpt], r1[kScatterWpt];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= (unsigned)o) incl += v;
-    }
-    if (lane == 31) s_wsum[warp] = incl;
-    __syncthreads();
-    // prefix of the warp totals (every warp scans the 16 sums itself)
-    unsigned ws = s_wsum[lane], wincl = ws;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned v = __shfl_up_sync(0xffffffffu, wincl, o);
-      if (lane >= (unsigned)o) wincl += v;
-    }
-    const unsigned total = __shfl_sync(0xffffffffu, wincl, kWarps - 1);  // records in this tile
-    unsigned run = __shfl_sync(0xffffffffu, wincl - ws, warp) + incl - local;
-#pragma unroll
-    for (unsigned x = 0; x < kScatterMaxChunk; ++x) {
-      const unsigned p = p0 + x;
-      if (p < p1) {
-        const unsigned c = s_cnt[p];
-        s_off[p] = run;
-        run += c;
-        if (c) {
-          const u64 b = res[x];
-          const u64 room = b < cap ? cap - b : 0;
-          const unsigned n1 = (unsigned)(room < c ? room : c);
-          s_gbase[p] = (unsigned)(b < cap ? b : 0);
-          s_n1[p] = n1;
-          s_obase[p] = n1 < c ? (unsigned)min(atomicAdd(&R.fill[P], (u64)(c - n1)), ocap) : 0u;
+    for (int j = 0; j < kScatterWpt; ++j) {
+      const unsigned slot = j * kScatterThreads + tid;
+      if (pr[j] != 0xFFFFFFFFu) {
+        if (KW == 1) {
+          r0[j] = s_rec[slot];
+        } else {
+          const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[slot];
+          r0[j] = v.x;
+          r1[j] = v.y;
         }
-        s_cnt[p] = 0;  // for the next tile
       }
     }
     __syncthreads();
-    // 3a: sorted order (partition-major) of the staged records
 #pragma unroll
     for (int j = 0; j < kScatterWpt; ++j) {
       if (pr[j] == 0xFFFFFFFFu) continue;
-      const unsigned p = pr[j] >> 13, r = pr[j] & 8191u;
-      s_order[s_off[p] + r] = (p << 13) | (j * kScatterThreads + tid);
+      const unsigned at = s_bin[pr[j] >> 13] + (pr[j] & 8191u);
+      if (KW == 1) s_rec[at] = r0[j];
+      else reinterpret_cast<ulonglong2*>(s_rec)[at] = make_ulonglong2(r0[j], r1[j]);
     }
+    fence_proxy_async_smem();
     __syncthreads();
-    // 3b: write out in sorted order (coalesced runs per bucket)
-    for (unsigned i = tid; i < total; i += kScatterThreads) {
-      const unsigned e = s_order[i];
-      const unsigned slot = e & 8191u, p = e >> 13;
-      const unsigned r = i - s_off[p], n1 = s_n1[p];
-      u64 gi;
-      if (r < n1) {
-        gi = (u64)p * cap + s_gbase[p] + r;
-      } else {
-        const u64 o = (u64)s_obase[p] + (r - n1);
-        if (o >= ocap) {  // overflow area full: reported, never dropped silently
-          atomicOr(&G.status->flags, kFlagFull);
-          continue;
-        }
-        gi = (u64)P * cap + o;
-      }
-      if (KW == 1) {
-        st_stream(reinterpret_cast<u64*>(R.keys) + gi, s_keys[slot], pol);
-      } else {
-        st_stream(reinterpret_cast<ulonglong2*>(R.keys) + gi, reinterpret_cast<const ulonglong2*>(s_keys)[slot], pol);
-      }
-      st_stream(R.info + gi, s_info[slot], pol);
+    if (tid == 0 && total) {
+      unsigned char* dst = reinterpret_cast<unsigned char*>(T.recs) + (T.tile0 + t) * (u64)(kScatterTile * KW * 8);
+      const unsigned bytes = (total * KW * 8 + 15u) & ~15u;
+      for (unsigned o = 0; o < bytes; o += 16384u)
+        tma_store_1d(dst + o, smem_u32(s_rec) + o, bytes - o < 16384u ? bytes - o : 16384u);
+      tma_store_commit();
     }
-    __syncthreads();  // staged records and per-partition runs are reused by the next tile
   }
-  // valid windows: reduce inside the warp first
+  if (tid == 0) tma_store_wait();  // complete before the CTA may leave
+#pragma unroll
+  for (unsigned x = 0; x < kScatterMaxPer; ++x)
+    if (acc_bucket[x]) atomicAdd(&T.totals[tid * per + x], (u64)acc_bucket[x]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc_valid += __shfl_down_sync(0xffffffffu, acc_valid, o);
   if (lane == 0 && acc_valid) atomicAdd(&G.status->valid_windows, (u64)acc_valid);
 }
 
-// ------------------------------------------------------------------ record pass
+// ------------------------------------------------------------------ split
 //
-// Tiles walk the buckets in partition order (then the overflow area), so at any moment the
-// CTAs work on one or two partitions whose sub-filter and sub-table sit in L2. Every warp
-// works on its own tiles of 32 * RPT records, staged in shared memory with 1-D bulk copies
-// and double-buffered: while the lanes resolve the atomics of one tile, the warp's next tile
-// is on its way. Warps never wait for each other (no block barriers), so a warp whose
-// probes take long does not hold up the others.
+// One work item = a chunk of scatter tiles x kSplitBuckets adjacent buckets. The offset rows of
+// the chunk's tiles are read once for all of the item's buckets (adjacent entries of a row).
+// Per bucket: the lengths of its runs are scanned, the records gathered into shared memory (a
+// few lanes per run, 8- or 16-byte asynchronous copies) and sorted by sub-bucket like a scatter
+// tile, at most kPartSubTile at a time (a chunk is sized so that one such sub-tile is the rule).
+// Each sub-bucket's run then takes the next places of its sub-bucket (one atomic per run) and is
+// written there, so that the count kernel finds a sub-bucket in one piece: gathering it there, a
+// handful of records per run, took more instructions than the counting. Items go through the
+// buckets in order, so the pieces of one line meet in L2. A sub-bucket has room for G.cap
+// records; what does not fit (very frequent k-mers) goes to an overflow segment of the bucket.
 
-template <int KW, int RPT>
-struct WarpStage {
-  static constexpr int kTile = 32 * RPT;  // a multiple of 16
-  u64 keys[2][kTile * KW];
-  unsigned char info[2][kTile];
-  unsigned char dup[64];                  // equal keys among a round of 32 records: a lane per hash slot
-  unsigned acc[32][10];                   // per group leader: occurrences by left / right outcome
-  unsigned walk[8];                       // lane 0's tile walk: t, c_end, c_next, cb, cf, kept
-                                          // here: as registers they took five in every lane
-                                          // and the Bloom pass spilled
-  unsigned long long bar[2];
-};
-static_assert(sizeof(WarpStage<1, 2>) % 16 == 0 && sizeof(WarpStage<2, 2>) % 16 == 0 &&
-                  sizeof(WarpStage<1, 4>) % 16 == 0 && sizeof(WarpStage<2, 4>) % 16 == 0,
-              "every warp's staging buffers must start on a 16-byte boundary");
+constexpr int kSplitThreads = 512;
+constexpr int kSplitItems = kPartSubTile / kSplitThreads;
+constexpr int kSplitMaxPer = kMaxSubBuckets / kSplitThreads;  // sub-buckets per thread
+static_assert(kPartSubTile <= 8192, "ranks are 13 bits");
 
-// Records of launch tile t: the first one (base) and their number, 0 if the tile is empty.
-// The launch numbers its tiles from 0: first the nb tiles of the buckets of partitions
-// [p_begin, p_end), tpb per bucket, then the tiles of the overflow area (if the launch covers
-// it). Tile numbers, bucket numbers and record counts within a bucket fit 32 bits (the host
-// checks each record batch). cb / cf: the bucket whose record count was loaded last.
-// tinv: 0, or tile_inverse(tpb), with which the bucket number is a multiply-high instead of a
-// division.
-template <int TILE>
-__device__ __forceinline__ unsigned rec_tile(const PartGeom& G, const PartRecords& R, unsigned tpb, unsigned nb,
-                                             unsigned t, u64& base, unsigned& cb, unsigned& cf, u64 tinv) {
-  unsigned f, lo;
-  u64 b0;
-  if (t < nb) {
-    const unsigned q = tinv ? (tpb == 1 ? t : (unsigned)__umul64hi((u64)t, tinv)) : t / tpb;
-    const unsigned b = R.p_begin + q;
-    if (b != cb) {
-      const u64 x = R.fill[b];
-      cb = b;
-      cf = (unsigned)(x < R.cap ? x : R.cap);
-    }
-    f = cf;
-    lo = (t - q * tpb) * TILE;
-    b0 = (u64)b * R.cap;
-  } else {
-    const u64 x = R.fill[G.P];
-    f = (unsigned)(x < R.ocap ? x : R.ocap);
-    lo = (t - nb) * TILE;
-    b0 = (u64)G.P * R.cap;
+// First overflow segment of each bucket of [b0, b1): a sub-tile makes one at most.
+constexpr int kBaseThreads = 1024;
+__global__ void __launch_bounds__(kBaseThreads) part_base_kernel(const u64* totals, unsigned b0, unsigned b1,
+                                                                 unsigned n_chunks, unsigned* seg_base) {
+  __shared__ unsigned s_sum[32];
+  constexpr unsigned kPer = (1u << kMaxLogBuckets) / kBaseThreads;
+  unsigned v[kPer], local = 0, total;
+#pragma unroll
+  for (unsigned x = 0; x < kPer; ++x) {
+    const unsigned b = b0 + threadIdx.x * kPer + x;
+    v[x] = b < b1 ? (unsigned)(totals[b] / kPartSubTile) + n_chunks : 0u;
+    local += v[x];
   }
-  if (lo >= f) return 0;
-  base = b0 + lo;
-  return f - lo < (unsigned)TILE ? f - lo : (unsigned)TILE;
-}
-
-// Tiles are handed out in launch order from a global queue, kQueueChunk consecutive tiles at a
-// time, so every warp works at the front of the partition sequence: the warps never spread
-// over more partitions than the front touches, and those partitions' sub-filters and
-// sub-tables stay in L2. (Tiles assigned to warps in a fixed pattern let fast and slow warps
-// drift apart over the partitions, and their structures evicted one another from L2.)
-// Lane 0 holds the warp's current chunk (tiles up to c_end) and the next chunk, grabbed one
-// ahead so that its queue round trip is hidden.
-constexpr unsigned kQueueChunk = 8;
-
-// floor(t / d) = high word of t * (floor((2^64 - 1) / d) + 1) for every t < 2^32 and 2 <= d <
-// 2^32 (division by an invariant integer through a rounded-up reciprocal, Granlund and
-// Montgomery, PLDI 1994): the product's error t * e / 2^64, e <= 1, stays below 1 / d.
-__device__ __forceinline__ u64 tile_inverse(unsigned d) { return d > 1 ? ~0ull / d + 1 : 0ull; }
-
-// Lane 0: the next non-empty tile from t on (its first record in base, t moved past it),
-// moving through the warp's chunks; returns its record count, 0 when no tile is left.
-template <int TILE>
-__device__ __forceinline__ unsigned rec_next(const PartGeom& G, const PartRecords& R, unsigned tpb, unsigned nb,
-                                             unsigned n_tiles, unsigned& t, unsigned& c_end, unsigned& c_next,
-                                             u64& base, unsigned& cb, unsigned& cf, u64 tinv = 0) {
-  while (true) {
-    if (t >= c_end) {  // chunk done: take the one grabbed ahead, grab the following one
-      t = c_next * kQueueChunk;
-      c_end = t + kQueueChunk;
-      c_next = atomicAdd(R.queue, 1u);
-    }
-    if (t >= n_tiles) return 0;
-    const unsigned n = rec_tile<TILE>(G, R, tpb, nb, t, base, cb, cf, tinv);
-    ++t;
-    if (n) return n;
+  unsigned run = block_scan<kBaseThreads>(local, s_sum, total);
+#pragma unroll
+  for (unsigned x = 0; x < kPer; ++x) {
+    const unsigned b = b0 + threadIdx.x * kPer + x;
+    if (b < b1) seg_base[b - b0] = run;
+    run += v[x];
   }
 }
 
-// Lane 0: stage the n records from `base` into buffer `buf` (sizes rounded up to 16 records,
-// which stays inside the bucket because cap and ocap are multiples of 16).
-template <int KW, int RPT>
-__device__ __forceinline__ void rec_issue(WarpStage<KW, RPT>& S, const PartRecords& R, int buf, u64 base, unsigned n,
-                                          u64 pol) {
-  const unsigned n16 = (n + 15u) & ~15u;
-  const unsigned kb = n16 * 8u * KW;
-  const unsigned bar = smem_u32(&S.bar[buf]);
-  fence_proxy_async_smem();
-  mbar_expect_tx(bar, kb + n16);
-  tma_load_1d_hint(smem_u32(S.keys[buf]), reinterpret_cast<const u64*>(R.keys) + base * KW, kb, bar, pol);
-  tma_load_1d_hint(smem_u32(S.info[buf]), R.info + base, n16, bar, pol);
+__host__ __device__ constexpr size_t split_smem(unsigned chunk_tiles, unsigned sub_max, int kw) {
+  return (size_t)kPartSubTile * kw * 8 + (size_t)sub_max * (4 + 4 + 2) + 32 * 4 + (size_t)chunk_tiles * 4 +
+         (((size_t)chunk_tiles * (kSplitBuckets + 1) * 2 + 15) & ~(size_t)15);
 }
 
-// Lane 0: the same staging copy into explicit buffers (keys, info) completing on `bar`.
 template <int KW>
-__device__ __forceinline__ void rec_issue_raw(u64* keys, unsigned char* info, unsigned bar, const PartRecords& R,
-                                              u64 base, unsigned n, u64 pol) {
-  const unsigned n16 = (n + 15u) & ~15u;
-  const unsigned kb = n16 * 8u * KW;
-  fence_proxy_async_smem();
-  mbar_expect_tx(bar, kb + n16);
-  tma_load_1d_hint(smem_u32(keys), reinterpret_cast<const u64*>(R.keys) + base * KW, kb, bar, pol);
-  tma_load_1d_hint(smem_u32(info), R.info + base, n16, bar, pol);
-}
-
-__device__ __forceinline__ u64 shfl0(u64 v) { return __shfl_sync(0xffffffffu, v, 0); }
-
-template <int KW, int RPT, unsigned MODE, bool GROUP>
-__global__ void __launch_bounds__(kPartThreads, RPT == 2 ? 4 : 2) part_pass_kernel(const __grid_constant__ PartGeom G,
-                                                                                  const __grid_constant__ PartRecords R) {
-  static_assert(MODE == kModeBloom || MODE == kModeCount, "the recount has its own kernel");
-  constexpr int kTile = WarpStage<KW, RPT>::kTile;
-  constexpr int kWarps = kPartThreads / 32;
-  __shared__ __align__(128) WarpStage<KW, RPT> stage[kWarps];
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  WarpStage<KW, RPT>& S = stage[warp];
-  const unsigned tpb = (unsigned)((R.cap + kTile - 1) / kTile);  // tiles per bucket
-  const unsigned ofill = (unsigned)(R.fill[G.P] < R.ocap ? R.fill[G.P] : R.ocap);
-  const unsigned nb = (R.p_end - R.p_begin) * tpb;  // bucket tiles of this launch
-  const unsigned n_tiles = nb + (R.overflow ? (ofill + kTile - 1) / kTile : 0u);
-  const u64 pol = policy_evict_first();
-  unsigned acc_ins = 0, acc_first = 0;  // per warp: below 2^32
-  unsigned phases = 0;  // bit b: parity to wait for on buffer b (same in every lane)
-
-  // lane 0's walk over the queue's chunks
-  unsigned& t = S.walk[0];
-  unsigned& c_end = S.walk[1];
-  unsigned& c_next = S.walk[2];
-  unsigned& cb = S.walk[3];
-  unsigned& cf = S.walk[4];
-  u64 base = 0;
-  unsigned n = 0;
-  if (lane == 0) {
-    t = 0;
-    cb = ~0u;
-    cf = 0;
-    c_end = 0;
-    mbar_init(smem_u32(&S.bar[0]), 1);
-    mbar_init(smem_u32(&S.bar[1]), 1);
-    c_next = atomicAdd(R.queue, 1u);
-    n = rec_next<kTile>(G, R, tpb, nb, n_tiles, t, c_end, c_next, base, cb, cf);
-    if (n) rec_issue(S, R, 0, base, n, pol);
-  }
-  __syncwarp();  // barriers initialised before any lane polls them
-  n = __shfl_sync(0xffffffffu, n, 0);
-  base = shfl0(base);
-  int buf = 0;
-  while (n) {
-    // stage the warp's next non-empty tile into the other buffer, then wait for this one
-    u64 nbase = 0;
-    unsigned nn = 0;
-    if (lane == 0) {
-      nn = rec_next<kTile>(G, R, tpb, nb, n_tiles, t, c_end, c_next, nbase, cb, cf);
-      if (nn) rec_issue(S, R, buf ^ 1, nbase, nn, pol);
+__global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __grid_constant__ PartGeom G,
+                                                                      const __grid_constant__ PartTiles T,
+                                                                      const __grid_constant__ PartSplit S) {
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  __shared__ u64 s_over;
+  u64* s_rec = reinterpret_cast<u64*>(s_raw);                                  // [sub-tile * KW]
+  unsigned* s_bin = reinterpret_cast<unsigned*>(s_rec + kPartSubTile * KW);    // [sub_max] counts, then offsets
+  unsigned* s_to = s_bin + G.sub_max;                                          // [sub_max] place minus sorted position
+  unsigned* s_wsum = s_to + G.sub_max;                                         // [32]
+  unsigned* s_dst = s_wsum + 32;                                               // [chunk tiles] first record of the run
+  unsigned short* s_lim = reinterpret_cast<unsigned short*>(s_dst + S.chunk_tiles);  // [sub_max] end of what fits
+  unsigned short* s_off = s_lim + G.sub_max;                                   // [chunk tiles][buckets + 1]
+  const unsigned tid = threadIdx.x;
+  const unsigned n_sub = sub_buckets(G);
+  const unsigned per_sub = (n_sub + kSplitThreads - 1) / kSplitThreads;
+  const unsigned n_blocks = (S.b1 - S.b0 + kSplitBuckets - 1) / kSplitBuckets;
+  const unsigned n_chunks = (T.n_tiles + S.chunk_tiles - 1) / S.chunk_tiles;
+  const u64 n_items = (u64)n_chunks * n_blocks;
+  const unsigned glanes = 1u << S.log_lanes, gl = tid & (glanes - 1), gi = tid >> S.log_lanes,
+                 gn = kSplitThreads >> S.log_lanes;
+  for (u64 item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const unsigned chunk = (unsigned)(item % n_chunks);
+    const unsigned bb = S.b0 + (unsigned)(item / n_chunks) * kSplitBuckets;
+    const unsigned nb = S.b1 - bb < kSplitBuckets ? S.b1 - bb : kSplitBuckets;
+    const unsigned t0 = chunk * S.chunk_tiles;
+    const unsigned nt = T.n_tiles - t0 < S.chunk_tiles ? T.n_tiles - t0 : S.chunk_tiles;
+    __syncthreads();  // the previous item's offsets are no longer read
+    for (unsigned x = tid; x < nt * (kSplitBuckets + 1); x += kSplitThreads) {
+      const unsigned i = x / (kSplitBuckets + 1), j = x - i * (kSplitBuckets + 1);
+      s_off[x] = j <= nb ? T.offs[(u64)(t0 + i) * T.stride + bb + j] : 0;
     }
-    nn = __shfl_sync(0xffffffffu, nn, 0);
-    nbase = shfl0(nbase);
-    const unsigned bar = smem_u32(&S.bar[buf]);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, (phases >> buf) & 1u, G.wait_limit));
-    if (!ok) {  // give up: report, let the copies in flight land (bounded), stop the warp
-      if (lane == 0) {
-        atomicOr(&G.status->flags, kFlagTimeout);
-        mbar_drain(bar, (phases >> buf) & 1u, G.wait_limit);
-        if (nn) mbar_drain(smem_u32(&S.bar[buf ^ 1]), (phases >> (buf ^ 1)) & 1u, G.wait_limit);
+    __syncthreads();
+    const unsigned per = (nt + kSplitThreads - 1) / kSplitThreads;  // runs per thread
+    for (unsigned j = 0; j < nb; ++j) {
+      unsigned local = 0, total;
+      for (unsigned x = 0; x < per; ++x) {
+        const unsigned i = tid * per + x;
+        if (i < nt) local += s_off[i * (kSplitBuckets + 1) + j + 1] - s_off[i * (kSplitBuckets + 1) + j];
       }
-      return;
-    }
-    phases ^= 1u << buf;
-    const u64* sk = S.keys[buf];
-    const unsigned char* si = S.info[buf];
-
-    Window w[RPT];
-    u64 h[RPT];
-    unsigned p[RPT], rec[RPT];
-    bool act[RPT];
-    // stage 1: records from shared memory
-#pragma unroll
-    for (int j = 0; j < RPT; ++j) {
-      const unsigned k = j * 32 + lane;
-      act[j] = k < n;
-      rec[j] = k;
-      h[j] = 0;
-      p[j] = 0;
-      if (act[j]) {
-        const unsigned i = rec[j];
-        if (KW == 1) {
-          w[j].lo = sk[i];
-          w[j].hi = 0;
-        } else {
-          const ulonglong2 kk = reinterpret_cast<const ulonglong2*>(sk)[i];
-          w[j].lo = kk.x;
-          w[j].hi = kk.y;
-        }
-        window_of(si[i], w[j]);
-        h[j] = key_hash(w[j].lo, w[j].hi);
-        p[j] = part_of(h[j], G.P);
-      }
-    }
-    // Equal keys in a round of 32 records (frequent k-mers: satellites, low-complexity
-    // sequence) act as one group: only its leader does the Bloom test-and-set and the table
-    // probe, and the group's counter updates are summed in shared memory and applied once
-    // (the paper accumulates frequent k-mers locally before a global reduction, Section 5.1;
-    // here the locality is the warp). Each lane writes its lane number at a slot chosen by its
-    // hash; a lane whose slot holds another lane with the same key joins that lane's group.
-    // Only with GROUP (the heavy_hitters parameter): elsewhere every lane is its own group.
-    bool dup[RPT];
-    unsigned ldr[RPT];
-    bool anydup = false;
-#pragma unroll
-    for (int j = 0; j < RPT; ++j) {
-      dup[j] = false;
-      ldr[j] = lane;
-    }
-    if (GROUP) {
-#pragma unroll
-      for (int j = 0; j < RPT; ++j) {
-        const unsigned slot = (unsigned)h[j] & 63u;
-        if (act[j]) S.dup[slot] = (unsigned char)lane;
-        __syncwarp();
-        const unsigned wl = act[j] ? S.dup[slot] : lane;
-        const u64 wlo = __shfl_sync(0xffffffffu, w[j].lo, wl), whi = __shfl_sync(0xffffffffu, w[j].hi, wl);
-        dup[j] = act[j] && wl != lane && wlo == w[j].lo && whi == w[j].hi;
-        ldr[j] = dup[j] ? wl : lane;
-        anydup |= __any_sync(0xffffffffu, dup[j]);
-        __syncwarp();  // the slots are rewritten by the next round
-      }
-    }
-    // stage 2: Bloom test-and-set in the partition's sub-filter; first sightings flagged
-    if (MODE == kModeBloom) {
-      u64 old[RPT], msk[RPT];
-#pragma unroll
-      for (int j = 0; j < RPT; ++j) {
-        old[j] = msk[j] = 0;
-        if (act[j]) {
-          msk[j] = bloom_mask(h[j], G.bloom_h);
-          if (!dup[j]) old[j] = atomicOr(G.bloom + (u64)p[j] * G.Wp + bloom_index(h[j], G.Wp), msk[j]);
+      unsigned run = block_scan<kSplitThreads>(local, s_wsum, total);
+      for (unsigned x = 0; x < per; ++x) {
+        const unsigned i = tid * per + x;
+        if (i < nt) {
+          s_dst[i] = run;
+          run += s_off[i * (kSplitBuckets + 1) + j + 1] - s_off[i * (kSplitBuckets + 1) + j];
         }
       }
-#pragma unroll
-      for (int j = 0; j < RPT; ++j) {
-        // a group's members come after its leader: they have been seen
-        const bool first = act[j] && !dup[j] && (old[j] & msk[j]) != msk[j];
-        if (first) st_stream(R.info + base + rec[j], (unsigned)si[rec[j]] | kInfoFirst, pol);
-        acc_first += __popc(__ballot_sync(0xffffffffu, first));
-        act[j] = act[j] && !first;
-        // a group whose leader was the first sighting: its members resolve on their own
-        if (GROUP && __shfl_sync(0xffffffffu, first, ldr[j])) {
-          dup[j] = false;
-          ldr[j] = lane;
+      const u64 sub0 = (u64)(bb + j - S.b0) * n_sub;  // the bucket's first sub-bucket
+      u64* out = S.recs + sub0 * G.cap * KW;
+      for (unsigned w0 = 0; w0 < total; w0 += kPartSubTile) {
+        const unsigned n = total - w0 < kPartSubTile ? total - w0 : kPartSubTile;
+        for (unsigned p = tid; p < n_sub; p += kSplitThreads) s_bin[p] = 0;
+        __syncthreads();  // also: s_dst is set, the previous sub-tile has been written
+        // gather the window [w0, w0 + n) of the bucket's records
+        for (unsigned i = gi; i < nt; i += gn) {
+          const unsigned a = s_off[i * (kSplitBuckets + 1) + j], len = s_off[i * (kSplitBuckets + 1) + j + 1] - a;
+          const unsigned d = s_dst[i];
+          if (d >= w0 + n || d + len <= w0) continue;
+          const unsigned x0 = d < w0 ? w0 - d : 0u, x1 = d + len > w0 + n ? w0 + n - d : len;
+          const u64* src = T.recs + ((u64)(t0 + i) * kPartTile + a) * KW;
+          for (unsigned x = x0 + gl; x < x1; x += glanes)
+            cp_async<8 * KW>(smem_u32(s_rec + (size_t)(d + x - w0) * KW), src + (u64)x * KW);
         }
-      }
-    }
-    // stage 3: first probe in the partition's sub-table (group leaders only)
-    ulonglong2 kv[RPT];
-    u64 idx[RPT];
+        cp_async_wait_all();
+        __syncthreads();
+        u64 r0[kSplitItems], r1[kSplitItems];
+        unsigned pr[kSplitItems];
 #pragma unroll
-    for (int j = 0; j < RPT; ++j) {
-      kv[j] = make_ulonglong2(0, 0);
-      idx[j] = 0;
-      if (act[j] && !dup[j]) {
-        idx[j] = table_index(h[j], G.Sp);
-        kv[j] = __ldcg(reinterpret_cast<const ulonglong2*>(G.table + (u64)p[j] * G.Sp + idx[j]));
-      }
-    }
-    // stage 4: resolve and count
-#pragma unroll
-    for (int j = 0; j < RPT; ++j) {
-      Slot* s = nullptr;
-      bool inserted = false;
-      if (act[j] && !dup[j]) {
-        Slot* sub = G.table + (u64)p[j] * G.Sp;
-        s = resolve_insert(sub, G.Sp, idx[j], kv[j], w[j].lo, w[j].hi, inserted);
-        if (!s) atomicOr(&G.status->flags, kFlagFull);
-      }
-      acc_ins += __popc(__ballot_sync(0xffffffffu, inserted));
-      if (GROUP && anydup) {
-        // sum each group's outcomes in its leader's block, then the leader applies them
-        unsigned* blk = S.acc[lane];
-#pragma unroll
-        for (int c = 0; c < 10; ++c) blk[c] = 0;
-        __syncwarp();
-        if (act[j]) {
-          atomicAdd(&S.acc[ldr[j]][w[j].lu ? w[j].lb : 4u], 1u);
-          atomicAdd(&S.acc[ldr[j]][5u + (w[j].ru ? w[j].rb : 4u)], 1u);
-        }
-        __syncwarp();
-        if (s) {
-#pragma unroll
-          for (int c = 0; c < 10; ++c) {
-            const unsigned v = blk[c];
-            if (!v) continue;
-            unsigned* ctr = c < 4 ? &s->ext[c] : c == 4 ? &s->none[0] : c < 9 ? &s->ext[c - 1] : &s->none[1];
-            if (G.no_overflow) red_add(ctr, v);
-            else if (atomicAdd(ctr, v) > 0xFFFFFFFFu - v) atomicOr(&G.status->flags, kFlagOverflow);
+        for (int y = 0; y < kSplitItems; ++y) {
+          const unsigned x = y * kSplitThreads + tid;
+          pr[y] = 0xFFFFFFFFu;
+          if (x < n) {
+            if (KW == 1) {
+              r0[y] = s_rec[x];
+            } else {
+              const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
+              r0[y] = v.x;
+              r1[y] = v.y;
+            }
+            const unsigned p = sub_of(r0[y], G.log_b, n_sub);
+            pr[y] = (p << 13) | atomicAdd(&s_bin[p], 1u);
           }
         }
-        __syncwarp();  // the blocks are cleared by the next round
-      } else if (s) {
-        if (G.no_overflow) add_occurrence_red(s, w[j]);
-        else add_occurrence(s, w[j], 1u, G.status);
+        __syncthreads();
+        unsigned c[kSplitMaxPer];
+        u64 at[kSplitMaxPer];
+        unsigned lc = 0, tot2;
+#pragma unroll
+        for (unsigned x = 0; x < kSplitMaxPer; ++x) {  // places taken; in flight during the scan
+          const unsigned p = tid * per_sub + x;
+          c[x] = x < per_sub && p < n_sub ? s_bin[p] : 0u;
+          at[x] = c[x] ? atomicAdd(&S.fill[sub0 + p], (u64)c[x]) : 0;
+          lc += c[x];
+        }
+        unsigned ro = block_scan<kSplitThreads>(lc, s_wsum, tot2);
+        unsigned over = 0;
+#pragma unroll
+        for (unsigned x = 0; x < kSplitMaxPer; ++x) {
+          const unsigned p = tid * per_sub + x;
+          if (x < per_sub && p < n_sub) {
+            const unsigned room = at[x] < G.cap ? G.cap - (unsigned)at[x] : 0u, fits = c[x] < room ? c[x] : room;
+            s_bin[p] = ro;
+            s_to[p] = p * G.cap + (unsigned)at[x] - ro;
+            s_lim[p] = (unsigned short)(ro + fits);
+            over += c[x] - fits;
+            c[x] -= fits;
+            ro += c[x] + fits;
+          }
+        }
+        const int any_over = __syncthreads_or(over != 0);
+#pragma unroll
+        for (int y = 0; y < kSplitItems; ++y) {
+          if (pr[y] == 0xFFFFFFFFu) continue;
+          const unsigned to = s_bin[pr[y] >> 13] + (pr[y] & 8191u);
+          if (KW == 1) s_rec[to] = r0[y];
+          else reinterpret_cast<ulonglong2*>(s_rec)[to] = make_ulonglong2(r0[y], r1[y]);
+        }
+        __syncthreads();
+        if (any_over) {  // the block's records that found no room: numbered, and a segment for them
+          unsigned n_over;
+          unsigned o = block_scan<kSplitThreads>(over, s_wsum, n_over);
+#pragma unroll
+          for (unsigned x = 0; x < kSplitMaxPer; ++x) {
+            const unsigned p = tid * per_sub + x;
+            if (x < per_sub && p < n_sub) {
+              s_bin[p] = o - s_lim[p];  // overflow number minus sorted position
+              o += c[x];
+            }
+          }
+          if (tid == 0) {
+            const u64 pos = atomicAdd(S.over_n, (u64)n_over);
+            const unsigned b = bb + j - S.b0;
+            PartSegment sg;
+            sg.pos = pos;
+            sg.n = n_over;
+            sg.pad = 0;
+            S.segs[S.seg_base[b] + atomicAdd(&S.n_segs[b], 1u)] = sg;
+            s_over = pos;
+          }
+          __syncthreads();
+        }
+        for (unsigned i = tid; i < n; i += kSplitThreads) {
+          u64 v0, v1 = 0;
+          if (KW == 1) {
+            v0 = s_rec[i];
+          } else {
+            const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[i];
+            v0 = v.x;
+            v1 = v.y;
+          }
+          const unsigned p = sub_of(v0, G.log_b, n_sub);
+          u64* to = i < s_lim[p] ? out + (u64)(s_to[p] + i) * KW : S.over + (s_over + (s_bin[p] + i)) * KW;
+          if (KW == 1) *to = v0;
+          else *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(v0, v1);
+        }
+        __syncthreads();  // s_bin, s_rec and s_wsum are rewritten
+      }
+      if (total == 0) __syncthreads();  // s_wsum
+    }
+  }
+}
+
+// ------------------------------------------------------------------ count
+//
+// One work item = one sub-bucket, brought into shared memory by bulk copies while the previous
+// one is counted (two buffers, two CTAs per SM). Then
+//  1. every record writes its number at the entry its hash picks, the last one wins; after a
+//     barrier it compares its key with the winner's: equal keys share the winner as their
+//     representative, without an atomic or a loop;
+//  2. the others (about one in eight) find theirs in a second table by compare-and-swap and
+//     probing, compacted into full warps first;
+//  3. representatives that another record joined take a block of ten 16-bit counters (a staged
+//     sub-bucket has fewer than 2^16 records), and
+//  4. every record of such a key adds its two outcomes;
+//  5. these keys with their counters (all keys without the singleton filter) are appended to a
+//     list, which part_insert_kernel puts into the HBM table: a few keys per sub-bucket would
+//     leave most threads waiting for the table's round trips here.
+// Sub-buckets that overflowed (very frequent k-mers) are counted by count_large.
+//
+// Bound by instruction issue. Rejected: a table with the keys and counters themselves that
+// records are added to from registers (a probe of a 16-byte key behind a 64-bit compare-and-swap
+// takes 70 instructions for 32 records, 12 in all per record and warp instead of 6).
+
+constexpr int kCountThreads = 512;
+constexpr int kCountCtas = 2;                // per SM
+constexpr unsigned kEntries = 4096;          // first entries, 16 bits
+constexpr unsigned kEntries2 = 2048;         // second table, 32 bits
+constexpr unsigned kNoEntry = 0xFFFFFFFFu;   // empty entry
+constexpr unsigned kOnce = 0xFFFFu;          // counter block of a representative nobody joined, and of no representative
+constexpr unsigned kJoined = 0xFFFEu;        // joined, block not taken yet
+constexpr unsigned kLone = 0x8000u;          // without the singleton filter: number among the keys seen once
+constexpr unsigned kRangeBits = 20;          // hash bits 21..40: count_large takes a range of them at a time
+
+// An entry of the list of counted keys: five words of 16-bit counter pairs (left A C G T none,
+// right A C G T none), then h and hi.
+template <int KW>
+constexpr unsigned kKeyWords = 5 + 2 * KW;
+
+template <int KW>
+struct CountShape {
+  static constexpr unsigned kCap = KW == 1 ? kCountCap1 : kCountCap2;
+  static constexpr unsigned kItems = (kCap + kCountThreads - 1) / kCountThreads;
+  static constexpr unsigned kCtrWords = 6;   // 16-bit counter pairs, then the key's representative
+  static constexpr size_t kRec = (size_t)kCap * KW * 8;
+  static constexpr size_t kIdx = ((size_t)kCap * 2 + 15) & ~(size_t)15;  // representative; counter block
+  // the counters take the room of the entries, the second table and the list of step 2
+  static constexpr size_t kTab = (size_t)kEntries * 2 + kEntries2 * 4 + kIdx;
+  static constexpr size_t kCtr = ((size_t)(kCap / 2) * kCtrWords * 4 + 15) & ~(size_t)15;
+  static constexpr size_t kSmem = 2 * kRec + 2 * kIdx + (kTab > kCtr ? kTab : kCtr);
+  // count_large: keys and left counters where the representatives begin, right counters in the
+  // buffer that is not being filled
+  static constexpr unsigned kLargeSlots = 1024;
+  static_assert(kCap < kLone && kCap % 2 == 0, "record numbers are 16 bits, bulk copies of 16 bytes");
+  static_assert((size_t)kLargeSlots * (KW * 8 + 20) <= kSmem - 2 * kRec && (size_t)kLargeSlots * 20 <= kRec, "room for count_large");
+};
+
+// Insert one key with its ten counters (left A C G T none, right A C G T none) into the table.
+// The key is in no slot yet and no other thread inserts it.
+__device__ __forceinline__ bool emit_key(const PartGeom& G, u64 h, u64 hi, const unsigned (&ctr)[10]) {
+  const u64 lo = key_lo(h, hi);
+  Slot* sub = G.table + (u64)part_of(h, G.P) * G.Sp;
+  u64 idx = table_index(h, G.Sp);
+  const u64 limit = G.Sp < kMaxProbe ? G.Sp : kMaxProbe;
+  for (u64 n = 0; n < limit; ++n) {
+    Slot* s = sub + idx;
+    u64 olo, ohi;
+    cas128(s, kEmpty, kEmpty, lo, hi, olo, ohi);
+    if (olo == kEmpty && ohi == kEmpty) {
+      *reinterpret_cast<uint4*>(&s->none[0]) = make_uint4(ctr[4], ctr[9], 0u, 0u);
+      *reinterpret_cast<uint4*>(&s->ext[0]) = make_uint4(ctr[0], ctr[1], ctr[2], ctr[3]);
+      *reinterpret_cast<uint4*>(&s->ext[4]) = make_uint4(ctr[5], ctr[6], ctr[7], ctr[8]);
+      return true;
+    }
+    idx = (idx + 1 == G.Sp) ? 0 : idx + 1;
+  }
+  atomicOr(&G.status->flags, kFlagFull);
+  return false;
+}
+
+constexpr u64 kFree = ~0ull;                 // count_large: first key word of an empty slot
+constexpr u64 kLock = 1ull << 63;            // slot taken, second key word not written yet
+constexpr unsigned kProbes = 128;
+
+// One probe of count_large's table at `pos` for key (h, hi): kSame (the slot holds the key, taken
+// for it now if it was empty), kOther, or (two-word keys) kAgain: a new key of two words is
+// written behind a lock bit, within this call, so a lane that meets the locked slot of its own
+// hash only has to come back.
+enum : unsigned { kOther = 0, kSame = 1, kAgain = 2 };
+template <int KW>
+__device__ __forceinline__ unsigned probe_slot(u64* k0, u64* k1, unsigned pos, u64 h, u64 hi) {
+  u64 e = *reinterpret_cast<volatile u64*>(&k0[pos]);
+  if (e == kFree) {
+    e = atomicCAS(&k0[pos], kFree, KW == 1 ? h : h | kLock);
+    if (e == kFree) {
+      if (KW == 2) {
+        *reinterpret_cast<volatile u64*>(&k1[pos]) = hi;
+        __threadfence_block();
+        *reinterpret_cast<volatile u64*>(&k0[pos]) = h;
+      }
+      return kSame;
+    }
+  }
+  if (KW == 1) return e == h ? kSame : kOther;
+  if (e == h) return *reinterpret_cast<volatile u64*>(&k1[pos]) == hi ? kSame : kOther;
+  return e == (h | kLock) ? kAgain : kOther;
+}
+
+// A sub-bucket of any size: its records (`n_in` in place, the rest among the bucket's overflow
+// segments) are streamed from HBM through a shared-memory table with 32-bit counters, as often as
+// its distinct keys need: one range of the hash at a time, halved when a probe of kProbes slots
+// finds no place. Lanes with equal outcomes of equal keys act as one (frequent k-mers are
+// accumulated in the warp first, Section 5.1). The keys go straight to the HBM table.
+template <int KW>
+__device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, u64* k0, unsigned* left, unsigned* right,
+                                         unsigned b, unsigned s, unsigned n_sub, unsigned n_in, unsigned& acc_ins,
+                                         unsigned& acc_first) {
+  using C = CountShape<KW>;
+  constexpr unsigned kSlots = C::kLargeSlots;
+  constexpr unsigned kWarps = kCountThreads / 32;
+  __shared__ unsigned s_bad;
+  u64* k1 = k0 + kSlots * (KW - 1);
+  const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const u64 htop = (u64)(b >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
+  const unsigned n_segs = S.n_segs[b - S.b0];
+  const PartSegment* segs = S.segs + S.seg_base[b - S.b0];
+  u64 lo = 0, width = 1ull << kRangeBits;
+  while (lo < (1ull << kRangeBits)) {
+    __syncthreads();
+    for (unsigned i = tid; i < kSlots; i += kCountThreads) k0[i] = kFree;
+    for (unsigned i = tid; i < kSlots * 5; i += kCountThreads) left[i] = right[i] = 0;
+    if (tid == 0) s_bad = 0;
+    __syncthreads();
+    // one row of 32 records: lane's record (if `in`)
+    auto row = [&](bool in, u64 r, u64 hi) {
+      const u64 h = r & kHashMask, x = (h >> 21) & ((1u << kRangeBits) - 1);
+      bool act = in && x >= lo && x < lo + width;
+      unsigned pos = (unsigned)h & (kSlots - 1), got = kOther;
+      const unsigned jump = (unsigned)(h >> 11) | 1u;
+      const bool mine = act;
+      for (unsigned step = 0; step < kProbes; ++step) {
+        if (act) {
+          got = probe_slot<KW>(k0, k1, pos, h, hi);
+          act = got != kSame;
+          if (got == kOther) pos = (pos + jump) & (kSlots - 1);
+        }
+        if (!__any_sync(0xffffffffu, act)) break;
+      }
+      const bool hit = mine && got == kSame;
+      if (mine && !hit) s_bad = 1;
+      const unsigned l = left_outcome(r), o = right_outcome(r);
+      const unsigned ml = __match_any_sync(0xffffffffu, hit ? pos * 8 + l : ~0u);
+      const unsigned mo = __match_any_sync(0xffffffffu, hit ? pos * 8 + o : ~0u);
+      if (hit) {
+        bool wrap = false;
+        if (lane == __ffs(ml) - 1) wrap |= atomicAdd(&left[pos * 5 + l], __popc(ml)) > 0xFFFFFFFFu - __popc(ml);
+        if (lane == __ffs(mo) - 1) wrap |= atomicAdd(&right[pos * 5 + o], __popc(mo)) > 0xFFFFFFFFu - __popc(mo);
+        if (wrap) atomicOr(&G.status->flags, kFlagOverflow);
+      }
+    };
+    auto load = [&](const u64* p, u64& r, u64& hi) {
+      if (KW == 1) {
+        r = __ldg(p);
+      } else {
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p));
+        r = v.x;
+        hi = v.y;
+      }
+    };
+    const u64* in = S.recs + ((u64)(b - S.b0) * n_sub + s) * G.cap * KW;
+    for (unsigned x0 = warp * 32; x0 < n_in; x0 += kCountThreads) {
+      u64 r = 0, hi = 0;
+      if (x0 + lane < n_in) load(in + (u64)(x0 + lane) * KW, r, hi);
+      row(x0 + lane < n_in, r, hi);
+    }
+    for (unsigned g = warp; g < n_segs; g += kWarps) {
+      const PartSegment sg = segs[g];
+      for (unsigned x0 = 0; x0 < sg.n; x0 += 32) {
+        u64 r = 0, hi = 0;
+        bool mine = x0 + lane < sg.n;
+        if (mine) {
+          load(S.over + (sg.pos + x0 + lane) * KW, r, hi);
+          mine = sub_of(r, G.log_b, n_sub) == s;
+        }
+        if (__any_sync(0xffffffffu, mine)) row(mine, r, hi);
       }
     }
-    __syncwarp();  // buffer `buf` (and the list) are free for the next copy
-    n = nn;
-    base = nbase;
-    buf ^= 1;
+    __syncthreads();
+    if (s_bad) {  // uniform
+      if (width > 1) {
+        width >>= 1;
+        continue;
+      }
+      if (tid == 0) atomicOr(&G.status->flags, kFlagFull);  // cannot be: the hash has more bits than the range
+    }
+    for (unsigned i = tid; i < kSlots; i += kCountThreads) {
+      const u64 h = k0[i];
+      if (h == kFree) continue;
+      ++acc_first;
+      unsigned v[10];
+      u64 n = 0;
+#pragma unroll
+      for (int x = 0; x < 5; ++x) {
+        v[x] = left[i * 5 + x];
+        v[5 + x] = right[i * 5 + x];
+        n += v[x];
+      }
+      if (n >= G.min_count) acc_ins += emit_key(G, h | htop, KW == 2 ? k1[i] : 0, v);
+    }
+    lo += width;
+  }
+  __syncthreads();
+}
+
+template <int KW>
+__global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(const __grid_constant__ PartGeom G,
+                                                                               const __grid_constant__ PartSplit S) {
+  using C = CountShape<KW>;
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  __shared__ __align__(8) unsigned long long s_bar[2];
+  __shared__ u64 s_fill[2], s_base;
+  __shared__ unsigned s_nctr, s_nlone, s_nlist, s_crowded;
+  const unsigned tid = threadIdx.x, lane = tid & 31;
+  unsigned char* s_var = s_raw + 2 * C::kRec + 2 * C::kIdx;
+  unsigned short* s_rep = reinterpret_cast<unsigned short*>(s_raw + 2 * C::kRec);           // [cap] representative
+  unsigned short* s_q = reinterpret_cast<unsigned short*>(s_raw + 2 * C::kRec + C::kIdx);   // [cap] its counter block
+  unsigned* s_ctr = reinterpret_cast<unsigned*>(s_var);                                     // [cap / 2][kCtrWords]
+  unsigned* s_ent2 = reinterpret_cast<unsigned*>(s_var);                                    // [entries2]
+  unsigned short* s_ent = reinterpret_cast<unsigned short*>(s_ent2 + kEntries2);            // [entries]
+  unsigned short* s_list = s_ent + kEntries;                                                // [cap] not settled yet
+  const unsigned n_sub = sub_buckets(G);
+  const u64 n_items = (u64)(S.b1 - S.b0) * n_sub;
+  unsigned acc_ins = 0, acc_first = 0;  // per thread: below 2^32
+  // thread 0: copy a sub-bucket's records into buffer `buf`
+  auto issue = [&](unsigned buf, u64 item, u64 fill) {
+    s_fill[buf] = fill;
+    const unsigned n = fill < G.cap ? (unsigned)fill : G.cap;
+    const unsigned bytes = (n * (8 * KW) + 15u) & ~15u, bar = smem_u32(&s_bar[buf]);
+    fence_proxy_async_smem();
+    mbar_expect_tx(bar, bytes);
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(S.recs + item * G.cap * KW);
+    const unsigned dst = smem_u32(s_raw) + buf * (unsigned)C::kRec;
+    for (unsigned o = 0; o < bytes; o += 16384u) tma_load_1d(dst + o, src + o, bytes - o < 16384u ? bytes - o : 16384u, bar);
+  };
+  u64 ahead = 0;  // thread 0: records of the item after the one whose copy is under way
+  if (tid == 0) {
+    mbar_init(smem_u32(&s_bar[0]), 1);
+    mbar_init(smem_u32(&s_bar[1]), 1);
+    if (blockIdx.x < n_items) issue(0, blockIdx.x, __ldcg(&S.fill[blockIdx.x]));
+    if (blockIdx.x + (u64)gridDim.x < n_items) ahead = __ldcg(&S.fill[blockIdx.x + gridDim.x]);
+  }
+  unsigned phases = 0, buf = 0;  // bit b: parity to wait for on buffer b
+  for (u64 item = blockIdx.x; item < n_items; item += gridDim.x, buf ^= 1) {
+    __syncthreads();  // the previous sub-bucket's memory is free (and the barriers are initialised)
+    if (tid == 0) {
+      const u64 next = item + gridDim.x;
+      if (next < n_items) issue(buf ^ 1, next, ahead);
+      if (next + gridDim.x < n_items) ahead = __ldcg(&S.fill[next + gridDim.x]);
+      s_nctr = s_nlone = s_nlist = s_crowded = 0;
+    }
+    const bool ok = mbar_wait_bounded(smem_u32(&s_bar[buf]), (phases >> buf) & 1u, kWaitPolls);
+    phases ^= 1u << buf;
+    if (!__syncthreads_and(ok)) {  // give up: report, let the copies in flight land (bounded)
+      if (tid == 0) {
+        atomicOr(&G.status->flags, kFlagTimeout);
+        mbar_drain(smem_u32(&s_bar[buf]), ((phases >> buf) & 1u) ^ 1u, kWaitPolls);
+        if (item + gridDim.x < n_items) mbar_drain(smem_u32(&s_bar[buf ^ 1]), (phases >> (buf ^ 1)) & 1u, kWaitPolls);
+      }
+      break;
+    }
+    const u64 fill = s_fill[buf];
+    const unsigned b = S.b0 + (unsigned)(item / n_sub);
+    u64* s_rec = reinterpret_cast<u64*>(s_raw + buf * C::kRec);  // [cap * KW]
+    const unsigned n = fill < G.cap ? (unsigned)fill : G.cap;
+    auto large = [&]() {
+      u64* keys = reinterpret_cast<u64*>(s_rep);
+      count_large<KW>(G, S, keys, reinterpret_cast<unsigned*>(keys + C::kLargeSlots * KW), reinterpret_cast<unsigned*>(s_rec),
+                      b, (unsigned)(item % n_sub), n_sub, n, acc_ins, acc_first);
+    };
+    if (fill > G.cap) {  // uniform
+      large();
+      continue;
+    }
+    if (n == 0) continue;
+    unsigned firsts = 0;  // representatives
+    // 1: a representative for every record
+    u64 h[C::kItems], hi[C::kItems];
+#pragma unroll
+    for (unsigned y = 0; y < C::kItems; ++y) {
+      const unsigned x = y * kCountThreads + tid;
+      h[y] = hi[y] = 0;
+      if (x < n) {
+        if (KW == 1) {
+          h[y] = s_rec[x] & kHashMask;
+        } else {
+          const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
+          h[y] = v.x & kHashMask;
+          hi[y] = v.y;
+        }
+        s_ent[(unsigned)h[y] & (kEntries - 1)] = (unsigned short)x;
+        s_q[x] = (unsigned short)kOnce;
+      }
+    }
+    reinterpret_cast<uint4*>(s_ent2)[tid] = make_uint4(kNoEntry, kNoEntry, kNoEntry, kNoEntry);
+    static_assert(kEntries2 == kCountThreads * 4, "one store per thread clears the second table");
+    __syncthreads();
+    // the key of record z is (ah, ahi)?
+    auto same_key = [&](unsigned z, u64 ah, u64 ahi) -> bool {
+      if (KW == 1) return (s_rec[z] & kHashMask) == ah;
+      const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[z];
+      return (v.x & kHashMask) == ah && v.y == ahi;
+    };
+#pragma unroll
+    for (unsigned y = 0; y < C::kItems; ++y) {
+      const unsigned x = y * kCountThreads + tid;
+      if (x - lane >= n) break;  // the same for the whole warp
+      bool left = false;
+      if (x < n) {
+        const unsigned z = s_ent[(unsigned)h[y] & (kEntries - 1)];
+        if (z == x) {
+          ++firsts;
+          s_rep[x] = (unsigned short)x;
+        } else if (same_key(z, h[y], hi[y])) {
+          s_q[z] = (unsigned short)kJoined;
+          s_rep[x] = (unsigned short)z;
+        } else {
+          left = true;
+        }
+      }
+      const unsigned lm = __ballot_sync(0xffffffffu, left);
+      if (lm) {
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&s_nlist, __popc(lm));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(lm & ((1u << lane) - 1u));
+        if (left) s_list[at] = (unsigned short)x;
+      }
+    }
+    __syncthreads();
+    // 2: the others
+    const unsigned nl = s_nlist;
+    for (unsigned i = tid; i < nl; i += kCountThreads) {
+      const unsigned x = s_list[i];
+      u64 kh, khi = 0;
+      if (KW == 1) {
+        kh = s_rec[x] & kHashMask;
+      } else {
+        const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
+        kh = v.x & kHashMask;
+        khi = v.y;
+      }
+      unsigned pos = (unsigned)(kh >> 12) & (kEntries2 - 1), z;
+      const unsigned jump = (unsigned)(kh >> 23) | 1u;  // odd: comes by every entry
+      unsigned step = 0;
+      for (; step < kEntries2; ++step) {
+        z = *reinterpret_cast<volatile unsigned*>(&s_ent2[pos]);
+        if (z == kNoEntry) {
+          z = atomicCAS(&s_ent2[pos], kNoEntry, x);
+          if (z == kNoEntry) {
+            z = x;
+            ++firsts;
+            break;
+          }
+        }
+        if (same_key(z, kh, khi)) {
+          s_q[z] = (unsigned short)kJoined;
+          break;
+        }
+        pos = (pos + jump) & (kEntries2 - 1);
+      }
+      if (step == kEntries2) s_crowded = 1;  // more keys than the second table holds
+      s_rep[x] = (unsigned short)z;
+    }
+    __syncthreads();
+    if (s_crowded) {  // uniform
+      large();
+      continue;
+    }
+    acc_first += firsts;
+    // 3: counter blocks
+#pragma unroll
+    for (unsigned y = 0; y < C::kItems; ++y) {
+      const unsigned x = y * kCountThreads + tid;
+      if (x - lane >= n) break;
+      const unsigned q0 = x < n ? s_q[x] : kOnce;
+      const unsigned mm = __ballot_sync(0xffffffffu, q0 == kJoined);
+      if (mm) {
+        unsigned q = 0;
+        if (lane == 0) q = atomicAdd(&s_nctr, __popc(mm));
+        q = __shfl_sync(0xffffffffu, q, 0) + __popc(mm & ((1u << lane) - 1u));
+        if (q0 == kJoined) {
+          s_q[x] = (unsigned short)q;
+          unsigned* c = s_ctr + q * C::kCtrWords;
+#pragma unroll
+          for (int w = 0; w < 5; ++w) c[w] = 0;
+          c[5] = x;
+        }
+      }
+      if (G.min_count <= 1) {
+        const bool lone = x < n && q0 == kOnce && s_rep[x] == x;
+        const unsigned lm = __ballot_sync(0xffffffffu, lone);
+        unsigned q = 0;
+        if (lane == 0 && lm) q = atomicAdd(&s_nlone, __popc(lm));
+        q = __shfl_sync(0xffffffffu, q, 0) + __popc(lm & ((1u << lane) - 1u));
+        if (lone) s_q[x] = (unsigned short)(kLone | q);
+      }
+    }
+    __syncthreads();
+    // 4: outcomes
+    if (tid == 0) s_base = s_nctr + s_nlone ? atomicAdd(S.n_keys, (u64)(s_nctr + s_nlone)) : 0;
+    for (unsigned x = tid; x < n; x += kCountThreads) {
+      const unsigned q = s_q[s_rep[x]];
+      if (q < kLone) {
+        const u64 r = s_rec[(size_t)x * KW];
+        const unsigned l = left_outcome(r), o = 5u + right_outcome(r);
+        unsigned* c = s_ctr + q * C::kCtrWords;
+        atomicAdd(&c[l >> 1], 1u << ((l & 1u) * 16));
+        atomicAdd(&c[o >> 1], 1u << ((o & 1u) * 16));
+      }
+    }
+    __syncthreads();
+    // 5: to the list
+    const unsigned nq = s_nctr;
+    const u64 htop = (u64)(b >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
+    unsigned* out = S.keys + s_base * kKeyWords<KW>;
+    for (unsigned e = tid; e < nq * kKeyWords<KW>; e += kCountThreads) {
+      const unsigned q = e / kKeyWords<KW>, w = e - q * kKeyWords<KW>;
+      const unsigned* c = s_ctr + q * C::kCtrWords;
+      unsigned v;
+      if (w < 5) {
+        v = c[w];
+      } else {
+        v = reinterpret_cast<const unsigned*>(s_rec + (size_t)c[5] * KW)[w - 5];
+        if (w == 6) v = (v & (unsigned)(kHashMask >> 32)) | (unsigned)(htop >> 32);
+      }
+      out[e] = v;
+    }
+    if (s_nlone) {
+      for (unsigned x = tid; x < n; x += kCountThreads) {
+        const unsigned q = s_q[x];
+        if (q < kLone || q >= kJoined) continue;
+        const u64 r = s_rec[(size_t)x * KW];
+        const unsigned l = left_outcome(r), o = 5u + right_outcome(r);
+        unsigned* c = out + (size_t)(nq + (q & ~kLone)) * kKeyWords<KW>;
+#pragma unroll
+        for (unsigned w = 0; w < 5; ++w)
+          c[w] = ((l >> 1) == w ? 1u << ((l & 1u) * 16) : 0u) + ((o >> 1) == w ? 1u << ((o & 1u) * 16) : 0u);
+        const u64 kh = (r & kHashMask) | htop;
+        c[5] = (unsigned)kh;
+        c[6] = (unsigned)(kh >> 32);
+        if (KW == 2) {
+          const u64 khi = s_rec[(size_t)x * KW + KW - 1];
+          c[kKeyWords<KW> - 2] = (unsigned)khi;
+          c[kKeyWords<KW> - 1] = (unsigned)(khi >> 32);
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
+    acc_first += __shfl_down_sync(0xffffffffu, acc_first, o);
   }
   if (lane == 0) {
     if (acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
-    if (acc_first) atomicAdd(&G.status->first_sightings, (u64)acc_first);
+    if (acc_first && G.min_count > 1) atomicAdd(&G.status->first_sightings, (u64)acc_first);
   }
 }
 
-// ------------------------------------------------------------------ recount
+// ------------------------------------------------------------------ insert
 //
-// The first sightings marked by the Bloom pass (about two in five records, most of them k-mers
-// seen once) are added to the k-mers that reached the table. Every warp stages its tiles like
-// the other record passes, copies each tile's marked records into a ring in shared memory
-// (the staging buffer is then free for the next copy), and resolves the ring in full rounds of
-// 32 records, one per lane: key filter, then (for the few that pass it) the table probe and the
-// count. Resolving tile by tile instead would leave most lanes idle in every round.
-
-constexpr int kRing = 128;  // entries; a tile adds at most 64 to fewer than 32 left over
+// One counted key per thread into the HBM table. The keys of the list are distinct, in no slot
+// yet, and in hash order roughly, so the slots written at one time lie in one or two partitions.
 
 template <int KW>
-struct RecountStage {
-  static constexpr int kTile = 64;
-  u64 keys[2][kTile * KW];
-  u64 rkeys[kRing * KW];
-  unsigned char info[2][kTile];
-  unsigned char rinfo[kRing];
-  unsigned walk[8];  // lane 0's tile walk: t, c_end, c_next, cb, cf (not in every lane's registers)
-  unsigned long long bar[2];
-};
-static_assert(sizeof(RecountStage<1>) % 16 == 0 && sizeof(RecountStage<2>) % 16 == 0,
-              "every warp's staging buffers must start on a 16-byte boundary");
-
-// One round: lane l resolves ring entry (head + l), if act.
-template <int KW>
-__device__ __forceinline__ void recount_round(const PartGeom& G, const RecountStage<KW>& S, unsigned e, bool act) {
-  if (!act) return;
-  Window w;
-  if (KW == 1) {
-    w.lo = S.rkeys[e];
-    w.hi = 0;
-  } else {
-    const ulonglong2 kk = reinterpret_cast<const ulonglong2*>(S.rkeys)[e];
-    w.lo = kk.x;
-    w.hi = kk.y;
-  }
-  const u64 h = key_hash(w.lo, w.hi);
-  const unsigned p = part_of(h, G.P);
-  // most first sightings are of k-mers seen once, which never reached the table: the key
-  // filter (every inserted key set its bits) rules them out without a probe
-  if (G.Wk) {
-    const u64 m = keyfilter_mask(h, G.bloom_h);
-    if ((__ldcg(G.keyfilter + (u64)p * G.Wk + keyfilter_index(h, G.Wk)) & m) != m) return;
-  }
-  window_of(S.rinfo[e], w);  // extension outcomes: only for the sightings that may count
-  Slot* sub = G.table + (u64)p * G.Sp;
-  const u64 idx = table_index(h, G.Sp);
-  const ulonglong2 kv = __ldcg(reinterpret_cast<const ulonglong2*>(sub + idx));
-  bool full;
-  Slot* s = resolve_find(sub, G.Sp, idx, kv, w.lo, w.hi, full);
-  if (full) atomicOr(&G.status->flags, kFlagFull);
-  if (s) {
-    if (G.no_overflow) add_occurrence_red(s, w);
-    else add_occurrence(s, w, 1u, G.status);
-  }
-}
-
-template <int KW>
-__global__ void __launch_bounds__(kPartThreads, 6) part_recount_kernel(const __grid_constant__ PartGeom G,
-                                                                    const __grid_constant__ PartRecords R) {
-  constexpr int kTile = RecountStage<KW>::kTile;
-  constexpr int kWarps = kPartThreads / 32;
-  __shared__ __align__(128) RecountStage<KW> stage[kWarps];
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  RecountStage<KW>& S = stage[warp];
-  const unsigned tpb = (unsigned)((R.cap + kTile - 1) / kTile);
-  const unsigned ofill = (unsigned)(R.fill[G.P] < R.ocap ? R.fill[G.P] : R.ocap);
-  const unsigned nb = (R.p_end - R.p_begin) * tpb;
-  const unsigned n_tiles = nb + (R.overflow ? (ofill + kTile - 1) / kTile : 0u);
-  const u64 pol = policy_evict_first();
-  unsigned phases = 0;
-  unsigned head = 0, tail = 0;  // ring: entries [head, tail) are waiting (same in every lane)
-  const u64 tinv = tile_inverse(tpb);  // lane 0's tile walk: bucket numbers without a division
-
-  unsigned& t = S.walk[0];
-  unsigned& c_end = S.walk[1];
-  unsigned& c_next = S.walk[2];
-  unsigned& cb = S.walk[3];
-  unsigned& cf = S.walk[4];
-  u64 base = 0;
-  unsigned n = 0;
-  if (lane == 0) {
-    t = 0;
-    cb = ~0u;
-    cf = 0;
-    c_end = 0;
-    mbar_init(smem_u32(&S.bar[0]), 1);
-    mbar_init(smem_u32(&S.bar[1]), 1);
-    c_next = atomicAdd(R.queue, 1u);
-    n = rec_next<kTile>(G, R, tpb, nb, n_tiles, t, c_end, c_next, base, cb, cf, tinv);
-    if (n) rec_issue_raw<KW>(S.keys[0], S.info[0], smem_u32(&S.bar[0]), R, base, n, pol);
-  }
-  __syncwarp();
-  n = __shfl_sync(0xffffffffu, n, 0);
-  base = shfl0(base);
-  int buf = 0;
-  while (n) {
-    u64 nbase = 0;
-    unsigned nn = 0;
-    if (lane == 0) {
-      nn = rec_next<kTile>(G, R, tpb, nb, n_tiles, t, c_end, c_next, nbase, cb, cf, tinv);
-      if (nn) rec_issue_raw<KW>(S.keys[buf ^ 1], S.info[buf ^ 1], smem_u32(&S.bar[buf ^ 1]), R, nbase, nn, pol);
-    }
-    nn = __shfl_sync(0xffffffffu, nn, 0);
-    nbase = shfl0(nbase);
-    const unsigned bar = smem_u32(&S.bar[buf]);
-    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, (phases >> buf) & 1u, G.wait_limit));
-    if (!ok) {  // give up: report, let the copies in flight land (bounded), stop the warp
-      if (lane == 0) {
-        atomicOr(&G.status->flags, kFlagTimeout);
-        mbar_drain(bar, (phases >> buf) & 1u, G.wait_limit);
-        if (nn) mbar_drain(smem_u32(&S.bar[buf ^ 1]), (phases >> (buf ^ 1)) & 1u, G.wait_limit);
-      }
-      return;
-    }
-    phases ^= 1u << buf;
-    // the tile's marked records into the ring
+__global__ void __launch_bounds__(256) part_insert_kernel(const __grid_constant__ PartGeom G, const unsigned* keys,
+                                                          const u64* n_keys) {
+  const u64 n = __ldcg(n_keys);
+  unsigned acc_ins = 0;
+  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
+    const unsigned* c = keys + i * kKeyWords<KW>;
+    unsigned w[kKeyWords<KW>];
 #pragma unroll
-    for (int j = 0; j < kTile / 32; ++j) {
-      const unsigned i = j * 32 + lane;
-      const bool f = i < n && (S.info[buf][i] & kInfoFirst);
-      const unsigned m = __ballot_sync(0xffffffffu, f);
-      if (f) {
-        const unsigned e = (tail + __popc(m & ((1u << lane) - 1u))) & (kRing - 1);
-        if (KW == 1) S.rkeys[e] = S.keys[buf][i];
-        else reinterpret_cast<ulonglong2*>(S.rkeys)[e] = reinterpret_cast<const ulonglong2*>(S.keys[buf])[i];
-        S.rinfo[e] = S.info[buf][i];
-      }
-      tail += __popc(m);
-    }
-    __syncwarp();  // ring entries visible to every lane; buffer `buf` free for the next copy
-    while (tail - head >= 32) {
-      recount_round<KW>(G, S, (head + lane) & (kRing - 1), true);
-      head += 32;
-    }
-    __syncwarp();  // ring slots are rewritten by the next tile
-    n = nn;
-    base = nbase;
-    buf ^= 1;
-  }
-  recount_round<KW>(G, S, (head + lane) & (kRing - 1), lane < tail - head);
-}
-
-// ------------------------------------------------------------------ key filter
-//
-// After the Bloom pass: every key in the table sets its bits in its partition's key filter.
-// One CTA chunk = kKeyChunk consecutive slots of one partition (slot keys read once, in order).
-
-constexpr int kKeyThreads = 256;
-constexpr int kKeyChunk = kKeyThreads * 8;
-
-__global__ void __launch_bounds__(kKeyThreads) keyfilter_build_kernel(const __grid_constant__ PartGeom G) {
-  const u64 chunks_per_part = (G.Sp + kKeyChunk - 1) / kKeyChunk;
-  const u64 n_chunks = chunks_per_part * G.P;
-  for (u64 c = blockIdx.x; c < n_chunks; c += gridDim.x) {
-    const u64 p = c / chunks_per_part;
-    const u64 s0 = (c - p * chunks_per_part) * kKeyChunk;
-    const Slot* sub = G.table + p * G.Sp;
-    u64* kf = G.keyfilter + p * G.Wk;
-    // all of the thread's slot keys are loaded before the first atomic: the loads of a chunk
-    // are in flight together instead of one round trip each
-    constexpr int kPer = kKeyChunk / kKeyThreads;
-    ulonglong2 kv[kPer];
+    for (int x = 0; x < kKeyWords<KW>; ++x) w[x] = __ldcs(c + x);
+    unsigned v[10];
 #pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      const u64 i = s0 + (u64)j * kKeyThreads + threadIdx.x;
-      kv[j] = i < G.Sp ? __ldcs(reinterpret_cast<const ulonglong2*>(sub + i)) : make_ulonglong2(kEmpty, kEmpty);
+    for (int x = 0; x < 5; ++x) {
+      v[2 * x] = w[x] & 0xFFFFu;
+      v[2 * x + 1] = w[x] >> 16;
     }
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      if (kv[j].x == kEmpty && kv[j].y == kEmpty) continue;
-      const u64 h = key_hash(kv[j].x, kv[j].y);
-      atomicOr(kf + keyfilter_index(h, G.Wk), keyfilter_mask(h, G.bloom_h));
-    }
+    const u64 h = ((u64)w[6] << 32) | w[5];
+    const u64 hi = KW == 2 ? ((u64)w[kKeyWords<KW> - 1] << 32) | w[kKeyWords<KW> - 2] : 0ull;
+    acc_ins += emit_key(G, h, hi, v);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
+  if ((threadIdx.x & 31) == 0 && acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -739,97 +969,71 @@ cudaError_t allow_dynamic_smem(const void* fn, size_t need) {
   return need <= (size_t)limit ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-static int grid_for(const void* fn, int threads, size_t smem, int num_sms) {
+static u64 grid_for(const void* fn, int threads, size_t smem, int num_sms, u64 items) {
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem) != cudaSuccess) {
     cudaGetLastError();
     per_sm = 1;
   }
-  return num_sms * (per_sm > 0 ? per_sm : 1);
+  const u64 g = (u64)num_sms * (per_sm > 0 ? per_sm : 1);
+  return items < g ? items : g;
 }
 
-cudaError_t launch_part_scatter(const PartGeom& g, const PartWindows& w, const PartRecords& r,
-                                cudaStream_t stream, int num_sms) {
+cudaError_t launch_part_scatter(const PartGeom& g, const PartWindows& w, const PartTiles& t, cudaStream_t stream,
+                                int num_sms) {
   if (w.q1 <= w.q0) return cudaSuccess;
   const int kw = g.k > 32 ? 2 : 1;
-  const size_t smem = scatter_smem(g.P, kw);
+  const size_t smem = scatter_smem(g.log_b, kw);
   const void* fn = kw == 2 ? (const void*)part_scatter_kernel<2> : (const void*)part_scatter_kernel<1>;
   cudaError_t e = allow_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  const u64 tiles = (w.q1 - w.q0 + kScatterTile - 1) / kScatterTile;
-  u64 grid = grid_for(fn, kScatterThreads, smem, num_sms);
-  if (grid > tiles) grid = tiles;
-  if (kw == 2) part_scatter_kernel<2><<<(unsigned)grid, kScatterThreads, smem, stream>>>(g, w, r);
-  else part_scatter_kernel<1><<<(unsigned)grid, kScatterThreads, smem, stream>>>(g, w, r);
+  const unsigned grid =
+      (unsigned)grid_for(fn, kScatterThreads, smem, num_sms, (w.q1 - w.q0 + kScatterTile - 1) / kScatterTile);
+  if (kw == 2) part_scatter_kernel<2><<<grid, kScatterThreads, smem, stream>>>(g, w, t);
+  else part_scatter_kernel<1><<<grid, kScatterThreads, smem, stream>>>(g, w, t);
   return cudaGetLastError();
 }
 
-template <int KW, int RPT, unsigned MODE, bool GROUP>
-static cudaError_t launch_pass_rt(const PartGeom& g, const PartRecords& r, cudaStream_t stream, int num_sms) {
-  constexpr int tile = 32 * RPT;
-  if (r.p_begin > r.p_end || r.p_end > g.P) return cudaErrorInvalidValue;
-  const u64 tiles = (u64)(r.p_end - r.p_begin) * ((r.cap + tile - 1) / tile) +
-                    (r.overflow ? (r.ocap + tile - 1) / tile : 0);
-  if (tiles == 0) return cudaSuccess;
-  if ((r.cap | r.ocap) & 15 || (reinterpret_cast<uintptr_t>(r.keys) | reinterpret_cast<uintptr_t>(r.info)) & 15)
-    return cudaErrorInvalidValue;  // staging needs 16-record buckets on 16-byte boundaries
-  const void* fn = (const void*)part_pass_kernel<KW, RPT, MODE, GROUP>;
-  u64 grid = grid_for(fn, kPartThreads, 0, num_sms);
-  if (grid > tiles) grid = tiles;
-  cudaError_t e = cudaMemsetAsync(r.queue, 0, sizeof(unsigned), stream);  // the launch's tile queue
+cudaError_t launch_part_base(const unsigned long long* totals, const PartSplit& s, cudaStream_t stream) {
+  part_base_kernel<<<1, kBaseThreads, 0, stream>>>(totals, s.b0, s.b1, s.n_chunks, s.seg_base);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartSplit& s, cudaStream_t stream,
+                              int num_sms) {
+  if (t.n_tiles == 0 || s.b1 <= s.b0) return cudaSuccess;
+  if (s.chunk_tiles == 0 || s.chunk_tiles > kMaxChunkTiles) return cudaErrorInvalidValue;
+  const int kw = g.k > 32 ? 2 : 1;
+  const size_t smem = split_smem(s.chunk_tiles, g.sub_max, kw);
+  const void* fn = kw == 2 ? (const void*)part_split_kernel<2> : (const void*)part_split_kernel<1>;
+  cudaError_t e = allow_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  part_pass_kernel<KW, RPT, MODE, GROUP><<<(unsigned)grid, kPartThreads, 0, stream>>>(g, r);
+  const u64 items = (u64)((t.n_tiles + s.chunk_tiles - 1) / s.chunk_tiles) *
+                    ((s.b1 - s.b0 + kSplitBuckets - 1) / kSplitBuckets);
+  const unsigned grid = (unsigned)grid_for(fn, kSplitThreads, smem, num_sms, items);
+  if (kw == 2) part_split_kernel<2><<<grid, kSplitThreads, smem, stream>>>(g, t, s);
+  else part_split_kernel<1><<<grid, kSplitThreads, smem, stream>>>(g, t, s);
   return cudaGetLastError();
 }
 
-template <int KW>
-static cudaError_t launch_recount(const PartGeom& g, const PartRecords& r, cudaStream_t stream, int num_sms) {
-  constexpr int tile = RecountStage<KW>::kTile;
-  if (r.p_begin > r.p_end || r.p_end > g.P) return cudaErrorInvalidValue;
-  const u64 tiles = (u64)(r.p_end - r.p_begin) * ((r.cap + tile - 1) / tile) +
-                    (r.overflow ? (r.ocap + tile - 1) / tile : 0);
-  if (tiles == 0) return cudaSuccess;
-  if ((r.cap | r.ocap) & 15 || (reinterpret_cast<uintptr_t>(r.keys) | reinterpret_cast<uintptr_t>(r.info)) & 15)
-    return cudaErrorInvalidValue;  // staging needs 16-record buckets on 16-byte boundaries
-  const void* fn = (const void*)part_recount_kernel<KW>;
-  u64 grid = grid_for(fn, kPartThreads, 0, num_sms);
-  if (grid > tiles) grid = tiles;
-  cudaError_t e = cudaMemsetAsync(r.queue, 0, sizeof(unsigned), stream);  // the launch's tile queue
+cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms) {
+  if (s.b1 <= s.b0) return cudaSuccess;
+  const int kw = g.k > 32 ? 2 : 1;
+  const size_t smem = kw == 2 ? CountShape<2>::kSmem : CountShape<1>::kSmem;
+  const void* fn = kw == 2 ? (const void*)part_count_kernel<2> : (const void*)part_count_kernel<1>;
+  cudaError_t e = allow_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  part_recount_kernel<KW><<<(unsigned)grid, kPartThreads, 0, stream>>>(g, r);
+  const unsigned grid = (unsigned)grid_for(fn, kCountThreads, smem, num_sms, (u64)(s.b1 - s.b0) * g.sub_max);
+  if (kw == 2) part_count_kernel<2><<<grid, kCountThreads, smem, stream>>>(g, s);
+  else part_count_kernel<1><<<grid, kCountThreads, smem, stream>>>(g, s);
   return cudaGetLastError();
 }
 
-template <int KW, int RPT>
-static cudaError_t launch_pass_mode(const PartGeom& g, const PartRecords& r, unsigned mode, cudaStream_t stream,
-                                    int num_sms) {
-  // equal-key grouping (heavy hitters) is built for the 2-records-per-lane passes that count
-  const bool group = g.group && RPT == 2;
-  if (mode == kModeBloom)
-    return group ? launch_pass_rt<KW, RPT, kModeBloom, true>(g, r, stream, num_sms)
-                 : launch_pass_rt<KW, RPT, kModeBloom, false>(g, r, stream, num_sms);
-  if (mode == kModeCount)
-    return group ? launch_pass_rt<KW, RPT, kModeCount, true>(g, r, stream, num_sms)
-                 : launch_pass_rt<KW, RPT, kModeCount, false>(g, r, stream, num_sms);
-  return launch_recount<KW>(g, r, stream, num_sms);
-}
-
-cudaError_t launch_keyfilter_build(const PartGeom& g, cudaStream_t stream, int num_sms) {
-  if (!g.Wk || !g.keyfilter) return cudaSuccess;
-  const u64 chunks = g.P * ((g.Sp + kKeyChunk - 1) / kKeyChunk);
-  u64 grid = grid_for((const void*)keyfilter_build_kernel, kKeyThreads, 0, num_sms);
-  if (grid > chunks) grid = chunks;
-  keyfilter_build_kernel<<<(unsigned)grid, kKeyThreads, 0, stream>>>(g);
+cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms) {
+  const unsigned grid = (unsigned)num_sms * 8;  // the number of keys is known on the device only
+  if (g.k > 32) part_insert_kernel<2><<<grid, 256, 0, stream>>>(g, s.keys, s.n_keys);
+  else part_insert_kernel<1><<<grid, 256, 0, stream>>>(g, s.keys, s.n_keys);
   return cudaGetLastError();
-}
-
-cudaError_t launch_part_pass(const PartGeom& g, const PartRecords& r, unsigned mode, cudaStream_t stream,
-                             int num_sms) {
-  if (g.rpt >= 4)
-    return g.k > 32 ? launch_pass_mode<2, 4>(g, r, mode, stream, num_sms)
-                    : launch_pass_mode<1, 4>(g, r, mode, stream, num_sms);
-  return g.k > 32 ? launch_pass_mode<2, 2>(g, r, mode, stream, num_sms)
-                  : launch_pass_mode<1, 2>(g, r, mode, stream, num_sms);
 }
 
 }  // namespace kma
