@@ -1518,7 +1518,7 @@ int kmer_analysis_estimate(const kma_params* params, const char* seq, const char
   // device temporaries: sketch registers, the CTAs' heavy-hitter summaries, and (host input)
   // the reads, copied whole so that they are packed as one batch (the sampled stream is
   // defined on the positions of one packed batch)
-  const unsigned grid = hll_grid(p, h->num_sms);
+  const unsigned grid = hll_grid(p, params->k, h->num_sms);
   const u64 mg_n = (u64)grid * kMgBuckets * kMgCounters;
   std::vector<void*> temps;
   auto finish = [&](int code) {

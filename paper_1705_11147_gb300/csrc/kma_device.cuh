@@ -224,94 +224,142 @@ __device__ __forceinline__ bool load_window(const PassDesc& D, u64 q, Window& w)
   return load_window(D.codes, D.rcodes, D.inv, D.hq, D.k, D.canonical, q, w);
 }
 
-// Consecutive windows starting at q (a multiple of 8), one at a time: the state
-// holds the forward k-mer F and its reverse complement R of the current window, the next
-// bases to enter (MSB first), and the invalid / high-quality bits around the windows.
-struct RollingWindows {
-  u64 fhi, flo, rhi, rlo;  // F and R as 2k-bit numbers (first base most / least significant)
-  u64 nxt;                 // bases q + k, q + k + 1, ... (MSB first)
-  u64 iv0, iv1;            // invalid bits from q (MSB first), 128 of them
-  u64 hl, hr;              // hq bits from q - 1 (left extensions) and from q + k (right)
-  unsigned left;           // base at q - 1 (left extension of window q)
-  unsigned k;
+// Eight consecutive windows starting at q (a multiple of 8), in 32-bit words. The base streams
+// are aligned once per run (one funnel shift per word): fw holds the forward stream so that
+// window 0 ends with fw[2 KW - 1] and the following bases are in fw[2 KW], rv the reverse
+// complement stream from window 0 on. Window j is then 2 KW funnel shifts by the constant 2 j of
+// each, right-aligned as it is needed (rolling the two 128-bit numbers base by base took about
+// twice the instructions). Valid windows are a range of j: invalid positions before the first
+// window's eighth one cut it from below, those behind the first window's end from above.
+// Extension outcomes of all eight windows are put together in bytes beforehand, for either
+// orientation.
+template <int KW>
+struct WindowRun {
+  unsigned fw[2 * KW + 1], rv[2 * KW + 1];
+  unsigned m_top, m_next;     // masks of the words that hold bits 2k and above
+  unsigned valid;             // bit j: window j has no invalid position
+  unsigned ext[2][2];         // [forward?][j & 1]: byte j / 2 = outcome bits << 2 (left, right << 3)
 
-  __device__ __forceinline__ void init(const PartWindows& W, unsigned kk, u64 q) {
-    k = kk;
+  __device__ __forceinline__ static unsigned spread2(unsigned x) {  // 8 pairs -> 8 nibbles
+    x = (x | (x << 8)) & 0x00FF00FFu;
+    x = (x | (x << 4)) & 0x0F0F0F0Fu;
+    return (x | (x << 2)) & 0x33333333u;
+  }
+  __device__ __forceinline__ static unsigned spread1(unsigned x) {  // 8 bits -> 8 nibbles
+    x = (x | (x << 12)) & 0x000F000Fu;
+    x = (x | (x << 6)) & 0x03030303u;
+    return (x | (x << 3)) & 0x11111111u;
+  }
+  // Outcome nibbles (0-3 base, 4 none) of eight positions: codes in the top 16 bits of c and
+  // high-quality flags in the top 8 bits of u, first position first; comp: of the complements.
+  __device__ __forceinline__ static unsigned outcomes(unsigned c, unsigned u, unsigned& comp) {
+    c = __brev(c) & 0xFFFFu;  // first position in the low pair, its bits swapped
+    c = ((c >> 1) & 0x5555u) | ((c & 0x5555u) << 1);
+    const unsigned on = spread1(__brev(u) & 0xFFu), on3 = on * 3u;
+    const unsigned n = (spread2(c) & on3) | ((on ^ 0x11111111u) << 2);
+    comp = n ^ on3;
+    return n;
+  }
+
+  // With outcomes = false only the keys are wanted.
+  __device__ __forceinline__ void init(const PartWindows& W, unsigned k, u64 q, bool with_outcomes) {
+    const unsigned* c32 = reinterpret_cast<const unsigned*>(W.codes);   // word w of 16 positions: c32[w ^ 1]
+    const unsigned* r32 = reinterpret_cast<const unsigned*>(W.rcodes);  // word w of 16 positions: r32[w]
+    const unsigned* h32 = reinterpret_cast<const unsigned*>(W.hq);      // word w of 32 positions: h32[w ^ 1]
+    // forward: the 16 * 2 KW positions that end where window 0 ends, and the 16 behind them
+    // (positions before the arena are masked off below)
+    const u64 e = q + k;
+    const long long ie = (long long)(e >> 4);
+    const unsigned se = 2 * (unsigned)(e & 15);
+    unsigned prev = 0;
+#pragma unroll
+    for (int m = 0; m <= 2 * KW + 1; ++m) {
+      const long long w = ie - 2 * KW + m;
+      const unsigned x = c32[(u64)(w > 0 ? w : 0) ^ 1];
+      if (m > 0) fw[m - 1] = __funnelshift_l(x, prev, se);
+      prev = x;
+    }
+    const u64 iq = q >> 4;
+    const unsigned sq = 2 * (unsigned)(q & 15);
+    prev = r32[iq];
+#pragma unroll
+    for (int m = 0; m <= 2 * KW; ++m) {
+      const unsigned x = r32[iq + m + 1];
+      rv[m] = __funnelshift_r(prev, x, sq);
+      prev = x;
+    }
+    const unsigned over = 64u * KW - 2u * k;  // bits above the key: 0 .. 62
+    m_top = over >= 32 ? 0u : 0xFFFFFFFFu >> over;
+    m_next = over >= 32 ? 0xFFFFFFFFu >> (over - 32) : 0xFFFFFFFFu;
+    // validity
     const u64 v = q >> 6;
     const unsigned t = (unsigned)(q & 63);
     const u64 i0 = W.inv[v], i1 = W.inv[v + 1], i2 = W.inv[v + 2];
-    iv0 = fshl(i0, i1, t);
-    iv1 = fshl(i1, i2, t);
-    const u64 h0 = W.hq[v];
-    if (q > 0) {
-      const u64 vl = (q - 1) >> 6;
-      hl = fshl(W.hq[vl], W.hq[vl + 1], (unsigned)((q - 1) & 63));
-      left = code_at(W.codes, q - 1);
+    const u64 b0 = fshl(i0, i1, t), b1 = fshl(i1, i2, t);  // invalid bits from q, first in the top bit
+    if (k >= 8) {
+      const unsigned low = (unsigned)(b0 >> 57);                             // positions 0 .. 6
+      const unsigned high = (unsigned)(((b0 << k) | (b1 >> (64 - k))) >> 57);  // positions k .. k + 6
+      const unsigned from = low ? 8u - (unsigned)__ffs(low) : 0u;            // behind the last of the former
+      const unsigned upto = high ? (unsigned)__clz(high) - 25u : 7u;         // the first of the latter ends it
+      const bool all_bad = k > 7 && ((b0 << 7) >> (71 - k)) != 0;            // positions 7 .. k - 1
+      valid = all_bad ? 0u : (0xFFu << from) & (0xFFu >> (7 - upto));
     } else {
-      hl = h0 >> 1;  // no position before the arena: unusable
-      left = 0;
+      valid = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) valid |= (((b0 << j) >> (64 - k)) == 0 ? 1u : 0u) << j;
     }
-    const u64 qr = q + k, vr = qr >> 6;
-    hr = fshl(W.hq[vr], W.hq[vr + 1], (unsigned)(qr & 63));
-    const u64 wr = qr >> 5;
-    nxt = fshl(W.codes[wr], W.codes[wr + 1], 2 * (unsigned)(qr & 31));
-    // window q itself, as in load_window
-    const u64 wi = q >> 5;
-    const unsigned sh2 = 2 * (unsigned)(q & 31);
-    const u64 a = W.codes[wi], b = W.codes[wi + 1];
-    const u64 top = fshl(a, b, sh2);
-    const u64 r0 = W.rcodes[wi], r1 = W.rcodes[wi + 1];
-    const u64 bot = fshr(r0, r1, sh2);
-    if (k > 32) {
-      const u64 mid = fshl(b, W.codes[wi + 2], sh2);
-      const unsigned sh = 128 - 2 * k;
-      flo = (mid >> sh) | (top << (64 - sh));
-      fhi = top >> sh;
-      rlo = bot;
-      rhi = fshr(r1, W.rcodes[wi + 2], sh2) & ((1ull << (2 * k - 64)) - 1);
-    } else {
-      flo = top >> (64 - 2 * k);
-      fhi = 0;
-      rlo = k == 32 ? bot : bot & ((1ull << (2 * k)) - 1);
-      rhi = 0;
+    if (with_outcomes) {
+      // left: positions q - 1 .. q + 6 (none before the arena), right: e .. e + 7
+      unsigned lc = 0, lu = 0;
+      if (q > 0) {
+        const u64 p = q - 1;
+        lc = __funnelshift_l(c32[((p >> 4) + 1) ^ 1], c32[(p >> 4) ^ 1], 2 * (unsigned)(p & 15));
+        lu = __funnelshift_l(h32[((p >> 5) + 1) ^ 1], h32[(p >> 5) ^ 1], (unsigned)(p & 31));
+      } else {
+        lc = c32[1] >> 2;
+        lu = h32[1] >> 1;
+      }
+      const unsigned ru = __funnelshift_l(h32[((e >> 5) + 1) ^ 1], h32[(e >> 5) ^ 1], (unsigned)(e & 31));
+      unsigned lcomp, rcomp;
+      const unsigned l = outcomes(lc, lu, lcomp), r = outcomes(fw[2 * KW], ru, rcomp);
+      constexpr unsigned kEven = 0x07070707u;
+      ext[1][0] = ((l & kEven) << 2) | ((r & kEven) << 5);
+      ext[1][1] = (((l >> 4) & kEven) << 2) | (((r >> 4) & kEven) << 5);
+      ext[0][0] = ((rcomp & kEven) << 2) | ((lcomp & kEven) << 5);
+      ext[0][1] = (((rcomp >> 4) & kEven) << 2) | (((lcomp >> 4) & kEven) << 5);
     }
   }
 
-  // Window j of the run (the state holds window j): valid flag and the canonical window.
-  __device__ __forceinline__ bool get(unsigned j, unsigned canonical, Window& w) const {
-    const u64 bad = (j ? (iv0 << j) | (iv1 >> (64 - j)) : iv0) >> (64 - k);
-    if (bad) return false;
-    const unsigned ab = (unsigned)(nxt >> 62);              // base q + j + k
-    const bool au = (hr >> (63 - j)) & 1u;
-    const bool bu = (hl >> (63 - j)) & 1u;                 // base q + j - 1
-    const bool forward = !canonical || (fhi < rhi) || (fhi == rhi && flo <= rlo);
-    if (forward) {
-      w.lo = flo; w.hi = fhi;
-      w.lb = left; w.lu = bu;
-      w.rb = ab; w.ru = au;
-    } else {
-      w.lo = rlo; w.hi = rhi;
-      w.lb = 3u - ab; w.lu = au;
-      w.rb = 3u - left; w.ru = bu;
+  // Canonical key of window j (a constant when unrolled); returns whether it is read forward.
+  __device__ __forceinline__ bool key(int j, unsigned canonical, u64& lo, u64& hi) const {
+    unsigned f[2 * KW], r[2 * KW];  // least significant word first
+#pragma unroll
+    for (int m = 0; m < 2 * KW; ++m) {
+      f[2 * KW - 1 - m] = __funnelshift_l(fw[m + 1], fw[m], 2 * j);
+      r[m] = __funnelshift_r(rv[m], rv[m + 1], 2 * j);
     }
-    return true;
+    f[2 * KW - 1] &= m_top;
+    r[2 * KW - 1] &= m_top;
+    f[2 * KW - 2] &= m_next;
+    r[2 * KW - 2] &= m_next;
+    const u64 f0 = ((u64)f[1] << 32) | f[0], r0 = ((u64)r[1] << 32) | r[0];
+    if (KW == 1) {
+      const bool forward = !canonical || f0 <= r0;
+      lo = forward ? f0 : r0;
+      hi = 0;
+      return forward;
+    }
+    const u64 f1 = ((u64)f[2 * KW - 1] << 32) | f[2 * KW - 2], r1 = ((u64)r[2 * KW - 1] << 32) | r[2 * KW - 2];
+    const bool forward = !canonical || f1 < r1 || (f1 == r1 && f0 <= r0);
+    lo = forward ? f0 : r0;
+    hi = forward ? f1 : r1;
+    return forward;
   }
 
-  // Move to the next window: the base at q + j + k enters, the first base leaves.
-  __device__ __forceinline__ void roll() {
-    const unsigned b = (unsigned)(nxt >> 62);
-    nxt <<= 2;
-    if (k > 32) {
-      left = (unsigned)(fhi >> (2 * k - 66)) & 3u;
-      fhi = ((fhi << 2) | (flo >> 62)) & ((1ull << (2 * k - 64)) - 1);
-      flo = (flo << 2) | b;
-      rlo = (rlo >> 2) | (rhi << 62);
-      rhi = (rhi >> 2) | ((u64)(3u - b) << (2 * k - 66));
-    } else {
-      left = (unsigned)(flo >> (2 * k - 2)) & 3u;
-      flo = ((flo << 2) | b) & (k == 32 ? ~0ull : ((1ull << (2 * k)) - 1));
-      rlo = (rlo >> 2) | ((u64)(3u - b) << (2 * k - 2));
-    }
+  // Outcome bits of window j in the top byte (<< 26), read forward or not.
+  __device__ __forceinline__ unsigned info(int j, bool forward) const {
+    const unsigned w = forward ? ext[1][j & 1] : ext[0][j & 1];
+    return __byte_perm(w, 0u, 0x0444u | ((unsigned)(j >> 1) << 12));
   }
 };
 

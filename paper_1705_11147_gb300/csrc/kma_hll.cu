@@ -10,7 +10,7 @@
 // maximum. The estimate itself is computed on the host (kma_api.cu).
 //
 // Each CTA keeps its own registers in shared memory (32-bit words, shared-memory atomicMax),
-// walks tiles of 4096 window starts with the same rolling extraction as the scatter, and
+// walks tiles of 4096 window starts with the same extraction as the scatter, and
 // merges its registers into the global ones once at the end.
 //
 // Heavy hitters (Section 5.1: frequent k-mers are identified during this same pass, so that
@@ -42,6 +42,7 @@ __host__ __device__ constexpr size_t hll_smem(unsigned p) {
          (size_t)kMgBuckets * 8 + 16;                         // items per bucket, item count
 }
 
+template <int KW>
 __global__ void __launch_bounds__(kHllThreads) hll_kernel(const __grid_constant__ PartWindows W, unsigned k,
                                                           unsigned canonical, unsigned n_parts, unsigned part,
                                                           unsigned p, unsigned* regs, DevStatus* st,
@@ -68,28 +69,26 @@ __global__ void __launch_bounds__(kHllThreads) hll_kernel(const __grid_constant_
   for (u64 t = blockIdx.x; t < n_tiles; t += gridDim.x) {
     const u64 q = W.q0 + t * kHllTile + (u64)threadIdx.x * kHllWpt;
     if (q < W.q1) {  // q1 - q0 is a multiple of 64: all kHllWpt starts are inside
-      RollingWindows rw;
-      rw.init(W, k, q);
+      WindowRun<KW> run;
+      run.init(W, k, q, false);
 #pragma unroll
       for (int j = 0; j < kHllWpt; ++j) {
-        Window w;
-        if (rw.get(j, canonical, w)) {
-          const u64 h = key_hash(w.lo, w.hi);
-          if (n_parts <= 1 || owner_of(h, n_parts) == part) {
-            ++acc_valid;
-            const unsigned idx = (unsigned)(h >> (64 - p));
-            const u64 rest = h << p;
-            const unsigned rank = rest ? (unsigned)__clzll(rest) + 1u : 64u - p + 1u;
-            atomicMax(&s_reg[idx], rank);
-            if (mg.lo && (((q + j) & ((1u << kMgSampleShift) - 1)) == 0)) {  // sampled window
-              const unsigned slot = atomicAdd(s_nit, 1u);
-              it_lo[slot] = w.lo;
-              it_hi[slot] = w.hi;
-              it_b[slot] = (unsigned)(h >> (64 - kMgBucketBits));
-            }
-          }
+        if (!((run.valid >> j) & 1u)) continue;
+        u64 lo, hi;
+        run.key(j, canonical, lo, hi);
+        const u64 h = key_hash(lo, hi);
+        if (n_parts > 1 && owner_of(h, n_parts) != part) continue;
+        ++acc_valid;
+        const unsigned idx = (unsigned)(h >> (64 - p));
+        const u64 rest = h << p;
+        const unsigned rank = rest ? (unsigned)__clzll(rest) + 1u : 64u - p + 1u;
+        atomicMax(&s_reg[idx], rank);
+        if (mg.lo && (((q + j) & ((1u << kMgSampleShift) - 1)) == 0)) {  // sampled window
+          const unsigned slot = atomicAdd(s_nit, 1u);
+          it_lo[slot] = lo;
+          it_hi[slot] = hi;
+          it_b[slot] = (unsigned)(h >> (64 - kMgBucketBits));
         }
-        if (j + 1 < kHllWpt) rw.roll();
       }
     }
     if (!mg.lo) continue;  // block-uniform
@@ -147,10 +146,11 @@ __global__ void __launch_bounds__(kHllThreads) hll_kernel(const __grid_constant_
   if ((threadIdx.x & 31) == 0 && acc_valid) atomicAdd(&st->valid_windows, (u64)acc_valid);
 }
 
-unsigned hll_grid(unsigned p, int num_sms) {
+unsigned hll_grid(unsigned p, unsigned k, int num_sms) {
   int per_sm = 0;
-  if (allow_dynamic_smem((const void*)hll_kernel, hll_smem(p)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hll_kernel, kHllThreads, hll_smem(p)) != cudaSuccess) {
+  const void* fn = k > 32 ? (const void*)hll_kernel<2> : (const void*)hll_kernel<1>;
+  if (allow_dynamic_smem(fn, hll_smem(p)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kHllThreads, hll_smem(p)) != cudaSuccess) {
     cudaGetLastError();
     per_sm = 1;
   }
@@ -161,10 +161,11 @@ cudaError_t launch_hll(const PartWindows& w, unsigned k, unsigned canonical, uns
                        unsigned p, unsigned* regs, DevStatus* st, const MgOut& mg, unsigned grid,
                        cudaStream_t stream) {
   const size_t smem = hll_smem(p);
-  cudaError_t e = allow_dynamic_smem((const void*)hll_kernel, smem);
+  cudaError_t e = allow_dynamic_smem(k > 32 ? (const void*)hll_kernel<2> : (const void*)hll_kernel<1>, smem);
   if (e != cudaSuccess) return e;
   // every CTA runs (and writes its summaries) even when there are fewer tiles than CTAs
-  hll_kernel<<<grid, kHllThreads, smem, stream>>>(w, k, canonical, n_parts, part, p, regs, st, mg);
+  if (k > 32) hll_kernel<2><<<grid, kHllThreads, smem, stream>>>(w, k, canonical, n_parts, part, p, regs, st, mg);
+  else hll_kernel<1><<<grid, kHllThreads, smem, stream>>>(w, k, canonical, n_parts, part, p, regs, st, mg);
   return cudaGetLastError();
 }
 

@@ -235,7 +235,7 @@ cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartS
                               int num_sms);
 cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
 cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
-constexpr unsigned kMaxKeyWords = 9;           // words of one counted key in the list
+constexpr unsigned kMaxKeyWords = 10;          // words of one counted key in the list
 
 // FASTQ parsing (kma_fastq.cu) and the device-wide exclusive scan it uses.
 unsigned long long scan_scratch_items(unsigned long long n);
@@ -289,7 +289,7 @@ cudaError_t allow_dynamic_smem(const void* fn, size_t need);
 
 // HyperLogLog registers (2^p, 32-bit each) of the windows [w.q0, w.q1), and the heavy-hitter
 // summaries of `grid` CTAs (kma_hll.cu); hll_grid gives the number of resident CTAs.
-unsigned hll_grid(unsigned p, int num_sms);
+unsigned hll_grid(unsigned p, unsigned k, int num_sms);
 cudaError_t launch_hll(const PartWindows& w, unsigned k, unsigned canonical, unsigned n_parts, unsigned part,
                        unsigned p, unsigned* regs, DevStatus* st, const MgOut& mg, unsigned grid,
                        cudaStream_t stream);

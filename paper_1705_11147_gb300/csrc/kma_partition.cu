@@ -112,9 +112,8 @@ __device__ __forceinline__ unsigned block_scan(unsigned v, unsigned* wsum, unsig
 //
 // One tile = 8192 consecutive window starts; thread t takes the kScatterWpt consecutive starts
 // t * kScatterWpt + j.
-//  1. extract the windows (one set of word loads per thread, then the forward k-mer and its
-//     reverse complement are rolled one base at a time), stage the records in shared memory,
-//     rank each inside its bucket for this tile (shared-memory atomics);
+//  1. extract the windows (WindowRun), stage the records in shared memory, rank each inside its
+//     bucket for this tile (shared-memory atomics);
 //  2. exclusive scan of the bucket counts: the tile's offset row;
 //  3. the staged records into bucket order (through registers, in place), and the sorted tile to
 //     HBM with bulk copies.
@@ -154,25 +153,22 @@ __global__ void __launch_bounds__(kScatterThreads, 1) part_scatter_kernel(const 
     for (int j = 0; j < kScatterWpt; ++j) pr[j] = 0xFFFFFFFFu;
     const u64 q = W.q0 + (u64)t * kScatterTile + (u64)tid * kScatterWpt;
     if (q < W.q1) {  // q1 - q0 is a multiple of 64: all kScatterWpt starts are inside
-      RollingWindows rw;
-      rw.init(W, G.k, q);
+      WindowRun<KW> run;
+      run.init(W, G.k, q, true);
 #pragma unroll
       for (int j = 0; j < kScatterWpt; ++j) {
-        Window w;
-        if (rw.get(j, G.canonical, w)) {
-          const u64 h = key_hash(w.lo, w.hi);
-          if (G.n_parts <= 1 || owner_of(h, G.n_parts) == G.part) {
-            ++acc_valid;
-            const unsigned slot = j * kScatterThreads + tid;
-            const unsigned p = (unsigned)(h >> (64 - G.log_b));
-            pr[j] = (p << 13) | atomicAdd(&s_bin[p], 1u);
-            const unsigned info = (w.lu ? w.lb : 4u) | ((w.ru ? w.rb : 4u) << 3);
-            const u64 r = (h & kHashMask) | ((u64)info << (64 - kInfoBits));
-            if (KW == 1) s_rec[slot] = r;
-            else reinterpret_cast<ulonglong2*>(s_rec)[slot] = make_ulonglong2(r, w.hi);
-          }
-        }
-        if (j + 1 < kScatterWpt) rw.roll();
+        if (!((run.valid >> j) & 1u)) continue;
+        u64 lo, hi;
+        const bool forward = run.key(j, G.canonical, lo, hi);
+        const u64 h = key_hash(lo, hi);
+        if (G.n_parts > 1 && owner_of(h, G.n_parts) != G.part) continue;
+        ++acc_valid;
+        const unsigned slot = j * kScatterThreads + tid, top = (unsigned)(h >> 32);
+        const unsigned p = top >> (32 - G.log_b);
+        pr[j] = (p << 13) | atomicAdd(&s_bin[p], 1u);
+        const u64 r = ((u64)((top & (unsigned)(kHashMask >> 32)) | run.info(j, forward)) << 32) | (unsigned)h;
+        if (KW == 1) s_rec[slot] = r;
+        else reinterpret_cast<ulonglong2*>(s_rec)[slot] = make_ulonglong2(r, hi);
       }
     }
     __syncthreads();
@@ -453,13 +449,12 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 //
 // One work item = one sub-bucket, brought into shared memory by bulk copies while the previous
 // one is counted (two buffers, two CTAs per SM). Then
-//  1. every record writes its number at the entry its hash picks, the last one wins; after a
-//     barrier it compares its key with the winner's: equal keys share the winner as their
-//     representative, without an atomic or a loop;
-//  2. the others (about one in eight) find theirs in a second table by compare-and-swap and
-//     probing, compacted into full warps first;
+//  1. every record writes its number at the entry its hash picks, the last one wins;
+//  2. it compares its key with the winner's: equal keys share the winner as their representative,
+//     without an atomic or a loop. The others (about one in eight) find theirs in a second table
+//     by compare-and-swap and probing, compacted into full warps first;
 //  3. representatives that another record joined take a block of ten 16-bit counters (a staged
-//     sub-bucket has fewer than 2^16 records), and
+//     sub-bucket has fewer than 2^16 records);
 //  4. every record of such a key adds its two outcomes;
 //  5. these keys with their counters (all keys without the singleton filter) are appended to a
 //     list, which part_insert_kernel puts into the HBM table: a few keys per sub-bucket would
@@ -473,29 +468,35 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 constexpr int kCountThreads = 512;
 constexpr int kCountCtas = 2;                // per SM
 constexpr unsigned kEntries = 4096;          // first entries, 16 bits
-constexpr unsigned kEntries2 = 2048;         // second table, 32 bits
+constexpr unsigned kEntries2 = 1024;         // second table, 32 bits
 constexpr unsigned kNoEntry = 0xFFFFFFFFu;   // empty entry
 constexpr unsigned kOnce = 0xFFFFu;          // counter block of a representative nobody joined, and of no representative
 constexpr unsigned kJoined = 0xFFFEu;        // joined, block not taken yet
 constexpr unsigned kLone = 0x8000u;          // without the singleton filter: number among the keys seen once
 constexpr unsigned kRangeBits = 20;          // hash bits 21..40: count_large takes a range of them at a time
 
-// An entry of the list of counted keys: five words of 16-bit counter pairs (left A C G T none,
-// right A C G T none), then h and hi.
+// Counters of a key in 16-bit halves of six words: left A C G T none, (a half not used), right
+// A C G T none, (not used). The outcome bits of a record lie in the top byte of its first word:
+// v = outcome bits << 2. Byte offset of the counter's word, and 1 in the counter's half of it:
+__device__ __forceinline__ unsigned left_word(unsigned v) { return (v >> 1) & 12u; }
+__device__ __forceinline__ unsigned left_one(unsigned v) { return 1u << ((v << 2) & 16u); }
+__device__ __forceinline__ unsigned right_word(unsigned v) { return 12u + ((v >> 4) & 12u); }
+__device__ __forceinline__ unsigned right_one(unsigned v) { return 1u << ((v >> 1) & 16u); }
+constexpr unsigned kCtrWords = 6;
+
+// An entry of the list of counted keys: the six counter words (the half not used of the third
+// one is undefined), then h and hi.
 template <int KW>
-constexpr unsigned kKeyWords = 5 + 2 * KW;
+constexpr unsigned kKeyWords = kCtrWords + 2 * KW;
 
 template <int KW>
 struct CountShape {
   static constexpr unsigned kCap = KW == 1 ? kCountCap1 : kCountCap2;
-  static constexpr unsigned kItems = (kCap + kCountThreads - 1) / kCountThreads;
-  static constexpr unsigned kCtrWords = 6;   // 16-bit counter pairs, then the key's representative
   static constexpr size_t kRec = (size_t)kCap * KW * 8;
   static constexpr size_t kIdx = ((size_t)kCap * 2 + 15) & ~(size_t)15;  // representative; counter block
-  // the counters take the room of the entries, the second table and the list of step 2
-  static constexpr size_t kTab = (size_t)kEntries * 2 + kEntries2 * 4 + kIdx;
+  static constexpr size_t kTab = (size_t)kEntries * 2 + kEntries2 * 4 + kIdx;  // entries, second table, list of step 2
   static constexpr size_t kCtr = ((size_t)(kCap / 2) * kCtrWords * 4 + 15) & ~(size_t)15;
-  static constexpr size_t kSmem = 2 * kRec + 2 * kIdx + (kTab > kCtr ? kTab : kCtr);
+  static constexpr size_t kSmem = 2 * kRec + 2 * kIdx + (kTab > kCtr ? kTab : kCtr);  // steps 1 and 2 share the counters' room
   // count_large: keys and left counters where the representatives begin, right counters in the
   // buffer that is not being filled
   static constexpr unsigned kLargeSlots = 1024;
@@ -666,114 +667,102 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
   using C = CountShape<KW>;
   extern __shared__ __align__(128) unsigned char s_raw[];
   __shared__ __align__(8) unsigned long long s_bar[2];
-  __shared__ u64 s_fill[2], s_base;
-  __shared__ unsigned s_nctr, s_nlone, s_nlist, s_crowded;
-  const unsigned tid = threadIdx.x, lane = tid & 31;
-  unsigned char* s_var = s_raw + 2 * C::kRec + 2 * C::kIdx;
+  __shared__ u64 s_fill[2], s_ahead, s_base;  // s_ahead: records of the item after the one whose copy is under way
+  __shared__ unsigned s_nctr, s_nlone, s_nlist, s_state;
+  const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   unsigned short* s_rep = reinterpret_cast<unsigned short*>(s_raw + 2 * C::kRec);           // [cap] representative
   unsigned short* s_q = reinterpret_cast<unsigned short*>(s_raw + 2 * C::kRec + C::kIdx);   // [cap] its counter block
-  unsigned* s_ctr = reinterpret_cast<unsigned*>(s_var);                                     // [cap / 2][kCtrWords]
-  unsigned* s_ent2 = reinterpret_cast<unsigned*>(s_var);                                    // [entries2]
+  unsigned* s_ent2 = reinterpret_cast<unsigned*>(s_raw + 2 * C::kRec + 2 * C::kIdx);        // [entries2]
   unsigned short* s_ent = reinterpret_cast<unsigned short*>(s_ent2 + kEntries2);            // [entries]
-  unsigned short* s_list = s_ent + kEntries;                                                // [cap] not settled yet
+  unsigned short* s_list = s_ent + kEntries;                                                // [cap] not settled yet (step 2)
+  unsigned char* s_ctr = s_raw + 2 * C::kRec + 2 * C::kIdx;                                 // [cap / 2][kCtrWords * 4]
   const unsigned n_sub = sub_buckets(G);
-  const u64 n_items = (u64)(S.b1 - S.b0) * n_sub;
+  const unsigned n_items = (S.b1 - S.b0) * n_sub;  // at most 2^22
   unsigned acc_ins = 0, acc_first = 0;  // per thread: below 2^32
   // thread 0: copy a sub-bucket's records into buffer `buf`
-  auto issue = [&](unsigned buf, u64 item, u64 fill) {
+  auto issue = [&](unsigned buf, unsigned item, u64 fill) {
     s_fill[buf] = fill;
     const unsigned n = fill < G.cap ? (unsigned)fill : G.cap;
     const unsigned bytes = (n * (8 * KW) + 15u) & ~15u, bar = smem_u32(&s_bar[buf]);
     fence_proxy_async_smem();
     mbar_expect_tx(bar, bytes);
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(S.recs + item * G.cap * KW);
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(S.recs + (u64)item * G.cap * KW);
     const unsigned dst = smem_u32(s_raw) + buf * (unsigned)C::kRec;
     for (unsigned o = 0; o < bytes; o += 16384u) tma_load_1d(dst + o, src + o, bytes - o < 16384u ? bytes - o : 16384u, bar);
   };
-  u64 ahead = 0;  // thread 0: records of the item after the one whose copy is under way
   if (tid == 0) {
     mbar_init(smem_u32(&s_bar[0]), 1);
     mbar_init(smem_u32(&s_bar[1]), 1);
+    s_state = s_nlist = 0;
     if (blockIdx.x < n_items) issue(0, blockIdx.x, __ldcg(&S.fill[blockIdx.x]));
-    if (blockIdx.x + (u64)gridDim.x < n_items) ahead = __ldcg(&S.fill[blockIdx.x + gridDim.x]);
+    if (blockIdx.x + gridDim.x < n_items) s_ahead = __ldcg(&S.fill[blockIdx.x + gridDim.x]);
   }
+  __syncthreads();
   unsigned phases = 0, buf = 0;  // bit b: parity to wait for on buffer b
-  for (u64 item = blockIdx.x; item < n_items; item += gridDim.x, buf ^= 1) {
-    __syncthreads();  // the previous sub-bucket's memory is free (and the barriers are initialised)
-    if (tid == 0) {
-      const u64 next = item + gridDim.x;
-      if (next < n_items) issue(buf ^ 1, next, ahead);
-      if (next + gridDim.x < n_items) ahead = __ldcg(&S.fill[next + gridDim.x]);
-      s_nctr = s_nlone = s_nlist = s_crowded = 0;
+  for (unsigned item = blockIdx.x; item < n_items; item += gridDim.x, buf ^= 1) {
+    // bit 0 of s_state: a wait gave up; bit 1: the second table is full
+    if (!mbar_wait_bounded(smem_u32(&s_bar[buf]), (phases >> buf) & 1u, kWaitPolls)) atomicOr(&s_state, 1u);
+    __syncthreads();  // everyone is done with the previous sub-bucket
+    const u64 fill = s_fill[buf];
+    const unsigned n = fill < G.cap ? (unsigned)fill : G.cap;
+    u64* s_rec = reinterpret_cast<u64*>(s_raw + buf * C::kRec);  // [cap * KW]
+    // 1: numbers to the first entries
+#pragma unroll 2
+    for (unsigned x = tid; x < n; x += kCountThreads) {
+      s_ent[(unsigned)s_rec[(size_t)x * KW] & (kEntries - 1)] = (unsigned short)x;
+      s_q[x] = (unsigned short)kOnce;
     }
-    const bool ok = mbar_wait_bounded(smem_u32(&s_bar[buf]), (phases >> buf) & 1u, kWaitPolls);
-    phases ^= 1u << buf;
-    if (!__syncthreads_and(ok)) {  // give up: report, let the copies in flight land (bounded)
+    if (tid < kEntries2 / 4) reinterpret_cast<uint4*>(s_ent2)[tid] = make_uint4(kNoEntry, kNoEntry, kNoEntry, kNoEntry);
+    __syncthreads();
+    if (s_state) {  // uniform: a copy did not land. Report; those in flight land now (bounded)
       if (tid == 0) {
         atomicOr(&G.status->flags, kFlagTimeout);
-        mbar_drain(smem_u32(&s_bar[buf]), ((phases >> buf) & 1u) ^ 1u, kWaitPolls);
-        if (item + gridDim.x < n_items) mbar_drain(smem_u32(&s_bar[buf ^ 1]), (phases >> (buf ^ 1)) & 1u, kWaitPolls);
+        mbar_drain(smem_u32(&s_bar[buf]), (phases >> buf) & 1u, kWaitPolls);
       }
       break;
     }
-    const u64 fill = s_fill[buf];
-    const unsigned b = S.b0 + (unsigned)(item / n_sub);
-    u64* s_rec = reinterpret_cast<u64*>(s_raw + buf * C::kRec);  // [cap * KW]
-    const unsigned n = fill < G.cap ? (unsigned)fill : G.cap;
+    phases ^= 1u << buf;
+    if (tid == 0) {
+      const unsigned next = item + gridDim.x;
+      if (next < n_items) issue(buf ^ 1, next, s_ahead);
+      if (next + gridDim.x < n_items) s_ahead = __ldcg(&S.fill[next + gridDim.x]);
+      s_nctr = s_nlone = 0;
+    }
     auto large = [&]() {
       u64* keys = reinterpret_cast<u64*>(s_rep);
       count_large<KW>(G, S, keys, reinterpret_cast<unsigned*>(keys + C::kLargeSlots * KW), reinterpret_cast<unsigned*>(s_rec),
-                      b, (unsigned)(item % n_sub), n_sub, n, acc_ins, acc_first);
+                      S.b0 + item / n_sub, item % n_sub, n_sub, n, acc_ins, acc_first);
     };
     if (fill > G.cap) {  // uniform
       large();
       continue;
     }
-    if (n == 0) continue;
-    unsigned firsts = 0;  // representatives
-    // 1: a representative for every record
-    u64 h[C::kItems], hi[C::kItems];
-#pragma unroll
-    for (unsigned y = 0; y < C::kItems; ++y) {
-      const unsigned x = y * kCountThreads + tid;
-      h[y] = hi[y] = 0;
-      if (x < n) {
-        if (KW == 1) {
-          h[y] = s_rec[x] & kHashMask;
-        } else {
-          const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
-          h[y] = v.x & kHashMask;
-          hi[y] = v.y;
-        }
-        s_ent[(unsigned)h[y] & (kEntries - 1)] = (unsigned short)x;
-        s_q[x] = (unsigned short)kOnce;
-      }
-    }
-    reinterpret_cast<uint4*>(s_ent2)[tid] = make_uint4(kNoEntry, kNoEntry, kNoEntry, kNoEntry);
-    static_assert(kEntries2 == kCountThreads * 4, "one store per thread clears the second table");
-    __syncthreads();
-    // the key of record z is (ah, ahi)?
-    auto same_key = [&](unsigned z, u64 ah, u64 ahi) -> bool {
-      if (KW == 1) return (s_rec[z] & kHashMask) == ah;
+    // 2: a representative for every record. The key of record z is (a0, a1)?
+    auto same_key = [&](unsigned z, u64 a0, u64 a1) -> bool {
+      if (KW == 1) return ((s_rec[z] ^ a0) & kHashMask) == 0;
       const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[z];
-      return (v.x & kHashMask) == ah && v.y == ahi;
+      return (((v.x ^ a0) & kHashMask) | (v.y ^ a1)) == 0;
     };
-#pragma unroll
-    for (unsigned y = 0; y < C::kItems; ++y) {
-      const unsigned x = y * kCountThreads + tid;
-      if (x - lane >= n) break;  // the same for the whole warp
+    unsigned firsts = 0;
+#pragma unroll 1
+    for (unsigned x0 = tid - lane; x0 < n; x0 += kCountThreads) {
+      const unsigned x = x0 + lane;
       bool left = false;
       if (x < n) {
-        const unsigned z = s_ent[(unsigned)h[y] & (kEntries - 1)];
-        if (z == x) {
-          ++firsts;
-          s_rep[x] = (unsigned short)x;
-        } else if (same_key(z, h[y], hi[y])) {
-          s_q[z] = (unsigned short)kJoined;
-          s_rep[x] = (unsigned short)z;
+        u64 a0, a1 = 0;
+        if (KW == 1) {
+          a0 = s_rec[x];
         } else {
-          left = true;
+          const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
+          a0 = v.x;
+          a1 = v.y;
         }
+        const unsigned z = s_ent[(unsigned)a0 & (kEntries - 1)];
+        const bool same = same_key(z, a0, a1);
+        left = !same;
+        firsts += z == x;
+        if (same) s_rep[x] = (unsigned short)z;
+        if (same && z != x) s_q[z] = (unsigned short)kJoined;
       }
       const unsigned lm = __ballot_sync(0xffffffffu, left);
       if (lm) {
@@ -784,21 +773,18 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
       }
     }
     __syncthreads();
-    // 2: the others
-    const unsigned nl = s_nlist;
-    for (unsigned i = tid; i < nl; i += kCountThreads) {
+    for (unsigned i = tid; i < s_nlist; i += kCountThreads) {
       const unsigned x = s_list[i];
-      u64 kh, khi = 0;
+      u64 a0, a1 = 0;
       if (KW == 1) {
-        kh = s_rec[x] & kHashMask;
+        a0 = s_rec[x];
       } else {
         const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
-        kh = v.x & kHashMask;
-        khi = v.y;
+        a0 = v.x;
+        a1 = v.y;
       }
-      unsigned pos = (unsigned)(kh >> 12) & (kEntries2 - 1), z;
-      const unsigned jump = (unsigned)(kh >> 23) | 1u;  // odd: comes by every entry
-      unsigned step = 0;
+      unsigned pos = (unsigned)(a0 >> 12) & (kEntries2 - 1), z = x, step = 0;
+      const unsigned jump = (unsigned)(a0 >> 22) | 1u;  // odd: comes by every entry
       for (; step < kEntries2; ++step) {
         z = *reinterpret_cast<volatile unsigned*>(&s_ent2[pos]);
         if (z == kNoEntry) {
@@ -809,26 +795,26 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
             break;
           }
         }
-        if (same_key(z, kh, khi)) {
+        if (same_key(z, a0, a1)) {
           s_q[z] = (unsigned short)kJoined;
           break;
         }
         pos = (pos + jump) & (kEntries2 - 1);
       }
-      if (step == kEntries2) s_crowded = 1;  // more keys than the second table holds
+      if (step == kEntries2) atomicOr(&s_state, 2u);  // more keys than the second table holds
       s_rep[x] = (unsigned short)z;
     }
     __syncthreads();
-    if (s_crowded) {  // uniform
+    if (s_state) {  // uniform
+      __syncthreads();
+      if (tid == 0) s_state = s_nlist = 0;
       large();
       continue;
     }
     acc_first += firsts;
     // 3: counter blocks
-#pragma unroll
-    for (unsigned y = 0; y < C::kItems; ++y) {
-      const unsigned x = y * kCountThreads + tid;
-      if (x - lane >= n) break;
+    for (unsigned x0 = warp * 32; x0 < n; x0 += kCountThreads) {
+      const unsigned x = x0 + lane;
       const unsigned q0 = x < n ? s_q[x] : kOnce;
       const unsigned mm = __ballot_sync(0xffffffffu, q0 == kJoined);
       if (mm) {
@@ -837,10 +823,10 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
         q = __shfl_sync(0xffffffffu, q, 0) + __popc(mm & ((1u << lane) - 1u));
         if (q0 == kJoined) {
           s_q[x] = (unsigned short)q;
-          unsigned* c = s_ctr + q * C::kCtrWords;
-#pragma unroll
-          for (int w = 0; w < 5; ++w) c[w] = 0;
-          c[5] = x;
+          uint2* c = reinterpret_cast<uint2*>(s_ctr + q * (kCtrWords * 4));
+          c[0] = make_uint2(0, 0);
+          c[1] = make_uint2(x << 16, 0);  // the representative's number, in the half not used
+          c[2] = make_uint2(0, 0);
         }
       }
       if (G.min_count <= 1) {
@@ -854,31 +840,31 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     }
     __syncthreads();
     // 4: outcomes
+    if (tid == 0) s_nlist = 0;
     if (tid == 0) s_base = s_nctr + s_nlone ? atomicAdd(S.n_keys, (u64)(s_nctr + s_nlone)) : 0;
     for (unsigned x = tid; x < n; x += kCountThreads) {
       const unsigned q = s_q[s_rep[x]];
       if (q < kLone) {
-        const u64 r = s_rec[(size_t)x * KW];
-        const unsigned l = left_outcome(r), o = 5u + right_outcome(r);
-        unsigned* c = s_ctr + q * C::kCtrWords;
-        atomicAdd(&c[l >> 1], 1u << ((l & 1u) * 16));
-        atomicAdd(&c[o >> 1], 1u << ((o & 1u) * 16));
+        const unsigned v = reinterpret_cast<const unsigned char*>(s_rec)[(size_t)x * (8 * KW) + 7];
+        unsigned char* c = s_ctr + q * (kCtrWords * 4);
+        atomicAdd(reinterpret_cast<unsigned*>(c + left_word(v)), left_one(v));
+        atomicAdd(reinterpret_cast<unsigned*>(c + right_word(v)), right_one(v));
       }
     }
     __syncthreads();
     // 5: to the list
     const unsigned nq = s_nctr;
-    const u64 htop = (u64)(b >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
+    const u64 htop = (u64)((S.b0 + item / n_sub) >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
     unsigned* out = S.keys + s_base * kKeyWords<KW>;
     for (unsigned e = tid; e < nq * kKeyWords<KW>; e += kCountThreads) {
       const unsigned q = e / kKeyWords<KW>, w = e - q * kKeyWords<KW>;
-      const unsigned* c = s_ctr + q * C::kCtrWords;
+      const unsigned* c = reinterpret_cast<const unsigned*>(s_ctr) + q * kCtrWords;
       unsigned v;
-      if (w < 5) {
+      if (w < kCtrWords) {
         v = c[w];
       } else {
-        v = reinterpret_cast<const unsigned*>(s_rec + (size_t)c[5] * KW)[w - 5];
-        if (w == 6) v = (v & (unsigned)(kHashMask >> 32)) | (unsigned)(htop >> 32);
+        v = reinterpret_cast<const unsigned*>(s_rec + (size_t)(c[2] >> 16) * KW)[w - kCtrWords];
+        if (w == kCtrWords + 1) v = (v & (unsigned)(kHashMask >> 32)) | (unsigned)(htop >> 32);
       }
       out[e] = v;
     }
@@ -887,14 +873,14 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
         const unsigned q = s_q[x];
         if (q < kLone || q >= kJoined) continue;
         const u64 r = s_rec[(size_t)x * KW];
-        const unsigned l = left_outcome(r), o = 5u + right_outcome(r);
+        const unsigned v = (unsigned)(r >> 56);
         unsigned* c = out + (size_t)(nq + (q & ~kLone)) * kKeyWords<KW>;
 #pragma unroll
-        for (unsigned w = 0; w < 5; ++w)
-          c[w] = ((l >> 1) == w ? 1u << ((l & 1u) * 16) : 0u) + ((o >> 1) == w ? 1u << ((o & 1u) * 16) : 0u);
+        for (unsigned w = 0; w < kCtrWords; ++w)
+          c[w] = (left_word(v) == 4 * w ? left_one(v) : 0u) + (right_word(v) == 4 * w ? right_one(v) : 0u);
         const u64 kh = (r & kHashMask) | htop;
-        c[5] = (unsigned)kh;
-        c[6] = (unsigned)(kh >> 32);
+        c[kCtrWords] = (unsigned)kh;
+        c[kCtrWords + 1] = (unsigned)(kh >> 32);
         if (KW == 2) {
           const u64 khi = s_rec[(size_t)x * KW + KW - 1];
           c[kKeyWords<KW> - 2] = (unsigned)khi;
@@ -926,17 +912,13 @@ __global__ void __launch_bounds__(256) part_insert_kernel(const __grid_constant_
   unsigned acc_ins = 0;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
     const unsigned* c = keys + i * kKeyWords<KW>;
-    unsigned w[kKeyWords<KW>];
+    uint2 w[kKeyWords<KW> / 2];
 #pragma unroll
-    for (int x = 0; x < kKeyWords<KW>; ++x) w[x] = __ldcs(c + x);
-    unsigned v[10];
-#pragma unroll
-    for (int x = 0; x < 5; ++x) {
-      v[2 * x] = w[x] & 0xFFFFu;
-      v[2 * x + 1] = w[x] >> 16;
-    }
-    const u64 h = ((u64)w[6] << 32) | w[5];
-    const u64 hi = KW == 2 ? ((u64)w[kKeyWords<KW> - 1] << 32) | w[kKeyWords<KW> - 2] : 0ull;
+    for (unsigned x = 0; x < kKeyWords<KW> / 2; ++x) w[x] = __ldcs(reinterpret_cast<const uint2*>(c) + x);
+    const unsigned v[10] = {w[0].x & 0xFFFFu, w[0].x >> 16, w[0].y & 0xFFFFu, w[0].y >> 16, w[1].x & 0xFFFFu,
+                            w[1].y & 0xFFFFu, w[1].y >> 16, w[2].x & 0xFFFFu, w[2].x >> 16, w[2].y & 0xFFFFu};
+    const u64 h = ((u64)w[3].y << 32) | w[3].x;
+    const u64 hi = KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull;
     acc_ins += emit_key(G, h, hi, v);
   }
 #pragma unroll
