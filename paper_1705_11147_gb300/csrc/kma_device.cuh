@@ -261,11 +261,13 @@ struct WindowRun {
     return n;
   }
 
-  // With outcomes = false only the keys are wanted.
-  __device__ __forceinline__ void init(const PartWindows& W, unsigned k, u64 q, bool with_outcomes) {
-    const unsigned* c32 = reinterpret_cast<const unsigned*>(W.codes);   // word w of 16 positions: c32[w ^ 1]
-    const unsigned* r32 = reinterpret_cast<const unsigned*>(W.rcodes);  // word w of 16 positions: r32[w]
-    const unsigned* h32 = reinterpret_cast<const unsigned*>(W.hq);      // word w of 32 positions: h32[w ^ 1]
+  // q counts from the first position of the words given (the arena's or a staged part of it),
+  // `first`: window q starts the arena. With outcomes = false only the keys are wanted.
+  __device__ __forceinline__ void init(const u64* codes, const u64* rcodes, const u64* inv, const u64* hq, unsigned k,
+                                       u64 q, bool first, bool with_outcomes) {
+    const unsigned* c32 = reinterpret_cast<const unsigned*>(codes);   // word w of 16 positions: c32[w ^ 1]
+    const unsigned* r32 = reinterpret_cast<const unsigned*>(rcodes);  // word w of 16 positions: r32[w]
+    const unsigned* h32 = reinterpret_cast<const unsigned*>(hq);      // word w of 32 positions: h32[w ^ 1]
     // forward: the 16 * 2 KW positions that end where window 0 ends, and the 16 behind them
     // (positions before the arena are masked off below)
     const u64 e = q + k;
@@ -294,7 +296,7 @@ struct WindowRun {
     // validity
     const u64 v = q >> 6;
     const unsigned t = (unsigned)(q & 63);
-    const u64 i0 = W.inv[v], i1 = W.inv[v + 1], i2 = W.inv[v + 2];
+    const u64 i0 = inv[v], i1 = inv[v + 1], i2 = inv[v + 2];
     const u64 b0 = fshl(i0, i1, t), b1 = fshl(i1, i2, t);  // invalid bits from q, first in the top bit
     if (k >= 8) {
       const unsigned low = (unsigned)(b0 >> 57);                             // positions 0 .. 6
@@ -311,7 +313,7 @@ struct WindowRun {
     if (with_outcomes) {
       // left: positions q - 1 .. q + 6 (none before the arena), right: e .. e + 7
       unsigned lc = 0, lu = 0;
-      if (q > 0) {
+      if (!first) {
         const u64 p = q - 1;
         lc = __funnelshift_l(c32[((p >> 4) + 1) ^ 1], c32[(p >> 4) ^ 1], 2 * (unsigned)(p & 15));
         lu = __funnelshift_l(h32[((p >> 5) + 1) ^ 1], h32[(p >> 5) ^ 1], (unsigned)(p & 31));

@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(kHllThreads) hll_kernel(const __grid_constant_
     const u64 q = W.q0 + t * kHllTile + (u64)threadIdx.x * kHllWpt;
     if (q < W.q1) {  // q1 - q0 is a multiple of 64: all kHllWpt starts are inside
       WindowRun<KW> run;
-      run.init(W, k, q, false);
+      run.init(W.codes, W.rcodes, W.inv, W.hq, k, q, q == 0, false);
 #pragma unroll
       for (int j = 0; j < kHllWpt; ++j) {
         if (!((run.valid >> j) & 1u)) continue;

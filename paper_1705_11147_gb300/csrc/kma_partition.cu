@@ -126,8 +126,15 @@ constexpr int kScatterTile = kScatterThreads * kScatterWpt;
 static_assert(kScatterTile == kPartTile && kScatterTile <= 8192, "ranks are 13 bits");
 constexpr int kScatterMaxPer = (1 << kMaxLogBuckets) / kScatterThreads;  // buckets per thread
 
+// The packed reads of the next tile are brought into shared memory while this one is sorted (as
+// loads from L2 they took a third of a tile's time): the tile's positions with up to 256 before
+// and 384 behind, in words of 128 positions from a multiple of 128 on.
+constexpr unsigned kArenaPositions = kScatterTile + 256 + 384;
+constexpr size_t kArenaStage = kArenaPositions / 4 * 2 + kArenaPositions / 8 * 2;  // codes, rcodes, inv, hq
+static_assert(kArenaPositions % 128 == 0, "every staged array starts on 16 bytes");
+
 __host__ __device__ constexpr size_t scatter_smem(unsigned log_b, int kw) {
-  return (size_t)kScatterTile * kw * 8 + ((size_t)4 << log_b) + 32 * 4;
+  return (size_t)kScatterTile * kw * 8 + 2 * kArenaStage + ((size_t)4 << log_b) + 32 * 4;
 }
 
 template <int KW>
@@ -136,40 +143,84 @@ __global__ void __launch_bounds__(kScatterThreads, 1) part_scatter_kernel(const 
                                                                           const __grid_constant__ PartTiles T) {
   extern __shared__ __align__(128) unsigned char s_raw[];
   const unsigned B = 1u << G.log_b;
+  __shared__ __align__(8) unsigned long long s_bar[2];
+  __shared__ unsigned s_lost;
   u64* s_rec = reinterpret_cast<u64*>(s_raw);                                  // [tile * KW]
-  unsigned* s_bin = reinterpret_cast<unsigned*>(s_rec + kScatterTile * KW);    // [B] counts, then offsets
+  unsigned char* s_arena = s_raw + (size_t)kScatterTile * KW * 8;              // [2][codes, rcodes, inv, hq]
+  unsigned* s_bin = reinterpret_cast<unsigned*>(s_arena + 2 * kArenaStage);    // [B] counts, then offsets
   unsigned* s_wsum = s_bin + B;                                                // [32]
   const unsigned tid = threadIdx.x, lane = tid & 31;
   const unsigned n_tiles = (unsigned)((W.q1 - W.q0 + kScatterTile - 1) / kScatterTile);
   const unsigned per = (B + kScatterThreads - 1) / kScatterThreads;
-  unsigned acc_valid = 0;
+  // first staged position of tile t, and (thread 0) its copies into buffer `buf`
+  auto stage_from = [&](unsigned t) -> u64 {
+    const u64 q = W.q0 + (u64)t * kScatterTile;
+    return (q > 128 ? q - 128 : 0) & ~127ull;
+  };
+  auto issue = [&](unsigned t, unsigned buf) {
+    const u64 q = W.q0 + (u64)t * kScatterTile, from = stage_from(t);
+    const u64 end = ((q + kScatterTile < W.q1 ? q + kScatterTile : W.q1) + 256 + 127) & ~127ull;
+    const unsigned n = (unsigned)(end - from);  // a multiple of 128, at most kArenaPositions
+    const unsigned bar = smem_u32(&s_bar[buf]), dst = smem_u32(s_arena) + buf * (unsigned)kArenaStage;
+    fence_proxy_async_smem();
+    mbar_expect_tx(bar, n / 4 * 2 + n / 8 * 2);
+    tma_load_1d(dst, W.codes + from / 32, n / 4, bar);
+    tma_load_1d(dst + kArenaPositions / 4, W.rcodes + from / 32, n / 4, bar);
+    tma_load_1d(dst + kArenaPositions / 2, W.inv + from / 64, n / 8, bar);
+    tma_load_1d(dst + kArenaPositions / 2 + kArenaPositions / 8, W.hq + from / 64, n / 8, bar);
+  };
+  if (tid == 0) {
+    s_lost = 0;
+    mbar_init(smem_u32(&s_bar[0]), 1);
+    mbar_init(smem_u32(&s_bar[1]), 1);
+    if (blockIdx.x < n_tiles) issue(blockIdx.x, 0);
+  }
+  __syncthreads();
+  unsigned acc_valid = 0, phases = 0, buf = 0;
   unsigned acc_bucket[kScatterMaxPer] = {};  // records of this thread's buckets, over the CTA's tiles
-  for (unsigned t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+  for (unsigned t = blockIdx.x; t < n_tiles; t += gridDim.x, buf ^= 1) {
+    // everyone is done with the other buffer: the previous tile was extracted some barriers ago
+    if (tid == 0 && t + gridDim.x < n_tiles) issue(t + gridDim.x, buf ^ 1);
+    if (!mbar_wait_bounded(smem_u32(&s_bar[buf]), (phases >> buf) & 1u, kWaitPolls)) s_lost = 1;
+    const u64 q = W.q0 + (u64)t * kScatterTile + (u64)tid * kScatterWpt;
+    WindowRun<KW> win;
+    win.valid = 0;
+    if (q < W.q1) {  // q1 - q0 is a multiple of 64: all kScatterWpt starts are inside
+      const unsigned char* a = s_arena + buf * kArenaStage;
+      win.init(reinterpret_cast<const u64*>(a), reinterpret_cast<const u64*>(a + kArenaPositions / 4),
+               reinterpret_cast<const u64*>(a + kArenaPositions / 2),
+               reinterpret_cast<const u64*>(a + kArenaPositions / 2 + kArenaPositions / 8), G.k, q - stage_from(t),
+               q == 0, true);
+    }
     if (tid == 0) tma_store_wait_read();  // the previous tile has left shared memory
     for (unsigned p = tid; p < B; p += kScatterThreads) s_bin[p] = 0;
     __syncthreads();
+    if (s_lost) {  // uniform: a copy did not land. Report; those in flight land now (bounded)
+      if (tid == 0) {
+        atomicOr(&G.status->flags, kFlagTimeout);
+        mbar_drain(smem_u32(&s_bar[buf]), (phases >> buf) & 1u, kWaitPolls);
+        if (t + gridDim.x < n_tiles) mbar_drain(smem_u32(&s_bar[buf ^ 1]), (phases >> (buf ^ 1)) & 1u, kWaitPolls);
+      }
+      break;
+    }
+    phases ^= 1u << buf;
     unsigned pr[kScatterWpt];  // bucket << 13 | rank, or ~0u
 #pragma unroll
     for (int j = 0; j < kScatterWpt; ++j) pr[j] = 0xFFFFFFFFu;
-    const u64 q = W.q0 + (u64)t * kScatterTile + (u64)tid * kScatterWpt;
-    if (q < W.q1) {  // q1 - q0 is a multiple of 64: all kScatterWpt starts are inside
-      WindowRun<KW> run;
-      run.init(W, G.k, q, true);
 #pragma unroll
-      for (int j = 0; j < kScatterWpt; ++j) {
-        if (!((run.valid >> j) & 1u)) continue;
-        u64 lo, hi;
-        const bool forward = run.key(j, G.canonical, lo, hi);
-        const u64 h = key_hash(lo, hi);
-        if (G.n_parts > 1 && owner_of(h, G.n_parts) != G.part) continue;
-        ++acc_valid;
-        const unsigned slot = j * kScatterThreads + tid, top = (unsigned)(h >> 32);
-        const unsigned p = top >> (32 - G.log_b);
-        pr[j] = (p << 13) | atomicAdd(&s_bin[p], 1u);
-        const u64 r = ((u64)((top & (unsigned)(kHashMask >> 32)) | run.info(j, forward)) << 32) | (unsigned)h;
-        if (KW == 1) s_rec[slot] = r;
-        else reinterpret_cast<ulonglong2*>(s_rec)[slot] = make_ulonglong2(r, hi);
-      }
+    for (int j = 0; j < kScatterWpt; ++j) {
+      if (!((win.valid >> j) & 1u)) continue;
+      u64 lo, hi;
+      const bool forward = win.key(j, G.canonical, lo, hi);
+      const u64 h = key_hash(lo, hi);
+      if (G.n_parts > 1 && owner_of(h, G.n_parts) != G.part) continue;
+      ++acc_valid;
+      const unsigned slot = j * kScatterThreads + tid, top = (unsigned)(h >> 32);
+      const unsigned p = top >> (32 - G.log_b);
+      pr[j] = (p << 13) | atomicAdd(&s_bin[p], 1u);
+      const u64 r = ((u64)((top & (unsigned)(kHashMask >> 32)) | win.info(j, forward)) << 32) | (unsigned)h;
+      if (KW == 1) s_rec[slot] = r;
+      else reinterpret_cast<ulonglong2*>(s_rec)[slot] = make_ulonglong2(r, hi);
     }
     __syncthreads();
     // bucket offsets (thread t: buckets t * per ..), written as the tile's row
