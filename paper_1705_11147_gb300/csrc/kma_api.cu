@@ -655,12 +655,13 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     positions += sl.positions;
   }
   if (n_chunks == 0) return after(B);
-  if (parts > B) parts = B;
+  constexpr unsigned kStep = kSplitBuckets;  // groups are whole work items of the split
+  parts = std::min(parts, B / kStep);
   std::vector<unsigned> ends;
   u64 most = bound;        // records of a group
   unsigned most_buckets = 0;
   if (!may_sync || bound * h->d.rec_bytes <= kSplitAtOnce) {
-    for (unsigned i = 0; i < parts; ++i) ends.push_back((unsigned)((u64)B * (i + 1) / parts));
+    for (unsigned i = 0; i < parts; ++i) ends.push_back((unsigned)((u64)(B / kStep) * (i + 1) / parts) * kStep);
   } else {
     std::vector<u64> totals(B);
     KMA_CUDA(cudaMemcpyAsync(totals.data(), h->totals, B * sizeof(u64), cudaMemcpyDeviceToHost, st));
@@ -668,14 +669,16 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     u64 all = 0;
     for (u64 t : totals) all += t;
     const u64 aim = std::max(kSplitAtOnce / h->d.rec_bytes, all / kSplitGroups);
-    const unsigned widest = (B + parts - 1) / parts;
+    std::vector<u64> step(B / kStep, 0);  // records per step of buckets
+    for (unsigned b = 0; b < B; ++b) step[b / kStep] += totals[b];
+    const unsigned widest = (B / kStep + parts - 1) / parts;
     most = 0;
-    for (unsigned b = 0; b < B;) {
+    for (unsigned b = 0; b < B / kStep;) {
       unsigned e = b;
       u64 sum = 0;
-      do sum += totals[e++];
-      while (e < B && e - b < widest && sum + totals[e] <= aim);
-      ends.push_back(e);
+      do sum += step[e++];
+      while (e < B / kStep && e - b < widest && sum + step[e] <= aim);
+      ends.push_back(e * kStep);
       most = std::max(most, sum);
       b = e;
     }

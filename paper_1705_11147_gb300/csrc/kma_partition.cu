@@ -361,9 +361,16 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
     const unsigned t0 = chunk * S.chunk_tiles;
     const unsigned nt = T.n_tiles - t0 < S.chunk_tiles ? T.n_tiles - t0 : S.chunk_tiles;
     __syncthreads();  // the previous item's offsets are no longer read
-    for (unsigned x = tid; x < nt * (kSplitBuckets + 1); x += kSplitThreads) {
-      const unsigned i = x / (kSplitBuckets + 1), j = x - i * (kSplitBuckets + 1);
-      s_off[x] = j <= nb ? T.offs[(u64)(t0 + i) * T.stride + bb + j] : 0;
+    for (unsigned i = tid; i < nt; i += kSplitThreads) {
+      // eight entries in one load (groups of buckets start at multiples of 8, rows are padded), and the next one
+      static_assert(kSplitBuckets == 8, "an item's offsets are one 16-byte load");
+      const unsigned short* row = T.offs + (u64)(t0 + i) * T.stride + bb;
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(row));
+      const unsigned next = __ldg(row + kSplitBuckets);  // inside the row's padding for the last buckets
+      unsigned short* o = s_off + i * (kSplitBuckets + 1);
+      o[0] = (unsigned short)v.x, o[1] = (unsigned short)(v.x >> 16), o[2] = (unsigned short)v.y, o[3] = (unsigned short)(v.y >> 16);
+      o[4] = (unsigned short)v.z, o[5] = (unsigned short)(v.z >> 16), o[6] = (unsigned short)v.w, o[7] = (unsigned short)(v.w >> 16);
+      o[8] = (unsigned short)next;
     }
     __syncthreads();
     const unsigned per = (nt + kSplitThreads - 1) / kSplitThreads;  // runs per thread
@@ -429,21 +436,15 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
           lc += c[x];
         }
         unsigned ro = block_scan<kSplitThreads>(lc, s_wsum, tot2);
-        unsigned over = 0;
 #pragma unroll
         for (unsigned x = 0; x < kSplitMaxPer; ++x) {
           const unsigned p = tid * per_sub + x;
           if (x < per_sub && p < n_sub) {
-            const unsigned room = at[x] < G.cap ? G.cap - (unsigned)at[x] : 0u, fits = c[x] < room ? c[x] : room;
             s_bin[p] = ro;
-            s_to[p] = p * G.cap + (unsigned)at[x] - ro;
-            s_lim[p] = (unsigned short)(ro + fits);
-            over += c[x] - fits;
-            c[x] -= fits;
-            ro += c[x] + fits;
+            ro += c[x];
           }
         }
-        const int any_over = __syncthreads_or(over != 0);
+        __syncthreads();
 #pragma unroll
         for (int y = 0; y < kSplitItems; ++y) {
           if (pr[y] == 0xFFFFFFFFu) continue;
@@ -451,7 +452,20 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
           if (KW == 1) s_rec[to] = r0[y];
           else reinterpret_cast<ulonglong2*>(s_rec)[to] = make_ulonglong2(r0[y], r1[y]);
         }
-        __syncthreads();
+        unsigned over = 0;  // the places, taken by now
+#pragma unroll
+        for (unsigned x = 0; x < kSplitMaxPer; ++x) {
+          const unsigned p = tid * per_sub + x;
+          if (x < per_sub && p < n_sub) {
+            const unsigned room = at[x] < G.cap ? G.cap - (unsigned)at[x] : 0u, fits = c[x] < room ? c[x] : room;
+            const unsigned o = s_bin[p];
+            s_to[p] = p * G.cap + (unsigned)at[x] - o;
+            s_lim[p] = (unsigned short)(o + fits);
+            c[x] -= fits;
+            over += c[x];
+          }
+        }
+        const int any_over = __syncthreads_or(over != 0);
         if (any_over) {  // the block's records that found no room: numbered, and a segment for them
           unsigned n_over;
           unsigned o = block_scan<kSplitThreads>(over, s_wsum, n_over);
@@ -1035,7 +1049,7 @@ cudaError_t launch_part_base(const unsigned long long* totals, const PartSplit& 
 cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartSplit& s, cudaStream_t stream,
                               int num_sms) {
   if (t.n_tiles == 0 || s.b1 <= s.b0) return cudaSuccess;
-  if (s.chunk_tiles == 0 || s.chunk_tiles > kMaxChunkTiles) return cudaErrorInvalidValue;
+  if (s.chunk_tiles == 0 || s.chunk_tiles > kMaxChunkTiles || s.b0 % kSplitBuckets || t.stride % 8) return cudaErrorInvalidValue;
   const int kw = g.k > 32 ? 2 : 1;
   const size_t smem = split_smem(s.chunk_tiles, g.sub_max, kw);
   const void* fn = kw == 2 ? (const void*)part_split_kernel<2> : (const void*)part_split_kernel<1>;
