@@ -626,15 +626,61 @@ int scatter_windows(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, 
                       [&] { return launch_part_scatter(g, w, t, st, h->num_sms); });
 }
 
+int ensure_output(kma_handle* h, u64 need) {
+  if (need <= h->out_cap && h->out_keys) return KMA_OK;
+  dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
+  h->out_cap = 0;
+  u64 cap = std::max<u64>(need + need / 8, 1024);
+  int rc;
+  if ((rc = dalloc(h, &h->out_keys, 2 * cap))) return rc;
+  if ((rc = dalloc(h, &h->out_counts, cap))) return rc;
+  if ((rc = dalloc(h, &h->out_ext, 8 * cap))) return rc;
+  if ((rc = dalloc(h, &h->out_codes, 2 * cap))) return rc;
+  h->out_cap = cap;
+  return KMA_OK;
+}
+
+ClassDesc class_desc(kma_handle* h) {
+  ClassDesc c;
+  std::memset(&c, 0, sizeof(c));
+  c.table = h->table; c.status = h->status; c.slots = h->d.plan.table_slots;
+  c.out_keys = h->out_keys; c.out_counts = h->out_counts; c.out_ext = h->out_ext;
+  c.out_codes = h->out_codes; c.out_cap = h->out_cap;
+  c.min_depth = h->p.min_depth;
+  c.min_ext = h->p.min_ext_count ? h->p.min_ext_count : 1;
+  return c;
+}
+
+PartOut part_out(kma_handle* h) {
+  PartOut o;
+  std::memset(&o, 0, sizeof(o));
+  o.keys = h->out_keys;
+  o.counts = h->out_counts;
+  o.ext = h->out_ext;
+  o.codes = h->out_codes;
+  o.cap = h->out_keys ? h->out_cap : 0;
+  o.min_depth = h->p.min_depth;
+  o.min_ext = h->p.min_ext_count ? h->p.min_ext_count : 1;
+  return o;
+}
+
+// Partitioned mode: output room before anything is in the table, for as many keys as it was
+// sized for (or as much as there is: more records than fit are classified again afterwards).
+int guess_output(kma_handle* h) {
+  const double load = h->p.load_factor > 0 ? h->p.load_factor : 0.5;
+  const int rc = ensure_output(h, (u64)((double)h->d.plan.table_slots * load));
+  return rc == KMA_ENOMEM ? KMA_OK : rc;
+}
+
 // Lanes (log2) that copy one run of `len` records on average.
 unsigned lanes_for(double len) {
   const double l = std::floor(std::log2(std::max(len, 1.0)) + 0.3);
   return (unsigned)std::min(5.0, l);
 }
 
-// Partitioned mode: counts the handle's records into its table on stream `st`, the buckets in
-// order, `parts` groups of them or more, and calls after(end) when the buckets below `end` have
-// been enqueued. The sorted copy of the split is sized for all records when they are few or
+// Partitioned mode: counts the handle's records into its table and output records on stream `st`,
+// the buckets in order, `parts` groups of them or more, and calls after(end) when the buckets
+// below `end` have been enqueued. The sorted copy of the split is sized for all records when they are few or
 // when the call may not wait for the GPU (may_sync = false, capture); otherwise from the bucket
 // totals, a twelfth of the records or the largest bucket.
 template <typename F>
@@ -687,6 +733,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   PartSplit s;
   std::memset(&s, 0, sizeof(s));
   PartGeom g = part_geom(h);
+  const PartOut o = part_out(h);
   // sub-buckets for the windows expected (one more than that for reads shorter than k)
   g.sub_max = (unsigned)std::min<double>(g.sub_max, std::ceil(1.05 * windows / ((double)g.avg * B)) + 1.0);
   const u64 n_subs = (u64)most_buckets * g.sub_max;
@@ -735,9 +782,9 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
           return rc;
       }
       if ((rc = timed_launch(timed, KMA_KERNEL_PASS, st, true,
-                             [&] { return launch_part_count(g, s, st, h->num_sms); })) ||
+                             [&] { return launch_part_count(g, s, o, st, h->num_sms); })) ||
           (rc = timed_launch(timed, KMA_KERNEL_RECOUNT, st, true,
-                             [&] { return launch_part_insert(g, s, st, h->num_sms); })))
+                             [&] { return launch_part_insert(g, s, o, st, h->num_sms); })))
         return rc;
       if ((rc = after(s.b1))) return rc;
     }
@@ -783,31 +830,6 @@ int run_pack_and_pass(kma_handle* h, const PackDesc& pd) {
   if (rc) return rc;
   if (h->pack_only) return KMA_OK;
   return first_pass(h, pd.q0, pd.n_pos, pd.n_reads, pd.n_bases, h->stream);
-}
-
-int ensure_output(kma_handle* h, u64 need) {
-  if (need <= h->out_cap && h->out_keys) return KMA_OK;
-  dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
-  h->out_cap = 0;
-  u64 cap = std::max<u64>(need + need / 8, 1024);
-  int rc;
-  if ((rc = dalloc(h, &h->out_keys, 2 * cap))) return rc;
-  if ((rc = dalloc(h, &h->out_counts, cap))) return rc;
-  if ((rc = dalloc(h, &h->out_ext, 8 * cap))) return rc;
-  if ((rc = dalloc(h, &h->out_codes, 2 * cap))) return rc;
-  h->out_cap = cap;
-  return KMA_OK;
-}
-
-ClassDesc class_desc(kma_handle* h) {
-  ClassDesc c;
-  std::memset(&c, 0, sizeof(c));
-  c.table = h->table; c.status = h->status; c.slots = h->d.plan.table_slots;
-  c.out_keys = h->out_keys; c.out_counts = h->out_counts; c.out_ext = h->out_ext;
-  c.out_codes = h->out_codes; c.out_cap = h->out_cap;
-  c.min_depth = h->p.min_depth;
-  c.min_ext = h->p.min_ext_count ? h->p.min_ext_count : 1;
-  return c;
 }
 
 constexpr u64 kClassTile = 256 * 4;  // slots per classify block tile (kernel constants)
@@ -1034,6 +1056,7 @@ static int enqueue_recount(kma_handle* const* hs, uint32_t n, bool may_sync) {
   for (uint32_t i = 0; i < n; ++i) {
     kma_handle* h = hs[i];
     if (h->d.P <= 1) continue;
+    KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h0->stream));
     if ((rc = count_records(h, h0, h0->stream, may_sync, 1, [](unsigned) { return (int)KMA_OK; }))) return rc;
   }
   return KMA_OK;
@@ -1095,28 +1118,40 @@ static int finalize_many(kma_handle* const* hs, uint32_t n, kma_result* out) {
       if (e != cudaSuccess) return cuda_fail(e, "stream ordering");
     }
   }
+  for (uint32_t i = 0; i < n; ++i) {
+    if (hs[i]->d.P <= 1) continue;
+    cudaStream_t saved = hs[i]->stream;
+    hs[i]->stream = h0->stream;
+    rc = guess_output(hs[i]);
+    hs[i]->stream = saved;
+    if (rc) return rc;
+  }
   if ((rc = enqueue_recount(hs, n, true))) return rc;
-  // statuses -> output capacities (table_keys bounds the records)
+  // statuses -> output capacities (table_keys bounds the records). The partitioned handles have
+  // their records already, unless there was not enough room.
   for (uint32_t i = 0; i < n; ++i)
     KMA_CUDA(cudaMemcpyAsync(hs[i]->host_status, hs[i]->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, h0->stream));
   KMA_CUDA(cudaStreamSynchronize(h0->stream));
   int first_err = KMA_OK;
-  std::vector<int> ok(n, 0);
+  std::vector<int> ok(n, 0), todo(n, 0);  // done without an error; to be classified
   for (uint32_t i = 0; i < n; ++i) {
     kma_handle* h = hs[i];
-    int e = flags_to_code(h->host_status->flags);
+    int e = flags_to_code(h->host_status->flags & ~(h->d.P > 1 ? kFlagOutput : 0u));
     if (e) { h->failed = true; if (!first_err) first_err = e; continue; }
+    ok[i] = 1;
+    if (h->d.P > 1 && !(h->host_status->flags & kFlagOutput)) continue;
     cudaStream_t saved = h->stream;
     h->stream = h0->stream;
     e = ensure_output(h, h->host_status->table_keys);
     h->stream = saved;
-    if (e) { h->failed = true; if (!first_err) first_err = e; continue; }
-    ok[i] = 1;
+    if (e) { h->failed = true; ok[i] = 0; if (!first_err) first_err = e; continue; }
+    if (h->d.P > 1) KMA_CUDA(cudaMemsetAsync(&h->status->flags, 0, sizeof(h->status->flags), h0->stream));
+    todo[i] = 1;
   }
-  if ((rc = enqueue_classify(hs, n, ok))) return rc;
+  if ((rc = enqueue_classify(hs, n, todo))) return rc;
   for (uint32_t i = 0; i < n; ++i)
-    if (ok[i]) KMA_CUDA(cudaMemcpyAsync(hs[i]->host_status, hs[i]->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, h0->stream));
-  KMA_CUDA(cudaStreamSynchronize(h0->stream));
+    if (todo[i]) KMA_CUDA(cudaMemcpyAsync(hs[i]->host_status, hs[i]->status, sizeof(DevStatus), cudaMemcpyDeviceToHost, h0->stream));
+  if (std::any_of(todo.begin(), todo.end(), [](int v) { return v != 0; })) KMA_CUDA(cudaStreamSynchronize(h0->stream));
   for (uint32_t i = 0; i < n; ++i) {
     kma_handle* h = hs[i];
     if (!ok[i]) { if (out) std::memset(&out[i], 0, sizeof(kma_result)); continue; }
@@ -1150,8 +1185,9 @@ int kmer_analysis_finalize_batch_async(kma_handle* const* hs, uint32_t n) {
   for (uint32_t i = 0; i < n; ++i)
     if (!hs[i]->out_keys) return KMA_ESTATE;  // kmer_analysis_reserve_output first
   if ((rc = enqueue_recount(hs, n, false))) return rc;
-  std::vector<int> ok(n, 1);
-  if ((rc = enqueue_classify(hs, n, ok))) return rc;
+  std::vector<int> todo(n, 0);  // the partitioned handles have their records already
+  for (uint32_t i = 0; i < n; ++i) todo[i] = hs[i]->d.P <= 1;
+  if ((rc = enqueue_classify(hs, n, todo))) return rc;
   for (uint32_t i = 0; i < n; ++i) hs[i]->finalized = true;
   return KMA_OK;
 }
@@ -1265,7 +1301,14 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
   KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
   const unsigned G = (unsigned)std::max<u64>(1, std::min<u64>(kFinalizeGroups, parts ? h->d.P : S / kClassTile));
   unsigned published = 0;  // groups whose records have been appended to the output
-  // Classify the table slots [s0, s1) and publish the record count so far.
+  // Publish the record count so far.
+  auto announce = [&]() -> int {
+    KMA_CUDA(cudaMemcpyAsync(&h->host_groups[published], &h->status->n_out, sizeof(u64), cudaMemcpyDeviceToHost, h->stream));
+    KMA_CUDA(cudaEventRecord(h->group_ev[published], h->stream));
+    ++published;
+    return KMA_OK;
+  };
+  // Classify the table slots [s0, s1), then the same.
   auto publish = [&](u64 s0, u64 s1) -> int {
     ClassBatch cb;
     std::memset(&cb, 0, sizeof(cb));
@@ -1277,11 +1320,7 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
     cb.total_blocks = (s1 - s0 + kClassTile - 1) / kClassTile;
     int rc2 = timed_launch(h, KMA_KERNEL_CLASSIFY, h->stream, cb.total_blocks > 0,
                            [&] { return launch_classify(cb, h->stream, h->num_sms); });
-    if (rc2) return rc2;
-    KMA_CUDA(cudaMemcpyAsync(&h->host_groups[published], &h->status->n_out, sizeof(u64), cudaMemcpyDeviceToHost, h->stream));
-    KMA_CUDA(cudaEventRecord(h->group_ev[published], h->stream));
-    ++published;
-    return KMA_OK;
+    return rc2 ? rc2 : announce();
   };
   if (!parts) {
     // the recount is a pass over the windows: the groups only split the classification
@@ -1292,16 +1331,11 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
     for (unsigned i = 0; i < G; ++i)
       if ((rc = publish(S * i / G, S * (i + 1) / G))) return rc;
   } else {
-    // Buckets and partitions are ranges of the same hash: with the buckets below `end` counted,
-    // the partitions below end * P / B are complete.
+    // the records are appended to the output as each group of buckets is counted
     const unsigned B = 1u << h->d.log_b;
-    u64 p0 = 0;
     rc = count_records(h, h, h->stream, true, G, [&](unsigned end) -> int {
-      const u64 p1 = (u64)end * h->d.P / B;
-      if (end != B && (p1 == p0 || (u64)end * G / B <= published)) return KMA_OK;
-      const u64 from = p0;
-      p0 = p1;
-      return publish(from * h->d.Sp, p1 * h->d.Sp);
+      if (end != B && (u64)end * G / B <= published) return KMA_OK;
+      return announce();
     });
     if (rc) return rc;
   }

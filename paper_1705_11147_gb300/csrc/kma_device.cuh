@@ -30,13 +30,16 @@ __device__ __forceinline__ u64 key_hash(u64 lo, u64 hi) {
 // more products, instead of further 64-bit mixes:
 //   on-chip partition   high 32 bits of h                  (part_of)
 //   Bloom word          low 32 bits of h                   (bloom_index; < 2^32 words)
-//   table slot          high 32 bits of h * phi            (table_index; < 2^32 slots per part)
+//   table slot          high 32 bits of h, the part behind the partition (table_index; < 2^32 slots per part)
 //   Bloom bit positions 6-bit fields from the top of (h ^ h >> 32) * c   (bloom_mask)
 // The bit positions must not depend on the low bits of h alone: those also pick the word, and
 // keys sharing a word would then share most of their bits (a much higher false-positive rate).
 __device__ __forceinline__ u64 scramble(u64 h) { return h * 0x9e3779b97f4a7c15ull; }
-__device__ __forceinline__ u64 table_index(u64 h, u64 slots) {
-  return __umulhi((unsigned)(scramble(h) >> 32), (unsigned)slots);
+// Slot of a key in its partition (of `parts`): in the order of the hash, so that the keys of one
+// sub-bucket (partitioned mode counts in hash order) go to neighbouring slots and every line of
+// the table is brought in and written back once.
+__device__ __forceinline__ u64 table_index(u64 h, u64 slots, unsigned parts = 1) {
+  return __umulhi((unsigned)(h >> 32) * parts, (unsigned)slots);
 }
 __device__ __forceinline__ u64 bloom_index(u64 h, u64 words) {
   return __umulhi((unsigned)h, (unsigned)words);
@@ -408,9 +411,9 @@ __device__ __forceinline__ Slot* find_or_insert(Slot* table, u64 slots, u64 lo, 
 
 // Lookup in a table no thread is modifying. nullptr if absent; sets `full` if the probe
 // limit was reached without finding an empty slot.
-__device__ __forceinline__ const Slot* find(const Slot* table, u64 slots, u64 lo, u64 hi, u64 h,
+__device__ __forceinline__ const Slot* find(const Slot* table, u64 slots, unsigned parts, u64 lo, u64 hi, u64 h,
                                             bool& full) {
-  u64 idx = table_index(h, slots);
+  u64 idx = table_index(h, slots, parts);
   const u64 limit = slots < kMaxProbe ? slots : kMaxProbe;
   full = false;
   for (u64 n = 0; n < limit; ++n) {

@@ -228,13 +228,24 @@ struct PartSplit {
   unsigned long long* n_keys;   // their number; starts at 0
 };
 
+// Output records of the keys inserted (as ClassDesc).
+struct PartOut {
+  unsigned long long* keys;
+  unsigned int* counts;
+  unsigned int* ext;
+  unsigned char* codes;
+  unsigned long long cap;
+  unsigned int min_depth;
+  unsigned int min_ext;
+};
+
 cudaError_t launch_part_scatter(const PartGeom& g, const PartWindows& w, const PartTiles& t, cudaStream_t stream,
                                 int num_sms);
 cudaError_t launch_part_base(const unsigned long long* totals, const PartSplit& s, cudaStream_t stream);
 cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartSplit& s, cudaStream_t stream,
                               int num_sms);
-cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
-cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
+cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
+cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
 constexpr unsigned kMaxKeyWords = 10;          // words of one counted key in the list
 
 // FASTQ parsing (kma_fastq.cu) and the device-wide exclusive scan it uses.

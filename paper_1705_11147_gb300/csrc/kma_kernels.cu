@@ -604,20 +604,16 @@ __global__ void __launch_bounds__(256) query_kernel(const Slot* table, u64 slots
       bool full;
       const u64 h = key_hash(lo, hi);
       const Slot* sub = parts > 1 ? table + (u64)part_of(h, parts) * slots : table;
-      const Slot* s = find(sub, slots, lo, hi, h, full);
+      const Slot* s = find(sub, slots, parts, lo, hi, h, full);
       if (full) atomicOr(&st->flags, kFlagFull);
-      const unsigned sc = s ? slot_count(s->none[0], *reinterpret_cast<const uint4*>(&s->ext[0]), st) : 0u;
-      if (s && sc >= min_depth) {
-        c = sc;
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          if (forward) {
-            e[b] = s->ext[b];
-            e[4 + b] = s->ext[4 + b];
-          } else {
-            e[3 - b] = s->ext[4 + b];   // query's left = complement of key's right
-            e[4 + 3 - b] = s->ext[b];   // query's right = complement of key's left
-          }
+      if (s) {
+        const uint4 l = *reinterpret_cast<const uint4*>(&s->ext[0]), r = *reinterpret_cast<const uint4*>(&s->ext[4]);
+        const unsigned sc = slot_count(s->none[0], l, st);
+        if (sc >= min_depth) {
+          c = sc;
+          // a query on the other strand: its left = complement of the key's right, and the reverse
+          e[0] = forward ? l.x : r.w; e[1] = forward ? l.y : r.z; e[2] = forward ? l.z : r.y; e[3] = forward ? l.w : r.x;
+          e[4] = forward ? r.x : l.w; e[5] = forward ? r.y : l.z; e[6] = forward ? r.z : l.y; e[7] = forward ? r.w : l.x;
         }
       }
     }

@@ -569,27 +569,59 @@ struct CountShape {
   static_assert((size_t)kLargeSlots * (KW * 8 + 20) <= kSmem - 2 * kRec && (size_t)kLargeSlots * 20 <= kRec, "room for count_large");
 };
 
-// Insert one key with its ten counters (left A C G T none, right A C G T none) into the table.
-// The key is in no slot yet and no other thread inserts it.
-__device__ __forceinline__ bool emit_key(const PartGeom& G, u64 h, u64 hi, const unsigned (&ctr)[10]) {
-  const u64 lo = key_lo(h, hi);
-  Slot* sub = G.table + (u64)part_of(h, G.P) * G.Sp;
-  u64 idx = table_index(h, G.Sp);
+// Slot-to-be of one key in the table: the key's words and where its probes begin.
+struct Place {
+  Slot* sub;
+  u64 lo, hi, idx;
+};
+__device__ __forceinline__ Place place_of(const PartGeom& G, u64 h, u64 hi) {
+  Place p;
+  p.lo = key_lo(h, hi);
+  p.hi = hi;
+  p.sub = G.table + (u64)part_of(h, G.P) * G.Sp;
+  p.idx = table_index(h, G.Sp, G.P);
+  return p;
+}
+
+// Puts a key with its ten counters (left A C G T none, right A C G T none) into the table. The
+// key is in no slot yet and no other thread inserts it, so the first empty slot takes it.
+// (olo, ohi): what a compare-and-swap of the first slot returned.
+__device__ __forceinline__ bool finish_insert(const PartGeom& G, Place& p, u64 olo, u64 ohi, const unsigned (&ctr)[10]) {
   const u64 limit = G.Sp < kMaxProbe ? G.Sp : kMaxProbe;
-  for (u64 n = 0; n < limit; ++n) {
-    Slot* s = sub + idx;
-    u64 olo, ohi;
-    cas128(s, kEmpty, kEmpty, lo, hi, olo, ohi);
+  for (u64 n = 1;; ++n) {
     if (olo == kEmpty && ohi == kEmpty) {
+      Slot* s = p.sub + p.idx;
       *reinterpret_cast<uint4*>(&s->none[0]) = make_uint4(ctr[4], ctr[9], 0u, 0u);
       *reinterpret_cast<uint4*>(&s->ext[0]) = make_uint4(ctr[0], ctr[1], ctr[2], ctr[3]);
       *reinterpret_cast<uint4*>(&s->ext[4]) = make_uint4(ctr[5], ctr[6], ctr[7], ctr[8]);
       return true;
     }
-    idx = (idx + 1 == G.Sp) ? 0 : idx + 1;
+    if (n >= limit) break;
+    p.idx = (p.idx + 1 == G.Sp) ? 0 : p.idx + 1;
+    cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
   }
   atomicOr(&G.status->flags, kFlagFull);
   return false;
+}
+
+// Count of a key (its left outcomes; 0xFFFFFFFF and a flag above 32 bits), and its record at place
+// `at` of the output. Returns whether both sides are unique.
+__device__ __forceinline__ unsigned key_count(const PartGeom& G, const unsigned (&ctr)[10]) {
+  return slot_count(ctr[4], make_uint4(ctr[0], ctr[1], ctr[2], ctr[3]), G.status);
+}
+__device__ __forceinline__ bool write_record(const PartGeom& G, const PartOut& O, u64 at, u64 lo, u64 hi, unsigned count,
+                                             const unsigned (&ctr)[10]) {
+  const unsigned l = side_code(ctr, O.min_ext), r = side_code(ctr + 5, O.min_ext);
+  if (at < O.cap) {
+    reinterpret_cast<ulonglong2*>(O.keys)[at] = make_ulonglong2(lo, hi);
+    O.counts[at] = count;
+    reinterpret_cast<uint4*>(O.ext)[2 * at] = make_uint4(ctr[0], ctr[1], ctr[2], ctr[3]);
+    reinterpret_cast<uint4*>(O.ext)[2 * at + 1] = make_uint4(ctr[5], ctr[6], ctr[7], ctr[8]);
+    reinterpret_cast<uchar2*>(O.codes)[at] = make_uchar2((unsigned char)l, (unsigned char)r);
+  } else {
+    atomicOr(&G.status->flags, kFlagOutput);
+  }
+  return l < 4 && r < 4;
 }
 
 constexpr u64 kFree = ~0ull;                 // count_large: first key word of an empty slot
@@ -626,7 +658,7 @@ __device__ __forceinline__ unsigned probe_slot(u64* k0, u64* k1, unsigned pos, u
 // finds no place. Lanes with equal outcomes of equal keys act as one (frequent k-mers are
 // accumulated in the warp first, Section 5.1). The keys go straight to the HBM table.
 template <int KW>
-__device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, u64* k0, unsigned* left, unsigned* right,
+__device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, const PartOut& O, u64* k0, unsigned* left, unsigned* right,
                                          unsigned b, unsigned s, unsigned n_sub, unsigned n_in, unsigned& acc_ins,
                                          unsigned& acc_first) {
   using C = CountShape<KW>;
@@ -719,7 +751,14 @@ __device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, 
         v[5 + x] = right[i * 5 + x];
         n += v[x];
       }
-      if (n >= G.min_count) acc_ins += emit_key(G, h | htop, KW == 2 ? k1[i] : 0, v);
+      if (n < G.min_count) continue;
+      Place p = place_of(G, h | htop, KW == 2 ? k1[i] : 0);
+      u64 olo, ohi;
+      cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
+      acc_ins += finish_insert(G, p, olo, ohi, v);
+      const unsigned count = key_count(G, v);
+      if (count >= O.min_depth && write_record(G, O, atomicAdd(&G.status->n_out, 1ull), p.lo, p.hi, count, v))
+        atomicAdd(&G.status->n_uu, 1ull);
     }
     lo += width;
   }
@@ -728,7 +767,8 @@ __device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, 
 
 template <int KW>
 __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(const __grid_constant__ PartGeom G,
-                                                                               const __grid_constant__ PartSplit S) {
+                                                                               const __grid_constant__ PartSplit S,
+                                                                               const __grid_constant__ PartOut O) {
   using C = CountShape<KW>;
   extern __shared__ __align__(128) unsigned char s_raw[];
   __shared__ __align__(8) unsigned long long s_bar[2];
@@ -795,7 +835,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     }
     auto large = [&]() {
       u64* keys = reinterpret_cast<u64*>(s_rep);
-      count_large<KW>(G, S, keys, reinterpret_cast<unsigned*>(keys + C::kLargeSlots * KW), reinterpret_cast<unsigned*>(s_rec),
+      count_large<KW>(G, S, O, keys, reinterpret_cast<unsigned*>(keys + C::kLargeSlots * KW), reinterpret_cast<unsigned*>(s_rec),
                       S.b0 + item / n_sub, item % n_sub, n_sub, n, acc_ins, acc_first);
     };
     if (fill > G.cap) {  // uniform
@@ -967,28 +1007,73 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
 
 // ------------------------------------------------------------------ insert
 //
-// One counted key per thread into the HBM table. The keys of the list are distinct, in no slot
-// yet, and in hash order roughly, so the slots written at one time lie in one or two partitions.
+// The counted keys of the list into the HBM table, and the records of those that are frequent
+// enough (Section 5.1's depth filter, the side codes of Sections 2 and 4.1) into the output. The
+// keys are distinct, in no slot yet, and in hash order roughly, so the slots written at one time
+// lie in one or two partitions. A tile's output places are reserved together: the atomics on that
+// one counter take 6 ns each. One key in flight per thread: with two or four the registers cost
+// more warps than the round trips gained (8.0, 8.5 and 16.5 ms for 115 M keys, 7.7 as it is). Writing the
+// records here saves the scan of the whole table (64 bytes per slot, half of them empty).
+
+constexpr int kInsertThreads = 256;
+constexpr int kInsertKeys = 2;
+constexpr unsigned kInsertTile = kInsertThreads * kInsertKeys;
 
 template <int KW>
-__global__ void __launch_bounds__(256) part_insert_kernel(const __grid_constant__ PartGeom G, const unsigned* keys,
-                                                          const u64* n_keys) {
+__global__ void __launch_bounds__(kInsertThreads) part_insert_kernel(const __grid_constant__ PartGeom G,
+                                                                     const __grid_constant__ PartOut O,
+                                                                     const unsigned* keys, const u64* n_keys) {
+  __shared__ unsigned s_wsum[32];
+  __shared__ u64 s_base;
   const u64 n = __ldcg(n_keys);
-  unsigned acc_ins = 0;
-  for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x) {
-    const unsigned* c = keys + i * kKeyWords<KW>;
-    uint2 w[kKeyWords<KW> / 2];
+  unsigned acc_ins = 0, acc_uu = 0;
+  for (u64 t = blockIdx.x; t * kInsertTile < n; t += gridDim.x) {
+    // the records this thread's keys make
+    unsigned keep = 0;
 #pragma unroll
-    for (unsigned x = 0; x < kKeyWords<KW> / 2; ++x) w[x] = __ldcs(reinterpret_cast<const uint2*>(c) + x);
-    const unsigned v[10] = {w[0].x & 0xFFFFu, w[0].x >> 16, w[0].y & 0xFFFFu, w[0].y >> 16, w[1].x & 0xFFFFu,
-                            w[1].y & 0xFFFFu, w[1].y >> 16, w[2].x & 0xFFFFu, w[2].x >> 16, w[2].y & 0xFFFFu};
-    const u64 h = ((u64)w[3].y << 32) | w[3].x;
-    const u64 hi = KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull;
-    acc_ins += emit_key(G, h, hi, v);
+    for (int y = 0; y < kInsertKeys; ++y) {
+      const u64 i = t * kInsertTile + y * kInsertThreads + threadIdx.x;
+      if (i < n) {
+        const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
+        const uint2 a = __ldg(c);
+        const unsigned none = __ldg(&c[1].x) & 0xFFFFu;
+        keep += (a.x & 0xFFFFu) + (a.x >> 16) + (a.y & 0xFFFFu) + (a.y >> 16) + none >= O.min_depth;
+      }
+    }
+    unsigned total;
+    const unsigned before = block_scan<kInsertThreads>(keep, s_wsum, total);
+    if (threadIdx.x == 0) s_base = total ? atomicAdd(&G.status->n_out, (u64)total) : 0;
+    __syncthreads();
+    u64 at = s_base + before;
+#pragma unroll 1
+    for (int y = 0; y < kInsertKeys; ++y) {
+      const u64 i = t * kInsertTile + y * kInsertThreads + threadIdx.x;
+      if (i >= n) break;
+      const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
+      uint2 w[kKeyWords<KW> / 2];
+#pragma unroll
+      for (unsigned x = 0; x < kKeyWords<KW> / 2; ++x) w[x] = __ldg(c + x);
+      const u64 h = ((u64)w[3].y << 32) | w[3].x;
+      Place p = place_of(G, h, KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull);
+      u64 olo, ohi;
+      cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
+      const unsigned v[10] = {w[0].x & 0xFFFFu, w[0].x >> 16, w[0].y & 0xFFFFu, w[0].y >> 16, w[1].x & 0xFFFFu,
+                              w[1].y & 0xFFFFu, w[1].y >> 16, w[2].x & 0xFFFFu, w[2].x >> 16, w[2].y & 0xFFFFu};
+      const unsigned count = key_count(G, v);
+      acc_ins += finish_insert(G, p, olo, ohi, v);
+      if (count >= O.min_depth) acc_uu += write_record(G, O, at++, p.lo, p.hi, count, v);
+    }
+    __syncthreads();  // s_wsum and s_base are rewritten
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
-  if ((threadIdx.x & 31) == 0 && acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
+  for (int o = 16; o > 0; o >>= 1) {
+    acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
+    acc_uu += __shfl_down_sync(0xffffffffu, acc_uu, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
+    if (acc_uu) atomicAdd(&G.status->n_uu, (u64)acc_uu);
+  }
 }
 
 // ------------------------------------------------------------------ launchers
@@ -1063,7 +1148,7 @@ cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartS
   return cudaGetLastError();
 }
 
-cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms) {
+cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms) {
   if (s.b1 <= s.b0) return cudaSuccess;
   const int kw = g.k > 32 ? 2 : 1;
   const size_t smem = kw == 2 ? CountShape<2>::kSmem : CountShape<1>::kSmem;
@@ -1071,15 +1156,17 @@ cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_
   cudaError_t e = allow_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)grid_for(fn, kCountThreads, smem, num_sms, (u64)(s.b1 - s.b0) * g.sub_max);
-  if (kw == 2) part_count_kernel<2><<<grid, kCountThreads, smem, stream>>>(g, s);
-  else part_count_kernel<1><<<grid, kCountThreads, smem, stream>>>(g, s);
+  if (kw == 2) part_count_kernel<2><<<grid, kCountThreads, smem, stream>>>(g, s, o);
+  else part_count_kernel<1><<<grid, kCountThreads, smem, stream>>>(g, s, o);
   return cudaGetLastError();
 }
 
-cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms) {
-  const unsigned grid = (unsigned)num_sms * 8;  // the number of keys is known on the device only
-  if (g.k > 32) part_insert_kernel<2><<<grid, 256, 0, stream>>>(g, s.keys, s.n_keys);
-  else part_insert_kernel<1><<<grid, 256, 0, stream>>>(g, s.keys, s.n_keys);
+cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms) {
+  // the number of keys is known on the device only: as many CTAs as run at a time
+  const void* fn = g.k > 32 ? (const void*)part_insert_kernel<2> : (const void*)part_insert_kernel<1>;
+  const unsigned grid = (unsigned)grid_for(fn, kInsertThreads, 0, num_sms, ~0ull);
+  if (g.k > 32) part_insert_kernel<2><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys);
+  else part_insert_kernel<1><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys);
   return cudaGetLastError();
 }
 
