@@ -101,41 +101,56 @@ cudaError_t scan_exclusive(u64* data, u64 n, u64* tmp, cudaStream_t stream) {
 
 // ------------------------------------------------------------------ FASTQ kernels
 
+// The 16 text bytes from position i on (i a multiple of 16 from the text's first aligned address:
+// `head` bytes before it belong to the same 16 bytes), with a bit per byte: bit j of the result is
+// set if byte i + j is a newline, or the text's last byte and none (the end of an unterminated
+// line). Bytes outside [0, n) count as none. Bound by the text's one read; a byte load per
+// thread and byte took 13 times as many requests.
+__device__ __forceinline__ unsigned newline_mask(const unsigned char* text, u64 n, long long i) {
+  if (i >= (long long)n) return 0;
+  uint4 v;
+  if (i >= 0 && i + 16 <= (long long)n) {
+    v = __ldg(reinterpret_cast<const uint4*>(text + i));
+  } else {  // the first or the last piece: byte by byte
+    unsigned w[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (i + j >= 0 && i + j < (long long)n) w[j >> 2] |= (unsigned)text[i + j] << (8 * (j & 3));
+    v = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+  // one bit per byte: compare, keep bit 0 of each byte, gather the four of a word
+  const unsigned nl = 0x0A0A0A0Au;
+  const unsigned m0 = ((__vcmpeq4(v.x, nl) & 0x01010101u) * 0x01020408u) >> 24, m1 = ((__vcmpeq4(v.y, nl) & 0x01010101u) * 0x01020408u) >> 24;
+  const unsigned m2 = ((__vcmpeq4(v.z, nl) & 0x01010101u) * 0x01020408u) >> 24, m3 = ((__vcmpeq4(v.w, nl) & 0x01010101u) * 0x01020408u) >> 24;
+  unsigned m = (m0 & 15u) | ((m1 & 15u) << 4) | ((m2 & 15u) << 8) | ((m3 & 15u) << 12);
+  const long long last = (long long)n - 1 - i;
+  if (last < 16) m |= 1u << last;  // the last byte ends a line either way
+  return m;
+}
+
 // Newlines in each 16 KiB chunk (plus one for a final line that does not end in '\n').
-__global__ void __launch_bounds__(kFqThreads) fastq_count_kernel(const unsigned char* text, u64 n,
+__global__ void __launch_bounds__(kFqThreads) fastq_count_kernel(const unsigned char* text, u64 n, unsigned head,
                                                                  u64* chunk_counts) {
   __shared__ unsigned warp_cnt[kFqThreads / 32];
   const u64 c = blockIdx.x;
-  const u64 b0 = c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread;
-  unsigned cnt = 0;
-#pragma unroll
-  for (int j = 0; j < kFqBytesPerThread; ++j) {
-    const u64 i = b0 + j;
-    if (i < n) cnt += (text[i] == '\n') | (i == n - 1 && text[i] != '\n');
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
+  unsigned cnt = __popc(newline_mask(text, n, (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head));
+  cnt = __reduce_add_sync(0xffffffffu, cnt);
   if ((threadIdx.x & 31) == 0) warp_cnt[threadIdx.x >> 5] = cnt;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    u64 t = 0;
-    for (int w = 0; w < kFqThreads / 32; ++w) t += warp_cnt[w];
-    chunk_counts[c] = t;
+  if (threadIdx.x < 32) {
+    const unsigned t = __reduce_add_sync(0xffffffffu, warp_cnt[threadIdx.x]);
+    if (threadIdx.x == 0) chunk_counts[c] = t;
   }
 }
 
 // Line ends (position of each '\n', or n for an unterminated last line), in text order.
-__global__ void __launch_bounds__(kFqThreads) fastq_lines_kernel(const unsigned char* text, u64 n,
+__global__ void __launch_bounds__(kFqThreads) fastq_lines_kernel(const unsigned char* text, u64 n, unsigned head,
                                                                  const u64* chunk_offsets, u64* line_end) {
   __shared__ unsigned warp_off[kFqThreads / 32];
   const u64 c = blockIdx.x;
-  const u64 b0 = c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread;
-  unsigned cnt = 0;
-#pragma unroll
-  for (int j = 0; j < kFqBytesPerThread; ++j) {
-    const u64 i = b0 + j;
-    if (i < n) cnt += (text[i] == '\n') | (i == n - 1 && text[i] != '\n');
-  }
+  const long long i = (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head;
+  unsigned m = newline_mask(text, n, i);
+  const unsigned cnt = __popc(m);
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned incl = cnt;
 #pragma unroll
@@ -145,21 +160,21 @@ __global__ void __launch_bounds__(kFqThreads) fastq_lines_kernel(const unsigned 
   }
   if (lane == 31) warp_off[warp] = incl;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned run = 0;
-    for (int w = 0; w < kFqThreads / 32; ++w) {
-      const unsigned t = warp_off[w];
-      warp_off[w] = run;
-      run += t;
+  if (warp == 0) {
+    const unsigned t = warp_off[lane];
+    unsigned run = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned x = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= (unsigned)o) run += x;
     }
+    warp_off[lane] = run - t;
   }
   __syncthreads();
   u64 out = chunk_offsets[c] + warp_off[warp] + incl - cnt;
-#pragma unroll
-  for (int j = 0; j < kFqBytesPerThread; ++j) {
-    const u64 i = b0 + j;
-    if (i < n && text[i] == '\n') line_end[out++] = i;
-    else if (i == n - 1 && i < n) line_end[out++] = n;  // unterminated last line
+  for (; m; m &= m - 1) {
+    const u64 at = (u64)(i + __ffs(m) - 1);
+    line_end[out++] = at == n - 1 && text[at] != '\n' ? n : at;  // unterminated last line
   }
 }
 
@@ -186,30 +201,53 @@ __global__ void fastq_record_kernel(const unsigned char* text, const u64* line_e
   if (!ok) atomicMin(bad, (unsigned long long)r);
 }
 
-// One warp per record: bases and qualities to their place in the output.
+// Eight text bytes starting at any address, from the two aligned words that hold them (the second
+// one is read only if it does).
+__device__ __forceinline__ u64 load8(const unsigned char* p, unsigned valid) {
+  const u64 a = reinterpret_cast<u64>(p);
+  const u64* w = reinterpret_cast<const u64*>(a & ~7ull);
+  const unsigned s = (unsigned)(a & 7) * 8;
+  u64 v = __ldg(w) >> s;
+  if (s && valid > 8 - s / 8) v |= __ldg(w + 1) << (64 - s);
+  return v;
+}
+
+// `len` bytes from src to dst by 16 lanes (`lane` 0 .. 15): bytes up to an 8-byte boundary of dst,
+// then a word per lane, then the bytes left. Reads and writes nothing outside the ranges but the
+// rest of the aligned words that hold source bytes.
+__device__ __forceinline__ void copy_line(const unsigned char* src, unsigned char* dst, u64 len, unsigned lane) {
+  u64 head = (8 - (reinterpret_cast<u64>(dst) & 7)) & 7;
+  if (head > len) head = len;
+  if (lane < head) dst[lane] = src[lane];
+  const u64 words = (len - head) / 8;
+  for (u64 w = lane; w < words; w += 16) *reinterpret_cast<u64*>(dst + head + 8 * w) = load8(src + head + 8 * w, 8);
+  const u64 done = head + 8 * words;
+  if (lane < len - done) dst[done + lane] = src[done + lane];
+}
+
+// One warp per record: bases (half of the warp) and qualities to their place in the output, eight
+// bytes a lane: a byte per lane took eight times the requests on both sides.
 __global__ void fastq_copy_kernel(const unsigned char* text, const u64* line_end, u64 n_reads, const u64* offsets,
                                   unsigned char* seq, unsigned char* qual) {
   const u64 r = ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned lane = threadIdx.x & 31;
+  const unsigned lane = threadIdx.x & 31, half = lane >> 4;
   if (r >= n_reads) return;
-  u64 s1, e1, s3, e3;
-  line_span(text, line_end, 4 * r + 1, s1, e1);
-  line_span(text, line_end, 4 * r + 3, s3, e3);
-  const u64 o = offsets[r], len = e1 - s1;
-  for (u64 i = lane; i < len; i += 32) {
-    seq[o + i] = text[s1 + i];
-    qual[o + i] = text[s3 + i];
-  }
+  const u64 o = offsets[r], len = offsets[r + 1] - o;
+  const u64 l = 4 * r + 1 + 2 * half;  // the bases' line, or the qualities'
+  copy_line(text + line_end[l - 1] + 1, (half ? qual : seq) + o, len, lane & 15);
 }
 
 // ------------------------------------------------------------------ launchers
 
-u64 fastq_chunks(u64 n_bytes) { return (n_bytes + kFqChunk - 1) / kFqChunk; }
+// Chunks begin at a 16-byte boundary: `head` bytes before the text belong to the first one.
+static unsigned fastq_head(const unsigned char* text) { return (unsigned)(reinterpret_cast<uintptr_t>(text) & 15); }
+
+u64 fastq_chunks(u64 n_bytes) { return n_bytes ? (n_bytes + 15 + kFqChunk - 1) / kFqChunk : 0; }
 
 cudaError_t launch_fastq_count(const unsigned char* text, u64 n, u64* chunk_counts, cudaStream_t stream) {
   const u64 chunks = fastq_chunks(n);
   if (!chunks) return cudaSuccess;
-  fastq_count_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, chunk_counts);
+  fastq_count_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, fastq_head(text), chunk_counts);
   return cudaGetLastError();
 }
 
@@ -217,7 +255,7 @@ cudaError_t launch_fastq_lines(const unsigned char* text, u64 n, const u64* chun
                                cudaStream_t stream) {
   const u64 chunks = fastq_chunks(n);
   if (!chunks) return cudaSuccess;
-  fastq_lines_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, chunk_offsets, line_end);
+  fastq_lines_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, fastq_head(text), chunk_offsets, line_end);
   return cudaGetLastError();
 }
 
