@@ -10,8 +10,8 @@
 //
 // GPU-native traversal instead of the paper's per-processor walks with conflict resolution:
 // the edges define a successor function on the 2m directed states (vertex, direction of
-// travel), and pointer jumping (Wyllie's list ranking, ceil(log2 2m) + 1 rounds) gives every
-// state its distance to the end of its chain and that end. A path appears as two opposite
+// travel), and pointer jumping (Wyllie's list ranking) gives every state its distance to the end
+// of its chain and that end. A path appears as two opposite
 // chains; every vertex picks the chain whose head has the smaller key (with forward keys:
 // always the forward chain), which fixes its contig, its position and its orientation.
 // Cycles (chains that never end) are cut at their smallest key, on that vertex's left side,
@@ -139,35 +139,48 @@ __global__ void cg_edge_kernel(const u64* keys, const unsigned char* codes, cons
 // State s = 2u + d: vertex u travelled forward (d = 0, leaving through its right side) or
 // backward (d = 1, leaving through its left). Its successor follows the edge on that side and
 // leaves the next vertex through the side opposite to the one it entered.
-__global__ void cg_succ_kernel(const unsigned* nbr, u64 m, unsigned* nxt, unsigned* dist, unsigned* endst) {
+//
+// A state's word (link) holds a state ahead of it on its chain (low half) and how many steps
+// ahead it is (high half); the last state of a chain points to itself, zero steps ahead. A jump
+// replaces it by what the state ahead knows: true whatever the other threads have done to their
+// words meanwhile, so the words are updated in place, and a thread jumps kHops times in one
+// launch. One 8-byte gather per jump; separate successor, distance and end arrays in rounds of
+// one jump each took three, and a launch and a host round trip per round (18 rounds for 2^18
+// steps, 7.0 ms for 4 M vertices; now 3 launches).
+
+constexpr int kHops = 16;
+
+__device__ __forceinline__ u64 cg_link(unsigned steps, unsigned ahead) { return ((u64)steps << 32) | ahead; }
+
+__global__ void cg_succ_kernel(const unsigned* nbr, u64 m, u64* link) {
   const u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= 2 * m) return;
   // edge (v << 1) | side of v entered: entering v on its left means leaving it on its right,
   // i.e. state 2v + 0, on its right state 2v + 1 -- the same number
   const unsigned n = nbr[(s & ~1ull) | (1u - (unsigned)(s & 1))];
-  nxt[s] = n;
-  dist[s] = n == kNil ? 0u : 1u;
-  endst[s] = (unsigned)s;
+  link[s] = n == kNil ? cg_link(0, (unsigned)s) : cg_link(1, n);
 }
 
-// One pointer-jumping round from (nxt, dist, endst) into the *2 arrays; *live is set when a
-// state still has a successor (every writer stores the same value).
-__global__ void cg_jump_kernel(const unsigned* nxt, const unsigned* dist, const unsigned* endst, u64 n_states,
-                               unsigned* nxt2, unsigned* dist2, unsigned* endst2, unsigned long long* live) {
+// The end of a chain has arrived in `l` if the state ahead points to itself.
+__device__ __forceinline__ bool cg_ends(u64 ahead_link, unsigned ahead) { return ahead_link == cg_link(0, ahead); }
+
+// kHops jumps of every state; *live is set when one is not at its chain's end yet (every writer
+// stores the same value). A state that has gone n_states steps without meeting an end is on a
+// cycle and stops.
+__global__ void cg_jump_kernel(u64* link, u64 n_states, unsigned long long* live) {
   const u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n_states) return;
-  const unsigned n = nxt[s];
-  if (n == kNil) {
-    nxt2[s] = kNil;
-    dist2[s] = dist[s];
-    endst2[s] = endst[s];
-    return;
+  volatile u64* v = link;
+  u64 l = v[s];
+  for (int hop = 0; hop < kHops; ++hop) {
+    const unsigned ahead = (unsigned)l;
+    const u64 steps = l >> 32, q = v[ahead];
+    if (cg_ends(q, ahead) || steps >= n_states) return;
+    const u64 sum = steps + (q >> 32);
+    l = cg_link((unsigned)(sum < n_states ? sum : n_states), (unsigned)q);  // capped: not used any more on a cycle
+    v[s] = l;
   }
-  const unsigned nn = nxt[n];
-  nxt2[s] = nn;
-  dist2[s] = dist[s] + dist[n];
-  endst2[s] = endst[n];
-  if (nn != kNil) *live = 1ull;
+  if (!cg_ends(v[(unsigned)l], (unsigned)l) && (l >> 32) < n_states) *live = 1ull;
 }
 
 __device__ __forceinline__ bool key_lt(const u64* keys, const unsigned* vrec, unsigned a, unsigned b) {
@@ -176,15 +189,23 @@ __device__ __forceinline__ bool key_lt(const u64* keys, const unsigned* vrec, un
   return ahi != bhi ? ahi < bhi : keys[2 * ra] < keys[2 * rb];
 }
 
-// Cycle minimum: states still live after ranking lie on cycles; carry the vertex with the
-// smallest key along the cycle by pointer jumping (mn = vertex index, nxt a fresh successor).
-__global__ void cg_min_init_kernel(const unsigned* live_nxt, const unsigned* succ, u64 n_states, unsigned* mn,
-                                   unsigned* nxt) {
+// Cycle minimum: states that have met no end lie on cycles; carry the vertex with the smallest
+// key along the cycle by pointer jumping (mn = vertex index, nxt the plain successor).
+__global__ void cg_min_init_kernel(const u64* link, const unsigned* nbr, u64 n_states, unsigned* mn, unsigned* nxt) {
   const u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n_states) return;
-  const bool on_cycle = live_nxt[s] != kNil;
+  const unsigned ahead = (unsigned)link[s];
+  const bool on_cycle = !cg_ends(link[ahead], ahead);
   mn[s] = on_cycle ? (unsigned)(s >> 1) : kNil;
-  nxt[s] = on_cycle ? succ[s] : kNil;
+  nxt[s] = on_cycle ? nbr[(s & ~1ull) | (1u - (unsigned)(s & 1))] : kNil;
+}
+
+// Whether any state is on a cycle.
+__global__ void cg_any_cycle_kernel(const u64* link, u64 n_states, unsigned long long* cycles) {
+  const u64 s = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= n_states) return;
+  const unsigned ahead = (unsigned)link[s];
+  if (!cg_ends(link[ahead], ahead)) *cycles = 1ull;
 }
 
 __global__ void cg_min_jump_kernel(const u64* keys, const unsigned* vrec, const unsigned* mn, const unsigned* nxt,
@@ -216,8 +237,7 @@ __global__ void cg_cut_kernel(const unsigned* mn, u64 m, unsigned* nbr, unsigned
 
 // Per vertex: the chosen chain (head with the smaller key; forward keys: the forward chain),
 // position in it, and the contig length in bases (heads only) for the offset scan.
-__global__ void cg_place_kernel(const u64* keys, const unsigned* vrec, const unsigned* dist, const unsigned* endst,
-                                u64 m, unsigned k, unsigned canonical, unsigned* head, unsigned* pos,
+__global__ void cg_place_kernel(const u64* keys, const unsigned* vrec, const u64* link, u64 m, unsigned k, unsigned canonical, unsigned* head, unsigned* pos,
                                 unsigned char* dir, u64* head_flag, u64* head_len) {
   const u64 u = (u64)blockIdx.x * blockDim.x + threadIdx.x;
   if (u > m) return;
@@ -226,8 +246,9 @@ __global__ void cg_place_kernel(const u64* keys, const unsigned* vrec, const uns
     head_len[m] = 0;
     return;
   }
-  const unsigned endF = endst[2 * u] >> 1, endB = endst[2 * u + 1] >> 1;
-  const unsigned distF = dist[2 * u], distB = dist[2 * u + 1];
+  const ulonglong2 l = reinterpret_cast<const ulonglong2*>(link)[u];
+  const unsigned endF = (unsigned)l.x >> 1, endB = (unsigned)l.y >> 1;
+  const unsigned distF = (unsigned)(l.x >> 32), distB = (unsigned)(l.y >> 32);
   // chain (u, 0) starts at endB, chain (u, 1) at endF
   const bool fwd = !canonical || endB == endF || key_lt(keys, vrec, endB, endF);
   head[u] = fwd ? endB : endF;
@@ -323,46 +344,45 @@ int contig_pass(const u64* keys, const unsigned char* codes, u64 n, unsigned k, 
   CG_TRY(cudaGetLastError());
   // edges
   const u64 ns = 2 * m;
-  unsigned *nbr = nullptr, *nxt = nullptr, *dist = nullptr, *endst = nullptr, *nxt2 = nullptr, *dist2 = nullptr,
-           *endst2 = nullptr;
-  unsigned long long* cnt = nullptr;  // [0] live states, [1] cycles
-  if (!alloc((void**)&nbr, ns * 4) || !alloc((void**)&nxt, ns * 4) || !alloc((void**)&dist, ns * 4) ||
-      !alloc((void**)&endst, ns * 4) || !alloc((void**)&nxt2, ns * 4) || !alloc((void**)&dist2, ns * 4) ||
-      !alloc((void**)&endst2, ns * 4) || !alloc((void**)&cnt, 16))
-    return fail(-2);
+  unsigned* nbr = nullptr;
+  u64* link = nullptr;
+  unsigned long long* cnt = nullptr;  // [0] live states / cycles seen, [1] cycles cut
+  if (!alloc((void**)&nbr, ns * 4) || !alloc((void**)&link, ns * 8) || !alloc((void**)&cnt, 16)) return fail(-2);
   CG_TRY(cudaMemsetAsync(cnt, 0, 16, st));
   if (ns) cg_edge_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(keys, codes, vrec, m, k, canonical, mkey, midx,
                                                               log2s, nbr);
   CG_TRY(cudaGetLastError());
-  // list ranking (twice if there are cycles: rank, cut the cycles, rank again)
+  // list ranking (twice if there are cycles: rank, cut the cycles, rank again). A launch at least
+  // doubles the steps every state has gone, so `rounds` of them are enough.
   unsigned rounds = 1;
   while ((1ull << rounds) < ns + 1) ++rounds;
   ++rounds;
-  for (int attempt = 0; attempt < 2; ++attempt) {
-    if (ns) cg_succ_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(nbr, m, nxt, dist, endst);
+  for (int attempt = 0; attempt < 2 && ns; ++attempt) {
+    cg_succ_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(nbr, m, link);
     CG_TRY(cudaGetLastError());
-    unsigned long long live = 0;
-    for (unsigned it = 0; it < rounds && ns; ++it) {
+    unsigned long long flag0 = 1;
+    for (unsigned it = 0; it < rounds && flag0; ++it) {
       CG_TRY(cudaMemsetAsync(cnt, 0, 8, st));
-      cg_jump_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(nxt, dist, endst, ns, nxt2, dist2, endst2, cnt);
+      cg_jump_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(link, ns, cnt);
       CG_TRY(cudaGetLastError());
-      std::swap(nxt, nxt2);
-      std::swap(dist, dist2);
-      std::swap(endst, endst2);
-      CG_TRY(cudaMemcpyAsync(&live, cnt, 8, cudaMemcpyDeviceToHost, st));
+      if (it == 0) continue;  // one launch is never enough for the longest chains of a real sample
+      CG_TRY(cudaMemcpyAsync(&flag0, cnt, 8, cudaMemcpyDeviceToHost, st));
       CG_TRY(cudaStreamSynchronize(st));
-      if (live == 0) break;
     }
-    if (live == 0) break;
+    if (flag0) return fail(-1);  // cannot happen
+    CG_TRY(cudaMemsetAsync(cnt, 0, 8, st));
+    cg_any_cycle_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(link, ns, cnt);
+    CG_TRY(cudaGetLastError());
+    CG_TRY(cudaMemcpyAsync(&flag0, cnt, 8, cudaMemcpyDeviceToHost, st));
+    CG_TRY(cudaStreamSynchronize(st));
+    if (!flag0) break;
     if (attempt == 1) return fail(-1);  // cycles left after cutting: cannot happen
-    // states still live lie on cycles: find each cycle's smallest vertex and cut there
+    // find each cycle's smallest vertex and cut there
     unsigned *mnA = nullptr, *mnB = nullptr, *nxA = nullptr, *nxB = nullptr;
     if (!alloc((void**)&mnA, ns * 4) || !alloc((void**)&mnB, ns * 4) || !alloc((void**)&nxA, ns * 4) ||
         !alloc((void**)&nxB, ns * 4))
       return fail(-2);
-    cg_succ_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(nbr, m, nxB, dist2, endst2);  // fresh successors
-    CG_TRY(cudaGetLastError());
-    cg_min_init_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(nxt, nxB, ns, mnA, nxA);
+    cg_min_init_kernel<<<blocks_for(ns), kCgThreads, 0, st>>>(link, nbr, ns, mnA, nxA);
     CG_TRY(cudaGetLastError());
     unsigned* mn = mnA;
     for (unsigned it = 0; it < rounds; ++it) {
@@ -376,12 +396,12 @@ int contig_pass(const u64* keys, const unsigned char* codes, u64 n, unsigned k, 
     CG_TRY(cudaGetLastError());
   }
   // placement, offsets, bases
-  unsigned *head = nxt2, *pos = dist2;
+  unsigned *head = nullptr, *pos = nullptr;
   unsigned char* dir = nullptr;
   u64 *hflag = nullptr, *hlen = nullptr;
-  if (!alloc((void**)&dir, m) || !alloc((void**)&hflag, (m + 1) * 8) || !alloc((void**)&hlen, (m + 1) * 8))
+  if (!alloc((void**)&head, m * 4) || !alloc((void**)&pos, m * 4) || !alloc((void**)&dir, m) || !alloc((void**)&hflag, (m + 1) * 8) || !alloc((void**)&hlen, (m + 1) * 8))
     return fail(-2);
-  cg_place_kernel<<<blocks_for(m + 1), kCgThreads, 0, st>>>(keys, vrec, dist, endst, m, k, canonical, head, pos, dir,
+  cg_place_kernel<<<blocks_for(m + 1), kCgThreads, 0, st>>>(keys, vrec, link, m, k, canonical, head, pos, dir,
                                                            hflag, hlen);
   CG_TRY(cudaGetLastError());
   CG_TRY(scan_exclusive(hflag, m + 1, scan_tmp, st));
