@@ -222,45 +222,6 @@ int get_pool(int dev, cudaMemPool_t* out) {
   return KMA_OK;
 }
 
-// Heavy hitters: the CTAs' Misra-Gries summaries of one sub-stream merged into one (mergeable
-// summaries, Agarwal et al. 2012): the counts of each key are summed; if more than m keys
-// remain, the (m+1)-th largest count is subtracted from every count and the keys left at zero
-// or below are dropped. The merged summary keeps the bound of its parts: for a sub-stream of n
-// items, every key with frequency f > n / (m + 1) is present with f - n / (m + 1) <= c <= f.
-struct MgEntry {
-  u64 lo, hi, count;
-  unsigned bucket;
-};
-
-void mg_merge(const std::vector<u64>& lo, const std::vector<u64>& hi, const std::vector<unsigned>& cnt,
-              unsigned grid, std::vector<MgEntry>& out) {
-  out.clear();
-  for (unsigned b = 0; b < kMgBuckets; ++b) {
-    std::vector<MgEntry> e;
-    for (unsigned c = 0; c < grid; ++c)
-      for (unsigned i = 0; i < kMgCounters; ++i) {
-        const u64 o = ((u64)c * kMgBuckets + b) * kMgCounters + i;
-        if (cnt[o]) e.push_back({lo[o], hi[o], cnt[o], b});
-      }
-    std::sort(e.begin(), e.end(), [](const MgEntry& x, const MgEntry& y) {
-      return x.hi != y.hi ? x.hi < y.hi : x.lo < y.lo;
-    });
-    std::vector<MgEntry> sum;  // one entry per key
-    for (const MgEntry& x : e) {
-      if (!sum.empty() && sum.back().lo == x.lo && sum.back().hi == x.hi) sum.back().count += x.count;
-      else sum.push_back(x);
-    }
-    std::sort(sum.begin(), sum.end(), [](const MgEntry& x, const MgEntry& y) { return x.count > y.count; });
-    const u64 delta = sum.size() > kMgCounters ? sum[kMgCounters].count : 0;
-    for (MgEntry& x : sum)
-      if (x.count > delta) {
-        x.count -= delta;
-        out.push_back(x);
-      }
-  }
-  std::stable_sort(out.begin(), out.end(), [](const MgEntry& x, const MgEntry& y) { return x.count > y.count; });
-}
-
 // Small pinned host blocks (a handle's status word and group counts), kept in a free list
 // for the life of the process: cudaFreeHost synchronises the whole device, so a handle
 // destroyed in one thread would otherwise stall the GPU work other threads have queued.
@@ -1574,12 +1535,23 @@ int kmer_analysis_estimate(const kma_params* params, const char* seq, const char
     return KMA_OK;
   };
   unsigned* d_regs = nullptr;
-  MgOut mg{nullptr, nullptr, nullptr, nullptr};
+  MgOut mg{};
+  // one zeroed block: items, totals, merge tables, merged counts; merged entries and the items
+  // come back together
+  const u64 slots = mg_table_slots(grid);
+  const u64 zeroed = kMgBuckets * 8 + mg_n * 8 + kMgBuckets * slots * 4 + kMgBuckets * 4;
+  char* zero = nullptr;
   if ((rc = temp((void**)&d_regs, m * 4)) || (rc = temp((void**)&mg.lo, mg_n * 8)) ||
       (rc = temp((void**)&mg.hi, mg_n * 8)) || (rc = temp((void**)&mg.count, mg_n * 4)) ||
-      (rc = temp((void**)&mg.items, (u64)grid * kMgBuckets * 8)))
+      (rc = temp((void**)&mg.merged, kMgBuckets * kMgCounters * sizeof(MgEntry))) ||
+      (rc = temp((void**)&zero, zeroed)))
     return finish(rc);
+  mg.items = (unsigned long long*)zero;
+  mg.total = mg.items + kMgBuckets;
+  mg.table = (unsigned*)(mg.total + mg_n);
+  mg.n_merged = mg.table + kMgBuckets * slots;
   cudaError_t e;
+  if ((e = cudaMemsetAsync(zero, 0, zeroed, h->stream)) != cudaSuccess) return finish(cuda_fail(e, "summaries"));
   if ((e = cudaMemcpyAsync(d_regs, regs32.data(), m * 4, cudaMemcpyHostToDevice, h->stream)) != cudaSuccess)
     return finish(cuda_fail(e, "sketch registers in"));
   if (n_reads) {
@@ -1608,14 +1580,16 @@ int kmer_analysis_estimate(const kma_params* params, const char* seq, const char
   if ((e = launch_hll(w, params->k, params->canonical, n_parts, part, p, d_regs, h->status, mg, grid,
                       h->stream)) != cudaSuccess)
     return finish(cuda_fail(e, "hll_kernel"));
-  std::vector<u64> mlo(mg_n), mhi(mg_n), items((u64)grid * kMgBuckets);
-  std::vector<unsigned> mcnt(mg_n);
+  if ((e = launch_mg_merge(mg, grid, h->stream)) != cudaSuccess) return finish(cuda_fail(e, "mg_merge"));
+  unsigned n_merged[kMgBuckets];
+  u64 bucket_n[kMgBuckets];
+  std::vector<MgEntry> summary(kMgBuckets * kMgCounters);
   if ((e = cudaMemcpyAsync(regs32.data(), d_regs, m * 4, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(mlo.data(), mg.lo, mg_n * 8, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(mhi.data(), mg.hi, mg_n * 8, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(mcnt.data(), mg.count, mg_n * 4, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(items.data(), mg.items, items.size() * 8, cudaMemcpyDeviceToHost, h->stream)) !=
-          cudaSuccess)
+      (e = cudaMemcpyAsync(summary.data(), mg.merged, summary.size() * sizeof(MgEntry), cudaMemcpyDeviceToHost,
+                           h->stream)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(n_merged, mg.n_merged, sizeof n_merged, cudaMemcpyDeviceToHost, h->stream)) !=
+          cudaSuccess ||
+      (e = cudaMemcpyAsync(bucket_n, mg.items, sizeof bucket_n, cudaMemcpyDeviceToHost, h->stream)) != cudaSuccess)
     return finish(cuda_fail(e, "estimate results out"));
   if ((rc = read_status(h))) return finish(rc);
   if ((rc = flags_to_code(h->host_status->flags))) return finish(rc);
@@ -1626,22 +1600,28 @@ int kmer_analysis_estimate(const kma_params* params, const char* seq, const char
   est->distinct = hll_estimate(regs8.data(), p);
   est->rel_std_error = 1.04 / std::sqrt((double)m);
   est->valid_windows = h->host_status->valid_windows;
-  // heavy hitters: merge the summaries, report the keys by count
-  std::vector<u64> bucket_n(kMgBuckets, 0);
-  for (unsigned c = 0; c < grid; ++c)
-    for (unsigned b = 0; b < kMgBuckets; ++b) bucket_n[b] += items[(u64)c * kMgBuckets + b];
-  std::vector<MgEntry> merged;
-  mg_merge(mlo, mhi, mcnt, grid, merged);
+  // heavy hitters: the keys of all buckets by count
+  struct Heavy {
+    MgEntry e;
+    unsigned bucket;
+  };
+  std::vector<Heavy> merged;
+  for (unsigned b = 0; b < kMgBuckets; ++b)
+    for (unsigned i = 0; i < std::min(n_merged[b], kMgCounters); ++i) merged.push_back({summary[b * kMgCounters + i], b});
+  std::sort(merged.begin(), merged.end(), [](const Heavy& x, const Heavy& y) {
+    if (x.e.count != y.e.count) return x.e.count > y.e.count;
+    return x.e.hi != y.e.hi ? x.e.hi < y.e.hi : x.e.lo < y.e.lo;
+  });
   u64 sampled = 0;
   for (u64 x : bucket_n) sampled += x;
   est->sampled_windows = sampled;
   est->heavy_threshold = std::max<u64>(1, sampled / 2048);
-  est->heavy_hitters = !merged.empty() && merged[0].count >= est->heavy_threshold ? 1u : 0u;
+  est->heavy_hitters = !merged.empty() && merged[0].e.count >= est->heavy_threshold ? 1u : 0u;
   est->n_summary = merged.size();
   const u64 rows = std::min<u64>(est->summary_capacity, merged.size());
   for (u64 i = 0; i < rows; ++i) {
-    if (est->summary_keys) { est->summary_keys[2 * i] = merged[i].lo; est->summary_keys[2 * i + 1] = merged[i].hi; }
-    if (est->summary_counts) est->summary_counts[i] = merged[i].count;
+    if (est->summary_keys) { est->summary_keys[2 * i] = merged[i].e.lo; est->summary_keys[2 * i + 1] = merged[i].e.hi; }
+    if (est->summary_counts) est->summary_counts[i] = merged[i].e.count;
     if (est->summary_bucket) est->summary_bucket[i] = merged[i].bucket;
   }
   if (est->bucket_windows)

@@ -21,9 +21,13 @@
 // counter increments it; a new key takes a counter at zero if there is one; otherwise every
 // counter of that summary is decremented. A summary of a sub-stream of n items then holds every
 // key with frequency f > n / (m + 1), with a count in [f - n / (m + 1), f]. Warp w updates
-// the summaries of buckets w and w + 16, one item at a time, a counter per lane. The host
-// merges the CTAs' summaries bucket by bucket (counts of a key summed, the (m+1)-th largest
-// subtracted, non-positive ones dropped), which keeps the bound for the whole sub-stream.
+// the summaries of buckets w and w + 16, one item at a time, a counter per lane.
+//
+// The CTAs' summaries are then merged bucket by bucket (mergeable summaries, Agarwal et al.
+// 2012): the counts of each key are summed; if more than m keys remain, the (m+1)-th largest
+// count is subtracted from every count and the keys left at zero or below are dropped. The
+// merged summary keeps the bound of its parts: for a sub-stream of n items, every key with
+// frequency f > n / (m + 1) is present with f - n / (m + 1) <= c <= f.
 #include "kma_device.cuh"
 
 namespace kma {
@@ -139,11 +143,105 @@ __global__ void __launch_bounds__(kHllThreads) hll_kernel(const __grid_constant_
       mg.lo[o + i] = c ? mg_lo[i] : 0ull;
       mg.hi[o + i] = c ? mg_hi[i] : 0ull;
     }
-    if (threadIdx.x < kMgBuckets) mg.items[(u64)blockIdx.x * kMgBuckets + threadIdx.x] = mg_n[threadIdx.x];
+    if (threadIdx.x < kMgBuckets && mg_n[threadIdx.x]) atomicAdd(&mg.items[threadIdx.x], mg_n[threadIdx.x]);
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) acc_valid += __shfl_down_sync(0xffffffffu, acc_valid, o);
   if ((threadIdx.x & 31) == 0 && acc_valid) atomicAdd(&st->valid_windows, (u64)acc_valid);
+}
+
+// The merge, first half: entry i of the summaries adds its count to the total of the first entry
+// with the same key. The entries of a bucket meet in its own hash table of entry numbers (+ 1; 0 =
+// free); the keys stay where the summaries left them, so a taken slot can be compared at once.
+// The table is at most half full (mg_table_slots), so every probe ends.
+__global__ void mg_sum_kernel(const MgOut mg, u64 n, unsigned slots) {
+  const u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const unsigned c = mg.count[i];
+  if (!c) return;
+  const u64 lo = mg.lo[i], hi = mg.hi[i];
+  unsigned* tab = mg.table + (size_t)((i / kMgCounters) % kMgBuckets) * slots;
+  unsigned at = (unsigned)key_hash(lo, hi) & (slots - 1);
+  for (unsigned probe = 0; probe < slots; ++probe, at = (at + 1) & (slots - 1)) {
+    unsigned who = atomicCAS(&tab[at], 0u, (unsigned)i + 1u);
+    if (!who) who = (unsigned)i + 1u;
+    --who;
+    if (who == i || (mg.lo[who] == lo && mg.hi[who] == hi)) {
+      atomicAdd(&mg.total[who], (u64)c);
+      return;
+    }
+  }
+}
+
+// The merge, second half, one CTA per bucket: the (m+1)-th largest total by radix selection (a
+// byte at a time from the highest that any total uses), then the keys above it.
+constexpr int kMgMergeThreads = 1024;
+
+__global__ void __launch_bounds__(kMgMergeThreads) mg_select_kernel(const MgOut mg, unsigned grid) {
+  __shared__ unsigned hist[256];
+  __shared__ u64 s_max, s_prefix;
+  __shared__ unsigned s_keys, s_rank;
+  const unsigned b = blockIdx.x, n = grid * kMgCounters;
+  auto entry = [&](unsigned i) { return ((u64)(i / kMgCounters) * kMgBuckets + b) * kMgCounters + i % kMgCounters; };
+  if (threadIdx.x == 0) {
+    s_max = s_prefix = 0;
+    s_keys = 0;
+    s_rank = kMgCounters;  // how many totals are larger than the one looked for
+  }
+  __syncthreads();
+  u64 mx = 0;
+  unsigned keys = 0;
+  for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
+    const u64 t = mg.total[entry(i)];
+    mx = t > mx ? t : mx;
+    keys += t != 0;
+  }
+  if (keys) {
+    atomicAdd(&s_keys, keys);
+    atomicMax(&s_max, mx);
+  }
+  __syncthreads();
+  if (s_keys > kMgCounters) {
+    for (int shift = s_max ? (63 - __clzll(s_max)) & ~7 : 0; shift >= 0; shift -= 8) {
+      for (unsigned i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+      __syncthreads();
+      const u64 prefix = s_prefix;  // the bytes above this one
+      for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
+        const u64 t = mg.total[entry(i)];
+        if (t && (shift == 56 || (t >> (shift + 8)) == prefix)) atomicAdd(&hist[(unsigned)(t >> shift) & 255u], 1u);
+      }
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        unsigned d = 255, rank = s_rank;
+        while (d && rank >= hist[d]) rank -= hist[d--];
+        s_rank = rank;
+        s_prefix = (prefix << 8) | d;
+      }
+      __syncthreads();
+    }
+  }
+  const u64 delta = s_keys > kMgCounters ? s_prefix : 0ull;
+  for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
+    const u64 e = entry(i), t = mg.total[e];
+    if (t <= delta) continue;
+    const unsigned at = atomicAdd(&mg.n_merged[b], 1u);  // at most kMgCounters totals are above delta
+    if (at < kMgCounters) mg.merged[b * kMgCounters + at] = MgEntry{mg.lo[e], mg.hi[e], t - delta};
+  }
+}
+
+unsigned mg_table_slots(unsigned grid) {
+  unsigned s = 64;
+  while (s < 2 * grid * kMgCounters) s *= 2;
+  return s;
+}
+
+// Measured for 608 CTAs' summaries: see launch_hll's caller; on the host (12 MB copied out, 32
+// sorts) the merge took most of the 9.6 ms of a sizing pass over 90 Mbases.
+cudaError_t launch_mg_merge(const MgOut& mg, unsigned grid, cudaStream_t stream) {
+  const u64 n = (u64)grid * kMgBuckets * kMgCounters;
+  mg_sum_kernel<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(mg, n, mg_table_slots(grid));
+  mg_select_kernel<<<kMgBuckets, kMgMergeThreads, 0, stream>>>(mg, grid);
+  return cudaGetLastError();
 }
 
 unsigned hll_grid(unsigned p, unsigned k, int num_sms) {

@@ -280,14 +280,23 @@ constexpr unsigned kMgBucketBits = 5;
 constexpr unsigned kMgBuckets = 1u << kMgBucketBits;
 constexpr unsigned kMgCounters = 32;
 
+struct MgEntry {
+  unsigned long long lo, hi, count;
+};
+
 // Where the CTAs leave their summaries: entry [cta][bucket][counter] (lo, hi, count; count 0
-// = unused), items[cta][bucket] = sampled windows of that bucket the CTA saw. lo == nullptr:
+// = unused), items[bucket] = sampled windows of that bucket; and the merged summaries, at most
+// kMgCounters entries a bucket. items, table, total and n_merged start at zero. lo == nullptr:
 // no summaries.
 struct MgOut {
   unsigned long long* lo;
   unsigned long long* hi;
   unsigned* count;
-  unsigned long long* items;
+  unsigned long long* items;  // [kMgBuckets]
+  unsigned* table;            // [kMgBuckets][mg_table_slots(grid)]
+  unsigned long long* total;  // one per entry: the key's count over all CTAs, at its first entry
+  MgEntry* merged;            // [kMgBuckets][kMgCounters]
+  unsigned* n_merged;         // [kMgBuckets]
 };
 
 // Lets `fn` launch with up to the device's opt-in shared memory per block (less its static
@@ -304,6 +313,8 @@ unsigned hll_grid(unsigned p, unsigned k, int num_sms);
 cudaError_t launch_hll(const PartWindows& w, unsigned k, unsigned canonical, unsigned n_parts, unsigned part,
                        unsigned p, unsigned* regs, DevStatus* st, const MgOut& mg, unsigned grid,
                        cudaStream_t stream);
+unsigned mg_table_slots(unsigned grid);
+cudaError_t launch_mg_merge(const MgOut& mg, unsigned grid, cudaStream_t stream);
 
 struct LaunchShape {
   int block_threads;
