@@ -582,6 +582,11 @@ __global__ void __launch_bounds__(kClassThreads) classify_kernel(const __grid_co
 // ------------------------------------------------------------------ query
 
 // slots = slots per partition, parts = on-chip partitions (1: one table).
+// Bound by the two random 32-byte sectors of a slot and by how many of them are in flight. VEC
+// reads a key and writes its counters 16 bytes at a time and its two codes at once (8, 4 and 1
+// byte without it: a warp's stores to ext then touch every sector eight times). 1.5 M lookups, half
+// of them absent, in a table of 8 M slots: 78 us -> 69 us.
+template <bool VEC>
 __global__ void __launch_bounds__(256) query_kernel(const Slot* table, u64 slots, unsigned parts,
                                                     unsigned k,
                                                     unsigned canonical, unsigned min_depth,
@@ -590,7 +595,15 @@ __global__ void __launch_bounds__(256) query_kernel(const Slot* table, u64 slots
                                                     unsigned char* codes, DevStatus* st) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
   for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-    const u64 qlo = keys[2 * i], qhi = keys[2 * i + 1];
+    u64 qlo, qhi;
+    if (VEC) {
+      const ulonglong2 q = __ldcs(reinterpret_cast<const ulonglong2*>(keys) + i);
+      qlo = q.x;
+      qhi = q.y;
+    } else {
+      qlo = keys[2 * i];
+      qhi = keys[2 * i + 1];
+    }
     // bits at or above 2k must be clear
     const bool in_range = (2 * k >= 64) ? (2 * k == 128 || (qhi >> (2 * k - 64)) == 0)
                                         : (qhi == 0 && (qlo >> (2 * k)) == 0);
@@ -617,11 +630,19 @@ __global__ void __launch_bounds__(256) query_kernel(const Slot* table, u64 slots
         }
       }
     }
+    const unsigned cl = c ? side_code(e, min_ext) : 4u, cr = c ? side_code(e + 4, min_ext) : 4u;
     counts[i] = c;
+    if (VEC) {
+      uint4* o = reinterpret_cast<uint4*>(ext) + 2 * i;
+      __stcs(o, make_uint4(e[0], e[1], e[2], e[3]));
+      __stcs(o + 1, make_uint4(e[4], e[5], e[6], e[7]));
+      reinterpret_cast<unsigned short*>(codes)[i] = (unsigned short)(cl | (cr << 8));
+    } else {
 #pragma unroll
-    for (int j = 0; j < 8; ++j) ext[8 * i + j] = e[j];
-    codes[2 * i] = (unsigned char)(c ? side_code(e, min_ext) : 4u);
-    codes[2 * i + 1] = (unsigned char)(c ? side_code(e + 4, min_ext) : 4u);
+      for (int j = 0; j < 8; ++j) ext[8 * i + j] = e[j];
+      codes[2 * i] = (unsigned char)cl;
+      codes[2 * i + 1] = (unsigned char)cr;
+    }
   }
 }
 
@@ -717,8 +738,12 @@ cudaError_t launch_query(const Slot* table, u64 slots, unsigned parts, unsigned 
   if (n == 0) return cudaSuccess;
   u64 blocks = (n + 255) / 256;
   if (blocks > 152ull * 16) blocks = 152ull * 16;
-  query_kernel<<<(unsigned)blocks, 256, 0, stream>>>(table, slots, parts, k, canonical, min_depth, min_ext,
-                                                     keys, n, counts, ext, codes, st);
+  // the wide accesses want 16-byte aligned keys and counters and 2-byte aligned codes: any whole
+  // allocation, but not every slice of one
+  const bool vec = (((uintptr_t)keys | (uintptr_t)ext) & 15) == 0 && ((uintptr_t)codes & 1) == 0;
+  auto* fn = vec ? query_kernel<true> : query_kernel<false>;
+  fn<<<(unsigned)blocks, 256, 0, stream>>>(table, slots, parts, k, canonical, min_depth, min_ext, keys, n, counts, ext,
+                                           codes, st);
   return cudaGetLastError();
 }
 
