@@ -39,6 +39,28 @@ def test_tile_edges(gpu, k, canonical):
         both(gpu, rs, f"k={k} n={n}", partitions=3)
 
 
+@pytest.mark.parametrize("threshold", [0, 20, 41, 300])
+def test_packing(gpu, threshold):
+    """Reads and qualities that start at different bytes of a 16-byte piece, reads of every length
+    from none to more than a word, and thresholds that all, some and no qualities reach."""
+    from paper_1705_11147_gb300 import KmerAnalysis, make_params
+    rng = np.random.default_rng(11)
+    lens = list(range(0, 70)) + [0] * 70 + [1, 2] * 40 + [63, 64, 65, 127, 128, 129, 20_000]
+    reads = [one_read(n, 70 + n, "ACGTACGTacgtNx") for n in lens] * 2
+    quals = ["".join(chr(33 + x) for x in rng.integers(0, 42, len(r))) for r in reads]
+    rs = readset(reads, quals, k=5, min_depth=1, min_ext_count=1, qual_threshold=threshold)
+    want = oracle_for(rs)
+    for a, b in ((0, 0), (1, 1), (3, 8), (15, 0), (0, 15), (7, 6)):
+        seq, qual = (gpu.zeros(rs.n_bases + 16, dtype=gpu.uint8, device="cuda")[o:o + rs.n_bases] for o in (a, b))
+        seq.copy_(gpu.from_numpy(rs.seq))
+        qual.copy_(gpu.from_numpy(rs.qual))
+        with KmerAnalysis(make_params(max_bases=rs.n_bases, max_reads=rs.n_reads, expected_distinct=rs.n_bases, use_bloom=False,
+                                      **rs.meta["params"])) as ka:
+            ka.count(seq, qual, gpu.from_numpy(rs.offsets.astype(np.int64)).cuda())
+            ka.finalize()
+            assert_same(ka.copy_result().sorted(), want, (a, b))
+
+
 @pytest.mark.parametrize("k", [31, 33])
 @pytest.mark.parametrize("kind", ["one key", "few keys", "crowded", "distinct", "mixed"])
 def test_sub_bucket_shapes(gpu, k, kind):
