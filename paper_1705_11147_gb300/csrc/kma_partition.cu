@@ -293,18 +293,29 @@ __global__ void __launch_bounds__(kScatterThreads, 1) part_scatter_kernel(const 
 // One work item = a chunk of scatter tiles x kSplitBuckets adjacent buckets. The offset rows of
 // the chunk's tiles are read once for all of the item's buckets (adjacent entries of a row).
 // Per bucket: the lengths of its runs are scanned, the records gathered into shared memory (a
-// few lanes per run, 8- or 16-byte asynchronous copies) and sorted by sub-bucket like a scatter
-// tile, at most kPartSubTile at a time (a chunk is sized so that one such sub-tile is the rule).
+// few lanes per run, 8- or 16-byte asynchronous copies) and ordered by sub-bucket (a list of
+// record numbers: the records stay where they are), at most kPartSubTile at a time (a chunk is
+// sized so that one such sub-tile is the rule).
 // Each sub-bucket's run then takes the next places of its sub-bucket (one atomic per run) and is
 // written there, so that the count kernel finds a sub-bucket in one piece: gathering it there, a
 // handful of records per run, took more instructions than the counting. Items go through the
 // buckets in order, so the pieces of one line meet in L2. A sub-bucket has room for G.cap
 // records; what does not fit (very frequent k-mers) goes to an overflow segment of the bucket.
+//
+// Bound by the instructions issued, about 150 a record; a third and a fourth CTA per SM (40 and 32
+// registers) and sub-tiles of 3072, 6144 or 8192 records were slower. 166 M records of 16 bytes:
+// 0.94 ms; 2.4 G of 8 bytes: 25 ms (1.17 and 27 ms when the records were moved to their sorted
+// places, from and to registers).
 
 constexpr int kSplitThreads = 512;
 constexpr int kSplitItems = kPartSubTile / kSplitThreads;
 constexpr int kSplitMaxPer = kMaxSubBuckets / kSplitThreads;  // sub-buckets per thread
 static_assert(kPartSubTile <= 8192, "ranks are 13 bits");
+
+// Where sub-bucket p of n comes in a sorted sub-tile: thread t sorts p = t, t + kSplitThreads, ..
+__device__ __forceinline__ unsigned sub_order(unsigned p, unsigned n) {
+  return (p % kSplitThreads) * ((n + kSplitThreads - 1) / kSplitThreads) + p / kSplitThreads;
+}
 
 // First overflow segment of each bucket of [b0, b1): a sub-tile makes one at most.
 constexpr int kBaseThreads = 1024;
@@ -329,7 +340,7 @@ __global__ void __launch_bounds__(kBaseThreads) part_base_kernel(const u64* tota
 }
 
 __host__ __device__ constexpr size_t split_smem(unsigned chunk_tiles, unsigned sub_max, int kw) {
-  return (size_t)kPartSubTile * kw * 8 + (size_t)sub_max * (4 + 4 + 2) + 32 * 4 + (size_t)chunk_tiles * 4 +
+  return (size_t)kPartSubTile * (kw * 8 + 2) + (size_t)sub_max * (4 + 4 + 2) + 32 * 4 + (size_t)chunk_tiles * 4 +
          (((size_t)chunk_tiles * (kSplitBuckets + 1) * 2 + 15) & ~(size_t)15);
 }
 
@@ -340,7 +351,8 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
   extern __shared__ __align__(128) unsigned char s_raw[];
   __shared__ u64 s_over;
   u64* s_rec = reinterpret_cast<u64*>(s_raw);                                  // [sub-tile * KW]
-  unsigned* s_bin = reinterpret_cast<unsigned*>(s_rec + kPartSubTile * KW);    // [sub_max] counts, then offsets
+  unsigned short* s_ord = reinterpret_cast<unsigned short*>(s_rec + kPartSubTile * KW);  // [sub-tile] the record at a sorted position
+  unsigned* s_bin = reinterpret_cast<unsigned*>(s_ord + kPartSubTile);         // [sub_max] counts, then offsets
   unsigned* s_to = s_bin + G.sub_max;                                          // [sub_max] place minus sorted position
   unsigned* s_wsum = s_to + G.sub_max;                                         // [32]
   unsigned* s_dst = s_wsum + 32;                                               // [chunk tiles] first record of the run
@@ -395,7 +407,14 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
         for (unsigned p = tid; p < n_sub; p += kSplitThreads) s_bin[p] = 0;
         __syncthreads();  // also: s_dst is set, the previous sub-tile has been written
         // gather the window [w0, w0 + n) of the bucket's records
-        for (unsigned i = gi; i < nt; i += gn) {
+        if (total <= kPartSubTile) {
+          for (unsigned i = gi; i < nt; i += gn) {
+            const unsigned a = s_off[i * (kSplitBuckets + 1) + j], len = s_off[i * (kSplitBuckets + 1) + j + 1] - a;
+            const u64* src = T.recs + ((u64)(t0 + i) * kPartTile + a + gl) * KW;
+            unsigned dst = smem_u32(s_rec) + (s_dst[i] + gl) * (8 * KW);
+            for (unsigned x = gl; x < len; x += glanes, src += glanes * KW, dst += glanes * 8 * KW) cp_async<8 * KW>(dst, src);
+          }
+        } else for (unsigned i = gi; i < nt; i += gn) {
           const unsigned a = s_off[i * (kSplitBuckets + 1) + j], len = s_off[i * (kSplitBuckets + 1) + j + 1] - a;
           const unsigned d = s_dst[i];
           if (d >= w0 + n || d + len <= w0) continue;
@@ -406,21 +425,13 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
         }
         cp_async_wait_all();
         __syncthreads();
-        u64 r0[kSplitItems], r1[kSplitItems];
         unsigned pr[kSplitItems];
 #pragma unroll
         for (int y = 0; y < kSplitItems; ++y) {
           const unsigned x = y * kSplitThreads + tid;
           pr[y] = 0xFFFFFFFFu;
           if (x < n) {
-            if (KW == 1) {
-              r0[y] = s_rec[x];
-            } else {
-              const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[x];
-              r0[y] = v.x;
-              r1[y] = v.y;
-            }
-            const unsigned p = sub_of(r0[y], G.log_b, n_sub);
+            const unsigned p = sub_of(s_rec[x * KW], G.log_b, n_sub);
             pr[y] = (p << 13) | atomicAdd(&s_bin[p], 1u);
           }
         }
@@ -430,16 +441,18 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
         unsigned lc = 0, tot2;
 #pragma unroll
         for (unsigned x = 0; x < kSplitMaxPer; ++x) {  // places taken; in flight during the scan
-          const unsigned p = tid * per_sub + x;
-          c[x] = x < per_sub && p < n_sub ? s_bin[p] : 0u;
+          if (x >= per_sub) break;
+          const unsigned p = x * kSplitThreads + tid;
+          c[x] = p < n_sub ? s_bin[p] : 0u;
           at[x] = c[x] ? atomicAdd(&S.fill[sub0 + p], (u64)c[x]) : 0;
           lc += c[x];
         }
         unsigned ro = block_scan<kSplitThreads>(lc, s_wsum, tot2);
 #pragma unroll
         for (unsigned x = 0; x < kSplitMaxPer; ++x) {
-          const unsigned p = tid * per_sub + x;
-          if (x < per_sub && p < n_sub) {
+          if (x >= per_sub) break;
+          const unsigned p = x * kSplitThreads + tid;
+          if (p < n_sub) {
             s_bin[p] = ro;
             ro += c[x];
           }
@@ -448,15 +461,14 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 #pragma unroll
         for (int y = 0; y < kSplitItems; ++y) {
           if (pr[y] == 0xFFFFFFFFu) continue;
-          const unsigned to = s_bin[pr[y] >> 13] + (pr[y] & 8191u);
-          if (KW == 1) s_rec[to] = r0[y];
-          else reinterpret_cast<ulonglong2*>(s_rec)[to] = make_ulonglong2(r0[y], r1[y]);
+          s_ord[s_bin[pr[y] >> 13] + (pr[y] & 8191u)] = (unsigned short)(y * kSplitThreads + tid);
         }
         unsigned over = 0;  // the places, taken by now
 #pragma unroll
         for (unsigned x = 0; x < kSplitMaxPer; ++x) {
-          const unsigned p = tid * per_sub + x;
-          if (x < per_sub && p < n_sub) {
+          if (x >= per_sub) break;
+          const unsigned p = x * kSplitThreads + tid;
+          if (p < n_sub) {
             const unsigned room = at[x] < G.cap ? G.cap - (unsigned)at[x] : 0u, fits = c[x] < room ? c[x] : room;
             const unsigned o = s_bin[p];
             s_to[p] = p * G.cap + (unsigned)at[x] - o;
@@ -471,8 +483,9 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
           unsigned o = block_scan<kSplitThreads>(over, s_wsum, n_over);
 #pragma unroll
           for (unsigned x = 0; x < kSplitMaxPer; ++x) {
-            const unsigned p = tid * per_sub + x;
-            if (x < per_sub && p < n_sub) {
+            if (x >= per_sub) break;
+            const unsigned p = x * kSplitThreads + tid;
+            if (p < n_sub) {
               s_bin[p] = o - s_lim[p];  // overflow number minus sorted position
               o += c[x];
             }
@@ -489,12 +502,30 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
           }
           __syncthreads();
         }
+        if (!any_over) {
+#pragma unroll
+          for (int y = 0; y < kSplitItems; ++y) {
+            const unsigned i = y * kSplitThreads + tid;
+            if (i >= n) break;
+            u64 v0, v1 = 0;
+            if (KW == 1) {
+              v0 = s_rec[s_ord[i]];
+            } else {
+              const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[s_ord[i]];
+              v0 = v.x;
+              v1 = v.y;
+            }
+            u64* to = out + (u64)(s_to[sub_of(v0, G.log_b, n_sub)] + i) * KW;
+            if (KW == 1) *to = v0;
+            else *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(v0, v1);
+          }
+        } else {
         for (unsigned i = tid; i < n; i += kSplitThreads) {
           u64 v0, v1 = 0;
           if (KW == 1) {
-            v0 = s_rec[i];
+            v0 = s_rec[s_ord[i]];
           } else {
-            const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[i];
+            const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[s_ord[i]];
             v0 = v.x;
             v1 = v.y;
           }
@@ -502,6 +533,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
           u64* to = i < s_lim[p] ? out + (u64)(s_to[p] + i) * KW : S.over + (s_over + (s_bin[p] + i)) * KW;
           if (KW == 1) *to = v0;
           else *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(v0, v1);
+        }
         }
         __syncthreads();  // s_bin, s_rec and s_wsum are rewritten
       }
@@ -663,12 +695,11 @@ __device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, 
                                          unsigned& acc_first) {
   using C = CountShape<KW>;
   constexpr unsigned kSlots = C::kLargeSlots;
-  constexpr unsigned kWarps = kCountThreads / 32;
   __shared__ unsigned s_bad;
   u64* k1 = k0 + kSlots * (KW - 1);
   const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const u64 htop = (u64)(b >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
-  const unsigned n_segs = S.n_segs[b - S.b0];
+  const unsigned n_segs = S.n_segs[b - S.b0], order = sub_order(s, n_sub);
   const PartSegment* segs = S.segs + S.seg_base[b - S.b0];
   u64 lo = 0, width = 1ull << kRangeBits;
   while (lo < (1ull << kRangeBits)) {
@@ -719,16 +750,36 @@ __device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, 
       if (x0 + lane < n_in) load(in + (u64)(x0 + lane) * KW, r, hi);
       row(x0 + lane < n_in, r, hi);
     }
-    for (unsigned g = warp; g < n_segs; g += kWarps) {
-      const PartSegment sg = segs[g];
-      for (unsigned x0 = 0; x0 < sg.n; x0 += 32) {
-        u64 r = 0, hi = 0;
-        bool mine = x0 + lane < sg.n;
-        if (mine) {
-          load(S.over + (sg.pos + x0 + lane) * KW, r, hi);
-          mine = sub_of(r, G.log_b, n_sub) == s;
+    // the sub-bucket's records in the segments: each lane searches one segment, which is ordered by
+    // sub-bucket, for the first of them; then the warp takes them segment by segment
+    for (unsigned g0 = warp * 32; g0 < n_segs; g0 += kCountThreads) {
+      PartSegment sg = {0, 0, 0};
+      unsigned from = 0;
+      if (g0 + lane < n_segs) {
+        sg = segs[g0 + lane];
+        unsigned end = sg.n;
+        while (from < end) {
+          const unsigned mid = (from + end) / 2;
+          if (sub_order(sub_of(__ldg(S.over + (sg.pos + mid) * KW), G.log_b, n_sub), n_sub) < order) from = mid + 1;
+          else end = mid;
         }
-        if (__any_sync(0xffffffffu, mine)) row(mine, r, hi);
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, from < sg.n);
+      for (; todo; todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const u64 pos = __shfl_sync(0xffffffffu, sg.pos, src);
+        const unsigned n = __shfl_sync(0xffffffffu, sg.n, src);
+        for (unsigned x0 = __shfl_sync(0xffffffffu, from, src); x0 < n; x0 += 32) {
+          u64 r = 0, hi = 0;
+          bool mine = x0 + lane < n;
+          if (mine) {
+            load(S.over + (pos + x0 + lane) * KW, r, hi);
+            mine = sub_of(r, G.log_b, n_sub) == s;
+          }
+          const unsigned m = __ballot_sync(0xffffffffu, mine);
+          if (m) row(mine, r, hi);
+          if (m != 0xffffffffu) break;  // the last of them
+        }
       }
     }
     __syncthreads();
