@@ -712,19 +712,22 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   };
   auto run = [&]() -> int {
     int rc;
-    u64* zero = nullptr;  // [sub-buckets], overflow records, list entries, then segments per bucket (32 bits)
-    const u64 n_zero = n_subs + 2 + (most_buckets + 1) / 2;
+    // [sub-buckets], overflow records, list entries, large sub-buckets and those taken, then segments per bucket (32 bits)
+    u64* zero = nullptr;
+    const u64 n_zero = n_subs + 4 + (most_buckets + 1) / 2;
     const unsigned key_words = kMaxKeyWords - (h->d.rec_bytes == 8 ? 2 : 0);
     const u64 keys = most / (h->p.use_bloom ? 2 : 1) + 1;
     if ((rc = temp((void**)&s.recs, n_subs * g.cap * h->d.rec_bytes)) || (rc = temp((void**)&s.over, most * h->d.rec_bytes)) ||
-        (rc = temp((void**)&s.keys, keys * key_words * 4)) || (rc = temp((void**)&zero, n_zero * 8)) ||
+        (rc = temp((void**)&s.keys, keys * key_words * 4)) || (rc = temp((void**)&zero, n_zero * 8)) || (rc = temp((void**)&s.large, n_subs * sizeof(unsigned))) ||
         (rc = temp((void**)&s.segs, n_segs * sizeof(PartSegment))) ||
         (rc = temp((void**)&s.seg_base, most_buckets * sizeof(unsigned))))
       return rc;
     s.fill = zero;
     s.over_n = zero + n_subs;
     s.n_keys = zero + n_subs + 1;
-    s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 2);
+    s.n_large = zero + n_subs + 2;
+    s.next_large = zero + n_subs + 3;
+    s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 4);
     s.n_chunks = (unsigned)n_chunks;
     const double occ = std::min(1.0, std::max(0.3, positions > 0 ? windows / positions : 1.0));
     s.log_lanes = lanes_for(kPartTile * occ / B);
@@ -743,7 +746,9 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
           return rc;
       }
       if ((rc = timed_launch(timed, KMA_KERNEL_PASS, st, true,
-                             [&] { return launch_part_count(g, s, o, st, h->num_sms); })) ||
+                             [&] { return launch_part_count(g, s, st, h->num_sms); })) ||
+          (rc = timed_launch(timed, KMA_KERNEL_PASS, st, true,
+                             [&] { return launch_part_large(g, s, o, st, h->num_sms); })) ||
           (rc = timed_launch(timed, KMA_KERNEL_RECOUNT, st, true,
                              [&] { return launch_part_insert(g, s, o, st, h->num_sms); })))
         return rc;

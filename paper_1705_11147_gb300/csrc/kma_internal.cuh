@@ -226,6 +226,9 @@ struct PartSplit {
   unsigned int pad;
   unsigned int* keys;           // count: the counted keys for the table (kma_partition.cu)
   unsigned long long* n_keys;   // their number; starts at 0
+  unsigned int* large;          // [sub-buckets] count: those left to part_large_kernel
+  unsigned long long* n_large;  // their number, and how many have been taken; start at 0
+  unsigned long long* next_large;
 };
 
 // Output records of the keys inserted (as ClassDesc).
@@ -244,7 +247,8 @@ cudaError_t launch_part_scatter(const PartGeom& g, const PartWindows& w, const P
 cudaError_t launch_part_base(const unsigned long long* totals, const PartSplit& s, cudaStream_t stream);
 cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartSplit& s, cudaStream_t stream,
                               int num_sms);
-cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
+cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
+cudaError_t launch_part_large(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
 cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
 constexpr unsigned kMaxKeyWords = 10;          // words of one counted key in the list
 

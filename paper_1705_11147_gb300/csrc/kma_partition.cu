@@ -556,13 +556,15 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 //  5. these keys with their counters (all keys without the singleton filter) are appended to a
 //     list, which part_insert_kernel puts into the HBM table: a few keys per sub-bucket would
 //     leave most threads waiting for the table's round trips here.
-// Sub-buckets that overflowed (very frequent k-mers) are counted by count_large.
+// Sub-buckets that overflowed (very frequent k-mers) and those with more keys than the second
+// table holds are listed for part_large_kernel.
 //
-// Bound by instruction issue. Rejected: a table with the keys and counters themselves that
+// Bound by instruction issue and, between the steps, by the barriers. 166 M records of 16 bytes:
+// 1.74 ms; 2.4 G of 8 bytes: 24.4 ms. Rejected: a table with the keys and counters themselves that
 // records are added to from registers (a probe of a 16-byte key behind a 64-bit compare-and-swap
 // takes 70 instructions for 32 records, 12 in all per record and warp instead of 6).
 
-constexpr int kCountThreads = 512;
+constexpr int kCountThreads = 640;  // 512 and 768: 1 % and 6 % slower
 constexpr int kCountCtas = 2;                // per SM
 constexpr unsigned kEntries = 4096;          // first entries, 16 bits
 constexpr unsigned kEntries2 = 1024;         // second table, 32 bits
@@ -570,7 +572,7 @@ constexpr unsigned kNoEntry = 0xFFFFFFFFu;   // empty entry
 constexpr unsigned kOnce = 0xFFFFu;          // counter block of a representative nobody joined, and of no representative
 constexpr unsigned kJoined = 0xFFFEu;        // joined, block not taken yet
 constexpr unsigned kLone = 0x8000u;          // without the singleton filter: number among the keys seen once
-constexpr unsigned kRangeBits = 20;          // hash bits 21..40: count_large takes a range of them at a time
+constexpr unsigned kRangeBits = 20;          // hash bits 21..40: part_large_kernel takes a range of them at a time
 
 // Counters of a key in 16-bit halves of six words: left A C G T none, (a half not used), right
 // A C G T none, (not used). The outcome bits of a record lie in the top byte of its first word:
@@ -594,11 +596,7 @@ struct CountShape {
   static constexpr size_t kTab = (size_t)kEntries * 2 + kEntries2 * 4 + kIdx;  // entries, second table, list of step 2
   static constexpr size_t kCtr = ((size_t)(kCap / 2) * kCtrWords * 4 + 15) & ~(size_t)15;
   static constexpr size_t kSmem = 2 * kRec + 2 * kIdx + (kTab > kCtr ? kTab : kCtr);  // steps 1 and 2 share the counters' room
-  // count_large: keys and left counters where the representatives begin, right counters in the
-  // buffer that is not being filled
-  static constexpr unsigned kLargeSlots = 1024;
   static_assert(kCap < kLone && kCap % 2 == 0, "record numbers are 16 bits, bulk copies of 16 bytes");
-  static_assert((size_t)kLargeSlots * (KW * 8 + 20) <= kSmem - 2 * kRec && (size_t)kLargeSlots * 20 <= kRec, "room for count_large");
 };
 
 // Slot-to-be of one key in the table: the key's words and where its probes begin.
@@ -656,11 +654,11 @@ __device__ __forceinline__ bool write_record(const PartGeom& G, const PartOut& O
   return l < 4 && r < 4;
 }
 
-constexpr u64 kFree = ~0ull;                 // count_large: first key word of an empty slot
+constexpr u64 kFree = ~0ull;                 // part_large_kernel: first key word of an empty slot
 constexpr u64 kLock = 1ull << 63;            // slot taken, second key word not written yet
 constexpr unsigned kProbes = 128;
 
-// One probe of count_large's table at `pos` for key (h, hi): kSame (the slot holds the key, taken
+// One probe of part_large_kernel's table at `pos` for key (h, hi): kSame (the slot holds the key, taken
 // for it now if it was empty), kOther, or (two-word keys) kAgain: a new key of two words is
 // written behind a lock bit, within this call, so a lane that meets the locked slot of its own
 // hash only has to come back.
@@ -689,137 +687,190 @@ __device__ __forceinline__ unsigned probe_slot(u64* k0, u64* k1, unsigned pos, u
 // its distinct keys need: one range of the hash at a time, halved when a probe of kProbes slots
 // finds no place. Lanes with equal outcomes of equal keys act as one (frequent k-mers are
 // accumulated in the warp first, Section 5.1). The keys go straight to the HBM table.
+//
+// Bound by the latency of the segments' records: a moderately frequent key has a few in every
+// segment (a lane per segment), a hot one thousands (four rows of them in flight). A kernel of
+// its own, whose CTAs take the next sub-bucket when they are done: as a function of the count
+// kernel it held that to 64 registers (now 40) and left most CTAs waiting for those with a hot
+// key. 343 M windows, 30 % of them a satellite's: 10.6 ms -> 5.4 ms with the counting.
+constexpr int kLargeThreads = 512;
+constexpr unsigned kLargeSlots = 2048;  // keys counted at a time
+
+__host__ __device__ constexpr size_t large_smem(int kw) { return (size_t)kLargeSlots * (kw * 8 + 2 * 5 * 4); }
+
 template <int KW>
-__device__ __noinline__ void count_large(const PartGeom& G, const PartSplit& S, const PartOut& O, u64* k0, unsigned* left, unsigned* right,
-                                         unsigned b, unsigned s, unsigned n_sub, unsigned n_in, unsigned& acc_ins,
-                                         unsigned& acc_first) {
-  using C = CountShape<KW>;
-  constexpr unsigned kSlots = C::kLargeSlots;
-  __shared__ unsigned s_bad;
-  u64* k1 = k0 + kSlots * (KW - 1);
+__global__ void __launch_bounds__(kLargeThreads, 2) part_large_kernel(const __grid_constant__ PartGeom G,
+                                                                      const __grid_constant__ PartSplit S,
+                                                                      const __grid_constant__ PartOut O) {
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  constexpr unsigned kSlots = kLargeSlots;
+  __shared__ unsigned s_bad, s_item;
+  u64* k0 = reinterpret_cast<u64*>(s_raw);                            // [slots] first key words
+  u64* k1 = k0 + kSlots * (KW - 1);                                   // [slots] second ones
+  unsigned* left = reinterpret_cast<unsigned*>(k0 + kSlots * KW);     // [slots * 5]
+  unsigned* right = left + kSlots * 5;                                // [slots * 5]
   const unsigned tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const u64 htop = (u64)(b >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
-  const unsigned n_segs = S.n_segs[b - S.b0], order = sub_order(s, n_sub);
-  const PartSegment* segs = S.segs + S.seg_base[b - S.b0];
-  u64 lo = 0, width = 1ull << kRangeBits;
-  while (lo < (1ull << kRangeBits)) {
+  const unsigned n_sub = sub_buckets(G), n_items = (unsigned)__ldcg(S.n_large);
+  unsigned acc_ins = 0, acc_first = 0;
+  for (;;) {
     __syncthreads();
-    for (unsigned i = tid; i < kSlots; i += kCountThreads) k0[i] = kFree;
-    for (unsigned i = tid; i < kSlots * 5; i += kCountThreads) left[i] = right[i] = 0;
-    if (tid == 0) s_bad = 0;
+    if (tid == 0) s_item = atomicAdd(reinterpret_cast<unsigned*>(S.next_large), 1u);
     __syncthreads();
-    // one row of 32 records: lane's record (if `in`)
-    auto row = [&](bool in, u64 r, u64 hi) {
-      const u64 h = r & kHashMask, x = (h >> 21) & ((1u << kRangeBits) - 1);
-      bool act = in && x >= lo && x < lo + width;
-      unsigned pos = (unsigned)h & (kSlots - 1), got = kOther;
-      const unsigned jump = (unsigned)(h >> 11) | 1u;
-      const bool mine = act;
-      for (unsigned step = 0; step < kProbes; ++step) {
-        if (act) {
-          got = probe_slot<KW>(k0, k1, pos, h, hi);
-          act = got != kSame;
-          if (got == kOther) pos = (pos + jump) & (kSlots - 1);
-        }
-        if (!__any_sync(0xffffffffu, act)) break;
-      }
-      const bool hit = mine && got == kSame;
-      if (mine && !hit) s_bad = 1;
-      const unsigned l = left_outcome(r), o = right_outcome(r);
-      const unsigned ml = __match_any_sync(0xffffffffu, hit ? pos * 8 + l : ~0u);
-      const unsigned mo = __match_any_sync(0xffffffffu, hit ? pos * 8 + o : ~0u);
-      if (hit) {
-        bool wrap = false;
-        if (lane == __ffs(ml) - 1) wrap |= atomicAdd(&left[pos * 5 + l], __popc(ml)) > 0xFFFFFFFFu - __popc(ml);
-        if (lane == __ffs(mo) - 1) wrap |= atomicAdd(&right[pos * 5 + o], __popc(mo)) > 0xFFFFFFFFu - __popc(mo);
-        if (wrap) atomicOr(&G.status->flags, kFlagOverflow);
-      }
-    };
-    auto load = [&](const u64* p, u64& r, u64& hi) {
-      if (KW == 1) {
-        r = __ldg(p);
-      } else {
-        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p));
-        r = v.x;
-        hi = v.y;
-      }
-    };
-    const u64* in = S.recs + ((u64)(b - S.b0) * n_sub + s) * G.cap * KW;
-    for (unsigned x0 = warp * 32; x0 < n_in; x0 += kCountThreads) {
-      u64 r = 0, hi = 0;
-      if (x0 + lane < n_in) load(in + (u64)(x0 + lane) * KW, r, hi);
-      row(x0 + lane < n_in, r, hi);
-    }
-    // the sub-bucket's records in the segments: each lane searches one segment, which is ordered by
-    // sub-bucket, for the first of them; then the warp takes them segment by segment
-    for (unsigned g0 = warp * 32; g0 < n_segs; g0 += kCountThreads) {
-      PartSegment sg = {0, 0, 0};
-      unsigned from = 0;
-      if (g0 + lane < n_segs) {
-        sg = segs[g0 + lane];
-        unsigned end = sg.n;
-        while (from < end) {
-          const unsigned mid = (from + end) / 2;
-          if (sub_order(sub_of(__ldg(S.over + (sg.pos + mid) * KW), G.log_b, n_sub), n_sub) < order) from = mid + 1;
-          else end = mid;
-        }
-      }
-      unsigned todo = __ballot_sync(0xffffffffu, from < sg.n);
-      for (; todo; todo &= todo - 1) {
-        const int src = __ffs(todo) - 1;
-        const u64 pos = __shfl_sync(0xffffffffu, sg.pos, src);
-        const unsigned n = __shfl_sync(0xffffffffu, sg.n, src);
-        for (unsigned x0 = __shfl_sync(0xffffffffu, from, src); x0 < n; x0 += 32) {
-          u64 r = 0, hi = 0;
-          bool mine = x0 + lane < n;
-          if (mine) {
-            load(S.over + (pos + x0 + lane) * KW, r, hi);
-            mine = sub_of(r, G.log_b, n_sub) == s;
+    if (s_item >= n_items) break;
+    const unsigned item = S.large[s_item], b = S.b0 + item / n_sub, s = item % n_sub;
+    const u64 fill = S.fill[item];
+    const unsigned n_in = fill < G.cap ? (unsigned)fill : G.cap;
+    const u64 htop = (u64)(b >> (G.log_b - kInfoBits)) << (64 - kInfoBits);
+    const unsigned n_segs = fill > G.cap ? S.n_segs[b - S.b0] : 0u, order = sub_order(s, n_sub);
+    const PartSegment* segs = S.segs + S.seg_base[b - S.b0];
+    u64 lo = 0, width = 1ull << kRangeBits;
+    while (lo < (1ull << kRangeBits)) {
+      __syncthreads();
+      for (unsigned i = tid; i < kSlots; i += kLargeThreads) k0[i] = kFree;
+      for (unsigned i = tid; i < kSlots * 5; i += kLargeThreads) left[i] = right[i] = 0;
+      if (tid == 0) s_bad = 0;
+      __syncthreads();
+      // one row of 32 records: lane's record (if `in`)
+      auto row = [&](bool in, u64 r, u64 hi) {
+        const u64 h = r & kHashMask, x = (h >> 21) & ((1u << kRangeBits) - 1);
+        bool act = in && x >= lo && x < lo + width;
+        if (*reinterpret_cast<volatile unsigned*>(&s_bad)) act = false;  // this range is counted again
+        if (!__any_sync(0xffffffffu, act)) return;
+        unsigned pos = (unsigned)h & (kSlots - 1), got = kOther;
+        const unsigned jump = (unsigned)(h >> 11) | 1u;
+        const bool mine = act;
+        for (unsigned step = 0; step < kProbes; ++step) {
+          if (act) {
+            got = probe_slot<KW>(k0, k1, pos, h, hi);
+            act = got != kSame;
+            if (got == kOther) pos = (pos + jump) & (kSlots - 1);
           }
-          const unsigned m = __ballot_sync(0xffffffffu, mine);
-          if (m) row(mine, r, hi);
-          if (m != 0xffffffffu) break;  // the last of them
+          if (!__any_sync(0xffffffffu, act)) break;
+        }
+        const bool hit = mine && got == kSame;
+        if (mine && !hit) s_bad = 1;
+        const unsigned l = left_outcome(r), o = right_outcome(r);
+        const unsigned ml = __match_any_sync(0xffffffffu, hit ? pos * 8 + l : ~0u);
+        const unsigned mo = __match_any_sync(0xffffffffu, hit ? pos * 8 + o : ~0u);
+        if (hit) {
+          bool wrap = false;
+          if (lane == __ffs(ml) - 1) wrap |= atomicAdd(&left[pos * 5 + l], __popc(ml)) > 0xFFFFFFFFu - __popc(ml);
+          if (lane == __ffs(mo) - 1) wrap |= atomicAdd(&right[pos * 5 + o], __popc(mo)) > 0xFFFFFFFFu - __popc(mo);
+          if (wrap) atomicOr(&G.status->flags, kFlagOverflow);
+        }
+      };
+      auto load = [&](const u64* p, u64& r, u64& hi) {
+        if (KW == 1) {
+          r = __ldg(p);
+        } else {
+          const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p));
+          r = v.x;
+          hi = v.y;
+        }
+      };
+      const u64* in = S.recs + ((u64)(b - S.b0) * n_sub + s) * G.cap * KW;
+      for (unsigned x0 = warp * 32; x0 < n_in; x0 += kLargeThreads) {
+        u64 r = 0, hi = 0;
+        if (x0 + lane < n_in) load(in + (u64)(x0 + lane) * KW, r, hi);
+        row(x0 + lane < n_in, r, hi);
+      }
+      // the sub-bucket's records in the segments: each lane searches one segment, which is ordered by
+      // sub-bucket, for the first of them
+      for (unsigned g0 = warp * 32; g0 < n_segs; g0 += kLargeThreads) {
+        PartSegment sg = {0, 0, 0};
+        unsigned from = 0;
+        if (g0 + lane < n_segs) {
+          sg = segs[g0 + lane];
+          unsigned end = sg.n;
+          while (from < end) {
+            const unsigned mid = (from + end) / 2;
+            if (sub_order(sub_of(__ldg(S.over + (sg.pos + mid) * KW), G.log_b, n_sub), n_sub) < order) from = mid + 1;
+            else end = mid;
+          }
+        }
+        // the first few of every segment, a lane each
+        constexpr int kFew = 4;
+        u64 r[kFew], hi[kFew];
+#pragma unroll
+        for (int y = 0; y < kFew; ++y) {
+          r[y] = hi[y] = 0;
+          if (from + y < sg.n) load(S.over + (sg.pos + from + y) * KW, r[y], hi[y]);
+        }
+        bool more = true;
+#pragma unroll
+        for (int y = 0; y < kFew; ++y) {
+          more = more && from + y < sg.n && sub_of(r[y], G.log_b, n_sub) == s;
+          if (__any_sync(0xffffffffu, more)) row(more, r[y], hi[y]);
+        }
+        // the rest of the long ones (a hot key's), the warp together
+        unsigned todo = __ballot_sync(0xffffffffu, more);
+        for (; todo; todo &= todo - 1) {
+          const int src = __ffs(todo) - 1;
+          const u64 pos = __shfl_sync(0xffffffffu, sg.pos, src);
+          const unsigned n = __shfl_sync(0xffffffffu, sg.n, src);
+          for (unsigned x0 = __shfl_sync(0xffffffffu, from, src) + kFew; x0 < n; x0 += kFew * 32) {
+#pragma unroll
+            for (int y = 0; y < kFew; ++y) {
+              const unsigned x = x0 + y * 32 + lane;
+              if (x < n) load(S.over + (pos + x) * KW, r[y], hi[y]);
+            }
+            unsigned m = 0;
+#pragma unroll
+            for (int y = 0; y < kFew; ++y) {
+              const bool mine = x0 + y * 32 + lane < n && sub_of(r[y], G.log_b, n_sub) == s;
+              m = __ballot_sync(0xffffffffu, mine);
+              if (m) row(mine, r[y], hi[y]);
+            }
+            if (m != 0xffffffffu) break;  // the last of them
+          }
         }
       }
-    }
-    __syncthreads();
-    if (s_bad) {  // uniform
-      if (width > 1) {
-        width >>= 1;
-        continue;
+      __syncthreads();
+      if (s_bad) {  // uniform
+        if (width > 1) {
+          width >>= 1;
+          continue;
+        }
+        if (tid == 0) atomicOr(&G.status->flags, kFlagFull);  // cannot be: the hash has more bits than the range
       }
-      if (tid == 0) atomicOr(&G.status->flags, kFlagFull);  // cannot be: the hash has more bits than the range
-    }
-    for (unsigned i = tid; i < kSlots; i += kCountThreads) {
-      const u64 h = k0[i];
-      if (h == kFree) continue;
-      ++acc_first;
-      unsigned v[10];
-      u64 n = 0;
+      for (unsigned i = tid; i < kSlots; i += kLargeThreads) {
+        const u64 h = k0[i];
+        if (h == kFree) continue;
+        ++acc_first;
+        unsigned v[10];
+        u64 n = 0;
 #pragma unroll
-      for (int x = 0; x < 5; ++x) {
-        v[x] = left[i * 5 + x];
-        v[5 + x] = right[i * 5 + x];
-        n += v[x];
+        for (int x = 0; x < 5; ++x) {
+          v[x] = left[i * 5 + x];
+          v[5 + x] = right[i * 5 + x];
+          n += v[x];
+        }
+        if (n < G.min_count) continue;
+        Place p = place_of(G, h | htop, KW == 2 ? k1[i] : 0);
+        u64 olo, ohi;
+        cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
+        acc_ins += finish_insert(G, p, olo, ohi, v);
+        const unsigned count = key_count(G, v);
+        if (count >= O.min_depth && write_record(G, O, atomicAdd(&G.status->n_out, 1ull), p.lo, p.hi, count, v))
+          atomicAdd(&G.status->n_uu, 1ull);
       }
-      if (n < G.min_count) continue;
-      Place p = place_of(G, h | htop, KW == 2 ? k1[i] : 0);
-      u64 olo, ohi;
-      cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
-      acc_ins += finish_insert(G, p, olo, ohi, v);
-      const unsigned count = key_count(G, v);
-      if (count >= O.min_depth && write_record(G, O, atomicAdd(&G.status->n_out, 1ull), p.lo, p.hi, count, v))
-        atomicAdd(&G.status->n_uu, 1ull);
+      lo += width;
     }
-    lo += width;
   }
-  __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
+    acc_first += __shfl_down_sync(0xffffffffu, acc_first, o);
+  }
+  if (lane == 0) {
+    if (acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
+    if (acc_first && G.min_count > 1) atomicAdd(&G.status->first_sightings, (u64)acc_first);
+  }
 }
 
 template <int KW>
 __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(const __grid_constant__ PartGeom G,
-                                                                               const __grid_constant__ PartSplit S,
-                                                                               const __grid_constant__ PartOut O) {
+                                                                               const __grid_constant__ PartSplit S) {
   using C = CountShape<KW>;
   extern __shared__ __align__(128) unsigned char s_raw[];
   __shared__ __align__(8) unsigned long long s_bar[2];
@@ -834,7 +885,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
   unsigned char* s_ctr = s_raw + 2 * C::kRec + 2 * C::kIdx;                                 // [cap / 2][kCtrWords * 4]
   const unsigned n_sub = sub_buckets(G);
   const unsigned n_items = (S.b1 - S.b0) * n_sub;  // at most 2^22
-  unsigned acc_ins = 0, acc_first = 0;  // per thread: below 2^32
+  unsigned acc_first = 0;  // per thread: below 2^32
   // thread 0: copy a sub-bucket's records into buffer `buf`
   auto issue = [&](unsigned buf, unsigned item, u64 fill) {
     s_fill[buf] = fill;
@@ -884,13 +935,8 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
       if (next + gridDim.x < n_items) s_ahead = __ldcg(&S.fill[next + gridDim.x]);
       s_nctr = s_nlone = 0;
     }
-    auto large = [&]() {
-      u64* keys = reinterpret_cast<u64*>(s_rep);
-      count_large<KW>(G, S, O, keys, reinterpret_cast<unsigned*>(keys + C::kLargeSlots * KW), reinterpret_cast<unsigned*>(s_rec),
-                      S.b0 + item / n_sub, item % n_sub, n_sub, n, acc_ins, acc_first);
-    };
-    if (fill > G.cap) {  // uniform
-      large();
+    if (fill > G.cap) {  // uniform: left to part_large_kernel
+      if (tid == 0) S.large[atomicAdd(S.n_large, 1ull)] = item;
       continue;
     }
     // 2: a representative for every record. The key of record z is (a0, a1)?
@@ -900,7 +946,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
       return (((v.x ^ a0) & kHashMask) | (v.y ^ a1)) == 0;
     };
     unsigned firsts = 0;
-#pragma unroll 1
+#pragma unroll 2
     for (unsigned x0 = tid - lane; x0 < n; x0 += kCountThreads) {
       const unsigned x = x0 + lane;
       bool left = false;
@@ -963,8 +1009,10 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     __syncthreads();
     if (s_state) {  // uniform
       __syncthreads();
-      if (tid == 0) s_state = s_nlist = 0;
-      large();
+      if (tid == 0) {
+        s_state = s_nlist = 0;
+        S.large[atomicAdd(S.n_large, 1ull)] = item;
+      }
       continue;
     }
     acc_first += firsts;
@@ -1046,14 +1094,8 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     }
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
-    acc_first += __shfl_down_sync(0xffffffffu, acc_first, o);
-  }
-  if (lane == 0) {
-    if (acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
-    if (acc_first && G.min_count > 1) atomicAdd(&G.status->first_sightings, (u64)acc_first);
-  }
+  for (int o = 16; o > 0; o >>= 1) acc_first += __shfl_down_sync(0xffffffffu, acc_first, o);
+  if (lane == 0 && acc_first && G.min_count > 1) atomicAdd(&G.status->first_sightings, (u64)acc_first);
 }
 
 // ------------------------------------------------------------------ insert
@@ -1199,7 +1241,7 @@ cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartS
   return cudaGetLastError();
 }
 
-cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms) {
+cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms) {
   if (s.b1 <= s.b0) return cudaSuccess;
   const int kw = g.k > 32 ? 2 : 1;
   const size_t smem = kw == 2 ? CountShape<2>::kSmem : CountShape<1>::kSmem;
@@ -1207,8 +1249,21 @@ cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, const PartO
   cudaError_t e = allow_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)grid_for(fn, kCountThreads, smem, num_sms, (u64)(s.b1 - s.b0) * g.sub_max);
-  if (kw == 2) part_count_kernel<2><<<grid, kCountThreads, smem, stream>>>(g, s, o);
-  else part_count_kernel<1><<<grid, kCountThreads, smem, stream>>>(g, s, o);
+  if (kw == 2) part_count_kernel<2><<<grid, kCountThreads, smem, stream>>>(g, s);
+  else part_count_kernel<1><<<grid, kCountThreads, smem, stream>>>(g, s);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_part_large(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms) {
+  if (s.b1 <= s.b0) return cudaSuccess;
+  const int kw = g.k > 32 ? 2 : 1;
+  const void* fn = kw == 2 ? (const void*)part_large_kernel<2> : (const void*)part_large_kernel<1>;
+  cudaError_t e = allow_dynamic_smem(fn, large_smem(kw));
+  if (e != cudaSuccess) return e;
+  // their number is known on the device only
+  const unsigned grid = (unsigned)grid_for(fn, kLargeThreads, large_smem(kw), num_sms, (u64)(s.b1 - s.b0) * g.sub_max);
+  if (kw == 2) part_large_kernel<2><<<grid, kLargeThreads, large_smem(2), stream>>>(g, s, o);
+  else part_large_kernel<1><<<grid, kLargeThreads, large_smem(1), stream>>>(g, s, o);
   return cudaGetLastError();
 }
 
