@@ -548,7 +548,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 // one is counted (two buffers, two CTAs per SM). Then
 //  1. every record writes its number at the entry its hash picks, the last one wins;
 //  2. it compares its key with the winner's: equal keys share the winner as their representative,
-//     without an atomic or a loop. The others (about one in eight) find theirs in a second table
+//     without an atomic or a loop. The others (fewer than one in ten) find theirs in a second table
 //     by compare-and-swap and probing, compacted into full warps first;
 //  3. representatives that another record joined take a block of ten 16-bit counters (a staged
 //     sub-bucket has fewer than 2^16 records);
@@ -560,13 +560,13 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 // table holds are listed for part_large_kernel.
 //
 // Bound by instruction issue and, between the steps, by the barriers. 166 M records of 16 bytes:
-// 1.74 ms; 2.4 G of 8 bytes: 24.4 ms. Rejected: a table with the keys and counters themselves that
+// 1.65 ms; 2.4 G of 8 bytes: 23.0 ms. Rejected: a table with the keys and counters themselves that
 // records are added to from registers (a probe of a 16-byte key behind a 64-bit compare-and-swap
 // takes 70 instructions for 32 records, 12 in all per record and warp instead of 6).
 
 constexpr int kCountThreads = 640;  // 512 and 768: 1 % and 6 % slower
 constexpr int kCountCtas = 2;                // per SM
-constexpr unsigned kEntries = 4096;          // first entries, 16 bits
+constexpr unsigned kEntries = 8192;          // first entries, 16 bits (4096: 4 % slower, more records for the second table)
 constexpr unsigned kEntries2 = 1024;         // second table, 32 bits
 constexpr unsigned kNoEntry = 0xFFFFFFFFu;   // empty entry
 constexpr unsigned kOnce = 0xFFFFu;          // counter block of a representative nobody joined, and of no representative
@@ -985,7 +985,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
         a0 = v.x;
         a1 = v.y;
       }
-      unsigned pos = (unsigned)(a0 >> 12) & (kEntries2 - 1), z = x, step = 0;
+      unsigned pos = (unsigned)(a0 >> 13) & (kEntries2 - 1), z = x, step = 0;
       const unsigned jump = (unsigned)(a0 >> 22) | 1u;  // odd: comes by every entry
       for (; step < kEntries2; ++step) {
         z = *reinterpret_cast<volatile unsigned*>(&s_ent2[pos]);
@@ -1046,6 +1046,7 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     // 4: outcomes
     if (tid == 0) s_nlist = 0;
     if (tid == 0) s_base = s_nctr + s_nlone ? atomicAdd(S.n_keys, (u64)(s_nctr + s_nlone)) : 0;
+#pragma unroll 2
     for (unsigned x = tid; x < n; x += kCountThreads) {
       const unsigned q = s_q[s_rep[x]];
       if (q < kLone) {
