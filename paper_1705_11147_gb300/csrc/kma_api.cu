@@ -712,9 +712,10 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   };
   auto run = [&]() -> int {
     int rc;
-    // [sub-buckets], overflow records, list entries, large sub-buckets and those taken, then segments per bucket (32 bits)
+    // [sub-buckets], overflow records, list entries, large sub-buckets, those taken, CTAs done,
+    // then segments per bucket (32 bits)
     u64* zero = nullptr;
-    const u64 n_zero = n_subs + 4 + (most_buckets + 1) / 2;
+    const u64 n_zero = n_subs + 5 + (most_buckets + 1) / 2;
     const unsigned key_words = kMaxKeyWords - (h->d.rec_bytes == 8 ? 2 : 0);
     const u64 keys = most / (h->p.use_bloom ? 2 : 1) + 1;
     if ((rc = temp((void**)&s.recs, n_subs * g.cap * h->d.rec_bytes)) || (rc = temp((void**)&s.over, most * h->d.rec_bytes)) ||
@@ -727,7 +728,8 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     s.n_keys = zero + n_subs + 1;
     s.n_large = zero + n_subs + 2;
     s.next_large = zero + n_subs + 3;
-    s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 4);
+    s.inserted = zero + n_subs + 4;
+    s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 5);
     s.n_chunks = (unsigned)n_chunks;
     const double occ = std::min(1.0, std::max(0.3, positions > 0 ? windows / positions : 1.0));
     s.log_lanes = lanes_for(kPartTile * occ / B);

@@ -229,6 +229,7 @@ struct PartSplit {
   unsigned int* large;          // [sub-buckets] count: those left to part_large_kernel
   unsigned long long* n_large;  // their number, and how many have been taken; start at 0
   unsigned long long* next_large;
+  unsigned long long* inserted; // CTAs of part_insert_kernel that are done; starts at 0
 };
 
 // Output records of the keys inserted (as ClassDesc).

@@ -1116,48 +1116,65 @@ constexpr unsigned kInsertTile = kInsertThreads * kInsertKeys;
 template <int KW>
 __global__ void __launch_bounds__(kInsertThreads) part_insert_kernel(const __grid_constant__ PartGeom G,
                                                                      const __grid_constant__ PartOut O,
-                                                                     const unsigned* keys, const u64* n_keys) {
+                                                                     const unsigned* keys, const u64* n_keys, unsigned* done) {
   __shared__ unsigned s_wsum[32];
   __shared__ u64 s_base;
   const u64 n = __ldcg(n_keys);
   unsigned acc_ins = 0, acc_uu = 0;
-  for (u64 t = blockIdx.x; t * kInsertTile < n; t += gridDim.x) {
-    // the records this thread's keys make
-    unsigned keep = 0;
+  // key i into the table; its record at `at` if it has the depth
+  auto put = [&](u64 i, u64 at) {
+    const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
+    uint2 w[kKeyWords<KW> / 2];
 #pragma unroll
-    for (int y = 0; y < kInsertKeys; ++y) {
-      const u64 i = t * kInsertTile + y * kInsertThreads + threadIdx.x;
-      if (i < n) {
-        const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
-        const uint2 a = __ldg(c);
-        const unsigned none = __ldg(&c[1].x) & 0xFFFFu;
-        keep += (a.x & 0xFFFFu) + (a.x >> 16) + (a.y & 0xFFFFu) + (a.y >> 16) + none >= O.min_depth;
+    for (unsigned x = 0; x < kKeyWords<KW> / 2; ++x) w[x] = __ldg(c + x);
+    const u64 h = ((u64)w[3].y << 32) | w[3].x;
+    Place p = place_of(G, h, KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull);
+    u64 olo, ohi;
+    cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
+    const unsigned v[10] = {w[0].x & 0xFFFFu, w[0].x >> 16, w[0].y & 0xFFFFu, w[0].y >> 16, w[1].x & 0xFFFFu,
+                            w[1].y & 0xFFFFu, w[1].y >> 16, w[2].x & 0xFFFFu, w[2].x >> 16, w[2].y & 0xFFFFu};
+    const unsigned count = key_count(G, v);
+    acc_ins += finish_insert(G, p, olo, ohi, v);
+    if (count < O.min_depth) return false;
+    acc_uu += write_record(G, O, at, p.lo, p.hi, count, v);
+    return true;
+  };
+  if (O.min_depth <= G.min_count) {
+    // every key of the list has the depth: records in list order, nothing to number
+    const u64 base = __ldcg(&G.status->n_out), stride = (u64)gridDim.x * kInsertThreads;
+    for (u64 i = (u64)blockIdx.x * kInsertThreads + threadIdx.x; i < n; i += stride) put(i, base + i);
+    __syncthreads();  // all of the block have read base
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(done, 1u) == gridDim.x - 1 && n) atomicAdd(&G.status->n_out, n);  // everyone has
+    }
+  } else {
+    for (u64 t = blockIdx.x; t * kInsertTile < n; t += gridDim.x) {
+      // the records this thread's keys make
+      unsigned keep = 0;
+#pragma unroll
+      for (int y = 0; y < kInsertKeys; ++y) {
+        const u64 i = t * kInsertTile + y * kInsertThreads + threadIdx.x;
+        if (i < n) {
+          const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
+          const uint2 a = __ldg(c);
+          const unsigned none = __ldg(&c[1].x) & 0xFFFFu;
+          keep += (a.x & 0xFFFFu) + (a.x >> 16) + (a.y & 0xFFFFu) + (a.y >> 16) + none >= O.min_depth;
+        }
       }
-    }
-    unsigned total;
-    const unsigned before = block_scan<kInsertThreads>(keep, s_wsum, total);
-    if (threadIdx.x == 0) s_base = total ? atomicAdd(&G.status->n_out, (u64)total) : 0;
-    __syncthreads();
-    u64 at = s_base + before;
+      unsigned total;
+      const unsigned before = block_scan<kInsertThreads>(keep, s_wsum, total);
+      if (threadIdx.x == 0) s_base = total ? atomicAdd(&G.status->n_out, (u64)total) : 0;
+      __syncthreads();
+      u64 at = s_base + before;
 #pragma unroll 1
-    for (int y = 0; y < kInsertKeys; ++y) {
-      const u64 i = t * kInsertTile + y * kInsertThreads + threadIdx.x;
-      if (i >= n) break;
-      const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
-      uint2 w[kKeyWords<KW> / 2];
-#pragma unroll
-      for (unsigned x = 0; x < kKeyWords<KW> / 2; ++x) w[x] = __ldg(c + x);
-      const u64 h = ((u64)w[3].y << 32) | w[3].x;
-      Place p = place_of(G, h, KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull);
-      u64 olo, ohi;
-      cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
-      const unsigned v[10] = {w[0].x & 0xFFFFu, w[0].x >> 16, w[0].y & 0xFFFFu, w[0].y >> 16, w[1].x & 0xFFFFu,
-                              w[1].y & 0xFFFFu, w[1].y >> 16, w[2].x & 0xFFFFu, w[2].x >> 16, w[2].y & 0xFFFFu};
-      const unsigned count = key_count(G, v);
-      acc_ins += finish_insert(G, p, olo, ohi, v);
-      if (count >= O.min_depth) acc_uu += write_record(G, O, at++, p.lo, p.hi, count, v);
+      for (int y = 0; y < kInsertKeys; ++y) {
+        const u64 i = t * kInsertTile + y * kInsertThreads + threadIdx.x;
+        if (i >= n) break;
+        at += put(i, at);
+      }
+      __syncthreads();  // s_wsum and s_base are rewritten
     }
-    __syncthreads();  // s_wsum and s_base are rewritten
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -1272,8 +1289,8 @@ cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, const Part
   // the number of keys is known on the device only: as many CTAs as run at a time
   const void* fn = g.k > 32 ? (const void*)part_insert_kernel<2> : (const void*)part_insert_kernel<1>;
   const unsigned grid = (unsigned)grid_for(fn, kInsertThreads, 0, num_sms, ~0ull);
-  if (g.k > 32) part_insert_kernel<2><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys);
-  else part_insert_kernel<1><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys);
+  if (g.k > 32) part_insert_kernel<2><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys, reinterpret_cast<unsigned*>(s.inserted));
+  else part_insert_kernel<1><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys, reinterpret_cast<unsigned*>(s.inserted));
   return cudaGetLastError();
 }
 
