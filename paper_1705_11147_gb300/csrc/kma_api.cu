@@ -1683,7 +1683,9 @@ int kmer_analysis_parse_fastq(const char* text, uint64_t n_bytes, int on_device,
   if ((rc = alloc((void**)&cc, (chunks + 1) * 8)) ||
       (rc = alloc((void**)&tmp, scan_scratch_items(std::max<u64>(chunks + 1, 1)) * 8)))
     return done(rc);
-  FQ_CUDA(launch_fastq_count(d_text, n_bytes, cc, st));
+  unsigned short* masks = nullptr;
+  if ((rc = alloc((void**)&masks, fastq_masks(n_bytes) * 2))) return done(rc);
+  FQ_CUDA(launch_fastq_count(d_text, n_bytes, masks, cc, st));
   FQ_CUDA(cudaMemsetAsync(cc + chunks, 0, 8, st));
   FQ_CUDA(scan_exclusive(cc, chunks + 1, tmp, st));
   u64 n_lines = 0;
@@ -1692,7 +1694,7 @@ int kmer_analysis_parse_fastq(const char* text, uint64_t n_bytes, int on_device,
   // 3: line ends
   u64* line_end = nullptr;
   if ((rc = alloc((void**)&line_end, n_lines * 8))) return done(rc);
-  FQ_CUDA(launch_fastq_lines(d_text, n_bytes, cc, line_end, st));
+  FQ_CUDA(launch_fastq_lines(d_text, n_bytes, masks, cc, line_end, st));
   // lines after the last complete record must be empty
   const u64 extra = n_lines % 4;
   if (extra) {

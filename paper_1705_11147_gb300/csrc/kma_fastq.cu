@@ -128,12 +128,16 @@ __device__ __forceinline__ unsigned newline_mask(const unsigned char* text, u64 
   return m;
 }
 
-// Newlines in each 16 KiB chunk (plus one for a final line that does not end in '\n').
+// Newlines in each 16 KiB chunk (plus one for a final line that does not end in '\n'), and their
+// masks, an eighth of the text, for the next pass (reading the text again took it 104 us of 516 for
+// 100 Mbases).
 __global__ void __launch_bounds__(kFqThreads) fastq_count_kernel(const unsigned char* text, u64 n, unsigned head,
-                                                                 u64* chunk_counts) {
+                                                                 unsigned short* masks, u64* chunk_counts) {
   __shared__ unsigned warp_cnt[kFqThreads / 32];
   const u64 c = blockIdx.x;
-  unsigned cnt = __popc(newline_mask(text, n, (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head));
+  const unsigned m = newline_mask(text, n, (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head);
+  masks[c * kFqThreads + threadIdx.x] = (unsigned short)m;
+  unsigned cnt = __popc(m);
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   if ((threadIdx.x & 31) == 0) warp_cnt[threadIdx.x >> 5] = cnt;
   __syncthreads();
@@ -145,11 +149,12 @@ __global__ void __launch_bounds__(kFqThreads) fastq_count_kernel(const unsigned 
 
 // Line ends (position of each '\n', or n for an unterminated last line), in text order.
 __global__ void __launch_bounds__(kFqThreads) fastq_lines_kernel(const unsigned char* text, u64 n, unsigned head,
-                                                                 const u64* chunk_offsets, u64* line_end) {
+                                                                 const unsigned short* masks, const u64* chunk_offsets,
+                                                                 u64* line_end) {
   __shared__ unsigned warp_off[kFqThreads / 32];
   const u64 c = blockIdx.x;
   const long long i = (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head;
-  unsigned m = newline_mask(text, n, i);
+  unsigned m = masks[c * kFqThreads + threadIdx.x];
   const unsigned cnt = __popc(m);
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned incl = cnt;
@@ -212,29 +217,31 @@ __device__ __forceinline__ u64 load8(const unsigned char* p, unsigned valid) {
   return v;
 }
 
-// `len` bytes from src to dst by 16 lanes (`lane` 0 .. 15): bytes up to an 8-byte boundary of dst,
+// `len` bytes from src to dst by kLineLanes lanes: bytes up to an 8-byte boundary of dst,
 // then a word per lane, then the bytes left. Reads and writes nothing outside the ranges but the
 // rest of the aligned words that hold source bytes.
+constexpr unsigned kLineLanes = 8;
 __device__ __forceinline__ void copy_line(const unsigned char* src, unsigned char* dst, u64 len, unsigned lane) {
   u64 head = (8 - (reinterpret_cast<u64>(dst) & 7)) & 7;
   if (head > len) head = len;
   if (lane < head) dst[lane] = src[lane];
   const u64 words = (len - head) / 8;
-  for (u64 w = lane; w < words; w += 16) *reinterpret_cast<u64*>(dst + head + 8 * w) = load8(src + head + 8 * w, 8);
+  for (u64 w = lane; w < words; w += kLineLanes) *reinterpret_cast<u64*>(dst + head + 8 * w) = load8(src + head + 8 * w, 8);
   const u64 done = head + 8 * words;
   if (lane < len - done) dst[done + lane] = src[done + lane];
 }
 
-// One warp per record: bases (half of the warp) and qualities to their place in the output, eight
-// bytes a lane: a byte per lane took eight times the requests on both sides.
+// A quarter of a warp per line, bases or qualities, to its place in the output, eight bytes a lane:
+// a byte per lane took eight times the requests on both sides, and with half a warp per line 41 %
+// of the lanes had nothing to do for lines of 150 bytes.
 __global__ void fastq_copy_kernel(const unsigned char* text, const u64* line_end, u64 n_reads, const u64* offsets,
                                   unsigned char* seq, unsigned char* qual) {
-  const u64 r = ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const unsigned lane = threadIdx.x & 31, half = lane >> 4;
+  const u64 line = ((u64)blockIdx.x * blockDim.x + threadIdx.x) / kLineLanes, r = line / 2;
+  const unsigned lane = threadIdx.x % kLineLanes, which = (unsigned)line & 1;
   if (r >= n_reads) return;
   const u64 o = offsets[r], len = offsets[r + 1] - o;
-  const u64 l = 4 * r + 1 + 2 * half;  // the bases' line, or the qualities'
-  copy_line(text + line_end[l - 1] + 1, (half ? qual : seq) + o, len, lane & 15);
+  const u64 l = 4 * r + 1 + 2 * which;  // the bases' line, or the qualities'
+  copy_line(text + line_end[l - 1] + 1, (which ? qual : seq) + o, len, lane);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -242,20 +249,23 @@ __global__ void fastq_copy_kernel(const unsigned char* text, const u64* line_end
 // Chunks begin at a 16-byte boundary: `head` bytes before the text belong to the first one.
 static unsigned fastq_head(const unsigned char* text) { return (unsigned)(reinterpret_cast<uintptr_t>(text) & 15); }
 
+u64 fastq_masks(u64 n_bytes) { return fastq_chunks(n_bytes) * kFqThreads; }
+
 u64 fastq_chunks(u64 n_bytes) { return n_bytes ? (n_bytes + 15 + kFqChunk - 1) / kFqChunk : 0; }
 
-cudaError_t launch_fastq_count(const unsigned char* text, u64 n, u64* chunk_counts, cudaStream_t stream) {
-  const u64 chunks = fastq_chunks(n);
-  if (!chunks) return cudaSuccess;
-  fastq_count_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, fastq_head(text), chunk_counts);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_fastq_lines(const unsigned char* text, u64 n, const u64* chunk_offsets, u64* line_end,
+cudaError_t launch_fastq_count(const unsigned char* text, u64 n, unsigned short* masks, u64* chunk_counts,
                                cudaStream_t stream) {
   const u64 chunks = fastq_chunks(n);
   if (!chunks) return cudaSuccess;
-  fastq_lines_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, fastq_head(text), chunk_offsets, line_end);
+  fastq_count_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, fastq_head(text), masks, chunk_counts);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fastq_lines(const unsigned char* text, u64 n, const unsigned short* masks, const u64* chunk_offsets,
+                               u64* line_end, cudaStream_t stream) {
+  const u64 chunks = fastq_chunks(n);
+  if (!chunks) return cudaSuccess;
+  fastq_lines_kernel<<<(unsigned)chunks, kFqThreads, 0, stream>>>(text, n, fastq_head(text), masks, chunk_offsets, line_end);
   return cudaGetLastError();
 }
 
@@ -269,7 +279,7 @@ cudaError_t launch_fastq_records(const unsigned char* text, const u64* line_end,
 cudaError_t launch_fastq_copy(const unsigned char* text, const u64* line_end, u64 n_reads, const u64* offsets,
                               unsigned char* seq, unsigned char* qual, cudaStream_t stream) {
   if (!n_reads) return cudaSuccess;
-  const u64 threads = n_reads * 32;
+  const u64 threads = n_reads * 2 * kLineLanes;
   fastq_copy_kernel<<<(unsigned)((threads + 255) / 256), 256, 0, stream>>>(text, line_end, n_reads, offsets, seq,
                                                                           qual);
   return cudaGetLastError();

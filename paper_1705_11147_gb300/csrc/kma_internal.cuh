@@ -258,9 +258,11 @@ unsigned long long scan_scratch_items(unsigned long long n);
 cudaError_t scan_exclusive(unsigned long long* data, unsigned long long n, unsigned long long* tmp,
                            cudaStream_t stream);
 unsigned long long fastq_chunks(unsigned long long n_bytes);
-cudaError_t launch_fastq_count(const unsigned char* text, unsigned long long n, unsigned long long* chunk_counts,
+unsigned long long fastq_masks(unsigned long long n_bytes);  // newline masks, one per 16 bytes
+cudaError_t launch_fastq_count(const unsigned char* text, unsigned long long n, unsigned short* masks,
+                               unsigned long long* chunk_counts,
                                cudaStream_t stream);
-cudaError_t launch_fastq_lines(const unsigned char* text, unsigned long long n,
+cudaError_t launch_fastq_lines(const unsigned char* text, unsigned long long n, const unsigned short* masks,
                                const unsigned long long* chunk_offsets, unsigned long long* line_end,
                                cudaStream_t stream);
 cudaError_t launch_fastq_records(const unsigned char* text, const unsigned long long* line_end,
