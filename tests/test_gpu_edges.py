@@ -167,6 +167,47 @@ def test_query_slices(gpu, partitions):
         assert np.array_equal(a[1][:len(want)].cpu().numpy().view(np.uint32), want.ext)
 
 
+def test_query_host_arrays(gpu):
+    """Host arrays of lookups below, at and above the size that is copied by several threads, and two
+    calls at once: as with device arrays."""
+    import threading
+
+    from paper_1705_11147_gb300 import KmerAnalysis, make_params
+    r = one_read(5000, 78)
+    rs = readset([r, r], k=31, min_depth=2, min_ext_count=2, qual_threshold=20)
+    edge = (8 << 20) // 38
+    with KmerAnalysis(make_params(max_bases=rs.n_bases, max_reads=rs.n_reads, expected_distinct=rs.n_bases,
+                                  **rs.meta["params"])) as ka:
+        ka.count(rs.seq, rs.qual, rs.offsets)
+        ka.finalize()
+        found = ka.copy_result().keys
+        for n in (1, edge, edge + 1, 700_001):
+            keys = found[np.random.default_rng(n).integers(0, len(found), n)]
+            keys[::3] ^= np.uint64(9)
+            want = [x.cpu().numpy() for x in ka.query(gpu.from_numpy(keys.view(np.int64)).cuda())]
+            got = [None, None]
+
+            def look(i):
+                got[i] = ka.query(keys)
+
+            threads = [threading.Thread(target=look, args=(i,)) for i in range(2 if n > edge else 1)]
+            [t.start() for t in threads]
+            [t.join() for t in threads]
+            for answer in got[:len(threads)]:
+                for x, y in zip(answer, want):
+                    assert np.array_equal(x.view(y.dtype), y), n
+
+
+@pytest.mark.parametrize("partitions", [1, 5])
+def test_host_pieces(gpu, partitions):
+    """Host reads that are copied in pieces, one read longer than a piece among them."""
+    piece = 8 << 20
+    reads = [one_read(n, 60 + i) for i, n in enumerate((1, piece + 5, 40, piece - 45, 200, 3, piece // 2))]
+    rs = readset(reads, k=31, min_depth=1, min_ext_count=1, qual_threshold=20)
+    kw = dict(use_bloom=False, partitions=partitions)
+    assert_same(run_gpu(gpu, rs, device_inputs=False, **kw), run_gpu(gpu, rs, **kw), "pieces")
+
+
 @pytest.mark.parametrize("k", [31, 51])
 def test_summary_merge(gpu, k):
     """Fewer and more keys than a summary holds, one key above all, the all-A key."""
