@@ -440,7 +440,8 @@ int clear_state(kma_handle* h) {
   KMA_CUDA(cudaMemsetAsync(h->status, 0, sizeof(DevStatus), h->stream));
   if (h->bloom) KMA_CUDA(cudaMemsetAsync(h->bloom, 0, h->d.plan.bloom_words * 8, h->stream));
   if (h->totals) KMA_CUDA(cudaMemsetAsync(h->totals, 0, sizeof(u64) << h->d.log_b, h->stream));
-  int rc = timed_launch(h, KMA_KERNEL_INIT, h->stream, h->d.plan.table_slots > 0,
+  // (partitioned mode: the table is written as a whole when its keys are known)
+  int rc = timed_launch(h, KMA_KERNEL_INIT, h->stream, h->d.P <= 1 && h->d.plan.table_slots > 0,
                         [&] { return launch_table_init(h->table, h->d.plan.table_slots, h->stream); });
   if (rc) return rc;
   h->q_used = h->reads_used = h->bases_used = 0;
@@ -670,7 +671,11 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     windows += sl.windows;
     positions += sl.positions;
   }
-  if (n_chunks == 0) return after(B);
+  if (n_chunks == 0) {
+    const int rc = timed_launch(timed, KMA_KERNEL_INIT, st, true,
+                                [&] { return launch_table_init(h->table, h->d.plan.table_slots, st); });
+    return rc ? rc : after(B);
+  }
   constexpr unsigned kStep = kSplitBuckets;  // groups are whole work items of the split
   parts = std::min(parts, B / kStep);
   std::vector<unsigned> ends;
@@ -722,13 +727,17 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   auto run = [&]() -> int {
     int rc;
     // [sub-buckets], overflow records, list entries, large sub-buckets, those taken, CTAs done,
-    // then segments per bucket (32 bits)
+    // then segments per bucket and keys per sub-bucket (32 bits)
     u64* zero = nullptr;
-    const u64 n_zero = n_subs + 5 + (most_buckets + 1) / 2;
+    const u64 n_zero = n_subs + 5 + (most_buckets + n_subs + 1) / 2;
+    u64* n_carry = nullptr;
+    unsigned* carry = nullptr;  // two lists, taken in turn
     const unsigned key_words = kMaxKeyWords - (h->d.rec_bytes == 8 ? 2 : 0);
     const u64 keys = most / (h->p.use_bloom ? 2 : 1) + 1;
     if ((rc = temp((void**)&s.recs, n_subs * g.cap * h->d.rec_bytes)) || (rc = temp((void**)&s.over, most * h->d.rec_bytes)) ||
         (rc = temp((void**)&s.keys, keys * key_words * 4)) || (rc = temp((void**)&zero, n_zero * 8)) || (rc = temp((void**)&s.large, n_subs * sizeof(unsigned))) ||
+        (rc = temp((void**)&s.key_base, n_subs * 8)) || (rc = temp((void**)&n_carry, 2 * 8)) ||
+        (rc = temp((void**)&carry, 2 * (u64)kMaxProbe * kCarryWords * 4)) ||
         (rc = temp((void**)&s.segs, n_segs * sizeof(PartSegment))) ||
         (rc = temp((void**)&s.seg_base, most_buckets * sizeof(unsigned))))
       return rc;
@@ -739,13 +748,23 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     s.next_large = zero + n_subs + 3;
     s.inserted = zero + n_subs + 4;
     s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 5);
+    s.key_n = s.n_segs + most_buckets;
     s.n_chunks = (unsigned)n_chunks;
+    KMA_CUDA(cudaMemsetAsync(n_carry, 0, 2 * 8, st));
     const double occ = std::min(1.0, std::max(0.3, positions > 0 ? windows / positions : 1.0));
     s.log_lanes = lanes_for(kPartTile * occ / B);
     for (size_t i = 0; i < ends.size(); ++i) {
       s.b0 = i ? ends[i - 1] : 0;
       s.b1 = ends[i];
       KMA_CUDA(cudaMemsetAsync(zero, 0, n_zero * 8, st));
+      // the group's slots end where the hashes of bucket b1 begin (part_of, table_index)
+      const u64 top = s.b1 < B ? (u64)s.b1 << (32 - h->d.log_b) : 0;
+      s.end = s.b1 < B ? (top * g.P >> 32) * g.Sp + ((top * g.P & 0xFFFFFFFFull) * g.Sp >> 32) : (u64)g.P * g.Sp;
+      s.carry_in = carry + (i & 1) * (u64)kMaxProbe * kCarryWords;
+      s.carry_out = carry + ((i + 1) & 1) * (u64)kMaxProbe * kCarryWords;
+      s.n_carry_in = n_carry + (i & 1);
+      s.n_carry_out = n_carry + ((i + 1) & 1);
+      KMA_CUDA(cudaMemsetAsync(s.n_carry_out, 0, 8, st));
       if ((rc = timed_launch(timed, KMA_KERNEL_SCATTER, st, true,
                              [&] { return launch_part_base(h->totals, s, st); })))
         return rc;
@@ -758,6 +777,8 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
       }
       if ((rc = timed_launch(timed, KMA_KERNEL_PASS, st, true,
                              [&] { return launch_part_count(g, s, st, h->num_sms); })) ||
+          (rc = timed_launch(timed, KMA_KERNEL_RECOUNT, st, true,
+                             [&] { return launch_part_build(g, s, st, h->num_sms); })) ||
           (rc = timed_launch(timed, KMA_KERNEL_PASS, st, true,
                              [&] { return launch_part_large(g, s, o, st, h->num_sms); })) ||
           (rc = timed_launch(timed, KMA_KERNEL_RECOUNT, st, true,

@@ -211,6 +211,8 @@ struct PartSegment {
   unsigned long long pos;
   unsigned int n, pad;
 };
+constexpr unsigned kCarryWords = 14;  // an entry of carry_in and carry_out: ten counters, h, hi
+
 struct PartSplit {
   unsigned long long* recs;
   unsigned long long* fill;     // starts at 0
@@ -229,6 +231,13 @@ struct PartSplit {
   unsigned int* large;          // [sub-buckets] count: those left to part_large_kernel
   unsigned long long* n_large;  // their number, and how many have been taken; start at 0
   unsigned long long* next_large;
+  unsigned long long* key_base; // [sub-buckets] count: the sub-bucket's first key in the list
+  unsigned int* key_n;          // [sub-buckets] and their number; starts at 0
+  unsigned long long end;       // first table slot behind the group's (all slots: the last group's)
+  unsigned int* carry_in;       // keys that go to a slot behind their group's, from the groups before
+  unsigned int* carry_out;      // and for the next one (kMaxProbe entries)
+  unsigned long long* n_carry_in;
+  unsigned long long* n_carry_out;  // starts at 0
   unsigned long long* inserted; // CTAs of part_insert_kernel that are done; starts at 0
 };
 
@@ -250,6 +259,7 @@ cudaError_t launch_part_split(const PartGeom& g, const PartTiles& t, const PartS
                               int num_sms);
 cudaError_t launch_part_count(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
 cudaError_t launch_part_large(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
+cudaError_t launch_part_build(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms);
 cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms);
 constexpr unsigned kMaxKeyWords = 10;          // words of one counted key in the list
 

@@ -613,22 +613,41 @@ __device__ __forceinline__ Place place_of(const PartGeom& G, u64 h, u64 hi) {
   return p;
 }
 
-// Puts a key with its ten counters (left A C G T none, right A C G T none) into the table. The
-// key is in no slot yet and no other thread inserts it, so the first empty slot takes it.
-// (olo, ohi): what a compare-and-swap of the first slot returned.
-__device__ __forceinline__ bool finish_insert(const PartGeom& G, Place& p, u64 olo, u64 ohi, const unsigned (&ctr)[10]) {
+// A slot of 64 bytes: key, counters without a neighbour, counters.
+__device__ __forceinline__ void write_slot(Slot* s, const unsigned (&ctr)[10]) {
+  *reinterpret_cast<uint4*>(&s->none[0]) = make_uint4(ctr[4], ctr[9], 0u, 0u);
+  *reinterpret_cast<uint4*>(&s->ext[0]) = make_uint4(ctr[0], ctr[1], ctr[2], ctr[3]);
+  *reinterpret_cast<uint4*>(&s->ext[4]) = make_uint4(ctr[5], ctr[6], ctr[7], ctr[8]);
+}
+
+// Puts a key with its ten counters (left A C G T none, right A C G T none) into the table, whose
+// slots below S.end have been written. The key is in no slot yet and no other thread inserts it, so
+// the first empty slot takes it. If that lies in the next group's part of the table the key is
+// carried over to it (no more than kMaxProbe can be: every one of them takes one of the next
+// kMaxProbe slots, or the table is full).
+__device__ __forceinline__ bool insert_key(const PartGeom& G, const PartSplit& S, u64 h, u64 hi, const unsigned (&ctr)[10]) {
+  Place p = place_of(G, h, hi);
   const u64 limit = G.Sp < kMaxProbe ? G.Sp : kMaxProbe;
-  for (u64 n = 1;; ++n) {
+  for (u64 n = 0; n < limit; ++n) {
+    if (p.sub + p.idx == G.table + S.end) {
+      const u64 at = atomicAdd(S.n_carry_out, 1ull);
+      if (at >= kMaxProbe) break;
+      unsigned* c = S.carry_out + at * kCarryWords;
+#pragma unroll
+      for (int x = 0; x < 10; ++x) c[x] = ctr[x];
+      c[10] = (unsigned)h;
+      c[11] = (unsigned)(h >> 32);
+      c[12] = (unsigned)hi;
+      c[13] = (unsigned)(hi >> 32);
+      return false;
+    }
+    u64 olo, ohi;
+    cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
     if (olo == kEmpty && ohi == kEmpty) {
-      Slot* s = p.sub + p.idx;
-      *reinterpret_cast<uint4*>(&s->none[0]) = make_uint4(ctr[4], ctr[9], 0u, 0u);
-      *reinterpret_cast<uint4*>(&s->ext[0]) = make_uint4(ctr[0], ctr[1], ctr[2], ctr[3]);
-      *reinterpret_cast<uint4*>(&s->ext[4]) = make_uint4(ctr[5], ctr[6], ctr[7], ctr[8]);
+      write_slot(p.sub + p.idx, ctr);
       return true;
     }
-    if (n >= limit) break;
     p.idx = (p.idx + 1 == G.Sp) ? 0 : p.idx + 1;
-    cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
   }
   atomicOr(&G.status->flags, kFlagFull);
   return false;
@@ -846,12 +865,10 @@ __global__ void __launch_bounds__(kLargeThreads, 2) part_large_kernel(const __gr
           n += v[x];
         }
         if (n < G.min_count) continue;
-        Place p = place_of(G, h | htop, KW == 2 ? k1[i] : 0);
-        u64 olo, ohi;
-        cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
-        acc_ins += finish_insert(G, p, olo, ohi, v);
+        const u64 hi = KW == 2 ? k1[i] : 0;
+        acc_ins += insert_key(G, S, h | htop, hi, v);
         const unsigned count = key_count(G, v);
-        if (count >= O.min_depth && write_record(G, O, atomicAdd(&G.status->n_out, 1ull), p.lo, p.hi, count, v))
+        if (count >= O.min_depth && write_record(G, O, atomicAdd(&G.status->n_out, 1ull), key_lo(h | htop, hi), hi, count, v))
           atomicAdd(&G.status->n_uu, 1ull);
       }
       lo += width;
@@ -1045,7 +1062,12 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     __syncthreads();
     // 4: outcomes
     if (tid == 0) s_nlist = 0;
-    if (tid == 0) s_base = s_nctr + s_nlone ? atomicAdd(S.n_keys, (u64)(s_nctr + s_nlone)) : 0;
+    if (tid == 0) {
+      const unsigned nk = s_nctr + s_nlone;
+      s_base = nk ? atomicAdd(S.n_keys, (u64)nk) : 0;
+      S.key_base[item] = s_base;
+      S.key_n[item] = nk;
+    }
 #pragma unroll 2
     for (unsigned x = tid; x < n; x += kCountThreads) {
       const unsigned q = s_q[s_rep[x]];
@@ -1099,15 +1121,137 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
   if (lane == 0 && acc_first && G.min_count > 1) atomicAdd(&G.status->first_sightings, (u64)acc_first);
 }
 
+// ------------------------------------------------------------------ table
+//
+// The table's slots follow the hash, so the keys of neighbouring sub-buckets go to a range of
+// slots of their own: one CTA makes that range in shared memory, empty slots and all, and writes
+// it with bulk copies (kBuildSlots at a time: as many sub-buckets as fill them, or a part of one).
+// Nothing is cleared before and no slot is claimed in HBM. A key that finds no empty slot in its
+// range (or whose first slot lies behind it) is marked; part_insert_kernel puts it into the table
+// when all ranges of the group have been written.
+//
+// Bound by the latency of an item's few loads behind one another and by the table's write; one
+// sub-bucket at a time was twice as slow. With the records (part_insert_kernel) 7.4 ms for 115 M
+// keys in 317 M slots; clearing the table and claiming every slot with a compare-and-swap took
+// 10.5 ms. 512 slots and 6 CTAs, 1024 and 3, 256 and 12: 7.5, 8.1, 7.4 ms.
+
+constexpr int kBuildThreads = 256;
+constexpr int kBuildCtas = 4;               // per SM
+constexpr unsigned kBuildSlots = 768;
+constexpr unsigned kBuildSubs = 16;         // sub-buckets at a time, at most
+constexpr size_t kBuildSmem = (size_t)kBuildSlots * (sizeof(Slot) + 4);
+
+// Slot of a hash in the whole table (never decreases with it), and the first one of sub-bucket s of
+// n of bucket b.
+__device__ __forceinline__ u64 slot_of(const PartGeom& G, u64 h) {
+  return (u64)part_of(h, G.P) * G.Sp + table_index(h, G.Sp, G.P);
+}
+__device__ __forceinline__ u64 first_slot(const PartGeom& G, unsigned b, unsigned s, unsigned n) {
+  if (b >> G.log_b) return (u64)G.P * G.Sp;
+  const u64 x = (((u64)s << 32) + n - 1) / n;  // the smallest that sub_of takes to s
+  return slot_of(G, ((u64)b << (64 - G.log_b)) | (x << (32 - G.log_b)));
+}
+
+template <int KW>
+__global__ void __launch_bounds__(kBuildThreads, kBuildCtas) part_build_kernel(const __grid_constant__ PartGeom G,
+                                                                      const __grid_constant__ PartSplit S) {
+  extern __shared__ __align__(128) unsigned char s_raw[];
+  uint4* s_slot = reinterpret_cast<uint4*>(s_raw);                                       // [slots][4]
+  unsigned* s_taken = reinterpret_cast<unsigned*>(s_raw + kBuildSlots * sizeof(Slot));   // [slots]
+  __shared__ u64 s_first[2][kBuildSubs];                 // first list entry of each sub-bucket, less the keys before it
+  __shared__ unsigned s_upto[2][kBuildSubs];             // keys up to and with it
+  const unsigned tid = threadIdx.x, n_sub = sub_buckets(G), n_subs = (S.b1 - S.b0) * n_sub;
+  // as many neighbouring sub-buckets as fill the slots in shared memory
+  const double ranges = (double)n_sub * (double)(1u << G.log_b), slots = (double)G.P * (double)G.Sp;
+  const double fit = 0.95 * kBuildSlots * ranges / slots;
+  const unsigned m = fit >= kBuildSubs ? kBuildSubs : fit < 2.0 ? 1u : (unsigned)fit;
+  const unsigned n_items = (n_subs + m - 1) / m;
+  unsigned acc_ins = 0, buf = 0;
+  // the first warp: lists of an item's sub-buckets (loaded an item ahead)
+  auto lists = [&](unsigned item, unsigned to) {
+    if (tid >= 32) return;
+    const unsigned sub = item * m + tid;
+    const bool in = tid < m && item < n_items && sub < n_subs;
+    const unsigned n = in ? S.key_n[sub] : 0u;
+    const u64 base = n ? S.key_base[sub] : 0ull;
+    unsigned upto = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned x = __shfl_up_sync(0xffffffffu, upto, o);
+      if (tid >= (unsigned)o) upto += x;
+    }
+    if (tid < m) {
+      s_upto[to][tid] = upto;
+      s_first[to][tid] = base - (upto - n);
+    }
+  };
+  lists(blockIdx.x, 0);
+  for (unsigned item = blockIdx.x; item < n_items; item += gridDim.x, buf ^= 1) {
+    const unsigned sub0 = item * m, sub1 = sub0 + m < n_subs ? sub0 + m : n_subs;
+    const u64 begin = first_slot(G, S.b0 + sub0 / n_sub, sub0 % n_sub, n_sub);
+    const u64 end = first_slot(G, S.b0 + sub1 / n_sub, sub1 % n_sub, n_sub);
+    for (u64 c0 = begin; c0 < end || c0 == begin; c0 += kBuildSlots) {
+      const unsigned ns = end - c0 < kBuildSlots ? (unsigned)(end - c0) : kBuildSlots;
+      if (tid == 0) tma_store_wait_read();  // the previous slots have left shared memory
+      __syncthreads();
+      for (unsigned i = tid; i < ns * 4; i += kBuildThreads) {
+        const unsigned v = i & 3 ? 0u : 0xFFFFFFFFu;
+        s_slot[i] = make_uint4(v, v, v, v);
+      }
+      for (unsigned i = tid; i < ns; i += kBuildThreads) s_taken[i] = 0;
+      __syncthreads();
+      if (c0 == begin) lists(item + gridDim.x, buf ^ 1);  // read after the next barriers
+      const unsigned nk = s_upto[buf][m - 1];
+      for (unsigned i = tid; i < nk; i += kBuildThreads) {
+        unsigned at = 0;
+        while (i >= s_upto[buf][at]) ++at;
+        unsigned* e = S.keys + (s_first[buf][at] + i) * kKeyWords<KW>;
+        const uint2 hw = *reinterpret_cast<const uint2*>(e + kCtrWords);
+        const u64 h = ((u64)hw.y << 32) | hw.x, g = slot_of(G, h);
+        if (g >= end ? c0 + ns < end : g - c0 >= ns) continue;  // not of these slots (g >= begin)
+        // probes go round at the end of the partition, which may lie inside the range
+        const u64 round = ((u64)part_of(h, G.P) + 1) * G.Sp - c0;
+        const unsigned last = round < ns ? (unsigned)round : ns;
+        unsigned x = g < end ? (unsigned)(g - c0) : ns;
+        while (x < last && atomicExch(&s_taken[x], 1u)) ++x;
+        const uint2* w = reinterpret_cast<const uint2*>(e);
+        const uint2 w2 = w[2];
+        if (x >= last) {
+          e[5] = w2.y | 0x10000u;  // marked, in the half not used
+          continue;
+        }
+        const uint2 w0 = w[0], w1 = w[1];
+        const u64 hi = KW == 2 ? *reinterpret_cast<const u64*>(e + kKeyWords<KW> - 2) : 0ull, lo = key_lo(h, hi);
+        s_slot[4 * x] = make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
+        s_slot[4 * x + 1] = make_uint4(w1.x & 0xFFFFu, w2.y & 0xFFFFu, 0u, 0u);
+        s_slot[4 * x + 2] = make_uint4(w0.x & 0xFFFFu, w0.x >> 16, w0.y & 0xFFFFu, w0.y >> 16);
+        s_slot[4 * x + 3] = make_uint4(w1.y & 0xFFFFu, w1.y >> 16, w2.x & 0xFFFFu, w2.x >> 16);
+        ++acc_ins;
+      }
+      fence_proxy_async_smem();
+      __syncthreads();
+      if (tid == 0 && ns) {
+        unsigned char* dst = reinterpret_cast<unsigned char*>(G.table + c0);
+        const unsigned bytes = ns * (unsigned)sizeof(Slot);
+        for (unsigned o = 0; o < bytes; o += 16384u)
+          tma_store_1d(dst + o, smem_u32(s_raw) + o, bytes - o < 16384u ? bytes - o : 16384u);
+        tma_store_commit();
+      }
+    }
+  }
+  if (tid == 0) tma_store_wait();  // complete before the CTA may leave
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc_ins += __shfl_down_sync(0xffffffffu, acc_ins, o);
+  if ((tid & 31) == 0 && acc_ins) atomicAdd(&G.status->table_keys, (u64)acc_ins);
+}
+
 // ------------------------------------------------------------------ insert
 //
-// The counted keys of the list into the HBM table, and the records of those that are frequent
-// enough (Section 5.1's depth filter, the side codes of Sections 2 and 4.1) into the output. The
-// keys are distinct, in no slot yet, and in hash order roughly, so the slots written at one time
-// lie in one or two partitions. A tile's output places are reserved together: the atomics on that
-// one counter take 6 ns each. One key in flight per thread: with two or four the registers cost
-// more warps than the round trips gained (8.0, 8.5 and 16.5 ms for 115 M keys, 7.7 as it is). Writing the
-// records here saves the scan of the whole table (64 bytes per slot, half of them empty).
+// The output records of the listed keys that are frequent enough (Section 5.1's depth filter, the
+// side codes of Sections 2 and 4.1), and the marked keys into the table: a few at the end of each
+// range, by compare-and-swap behind those that are there. A tile's output places are reserved
+// together: the atomics on that one counter take 6 ns each. Writing the records here saves the
+// scan of the whole table (64 bytes per slot, half of them empty).
 
 constexpr int kInsertThreads = 256;
 constexpr int kInsertKeys = 2;
@@ -1115,28 +1259,37 @@ constexpr unsigned kInsertTile = kInsertThreads * kInsertKeys;
 
 template <int KW>
 __global__ void __launch_bounds__(kInsertThreads) part_insert_kernel(const __grid_constant__ PartGeom G,
-                                                                     const __grid_constant__ PartOut O,
-                                                                     const unsigned* keys, const u64* n_keys, unsigned* done) {
+                                                                     const __grid_constant__ PartSplit S,
+                                                                     const __grid_constant__ PartOut O) {
   __shared__ unsigned s_wsum[32];
   __shared__ u64 s_base;
-  const u64 n = __ldcg(n_keys);
+  const u64 n = __ldcg(S.n_keys);
+  const unsigned* keys = S.keys;
   unsigned acc_ins = 0, acc_uu = 0;
-  // key i into the table; its record at `at` if it has the depth
+  // the keys carried over from the groups before
+  u64 carried = __ldcg(S.n_carry_in);
+  if (carried > kMaxProbe) carried = kMaxProbe;
+  for (u64 i = (u64)blockIdx.x * kInsertThreads + threadIdx.x; i < carried; i += (u64)gridDim.x * kInsertThreads) {
+    const unsigned* c = S.carry_in + i * kCarryWords;
+    unsigned v[10];
+#pragma unroll
+    for (int x = 0; x < 10; ++x) v[x] = c[x];
+    acc_ins += insert_key(G, S, ((u64)c[11] << 32) | c[10], ((u64)c[13] << 32) | c[12], v);
+  }
+  // key i into the table if it is marked; its record at `at` if it has the depth
   auto put = [&](u64 i, u64 at) {
     const uint2* c = reinterpret_cast<const uint2*>(keys + i * kKeyWords<KW>);
     uint2 w[kKeyWords<KW> / 2];
 #pragma unroll
     for (unsigned x = 0; x < kKeyWords<KW> / 2; ++x) w[x] = __ldg(c + x);
     const u64 h = ((u64)w[3].y << 32) | w[3].x;
-    Place p = place_of(G, h, KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull);
-    u64 olo, ohi;
-    cas128(p.sub + p.idx, kEmpty, kEmpty, p.lo, p.hi, olo, ohi);
+    const u64 hi = KW == 2 ? ((u64)w[kKeyWords<KW> / 2 - 1].y << 32) | w[kKeyWords<KW> / 2 - 1].x : 0ull;
     const unsigned v[10] = {w[0].x & 0xFFFFu, w[0].x >> 16, w[0].y & 0xFFFFu, w[0].y >> 16, w[1].x & 0xFFFFu,
                             w[1].y & 0xFFFFu, w[1].y >> 16, w[2].x & 0xFFFFu, w[2].x >> 16, w[2].y & 0xFFFFu};
+    if (w[2].y >> 16) acc_ins += insert_key(G, S, h, hi, v);
     const unsigned count = key_count(G, v);
-    acc_ins += finish_insert(G, p, olo, ohi, v);
     if (count < O.min_depth) return false;
-    acc_uu += write_record(G, O, at, p.lo, p.hi, count, v);
+    acc_uu += write_record(G, O, at, key_lo(h, hi), hi, count, v);
     return true;
   };
   if (O.min_depth <= G.min_count) {
@@ -1146,7 +1299,7 @@ __global__ void __launch_bounds__(kInsertThreads) part_insert_kernel(const __gri
     __syncthreads();  // all of the block have read base
     if (threadIdx.x == 0) {
       __threadfence();
-      if (atomicAdd(done, 1u) == gridDim.x - 1 && n) atomicAdd(&G.status->n_out, n);  // everyone has
+      if (atomicAdd(reinterpret_cast<unsigned*>(S.inserted), 1u) == gridDim.x - 1 && n) atomicAdd(&G.status->n_out, n);  // everyone has
     }
   } else {
     for (u64 t = blockIdx.x; t * kInsertTile < n; t += gridDim.x) {
@@ -1285,12 +1438,23 @@ cudaError_t launch_part_large(const PartGeom& g, const PartSplit& s, const PartO
   return cudaGetLastError();
 }
 
+cudaError_t launch_part_build(const PartGeom& g, const PartSplit& s, cudaStream_t stream, int num_sms) {
+  if (s.b1 <= s.b0) return cudaSuccess;
+  const void* fn = g.k > 32 ? (const void*)part_build_kernel<2> : (const void*)part_build_kernel<1>;
+  cudaError_t e = allow_dynamic_smem(fn, kBuildSmem);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = (unsigned)grid_for(fn, kBuildThreads, kBuildSmem, num_sms, (u64)(s.b1 - s.b0) * g.sub_max);
+  if (g.k > 32) part_build_kernel<2><<<grid, kBuildThreads, kBuildSmem, stream>>>(g, s);
+  else part_build_kernel<1><<<grid, kBuildThreads, kBuildSmem, stream>>>(g, s);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_part_insert(const PartGeom& g, const PartSplit& s, const PartOut& o, cudaStream_t stream, int num_sms) {
   // the number of keys is known on the device only: as many CTAs as run at a time
   const void* fn = g.k > 32 ? (const void*)part_insert_kernel<2> : (const void*)part_insert_kernel<1>;
   const unsigned grid = (unsigned)grid_for(fn, kInsertThreads, 0, num_sms, ~0ull);
-  if (g.k > 32) part_insert_kernel<2><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys, reinterpret_cast<unsigned*>(s.inserted));
-  else part_insert_kernel<1><<<grid, kInsertThreads, 0, stream>>>(g, o, s.keys, s.n_keys, reinterpret_cast<unsigned*>(s.inserted));
+  if (g.k > 32) part_insert_kernel<2><<<grid, kInsertThreads, 0, stream>>>(g, s, o);
+  else part_insert_kernel<1><<<grid, kInsertThreads, 0, stream>>>(g, s, o);
   return cudaGetLastError();
 }
 

@@ -19,6 +19,21 @@ def one_read(n, seed, alphabet="ACGT"):
     return "".join(np.array(list(alphabet))[rng.integers(0, len(alphabet), n)])
 
 
+def oracle_absent(keys, k):
+    """Keys of random k-mers that are not among `keys`."""
+    have = {(int(a), int(b)) for a, b in keys}
+    rng = np.random.default_rng(13)
+    out = [(int(rng.integers(0, 1 << min(2 * k, 62))), int(rng.integers(0, 1 << (2 * k - 64))) if 2 * k > 64 else 0) for _ in range(2000)]
+
+    def canonical(key):
+        x, y = key[0] | key[1] << 64, 0
+        for i in range(k):
+            y |= (3 - (x >> 2 * i & 3)) << 2 * (k - 1 - i)
+        x = min(x, y)
+        return x & (1 << 64) - 1, x >> 64
+    return np.array([q for q in out if canonical(q) not in have], np.uint64)
+
+
 def both(gpu, rs, what, **kw):
     """Partitioned and oracle, with and without the minimum of two sightings."""
     for depth in (1, 2, 3):
@@ -90,6 +105,37 @@ def test_more_records_than_room(gpu, k):
     want = oracle_for(rs)
     for load in (0.05, 0.9):
         assert_same(run_gpu(gpu, rs, use_bloom=False, partitions=8, load_factor=load, table_capacity=1 << 17), want, load)
+
+
+@pytest.mark.parametrize("k", [31, 51])
+@pytest.mark.parametrize("partitions", [2, 7, 64])
+def test_table_of_ranges(gpu, k, partitions):
+    """The table that is made a sub-bucket's range at a time, roomy and nearly full (keys that find no
+    slot in their range, go round a partition's end or into the next group's slots), in one group of
+    buckets and in eight: every key is found in it, and no other."""
+    from paper_1705_11147_gb300 import KmerAnalysis, make_params
+    rs = readset([one_read(3000, 500 + i) for i in range(20)], k=k, min_ext_count=1, qual_threshold=20, min_depth=1)
+    want = oracle_for(rs)
+    absent = oracle_absent(want.keys, k)
+    for slots in (1.02, 1.2, 12.0):
+        for to_host in (False, True):
+            # the partitions' shares of the keys differ by a few standard deviations
+            room = int(len(want) * slots) + int(6 * np.sqrt(len(want) * partitions))
+            with KmerAnalysis(make_params(max_bases=rs.n_bases, max_reads=rs.n_reads, use_bloom=False, partitions=partitions,
+                                          table_capacity=room, **rs.meta["params"])) as ka:
+                for _ in range(2):  # also over the table of a sample before
+                    ka.reset()
+                    ka.count(rs.seq, rs.qual, rs.offsets)
+                    if to_host:
+                        n = len(want) + 5
+                        ka.finalize_to_host((np.empty((n, 2), np.uint64), np.empty(n, np.uint32), np.empty((n, 8), np.uint32),
+                                             np.empty((n, 2), np.uint8)))
+                    else:
+                        ka.finalize()
+                    counts, ext, codes = ka.query(want.keys)
+                    assert np.array_equal(counts, want.counts) and np.array_equal(ext, want.ext)
+                    assert np.array_equal(codes, want.codes)
+                    assert not ka.query(absent)[0].any()
 
 
 @pytest.mark.parametrize("n_parts", [2, 7])
