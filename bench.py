@@ -242,29 +242,26 @@ def roofline(timing: dict, res_info, positions: int, peak_gbs: float, plan_used,
       64 B per valid window (Bloom word sector read + write-back), 128 B per window whose k-mer
       the filter had seen (slot key/count sector + extension sector, read + written back),
       0.625 B per arena position (codes, reverse codes... read, marks written).
-    partitions (part_pass_kernel, Bloom mode), the partitioned model of the hot-path table:
-      per record (one per valid window) its key + info byte read (17 B, 9 B for k <= 32), and
-      per first sighting the record written back (compacted for the recount). A second figure
-      adds each partition's Bloom sub-filter and sub-table brought from HBM once and written
-      back once (2 x filter + table bytes).
-    The partitioned pass keeps its random atomics in L2, so its ceiling is the L2 request
-    rate: `l2` gives the L2 requests per record from the ncu capture times the records, over
-    the live kernel time, against the L2's peak request rate (slices x L2 clock, from ncu)."""
+    partitions (part_scatter_kernel + part_split_kernel, the two sorts, over all launches of one
+      step): 0.75 B per arena position read, and per record (one per valid window, 8 B for
+      k <= 32, else 16) one write by the scatter and a read and a write by the split. A second
+      figure is the counting (part_count_kernel), which reads every record once."""
     W = int(res_info.valid_windows)
     F = int(timing["first_sightings"])
     ms = timing["ms_pass"] / max(timing["n_pass"], 1)
     extra = {}
     if plan_used.partitions > 1:
-        rec = (16 if k > 32 else 8) + 1
-        struct_bytes = plan_used.bloom_words * 8 + plan_used.table_slots * 64
-        algo = float(W) * rec + float(F) * rec
-        kernel, files, summary = ("part_pass_kernel (Bloom mode)", ["kma_partition.cu", "kma_device.cuh"],
-                                  "part_pass_kernel_large_200m.md")
-        with_struct = algo + 2.0 * struct_bytes
-        extra["with_partition_structures"] = {
-            "algo_bytes_per_launch": int(with_struct),
-            "achieved": round(with_struct / (ms * 1e-3) / 1e9, 1),
-            "frac": round(with_struct / (ms * 1e-3) / 1e9 / peak_gbs, 4)}
+        rec = 16 if k > 32 else 8
+        steps = max(timing["n_pack"], 1)
+        counted = timing["ms_pass"] / steps
+        extra["count"] = {"kernel": "part_count_kernel", "ms_per_step": round(counted, 3),
+                          "algo_bytes_per_step": W * rec,
+                          "achieved": round(W * rec / (counted * 1e-3) / 1e9, 1),
+                          "frac": round(W * rec / (counted * 1e-3) / 1e9 / peak_gbs, 4)}
+        ms = timing["ms_scatter"] / steps
+        algo = 0.75 * positions + 3.0 * rec * W
+        kernel, files, summary = ("part_scatter_kernel + part_split_kernel", ["kma_partition.cu", "kma_device.cuh"],
+                                  "part_sort_kernels_bacterial_5m.md")
     else:
         algo = 64.0 * W + 128.0 * (W - F) + 0.625 * positions
         kernel, files, summary = ("pass_kernel (Bloom mode)", ["kma_kernels.cu", "kma_device.cuh"],

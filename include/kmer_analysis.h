@@ -4,8 +4,8 @@
  * The library implements the k-mer analysis stage of HipMer / Meraculous (arXiv 1705.11147):
  *   - chopping reads into overlapping k-mers (Section 2, item 1; Figure "combined"(b)),
  *   - canonical form (lexicographic min of a k-mer and its reverse complement),
- *   - a Bloom-filter pass that keeps singleton (error) k-mers out of the hash table
- *     (Section 5.1),
+ *   - a pass that keeps singleton (error) k-mers out of the hash table (Section 5.1: by a
+ *     Bloom filter; with partitions by counting them exactly on chip),
  *   - exact counting in a device hash table with per-k-mer counts of high-quality left and
  *     right extension bases (Section 5.1: two arrays of four counters per k-mer),
  *   - the depth filter and classification of each side into A/C/G/T (unique), X (none,
@@ -65,8 +65,8 @@ typedef struct {
                                  (paper: more than t_hq) */
   uint8_t qual_threshold;     /* an extension base is counted only if its Phred >= this */
   uint8_t qual_offset;        /* quality encoding offset: 33 for ASCII Phred+33, 0 for raw */
-  uint8_t use_bloom;          /* 1: Bloom-filter singleton pass (requires min_depth >= 2);
-                                 0: every k-mer goes straight into the table */
+  uint8_t use_bloom;          /* 1: singletons are kept out of the table (requires min_depth >= 2;
+                                 with one table by a Bloom filter); 0: every k-mer goes into it */
   uint8_t canonical;          /* 1: canonical k-mers (default); 0: forward strand only */
   uint64_t max_bases;         /* arena capacity: total bases over all count() calls */
   uint64_t max_reads;         /* total reads over all count() calls (0: max_bases / 32) */
@@ -75,14 +75,14 @@ typedef struct {
   double bloom_fpr;           /* target false-positive rate of the Bloom filter (0: 0.01) */
   uint64_t table_capacity;    /* hash-table slots (0: expected_keys / load_factor) */
   uint64_t expected_keys;     /* keys the table must hold (0: expected_distinct, or the window
-                                 bound). With the Bloom pass only k-mers seen twice (plus
-                                 false positives) are inserted. */
+                                 bound). With use_bloom only k-mers seen twice (with one table
+                                 plus false positives) are inserted. */
   double load_factor;         /* target table load when table_capacity = 0 (0: 0.5) */
   uint64_t staging_bytes;     /* device staging buffer for host inputs (0: 256 MiB) */
   /* Launch shape (0 = library default; chosen by the autotuner per GPU and size class). */
   uint32_t block_threads;     /* threads per CTA of the counting kernels: 64..256, x32 */
   uint32_t windows_per_thread;/* window starts one thread handles per tile: 1, 2, 4 or 8
-                                 (with partitions: records per thread, 4 or 8 -> 4, else 2) */
+                                 (with partitions the launch shape is the library's) */
   uint32_t ctas_per_sm;       /* persistent grid = SMs x ctas_per_sm (0: occupancy bound) */
   uint32_t warp_aggregate;    /* 1: merge identical keys inside a warp before the atomics */
   /* Owner-computes partition (Section 5.1: a deterministic k-mer -> owner map makes every
@@ -97,26 +97,25 @@ typedef struct {
                                  staging copies it never issued, with a short poll limit, so
                                  its bounded wait gives up and the handle reports KMA_ETIMEOUT */
   uint32_t partitions;        /* on-chip owner-computes partitions (Section 5.1's owner map on
-                                 one GPU): the Bloom filter and table are split by a hash into
-                                 P parts, windows are first written to per-part record buckets,
-                                 and the buckets are counted part by part so one part's filter
-                                 and table stay in L2. 0: automatic (P >= 2 when filter + table
+                                 one GPU): windows are written as records, sorted by hash until
+                                 all occurrences of a k-mer lie in one small sub-bucket, and
+                                 counted there in shared memory; the table is laid out in P
+                                 parts of the same hash. 0: automatic (P >= 2 when filter + table
                                  exceed 32 MB, at most 64 MB per part); 1: one table, windows
                                  counted in place; P >= 2: that many parts (<= 4096 for
                                  k <= 32, <= 2048 for k > 32; more: KMA_EINVAL). Results
                                  do not depend on it. */
   uint32_t heavy_hitters;     /* 1: k-mers with very many occurrences (satellites, low-complexity
-                                 sequence) are expected. The partitioned counting passes then
-                                 look for equal keys among each warp's records and treat them
-                                 as one (one Bloom test-and-set and one table probe per group,
-                                 counter updates summed in shared memory first: Section 5.1's
-                                 local accumulation of heavy hitters, at warp level). 0: off.
-                                 Results do not depend on it. */
+                                 sequence) are expected. Partitioned counting accumulates them
+                                 locally (Section 5.1: lanes with equal outcomes of equal keys
+                                 act as one, in sub-buckets that overflow) whether this is set
+                                 or not. Results do not depend on it. */
 } kma_params;
 
 /* Sizes derived from a kma_params (pure host arithmetic, no GPU needed). */
 typedef struct {
-  uint64_t bloom_words;    /* 64-bit words of the blocked Bloom filter (0 without Bloom) */
+  uint64_t bloom_words;    /* 64-bit words of the blocked Bloom filter (0 without Bloom); with
+                              partitions it decides their number but is not allocated */
   uint32_t bloom_hashes;   /* bits set per k-mer, all inside one 64-bit word */
   uint32_t partitions;     /* on-chip partitions (1: one table) */
   double bloom_fpr_est;    /* predicted false-positive rate at expected_distinct k-mers */
@@ -156,7 +155,8 @@ int kmer_analysis_create(const kma_params* params, void* cuda_stream, kma_handle
  * offsets has n_reads + 1 non-decreasing entries. Bases other than A/C/G/T (either case)
  * make every window covering them invalid. Reads shorter than k add no windows.
  * Packs the reads 2 bits per base into the handle's arena and runs the first pass
- * (Bloom test-and-set, table insert of k-mers seen twice; without Bloom, the counting).
+ * (Bloom test-and-set, table insert of k-mers seen twice; without Bloom, the counting; with
+ * partitions, the windows become records, counted by finalize).
  * With on_device = 1 the call reads offsets[0] and offsets[n_reads] back, which waits for
  * the stream up to that point. Errors: KMA_EINVAL (decreasing offsets), KMA_EFULL (arena:
  * max_bases / max_reads exceeded; table overflow is reported by finalize), KMA_ESTATE
@@ -165,8 +165,8 @@ int kmer_analysis_count(kma_handle* h, const char* seq, const char* qual,
                         const uint64_t* offsets, uint64_t n_reads, int on_device);
 
 /* Finish counting: second pass over the retained reads (first sightings of k-mers the
- * Bloom pass left out of the table), depth filter, classification and compaction into
- * device arrays (see kma_result). Synchronises the stream. Errors: KMA_EFULL (table
+ * Bloom pass left out of the table; with partitions, the counting of the records), depth filter,
+ * classification and compaction into device arrays (see kma_result). Synchronises the stream. Errors: KMA_EFULL (table
  * overflow: no partial result), KMA_EOVERFLOW, KMA_EINVAL (inconsistent offsets seen on
  * the device), KMA_ESTATE (already finalized), KMA_ENOMEM, KMA_ECUDA. */
 int kmer_analysis_finalize(kma_handle* h, kma_result* out);
@@ -178,9 +178,9 @@ int kmer_analysis_copy_result(kma_handle* h, uint64_t* keys, uint32_t* counts, u
                               uint8_t* codes, uint64_t capacity, int on_device);
 
 /* kmer_analysis_finalize followed by kmer_analysis_copy_result into HOST buffers, with the
- * copies overlapped: the recount (Section 5.1's exact second pass) and the classification
- * run in groups of on-chip partitions (of table slots with one table), and each group's
- * records are copied to the host while the next group is recounted. The records, their
+ * copies overlapped: the counting of the records (with one table, after the recount, the
+ * classification) runs in groups of hash ranges, and each group's records are copied to the
+ * host while the next group is counted. The records, their
  * order aside, are those of finalize. Buffers hold `capacity` records each (keys[c][2],
  * counts[c], ext[c][8], codes[c][2] as in kma_result); any pointer may be NULL to skip that
  * array; pinned host memory gives full copy bandwidth. The device result stays valid
@@ -200,8 +200,8 @@ int kmer_analysis_query(kma_handle* h, const uint64_t* keys, uint64_t n, uint32_
                         uint32_t* ext, uint8_t* codes, int on_device);
 
 /* Empty the handle for a new read set with the same parameters, keeping its memory
- * (Bloom filter and table are cleared on the stream; the packed-read arena is rewritten by
- * the next count calls). */
+ * (with one table the Bloom filter and table are cleared on the stream; the packed-read arena,
+ * and with partitions the table, are rewritten by the next count and finalize calls). */
 int kmer_analysis_reset(kma_handle* h);
 
 /* Change the stream later calls enqueue on (the caller orders the two streams). */
@@ -226,12 +226,14 @@ typedef struct {
 } kma_timings;
 
 #define KMA_KERNEL_PACK 0
-#define KMA_KERNEL_PASS 1      /* first pass: Bloom test-and-set + table (or counting) */
-#define KMA_KERNEL_RECOUNT 2   /* second pass over first sightings */
+#define KMA_KERNEL_PASS 1      /* first pass: Bloom test-and-set + table (or counting);
+                                  partitioned mode: counting of the sub-buckets */
+#define KMA_KERNEL_RECOUNT 2   /* second pass over first sightings; partitioned mode: the table
+                                  and the output records */
 #define KMA_KERNEL_CLASSIFY 3
 #define KMA_KERNEL_QUERY 4
-#define KMA_KERNEL_INIT 5      /* table initialisation on create / reset */
-#define KMA_KERNEL_SCATTER 7   /* partitioned mode: windows -> per-partition record buckets */
+#define KMA_KERNEL_INIT 5      /* table initialisation on create / reset (one table) */
+#define KMA_KERNEL_SCATTER 7   /* partitioned mode: windows -> records, and both their sorts */
 
 int kmer_analysis_set_profiling(kma_handle* h, int enable);
 int kmer_analysis_timings(kma_handle* h, kma_timings* out, int reset);

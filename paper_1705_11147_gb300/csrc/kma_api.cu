@@ -202,7 +202,9 @@ int derive(const kma_params* p, Derived& d) {
   if (d.P > 1) {  // scatter tiles with their offset rows, and the split's sorted copy
     const u64 tiles = pos / kPartTile + 1, recs = tiles * kPartTile * d.rec_bytes;
     const u64 copy = recs <= kSplitAtOnce ? recs : std::max(kSplitAtOnce, recs / kSplitGroups);
-    d.plan.device_bytes += recs + tiles * (((u64)1 << d.log_b) + 8) * 2 + 4 * copy;
+    // sub-buckets, overflow segments, and the listed keys: all records may be one (a half, of two each)
+    const double keys = (p->use_bloom ? 0.5 : 1.0) * (d.rec_bytes == 8 ? 4.0 : 2.5);
+    d.plan.device_bytes += recs + tiles * (((u64)1 << d.log_b) + 8) * 2 + (u64)((2.5 + keys) * (double)copy);
   }
   return KMA_OK;
 }

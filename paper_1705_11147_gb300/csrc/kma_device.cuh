@@ -34,7 +34,6 @@ __device__ __forceinline__ u64 key_hash(u64 lo, u64 hi) {
 //   Bloom bit positions 6-bit fields from the top of (h ^ h >> 32) * c   (bloom_mask)
 // The bit positions must not depend on the low bits of h alone: those also pick the word, and
 // keys sharing a word would then share most of their bits (a much higher false-positive rate).
-__device__ __forceinline__ u64 scramble(u64 h) { return h * 0x9e3779b97f4a7c15ull; }
 // Slot of a key in its partition (of `parts`): in the order of the hash, so that the keys of one
 // sub-bucket (partitioned mode counts in hash order) go to neighbouring slots and every line of
 // the table is brought in and written back once.
@@ -383,30 +382,6 @@ __device__ __forceinline__ void cas128(Slot* s, u64 cmp_lo, u64 cmp_hi, u64 new_
       : "=l"(old_lo), "=l"(old_hi)
       : "l"(cmp_lo), "l"(cmp_hi), "l"(new_lo), "l"(new_hi), "l"(s)
       : "memory");
-}
-
-// Insert-if-absent. Keys are written once (empty -> key) by a 16-byte CAS and never change
-// again. A plain 16-byte load may observe a half-written slot; any value with a word still
-// equal to the empty pattern is therefore resolved by the CAS itself, which is atomic.
-// Returns the slot or nullptr (probe limit reached: the table is full).
-__device__ __forceinline__ Slot* find_or_insert(Slot* table, u64 slots, u64 lo, u64 hi, u64 h,
-                                                bool& inserted) {
-  u64 idx = table_index(h, slots);
-  const u64 limit = slots < kMaxProbe ? slots : kMaxProbe;
-  inserted = false;
-  for (u64 n = 0; n < limit; ++n) {
-    Slot* s = table + idx;
-    const ulonglong2 kv = __ldcg(reinterpret_cast<const ulonglong2*>(s));
-    if (kv.x == lo && kv.y == hi) return s;
-    if (kv.y == kEmpty || kv.x == kEmpty) {
-      u64 olo, ohi;
-      cas128(s, kEmpty, kEmpty, lo, hi, olo, ohi);
-      if (olo == kEmpty && ohi == kEmpty) { inserted = true; return s; }
-      if (olo == lo && ohi == hi) return s;
-    }
-    idx = (idx + 1 == slots) ? 0 : idx + 1;
-  }
-  return nullptr;
 }
 
 // Lookup in a table no thread is modifying. nullptr if absent; sets `full` if the probe

@@ -6,18 +6,22 @@
 //                        outcomes); each tile of 8192 window starts is sorted by bucket (the top
 //                        bits of the key hash) in shared memory and written out as it lies, with
 //                        a row of bucket offsets
-//   part_split_kernel    gathers a bucket's runs from many scatter tiles, sorts them by sub-bucket
-//                        (the next part of the hash) and writes them the same way
-//   part_count_kernel    gathers a sub-bucket's runs into shared memory: all occurrences of a few
-//                        hundred to a few thousand k-mers, counted there; only k-mers seen at
-//                        least twice (every k-mer without the singleton filter) go to the table
-//                        in HBM, each inserted once with its final counters
+//   part_split_kernel    gathers a bucket's runs from many scatter tiles, orders them by sub-bucket
+//                        (the next part of the hash) and appends each run to its sub-bucket
+//   part_count_kernel    brings a sub-bucket into shared memory: all occurrences of a few hundred
+//                        to a few thousand k-mers, counted there; only k-mers seen at least twice
+//                        (every k-mer without the singleton filter) are listed
+//   part_large_kernel    the same for sub-buckets that do not fit (very frequent k-mers)
+//   part_build_kernel    the listed keys with their counters into the table, a range of slots at a
+//                        time
+//   part_insert_kernel   the output records, and the keys that left their range
 //
 // Why two sorts and no filter in front of the table: a Bloom test-and-set plus table atomics in
 // L2 took 4.6 L2 requests per window, 21 ns per 1000 windows, and a second pass over the first
-// sightings another 8 ns. A sort pass reads and writes 16 bytes per window in whole lines, and
-// with all occurrences of a k-mer in one shared memory the singletons (error k-mers) are known
-// exactly, so they cost no memory traffic outside the SM.
+// sightings another 8 ns. A sort pass reads and writes 8 or 16 bytes per window in whole lines,
+// and with all occurrences of a k-mer in one shared memory the singletons (error k-mers) are known
+// exactly, so they cost no memory traffic outside the SM. 2.4 G windows, k = 31: 110 ms -> 79 ms
+// from reads to answers, 166 M windows, k = 51: 8.2 ms -> 5.7 ms.
 #include <mutex>
 #include <utility>
 #include <vector>
@@ -554,8 +558,8 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 //     sub-bucket has fewer than 2^16 records);
 //  4. every record of such a key adds its two outcomes;
 //  5. these keys with their counters (all keys without the singleton filter) are appended to a
-//     list, which part_insert_kernel puts into the HBM table: a few keys per sub-bucket would
-//     leave most threads waiting for the table's round trips here.
+//     list for part_build_kernel: inserted here, a few keys per sub-bucket would leave most threads
+//     waiting for the table's round trips (34 ms -> 47 ms for 2.4 G windows).
 // Sub-buckets that overflowed (very frequent k-mers) and those with more keys than the second
 // table holds are listed for part_large_kernel.
 //
