@@ -5,13 +5,13 @@
 // number (line 4r starts record r), never by scanning for markers.
 //
 // Device steps (all on the caller's stream):
-//   1. newlines per 16 KiB chunk of text            fastq_count_kernel
+//   1. newlines per 64 KiB chunk of text, masks      fastq_count_kernel
 //   2. exclusive scan of the chunk counts           scan kernels (device-wide, u64)
 //   3. newline positions, in order                  fastq_lines_kernel
 //   4. per record: check the '@' and '+' lines, base and quality line lengths equal
 //                                                   fastq_record_kernel
 //   5. exclusive scan of the base counts -> offsets scan kernels
-//   6. bases and qualities copied out, one warp per record
+//   6. bases and qualities copied out, 8 lanes a line
 //                                                   fastq_copy_kernel
 // A line may end in "\r\n"; the '\r' is not part of it. A final line without '\n' counts.
 #include "kma_device.cuh"
@@ -20,7 +20,8 @@ namespace kma {
 
 constexpr int kFqThreads = 1024;
 constexpr int kFqBytesPerThread = 16;
-constexpr u64 kFqChunk = (u64)kFqThreads * kFqBytesPerThread;  // 16 KiB of text per CTA
+constexpr int kFqPieces = 4;  // 16-byte pieces per thread; with one the two passes took 69 and 75 instead of 50 and 26 us
+constexpr u64 kFqChunk = (u64)kFqThreads * kFqBytesPerThread * kFqPieces;  // 64 KiB of text per CTA
 
 // ------------------------------------------------------------------ device-wide scan (u64)
 
@@ -128,16 +129,22 @@ __device__ __forceinline__ unsigned newline_mask(const unsigned char* text, u64 
   return m;
 }
 
-// Newlines in each 16 KiB chunk (plus one for a final line that does not end in '\n'), and their
+// Newlines in each chunk (plus one for a final line that does not end in '\n'), and their
 // masks, an eighth of the text, for the next pass (reading the text again took it 104 us of 516 for
 // 100 Mbases).
 __global__ void __launch_bounds__(kFqThreads) fastq_count_kernel(const unsigned char* text, u64 n, unsigned head,
                                                                  unsigned short* masks, u64* chunk_counts) {
   __shared__ unsigned warp_cnt[kFqThreads / 32];
   const u64 c = blockIdx.x;
-  const unsigned m = newline_mask(text, n, (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head);
-  masks[c * kFqThreads + threadIdx.x] = (unsigned short)m;
-  unsigned cnt = __popc(m);
+  unsigned cnt = 0, m[kFqPieces];
+#pragma unroll
+  for (int j = 0; j < kFqPieces; ++j)
+    m[j] = newline_mask(text, n, (long long)(c * kFqChunk + (u64)(j * kFqThreads + threadIdx.x) * kFqBytesPerThread) - head);
+#pragma unroll
+  for (int j = 0; j < kFqPieces; ++j) {
+    masks[(c * kFqPieces + j) * kFqThreads + threadIdx.x] = (unsigned short)m[j];
+    cnt += __popc(m[j]);
+  }
   cnt = __reduce_add_sync(0xffffffffu, cnt);
   if ((threadIdx.x & 31) == 0) warp_cnt[threadIdx.x >> 5] = cnt;
   __syncthreads();
@@ -153,9 +160,11 @@ __global__ void __launch_bounds__(kFqThreads) fastq_lines_kernel(const unsigned 
                                                                  u64* line_end) {
   __shared__ unsigned warp_off[kFqThreads / 32];
   const u64 c = blockIdx.x;
-  const long long i = (long long)(c * kFqChunk + (u64)threadIdx.x * kFqBytesPerThread) - head;
-  unsigned m = masks[c * kFqThreads + threadIdx.x];
-  const unsigned cnt = __popc(m);
+  // four pieces in a row
+  static_assert(kFqPieces == 4 && kFqBytesPerThread == 16, "a thread's masks are one 64-bit word");
+  const long long i = (long long)(c * kFqChunk + (u64)threadIdx.x * (kFqBytesPerThread * kFqPieces)) - head;
+  u64 m = reinterpret_cast<const u64*>(masks)[c * kFqThreads + threadIdx.x];
+  const unsigned cnt = __popcll(m);
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned incl = cnt;
 #pragma unroll
@@ -178,7 +187,7 @@ __global__ void __launch_bounds__(kFqThreads) fastq_lines_kernel(const unsigned 
   __syncthreads();
   u64 out = chunk_offsets[c] + warp_off[warp] + incl - cnt;
   for (; m; m &= m - 1) {
-    const u64 at = (u64)(i + __ffs(m) - 1);
+    const u64 at = (u64)(i + __ffsll((long long)m) - 1);
     line_end[out++] = at == n - 1 && text[at] != '\n' ? n : at;  // unterminated last line
   }
 }
@@ -249,7 +258,7 @@ __global__ void fastq_copy_kernel(const unsigned char* text, const u64* line_end
 // Chunks begin at a 16-byte boundary: `head` bytes before the text belong to the first one.
 static unsigned fastq_head(const unsigned char* text) { return (unsigned)(reinterpret_cast<uintptr_t>(text) & 15); }
 
-u64 fastq_masks(u64 n_bytes) { return fastq_chunks(n_bytes) * kFqThreads; }
+u64 fastq_masks(u64 n_bytes) { return fastq_chunks(n_bytes) * (kFqThreads * kFqPieces); }
 
 u64 fastq_chunks(u64 n_bytes) { return n_bytes ? (n_bytes + 15 + kFqChunk - 1) / kFqChunk : 0; }
 

@@ -172,7 +172,7 @@ def test_fastq_alignment(gpu, shift, final_newline):
     from paper_1705_11147_gb300 import parse_fastq
     for extra in range(0, 17, 2 if shift else 1):
         n = 40
-        lens = [0, 1, 7, 8, 9, 15, 16, 17, 127, 128, 129, 255 + extra] + [100 + i for i in range(n)]
+        lens = [0, 1, 7, 8, 9, 15, 16, 17, 127, 128, 129, 255 + extra] + [100 + i for i in range(n)] + [65_400 - 30 * extra]
         reads = [one_read(m, 1000 + m, "ACGTN") for m in lens]
         text = "".join(f"@r{i}\n{r}\n+\n{'I' * len(r)}\n" for i, r in enumerate(reads))
         text += "@last\nACGT\n+\nIIII" + ("\n" if final_newline else "")
