@@ -138,6 +138,21 @@ def test_table_of_ranges(gpu, k, partitions):
                     assert not ka.query(absent)[0].any()
 
 
+@pytest.mark.parametrize("partitions", [1, 6])
+def test_no_reads(gpu, partitions):
+    """A handle without a window, after one with some: an empty result and an empty table."""
+    from paper_1705_11147_gb300 import KmerAnalysis, make_params
+    rs = readset([one_read(500, 6)] * 2, k=31, min_depth=2, min_ext_count=1, qual_threshold=20)
+    keys = oracle_for(rs).keys
+    with KmerAnalysis(make_params(max_bases=rs.n_bases, max_reads=rs.n_reads, partitions=partitions, **rs.meta["params"])) as ka:
+        for some in (False, True, False):
+            ka.reset()
+            if some:
+                ka.count(rs.seq, rs.qual, rs.offsets)
+            assert ka.finalize().n == (len(keys) if some else 0)
+            assert ka.query(keys)[0].astype(bool).all() == some and ka.query(keys)[0].any() == some
+
+
 @pytest.mark.parametrize("n_parts", [2, 7])
 def test_batches_and_owners(gpu, n_parts):
     """Several count calls (slabs of scatter tiles) and the owner filter: the parts' records add up."""
