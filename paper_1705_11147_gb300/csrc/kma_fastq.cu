@@ -130,8 +130,8 @@ __device__ __forceinline__ unsigned newline_mask(const unsigned char* text, u64 
 }
 
 // Newlines in each chunk (plus one for a final line that does not end in '\n'), and their
-// masks, an eighth of the text, for the next pass (reading the text again took it 104 us of 516 for
-// 100 Mbases).
+// masks, an eighth of the text, for the next pass (reading the text again took it 104 us for 100
+// Mbases).
 __global__ void __launch_bounds__(kFqThreads) fastq_count_kernel(const unsigned char* text, u64 n, unsigned head,
                                                                  unsigned short* masks, u64* chunk_counts) {
   __shared__ unsigned warp_cnt[kFqThreads / 32];
