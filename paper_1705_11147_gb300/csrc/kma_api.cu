@@ -309,7 +309,7 @@ struct kma_handle {
 
   // partitioned mode: the scatter tiles of the count() calls, in slabs kept until finalize has
   // counted them, and the records per bucket
-  struct Slab { u64* recs; unsigned short* offs; u64 cap, used; double windows, positions; };
+  struct Slab { u64* recs; unsigned short* offs; u64 cap, used; double windows, positions, bases; };
   std::vector<Slab> slabs;
   u64* totals = nullptr;
 
@@ -570,7 +570,7 @@ int prepare_tiles(kma_handle* h, u64 tiles, cudaStream_t st) {
   const u64 left = tiles_for(h->d.plan.arena_positions - std::min<u64>(h->q_used, h->d.plan.arena_positions)) + 1;
   const u64 cap = std::max<u64>(tiles, std::min<u64>(left, 2048));
   if (cap >= (1ull << 31)) return KMA_EINVAL;  // tile numbers are 32-bit
-  kma_handle::Slab sl{nullptr, nullptr, cap, 0, 0.0, 0.0};
+  kma_handle::Slab sl{nullptr, nullptr, cap, 0, 0.0, 0.0, 0.0};
   cudaError_t e = cudaMallocFromPoolAsync((void**)&sl.recs, (size_t)cap * kPartTile * h->d.rec_bytes, h->pool, st);
   if (e == cudaSuccess)
     e = cudaMallocFromPoolAsync((void**)&sl.offs, (size_t)cap * (((u64)1 << h->d.log_b) + 8) * 2, h->pool, st);
@@ -594,6 +594,7 @@ int scatter_windows(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, 
   const PartTiles t = tiles_of(h, sl, sl.used);
   sl.used += tiles_for(n_pos);
   sl.positions += (double)n_pos;
+  sl.bases += (double)n_bases;
   const u64 k1 = h->p.k - 1;
   sl.windows += (n_bases > k1 * n_reads ? (double)(n_bases - k1 * n_reads) : 0.0) / std::max(1u, h->p.n_parts);
   return timed_launch(h, KMA_KERNEL_SCATTER, st, n_pos > 0,
@@ -661,7 +662,7 @@ template <typename F>
 int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sync, unsigned parts, F&& after) {
   const unsigned B = 1u << h->d.log_b;
   u64 bound = 0, n_chunks = 0;
-  double windows = 0, positions = 0;
+  double windows = 0, positions = 0, bases = 0;
   std::vector<unsigned> chunk_tiles;
   for (auto& sl : h->slabs) {
     const double least = 0.5 / std::max(1u, h->p.n_parts);  // against many reads shorter than k
@@ -673,6 +674,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     bound += sl.used * kPartTile;
     windows += sl.windows;
     positions += sl.positions;
+    bases += sl.bases;
   }
   if (n_chunks == 0) {
     const int rc = timed_launch(timed, KMA_KERNEL_INIT, st, true,
@@ -684,6 +686,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   std::vector<unsigned> ends;
   u64 most = bound;        // records of a group
   unsigned most_buckets = 0;
+  double counted = bases / std::max(1u, h->p.n_parts);  // windows there may be
   if (!may_sync || bound * h->d.rec_bytes <= kSplitAtOnce) {
     for (unsigned i = 0; i < parts; ++i) ends.push_back((unsigned)((u64)(B / kStep) * (i + 1) / parts) * kStep);
   } else {
@@ -692,6 +695,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     KMA_CUDA(cudaStreamSynchronize(st));
     u64 all = 0;
     for (u64 t : totals) all += t;
+    counted = (double)all;
     const u64 aim = std::max(kSplitAtOnce / h->d.rec_bytes, all / kSplitGroups);
     std::vector<u64> step(B / kStep, 0);  // records per step of buckets
     for (unsigned b = 0; b < B; ++b) step[b / kStep] += totals[b];
@@ -712,8 +716,11 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   std::memset(&s, 0, sizeof(s));
   PartGeom g = part_geom(h);
   const PartOut o = part_out(h);
-  // sub-buckets for the windows expected (one more than that for reads shorter than k)
-  g.sub_max = (unsigned)std::min<double>(g.sub_max, std::ceil(1.05 * windows / ((double)g.avg * B)) + 1.0);
+  // Room for the sub-buckets of the windows there may be (sub_buckets makes as many as there are
+  // windows for). Not of n_bases - (k - 1) * n_reads windows: reads shorter than k take from the
+  // others' there, and with too few sub-buckets all of them overflow (1 Mbp, 30x of 35 to 75 bases,
+  // k = 63: 3.80 ms instead of 0.48, 3.43 of them in part_large_kernel).
+  g.sub_max = (unsigned)std::min<double>(g.sub_max, std::ceil(1.05 * counted / ((double)g.avg * B)) + 1.0);
   const u64 n_subs = (u64)most_buckets * g.sub_max;
   const u64 n_segs = most / kPartSubTile + (u64)most_buckets * n_chunks + 1;
   if (n_chunks >= (1ull << 31) || n_segs >= (1ull << 32)) return KMA_EINVAL;

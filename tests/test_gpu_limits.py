@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import synth
-from test_gpu_parity import gpu, to_dev  # noqa: F401
+from test_gpu_parity import assert_same, gpu, to_dev  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +59,48 @@ def test_host_answers(gpu, stream):
                 want = [x.cpu().numpy() for x in ref.query(gpu.from_numpy(keys.view(np.int64)).cuda())]
                 for w, g in zip(want, host_query(ka, keys, fresh)):
                     np.testing.assert_array_equal(w.view(g.dtype), g, err_msg=f"{n} fresh={fresh}")
+
+
+def spent(ka, reads, what):
+    """Milliseconds in the counting kernels of one pass over the reads, the least of three."""
+    best = float("inf")
+    ka.set_profiling(True)
+    for _ in range(3):
+        ka.reset()
+        ka.timings(reset=True)
+        ka.count(*reads)
+        ka.finalize()
+        t = ka.timings(reset=True)
+        best = min(best, sum(t[f"ms_{w}"] for w in what))
+    return best
+
+
+@pytest.mark.parametrize("k", [31, 63])
+def test_reads_shorter_than_k(gpu, k):
+    """Short reads add no windows: with so many of them that n_bases - (k - 1) * n_reads is about 0,
+    the records are the long reads' own, and the sub-buckets are as many as for the long reads
+    alone (with one or two of them every record would be counted several times as slowly)."""
+    from paper_1705_11147_gb300 import KmerAnalysis, make_params
+    rng = np.random.default_rng(8)
+    genome = rng.integers(0, 4, 2_000_000).astype(np.uint8)
+    n, length, short = 20_000, 1000, 12
+    starts = rng.integers(0, len(genome) - length, n)
+    long = np.frombuffer(b"ACGT", np.uint8)[genome[starts[:, None] + np.arange(length)]]
+    m = n * (length - k + 1) // (k - 1 - short) // n * n
+    each = m // n  # short reads behind every long one
+    row = np.concatenate([long, np.full((n, each * short), ord("C"), np.uint8)], axis=1)
+    lens = np.tile(np.array([length] + [short] * each), n)
+    p = dict(k=k, min_depth=2, min_ext_count=2, qual_threshold=20, partitions=4, expected_distinct=5_000_000, expected_keys=2_500_000,
+             max_bases=row.size, max_reads=len(lens))
+    sets = [(row.reshape(-1), lens), (long.reshape(-1), np.full(n, length))]
+    got, ms = [], []
+    for seq, ln in sets:
+        offs = np.concatenate([[0], np.cumsum(ln)]).astype(np.int64)
+        reads = (gpu.from_numpy(seq.copy()).cuda(), gpu.full((seq.size,), 70, dtype=gpu.uint8, device="cuda"), gpu.from_numpy(offs).cuda())
+        assert seq.size <= p["max_bases"]
+        with KmerAnalysis(make_params(**p)) as ka:
+            ms.append(spent(ka, reads, ("pass", "recount")))
+            got.append(ka.copy_result().sorted())
+    assert_same(*got)
+    assert len(got[0]) > 1_000_000
+    assert ms[0] < 2.5 * ms[1], ms
