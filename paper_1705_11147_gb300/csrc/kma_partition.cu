@@ -798,12 +798,15 @@ __global__ void __launch_bounds__(kLargeThreads, 2) part_large_kernel(const __gr
         row(x0 + lane < n_in, r, hi);
       }
       // the sub-bucket's records in the segments: each lane searches one segment, which is ordered by
-      // sub-bucket, for the first of them
-      for (unsigned g0 = warp * 32; g0 < n_segs; g0 += kLargeThreads) {
+      // sub-bucket, for the first of them. Neighbouring segments go to different warps: a bucket of a
+      // small sample has a few of them, which one warp alone took one after another (4 Mbases,
+      // 30 % of them a satellite's: 203 us -> 54 us)
+      for (unsigned g0 = 0; g0 < n_segs; g0 += kLargeThreads) {
+        const unsigned g = g0 + lane * (kLargeThreads / 32) + warp;
         PartSegment sg = {0, 0, 0};
         unsigned from = 0;
-        if (g0 + lane < n_segs) {
-          sg = segs[g0 + lane];
+        if (g < n_segs) {
+          sg = segs[g];
           unsigned end = sg.n;
           while (from < end) {
             const unsigned mid = (from + end) / 2;

@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 import synth
-from test_gpu_parity import assert_same, gpu, to_dev  # noqa: F401
+from test_gpu_parity import assert_same, gpu, oracle_for, run_gpu, to_dev  # noqa: F401
 
 pytestmark = pytest.mark.gpu
 
@@ -104,3 +104,41 @@ def test_reads_shorter_than_k(gpu, k):
     assert_same(*got)
     assert len(got[0]) > 1_000_000
     assert ms[0] < 2.5 * ms[1], ms
+
+
+def hot_reads(n, unit, other, seed):
+    """n reads of 150 bases, every third from a tandem array of one 171-base unit, the others random."""
+    rng = np.random.default_rng(seed)
+    array = np.tile(rng.integers(0, 4, unit).astype(np.uint8), 3)
+    genome = rng.integers(0, 4, other).astype(np.uint8)
+    hot = np.arange(n) % 3 == 0
+    at = np.where(hot, rng.integers(0, unit, n), rng.integers(0, other - 150, n))[:, None] + np.arange(150)
+    codes = np.where(hot[:, None], array[np.minimum(at, len(array) - 1)], genome[at])
+    return readset_of(np.frombuffer(b"ACGT", np.uint8)[codes].reshape(-1), np.arange(n + 1) * 150)
+
+
+def readset_of(seq, offsets, **params):
+    return synth.ReadSet(seq.copy(), np.full(len(seq), 70, np.uint8), offsets.astype(np.uint64), {"params": params})
+
+
+@pytest.mark.parametrize("n", [2_000, 9_000, 30_000, 120_000])
+@pytest.mark.parametrize("k", [31, 63])
+def test_hot_keys_of_small_samples(gpu, n, k):
+    """Hot k-mers in few segments, in as many as there are warps, and in more, against the oracle."""
+    rs = hot_reads(n, 171, 20_000, n)
+    for depth, bloom in ((1, False), (2, True)):
+        rs.meta["params"] = dict(k=k, min_depth=depth, min_ext_count=2, qual_threshold=20)
+        assert_same(run_gpu(gpu, rs, use_bloom=bloom, partitions=3), oracle_for(rs), f"depth {depth}")
+
+
+def test_hot_keys_use_all_warps(gpu):
+    """A third of a small sample's windows from 171 k-mers: counted in less than three times the time of
+    as many windows without them (a single warp for a bucket's few segments: five times)."""
+    from paper_1705_11147_gb300 import KmerAnalysis, make_params
+    ms = []
+    for unit in (171, 60_000):
+        rs = hot_reads(40_000, unit, 120_000, 3)
+        with KmerAnalysis(make_params(k=31, min_depth=2, partitions=2, max_bases=rs.n_bases, max_reads=rs.n_reads,
+                                      expected_distinct=500_000)) as ka:
+            ms.append(spent(ka, to_dev(gpu, rs), ("pass",)))
+    assert ms[0] < 3 * ms[1], ms
