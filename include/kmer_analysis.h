@@ -100,9 +100,10 @@ typedef struct {
                                  one GPU): windows are written as records, sorted by hash until
                                  all occurrences of a k-mer lie in one small sub-bucket, and
                                  counted there in shared memory; the table is laid out in P
-                                 parts of the same hash. 0: automatic (P >= 2 when filter + table
-                                 exceed 32 MB, at most 64 MB per part); 1: one table, windows
-                                 counted in place; P >= 2: that many parts (<= 4096 for
+                                 parts of the same hash. 0: automatic (P >= 2, at most 64 MB per
+                                 part, when filter + table exceed 32 MB and max_bases 1.2 M, 4 M
+                                 without use_bloom, or filter + table reach 512 MB); 1: one
+                                 table, windows counted in place; P >= 2: that many parts (<= 4096 for
                                  k <= 32, <= 2048 for k > 32; more: KMA_EINVAL). Results
                                  do not depend on it. */
   uint32_t heavy_hitters;     /* 1: k-mers with very many occurrences (satellites, low-complexity

@@ -116,7 +116,18 @@ constexpr double kSubBucketFill = 0.72;
 constexpr u64 kSplitAtOnce = 2ull << 30;
 constexpr u64 kSplitGroups = 12;
 
-constexpr u64 kAutoPartitionAbove = 32ull << 20;   // partitioned above: filter + table bytes
+// Partitioned above these: filter + table bytes, and bases the kernels have to count; a table so
+// large that clearing and scanning it (one table) costs more than the seven kernels of the sorts
+// always. One table against partitions, us from reads to answers, 30x of 150 bases:
+//   with the singleton filter, 64 MB, k = 25: 0.6 Mbases 144 / 161, 1.2 174 / 172, 2.5 233 / 194, 10 655 / 341
+//     (k = 51: 142 / 173, 167 / 180, 218 / 205, 618 / 346)
+//   every k-mer: 1.2 Mbases, 64 MB 166 / 187, 2.5 Mbases, 128 MB 209 / 234 (with hot k-mers 206 / 301);
+//     10 Mbases, 512 MB 840 / 501 (787 / 550)
+//   512 MB: 0.3 Mbases 272 / 294, 0.6 292 / 236; every k-mer 268 / 334, 290 / 289, 1.2 316 / 266
+constexpr u64 kAutoPartitionAbove = 32ull << 20;
+constexpr u64 kAutoPartitionBases = 1200000;
+constexpr u64 kAutoPartitionBasesAll = 4000000;  // every k-mer goes into the table
+constexpr u64 kAutoPartitionAlways = 512ull << 20;
 constexpr u64 kPartitionTarget = 64ull << 20;      // filter + table bytes per partition
 
 int check_params(const kma_params* p) {
@@ -164,7 +175,11 @@ int derive(const kma_params* p, Derived& d) {
     const u64 W = d.plan.bloom_words, S = d.plan.table_slots;
     const u64 bytes = W * 8 + S * sizeof(Slot);
     u64 P = p->partitions;
-    if (P == 0) P = bytes > kAutoPartitionAbove ? std::max<u64>(2, (bytes + kPartitionTarget - 1) / kPartitionTarget) : 1;
+    if (P == 0) {
+      const bool large = p->max_bases >= (p->use_bloom ? kAutoPartitionBases : kAutoPartitionBasesAll);
+      const bool split = bytes > kAutoPartitionAbove && (large || bytes >= kAutoPartitionAlways);
+      P = split ? std::max<u64>(2, (bytes + kPartitionTarget - 1) / kPartitionTarget) : 1;
+    }
     const u64 max_parts = p->k > 32 ? kMaxPartitionsWide : kMaxPartitions;
     if (P > max_parts) P = max_parts;
     if (P < 1) P = 1;
