@@ -142,3 +142,38 @@ def test_hot_keys_use_all_warps(gpu):
                                       expected_distinct=500_000)) as ka:
             ms.append(spent(ka, to_dev(gpu, rs), ("pass",)))
     assert ms[0] < 3 * ms[1], ms
+
+
+def test_finalize_after_graphs(gpu):
+    """Every batch graph that has been in the process makes allocations from the library's pool on a
+    busy stream slower: a pass of another handle takes as long as before them, but for one such
+    allocation (with ten it took 35 us longer for each graph)."""
+    import time
+    from paper_1705_11147_gb300 import BatchGraph, KmerAnalysis, make_params
+    rs = synth.workload("plain_1m", scale=0.3)
+    reads = to_dev(gpu, rs)
+    kw = dict(k=33, min_depth=2, max_bases=rs.n_bases, max_reads=rs.n_reads, expected_distinct=4_000_000, partitions=4)
+
+    def passes():
+        with KmerAnalysis(make_params(**kw)) as a, KmerAnalysis(make_params(**kw)) as b, KmerAnalysis(make_params(**kw)) as c:
+            us = []
+            for i in range(60):
+                ka = (a, b, c)[i % 3]
+                t = time.perf_counter()
+                ka.reset()
+                ka.count(*reads)
+                ka.finalize()
+                us.append((time.perf_counter() - t) * 1e6)
+            return float(np.median(us[20:]))
+
+    before = passes()
+    small = [synth.workload("plain_1m", scale=0.05 * (1 + i % 4)) for i in range(12)]
+    for _ in range(8):
+        handles = [KmerAnalysis(make_params(k=31, min_depth=2, max_bases=s.n_bases, max_reads=s.n_reads, partitions=4,
+                                            expected_distinct=s.n_bases // 4, expected_keys=s.n_bases // 10)) for s in small]
+        graph = BatchGraph(handles, [to_dev(gpu, s) for s in small])
+        graph.replay()
+        assert all(int(r.n) > 0 for r in graph.results())
+        del handles, graph
+    after = passes()
+    assert after - before < 120, (before, after)
