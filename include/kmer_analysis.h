@@ -123,7 +123,10 @@ typedef struct {
   uint64_t table_slots;    /* hash-table slots, 64 bytes each */
   uint64_t arena_positions;/* packed positions: bases + one separator per read + padding */
   uint64_t device_bytes;   /* device memory a handle holds (all buffers; with partitions,
-                              including per-window records for max_bases windows) */
+                              including per-window records for max_bases windows and the
+                              temporaries of a finalize that counts 256 MB of them at a time:
+                              while there is memory it takes 2 GB, and in a graph, where it
+                              cannot ask, room for all of them once more) */
 } kma_plan;
 
 /* Result of finalize. Pointers are device memory owned by the handle, valid until the

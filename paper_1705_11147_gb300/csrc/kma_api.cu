@@ -112,9 +112,16 @@ struct Derived {
 // their sizes: at 30x coverage one in a thousand overflows.
 constexpr double kSubBucketFill = 0.72;
 // The sorted copy of the records made by the split: as large as all of them below this size, one
-// launch; above it the buckets are split and counted in groups that share a smaller copy.
+// launch; above it the buckets are split and counted in groups that share a smaller copy. Smaller
+// groups leave the GPU idle at each one's end (2 GiB, 1 GiB, 256 MiB: 250 Mbases, k = 51 5.41,
+// 5.47, 5.98 ms; 140 Mbases, 30 % of them a satellite's, 10.9, 11.7, 17.3 ms; 12 and 24 groups of 3
+// Gbases 78.0 and 78.9 ms), so they are taken only where there is no memory for more. A handle is
+// planned with the second pair.
 constexpr u64 kSplitAtOnce = 2ull << 30;
 constexpr u64 kSplitGroups = 12;
+constexpr u64 kSplitPlanned = 256ull << 20;
+constexpr u64 kSplitGroupsPlanned = 48;
+constexpr u64 kSplitLeast = 16ull << 20;
 
 // Partitioned above these: filter + table bytes, and bases the kernels have to count; a table so
 // large that clearing and scanning it (one table) costs more than the seven kernels of the sorts
@@ -215,12 +222,16 @@ int derive(const kma_params* p, Derived& d) {
   d.plan.device_bytes = 2 * d.codes_words * 8 + 2 * d.bit_words * 8 + d.mark_words * 4 +
                         (d.P > 1 ? 0 : d.plan.bloom_words * 8) + d.plan.table_slots * sizeof(Slot) +
                         sizeof(DevStatus) + 2 * (2 * d.staging + (d.staging / 16 + 2) * 8);
-  if (d.P > 1) {  // scatter tiles with their offset rows, and the split's sorted copy
-    const u64 tiles = pos / kPartTile + 1, recs = tiles * kPartTile * d.rec_bytes;
-    const u64 copy = recs <= kSplitAtOnce ? recs : std::max(kSplitAtOnce, recs / kSplitGroups);
-    // sub-buckets, overflow segments, and the listed keys: all records may be one (a half, of two each)
-    const double keys = (p->use_bloom ? 0.5 : 1.0) * (d.rec_bytes == 8 ? 4.0 : 2.5);
-    d.plan.device_bytes += recs + tiles * (((u64)1 << d.log_b) + 8) * 2 + (u64)((2.5 + keys) * (double)copy);
+  if (d.P > 1) {  // scatter tiles with their offset rows, and count_records' temporaries
+    const u64 tiles = pos / kPartTile + 1;
+    d.plan.device_bytes += tiles * (kPartTile * d.rec_bytes + (((u64)1 << d.log_b) + 8) * 2);
+    const double windows = (double)p->max_bases, all = windows * d.rec_bytes;  // any of them may be counted
+    const double group = all <= (double)kSplitPlanned ? 1.0 : std::max((double)kSplitPlanned / all, 1.0 / kSplitGroupsPlanned);
+    const double most = group * windows, subs = (most / d.avg + (1 << d.log_b)) * 1.05;
+    const double slots = group * (double)d.plan.table_slots + 2 * kMaxProbe;
+    d.plan.device_bytes += (u64)(subs * ((double)(p->k > 32 ? kCountCap2 : kCountCap1) * d.rec_bytes + 24) + most * d.rec_bytes +
+                                 std::min(most / (p->use_bloom ? 2 : 1), slots) * (d.rec_bytes == 8 ? 32 : 40) +
+                                 2 * kMaxProbe * kCarryWords * 4);
   }
   return KMA_OK;
 }
@@ -670,9 +681,11 @@ unsigned lanes_for(double len) {
 
 // Partitioned mode: counts the handle's records into its table and output records on stream `st`,
 // the buckets in order, `parts` groups of them or more, and calls after(end) when the buckets
-// below `end` have been enqueued. The sorted copy of the split is sized for all records when they are few or
-// when the call may not wait for the GPU (may_sync = false, capture); otherwise from the bucket
-// totals, a twelfth of the records or the largest bucket.
+// below `end` have been enqueued. The groups share the sorted copy of the split: all records at once when
+// they are few, otherwise from the bucket totals, a twelfth of the records or the largest bucket;
+// smaller ones when there is no memory for that. When the call may not wait for the GPU (may_sync
+// = false, capture) the groups are a twelfth of the buckets, and only the room for records without
+// a place in their sub-bucket is for all (any bucket may hold them).
 template <typename F>
 int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sync, unsigned parts, F&& after) {
   const unsigned B = 1u << h->d.log_b;
@@ -686,7 +699,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     const double c = 0.85 * kPartSubTile * B / (kPartTile * occ);
     chunk_tiles.push_back((unsigned)std::min<double>(std::max(1.0, std::floor(c)), kMaxChunkTiles));
     n_chunks += (sl.used + chunk_tiles.back() - 1) / chunk_tiles.back();
-    bound += sl.used * kPartTile;
+    bound += std::min<u64>(sl.used * kPartTile, (u64)sl.bases);
     windows += sl.windows;
     positions += sl.positions;
     bases += sl.bases;
@@ -697,74 +710,94 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     return rc ? rc : after(B);
   }
   constexpr unsigned kStep = kSplitBuckets;  // groups are whole work items of the split
+  if (!may_sync && bound * h->d.rec_bytes > kSplitAtOnce) parts = std::max<unsigned>(parts, kSplitGroups);
   parts = std::min(parts, B / kStep);
-  std::vector<unsigned> ends;
-  u64 most = bound;        // records of a group
-  unsigned most_buckets = 0;
   double counted = bases / std::max(1u, h->p.n_parts);  // windows there may be
-  if (!may_sync || bound * h->d.rec_bytes <= kSplitAtOnce) {
-    for (unsigned i = 0; i < parts; ++i) ends.push_back((unsigned)((u64)(B / kStep) * (i + 1) / parts) * kStep);
-  } else {
-    std::vector<u64> totals(B);
-    KMA_CUDA(cudaMemcpyAsync(totals.data(), h->totals, B * sizeof(u64), cudaMemcpyDeviceToHost, st));
-    KMA_CUDA(cudaStreamSynchronize(st));
-    u64 all = 0;
-    for (u64 t : totals) all += t;
-    counted = (double)all;
-    const u64 aim = std::max(kSplitAtOnce / h->d.rec_bytes, all / kSplitGroups);
-    std::vector<u64> step(B / kStep, 0);  // records per step of buckets
-    for (unsigned b = 0; b < B; ++b) step[b / kStep] += totals[b];
-    const unsigned widest = (B / kStep + parts - 1) / parts;
-    most = 0;
-    for (unsigned b = 0; b < B / kStep;) {
-      unsigned e = b;
-      u64 sum = 0;
-      do sum += step[e++];
-      while (e < B / kStep && e - b < widest && sum + step[e] <= aim);
-      ends.push_back(e * kStep);
-      most = std::max(most, sum);
-      b = e;
-    }
-  }
-  for (size_t i = 0; i < ends.size(); ++i) most_buckets = std::max(most_buckets, ends[i] - (i ? ends[i - 1] : 0));
   PartSplit s;
   std::memset(&s, 0, sizeof(s));
   PartGeom g = part_geom(h);
   const PartOut o = part_out(h);
-  // Room for the sub-buckets of the windows there may be (sub_buckets makes as many as there are
-  // windows for). Not of n_bases - (k - 1) * n_reads windows: reads shorter than k take from the
-  // others' there, and with too few sub-buckets all of them overflow (1 Mbp, 30x of 35 to 75 bases,
-  // k = 63: 3.80 ms instead of 0.48, 3.43 of them in part_large_kernel).
-  g.sub_max = (unsigned)std::min<double>(g.sub_max, std::ceil(1.05 * counted / ((double)g.avg * B)) + 1.0);
-  const u64 n_subs = (u64)most_buckets * g.sub_max;
-  const u64 n_segs = most / kPartSubTile + (u64)most_buckets * n_chunks + 1;
-  if (n_chunks >= (1ull << 31) || n_segs >= (1ull << 32)) return KMA_EINVAL;
+  // first slot of the hashes of bucket b (part_of, table_index)
+  auto first_slot = [&](unsigned b) -> u64 {
+    const u64 top = (u64)b << (32 - h->d.log_b);
+    return b < B ? (top * g.P >> 32) * g.Sp + ((top * g.P & 0xFFFFFFFFull) * g.Sp >> 32) : (u64)g.P * g.Sp;
+  };
   // Temporaries, in one allocation. While the stream is busy an allocation from the pool takes the
   // host 1 us, and 3.5 us more for every other stream that the pool's free memory was used on
   // (ten of them, after eight batch graphs on streams of their own: 0.72 -> 0.90 ms for 12 Mbases).
-  u64 block_bytes = 0;
-  auto room = [&](u64 bytes) -> u64 {
-    const u64 at = block_bytes;
-    block_bytes += (bytes + 255) & ~255ull;
-    return at;
-  };
-  // [sub-buckets], overflow records, list entries, large sub-buckets, those taken, CTAs done,
-  // then segments per bucket and keys per sub-bucket (32 bits)
-  const u64 n_zero = n_subs + 5 + (most_buckets + n_subs + 1) / 2;
-  const unsigned key_words = kMaxKeyWords - (h->d.rec_bytes == 8 ? 2 : 0);
-  const u64 n_keys = most / (h->p.use_bloom ? 2 : 1) + 1;
-  const u64 at_recs = room(n_subs * g.cap * h->d.rec_bytes), at_over = room(most * h->d.rec_bytes);
-  const u64 at_keys = room(n_keys * key_words * 4), at_zero = room(n_zero * 8), at_large = room(n_subs * sizeof(unsigned));
-  const u64 at_base = room(n_subs * 8), at_n_carry = room(2 * 8);
-  const u64 at_carry = room(2 * (u64)kMaxProbe * kCarryWords * 4);  // two lists, taken in turn
-  const u64 at_segs = room(n_segs * sizeof(PartSegment)), at_seg_base = room(most_buckets * sizeof(unsigned));
+  std::vector<u64> totals;     // records per bucket
+  std::vector<unsigned> ends;  // of the groups
+  unsigned most_buckets = 0;   // of a group
+  u64 n_subs = 0, n_zero = 0, n_keys = 0, block_bytes = 0;
+  u64 at_recs, at_over, at_keys, at_zero, at_large, at_base, at_n_carry, at_carry, at_segs, at_seg_base;
   unsigned char* block = nullptr;
-  {
-    const cudaError_t e = cudaMallocFromPoolAsync((void**)&block, block_bytes, h->pool, st);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return e == cudaErrorMemoryAllocation ? KMA_ENOMEM : cuda_fail(e, "split output");
+  for (u64 at_once = kSplitAtOnce, at_most = kSplitGroups;; at_once /= 2, at_most *= 2) {
+    u64 most = bound, most_slots = 0;  // records and table slots of a group
+    ends.clear();
+    if (!may_sync || bound * h->d.rec_bytes <= at_once) {
+      for (unsigned i = 0; i < parts; ++i) ends.push_back((unsigned)((u64)(B / kStep) * (i + 1) / parts) * kStep);
+    } else {
+      if (totals.empty()) {
+        totals.resize(B);
+        KMA_CUDA(cudaMemcpyAsync(totals.data(), h->totals, B * sizeof(u64), cudaMemcpyDeviceToHost, st));
+        KMA_CUDA(cudaStreamSynchronize(st));
+      }
+      u64 all = 0;
+      for (u64 t : totals) all += t;
+      counted = (double)all;
+      const u64 aim = std::max(at_once / h->d.rec_bytes, all / at_most);
+      std::vector<u64> step(B / kStep, 0);  // records per step of buckets
+      for (unsigned b = 0; b < B; ++b) step[b / kStep] += totals[b];
+      const unsigned widest = (B / kStep + parts - 1) / parts;
+      most = 0;
+      for (unsigned b = 0; b < B / kStep;) {
+        unsigned e = b;
+        u64 sum = 0;
+        do sum += step[e++];
+        while (e < B / kStep && e - b < widest && sum + step[e] <= aim);
+        ends.push_back(e * kStep);
+        most = std::max(most, sum);
+        b = e;
+      }
     }
+    most_buckets = 0;
+    for (size_t i = 0; i < ends.size(); ++i) {
+      const unsigned b0 = i ? ends[i - 1] : 0;
+      most_buckets = std::max(most_buckets, ends[i] - b0);
+      most_slots = std::max(most_slots, first_slot(ends[i]) - first_slot(b0));
+    }
+    // Room for the sub-buckets of the windows there may be (sub_buckets makes as many as there are
+    // windows for). Not of n_bases - (k - 1) * n_reads windows: reads shorter than k take from the
+    // others' there, and with too few sub-buckets all of them overflow (1 Mbp, 30x of 35 to 75 bases,
+    // k = 63: 3.80 ms instead of 0.48, 3.43 of them in part_large_kernel).
+    g.sub_max = (unsigned)std::min<double>(h->d.sub_max, std::ceil(1.05 * counted / ((double)g.avg * B)) + 1.0);
+    n_subs = (u64)most_buckets * g.sub_max;
+    const u64 n_segs = most / kPartSubTile + (u64)most_buckets * n_chunks + 1;
+    if (n_chunks >= (1ull << 31) || n_segs >= (1ull << 32)) return KMA_EINVAL;
+    // [sub-buckets], overflow records, list entries, large sub-buckets, those taken, CTAs done,
+    // then segments per bucket and keys per sub-bucket (32 bits)
+    n_zero = n_subs + 5 + (most_buckets + n_subs + 1) / 2;
+    const unsigned key_words = kMaxKeyWords - (h->d.rec_bytes == 8 ? 2 : 0);
+    // The keys of a group go to its slots, or kMaxProbe further on, or (round the end of a partition
+    // that began before it) to the first kMaxProbe of that: with more of them the table is full.
+    n_keys = std::min<u64>(most / (h->p.use_bloom ? 2 : 1), most_slots + 2 * kMaxProbe) + 1;
+    block_bytes = 0;
+    auto room = [&](u64 bytes) -> u64 {
+      const u64 at = block_bytes;
+      block_bytes += (bytes + 255) & ~255ull;
+      return at;
+    };
+    at_recs = room(n_subs * g.cap * h->d.rec_bytes), at_over = room(most * h->d.rec_bytes);
+    at_keys = room(n_keys * key_words * 4), at_zero = room(n_zero * 8), at_large = room(n_subs * sizeof(unsigned));
+    at_base = room(n_subs * 8), at_n_carry = room(2 * 8);
+    at_carry = room(2 * (u64)kMaxProbe * kCarryWords * 4);  // two lists, taken in turn
+    at_segs = room(n_segs * sizeof(PartSegment)), at_seg_base = room(most_buckets * sizeof(unsigned));
+    const cudaError_t e = cudaMallocFromPoolAsync((void**)&block, block_bytes, h->pool, st);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "split output");
+    if (!may_sync || at_once <= kSplitLeast) return KMA_ENOMEM;
+    KMA_CUDA(cudaStreamSynchronize(st));  // what has been freed on it is there for the next attempt
   }
   auto run = [&]() -> int {
     int rc;
@@ -786,6 +819,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     s.inserted = zero + n_subs + 4;
     s.n_segs = reinterpret_cast<unsigned*>(zero + n_subs + 5);
     s.key_n = s.n_segs + most_buckets;
+    s.keys_cap = n_keys;
     s.n_chunks = (unsigned)n_chunks;
     KMA_CUDA(cudaMemsetAsync(n_carry, 0, 2 * 8, st));
     const double occ = std::min(1.0, std::max(0.3, positions > 0 ? windows / positions : 1.0));
@@ -794,9 +828,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
       s.b0 = i ? ends[i - 1] : 0;
       s.b1 = ends[i];
       KMA_CUDA(cudaMemsetAsync(zero, 0, n_zero * 8, st));
-      // the group's slots end where the hashes of bucket b1 begin (part_of, table_index)
-      const u64 top = s.b1 < B ? (u64)s.b1 << (32 - h->d.log_b) : 0;
-      s.end = s.b1 < B ? (top * g.P >> 32) * g.Sp + ((top * g.P & 0xFFFFFFFFull) * g.Sp >> 32) : (u64)g.P * g.Sp;
+      s.end = first_slot(s.b1);  // the group's slots end there
       s.carry_in = carry + (i & 1) * (u64)kMaxProbe * kCarryWords;
       s.carry_out = carry + ((i + 1) & 1) * (u64)kMaxProbe * kCarryWords;
       s.n_carry_in = n_carry + (i & 1);

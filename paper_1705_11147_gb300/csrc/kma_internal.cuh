@@ -228,6 +228,7 @@ struct PartSplit {
   unsigned int pad;
   unsigned int* keys;           // count: the counted keys for the table (kma_partition.cu)
   unsigned long long* n_keys;   // their number; starts at 0
+  unsigned long long keys_cap;  // most that the table can take; the list has room for them
   unsigned int* large;          // [sub-buckets] count: those left to part_large_kernel
   unsigned long long* n_large;  // their number, and how many have been taken; start at 0
   unsigned long long* next_large;

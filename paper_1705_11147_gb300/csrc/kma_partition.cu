@@ -1070,8 +1070,12 @@ __global__ void __launch_bounds__(kCountThreads, kCountCtas) part_count_kernel(c
     // 4: outcomes
     if (tid == 0) s_nlist = 0;
     if (tid == 0) {
-      const unsigned nk = s_nctr + s_nlone;
+      unsigned nk = s_nctr + s_nlone;
       s_base = nk ? atomicAdd(S.n_keys, (u64)nk) : 0;
+      if (s_base + nk > S.keys_cap) {  // more keys than slots
+        atomicOr(&G.status->flags, kFlagFull);
+        nk = s_nctr = s_nlone = 0;
+      }
       S.key_base[item] = s_base;
       S.key_n[item] = nk;
     }
@@ -1270,7 +1274,7 @@ __global__ void __launch_bounds__(kInsertThreads) part_insert_kernel(const __gri
                                                                      const __grid_constant__ PartOut O) {
   __shared__ unsigned s_wsum[32];
   __shared__ u64 s_base;
-  const u64 n = __ldcg(S.n_keys);
+  const u64 listed = __ldcg(S.n_keys), n = listed < S.keys_cap ? listed : S.keys_cap;  // more: the table is full
   const unsigned* keys = S.keys;
   unsigned acc_ins = 0, acc_uu = 0;
   // the keys carried over from the groups before

@@ -177,3 +177,139 @@ def test_finalize_after_graphs(gpu):
         del handles, graph
     after = passes()
     assert after - before < 120, (before, after)
+
+
+def device_reads(gpu, n, length, unit, other, seed, quality=70):
+    """n reads of `length` bases on the device: every third from a tandem array of one `unit`, the others
+    from a random genome of `other` bases."""
+    g = gpu.Generator(device="cuda").manual_seed(seed)
+    codes = gpu.randint(0, 4, (other,), generator=g, device="cuda", dtype=gpu.uint8)
+    array = gpu.randint(0, 4, (unit,), generator=g, device="cuda", dtype=gpu.uint8).repeat(length // unit + 2)
+    letters = gpu.tensor(list(b"ACGT"), dtype=gpu.uint8, device="cuda")
+    seq = gpu.empty((n, length), dtype=gpu.uint8, device="cuda")
+    span = gpu.arange(length, device="cuda")
+    for a in range(0, n, 200_000):
+        b = min(n, a + 200_000)
+        at = gpu.randint(0, other - length, (b - a,), generator=g, device="cuda")
+        hot = gpu.arange(a, b, device="cuda") % 3 == 0
+        row = codes[at[:, None] + span]
+        row[hot] = array[(at[hot] % unit)[:, None] + span]
+        seq[a:b] = letters[row.long()]
+    offsets = gpu.arange(n + 1, device="cuda") * length
+    return seq.view(-1), gpu.full((n * length,), quality, dtype=gpu.uint8, device="cuda"), offsets
+
+
+def same_result(gpu, a, b):
+    """Two finalized handles hold the same records (in any order)."""
+    got = []
+    for ka in (a, b):
+        keys, counts, ext, codes = ka.copy_result_device()
+        order = gpu.argsort(keys[:, 0], stable=True)
+        order = order[gpu.argsort(keys[order, 1], stable=True)]
+        got.append([x[order] for x in (keys, counts, ext, codes)])
+    for x, y in zip(*got):
+        assert gpu.equal(x, y)
+    assert int(a.result_info.n_uu) == int(b.result_info.n_uu)
+    assert int(a.result_info.valid_windows) == int(b.result_info.valid_windows)
+
+
+@pytest.mark.parametrize("bloom", [True, False])
+def test_groups_of_buckets(gpu, bloom):
+    """More than 2 GiB of records, hot k-mers among them: counted in groups of buckets, by finalize (sizes
+    from the bucket totals), by finalize_to_host and in a graph (groups of a fixed number of
+    buckets), as in one table; and with no valid window at all."""
+    from paper_1705_11147_gb300 import BatchGraph, KmerAnalysis, host_result_buffers, make_params
+    reads = device_reads(gpu, 950_000, 150, 171, 1_500_000, 5)
+    kw = dict(k=51, min_depth=2 if bloom else 1, use_bloom=bloom, max_bases=reads[0].numel(), max_reads=950_000, expected_distinct=4_000_000,
+              expected_keys=3_000_000)
+    assert reads[0].numel() * 16 > 2 << 30
+    with KmerAnalysis(make_params(**kw, partitions=1)) as one, KmerAnalysis(make_params(**kw, partitions=8)) as ka:
+        one.count(*reads)
+        one.finalize()
+        assert int(one.result_info.n) > 1_400_000
+        ka.count(*reads)
+        ka.finalize()
+        same_result(gpu, one, ka)
+        ka.reset()
+        ka.count(*reads)
+        res = ka.finalize_to_host(host_result_buffers(4_000_000, pinned=True)).sorted()
+        np.testing.assert_array_equal(res.keys, one.copy_result().sorted().keys)
+        same_result(gpu, one, ka)
+        graph = BatchGraph([ka], [reads])
+        graph.replay()
+        graph.results()
+        same_result(gpu, one, ka)
+        del graph
+        ka.set_stream(gpu.cuda.current_stream())
+        ka.reset()
+        none = gpu.full_like(reads[0], ord("N"))
+        ka.count(none, reads[1], reads[2])
+        assert int(ka.finalize().n) == 0 and int(ka.result_info.valid_windows) == 0
+        assert not ka.query(one.copy_result_device()[0])[0].any()
+
+
+@pytest.mark.parametrize("k,bloom", [(31, True), (51, True), (51, False)])
+def test_more_keys_than_slots(gpu, k, bloom):
+    """A table with fewer slots than keys: KMA_EFULL, and the handle counts again after reset."""
+    from paper_1705_11147_gb300 import KmerAnalysis, capi, make_params
+    reads = device_reads(gpu, 40_000, 150, 171, 2_000_000, 6)
+    few = device_reads(gpu, 300, 150, 171, 1_000, 7)
+    kw = dict(k=k, min_depth=2 if bloom else 1, use_bloom=bloom, max_bases=reads[0].numel(), max_reads=40_000, expected_distinct=2_000_000)
+    for slots in (50_000, 200_000):
+        with KmerAnalysis(make_params(**kw, partitions=4, table_capacity=slots)) as ka, KmerAnalysis(make_params(**kw, partitions=1)) as one:
+            ka.count(*reads)
+            with pytest.raises(capi.KmaError) as e:
+                ka.finalize()
+            assert e.value.code == capi.KMA_EFULL
+            for h in (ka, one):
+                h.reset()
+                h.count(*few)
+                h.finalize()
+            same_result(gpu, one, ka)
+
+
+LITTLE_MEMORY = """
+import sys
+import torch as gpu
+from test_gpu_limits import device_reads, same_result
+from paper_1705_11147_gb300 import BatchGraph, KmerAnalysis, host_result_buffers, make_params
+k, keys, leave, host = (int(x) for x in sys.argv[1:])
+reads = device_reads(gpu, 600_000, 150, 171, 1_500_000, 5)
+kw = dict(k=k, min_depth=2, max_bases=reads[0].numel(), max_reads=600_000, expected_distinct=4_000_000)
+ka = KmerAnalysis(make_params(**kw, expected_keys=keys, partitions=8))
+one = KmerAnalysis(make_params(**kw, expected_keys=3_000_000, partitions=1))
+one.count(*reads)
+one.finalize()
+ka.count(*reads)
+gpu.cuda.synchronize()
+gpu.cuda.empty_cache()
+free = gpu.cuda.mem_get_info()[0]
+held = gpu.empty(free - (leave << 20), dtype=gpu.uint8, device="cuda")
+if host:
+    n = ka.finalize_to_host(host_result_buffers(4_000_000, pinned=True))
+else:
+    n = ka.finalize()
+del held
+gpu.cuda.empty_cache()
+same_result(gpu, one, ka)
+if host:
+    w, g = one.copy_result().sorted(), n.sorted()
+    assert (w.keys == g.keys).all() and (w.counts == g.counts).all() and (w.ext == g.ext).all() and (w.codes == g.codes).all()
+print("same")
+"""
+
+
+def little_memory(*args):
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    env = dict(os.environ, PYTHONPATH=os.pathsep.join([root, os.path.join(root, "tests")]))
+    r = subprocess.run([sys.executable, "-c", LITTLE_MEMORY, *map(str, args)], cwd=root, env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
+
+
+@pytest.mark.parametrize("k,leave", [(51, 1500), (31, 700)])
+def test_little_memory_for_the_sorts(gpu, k, leave):
+    """Not enough memory for the sorted copy of all records at once: smaller groups of buckets."""
+    little_memory(k, 3_000_000, leave, 0)
