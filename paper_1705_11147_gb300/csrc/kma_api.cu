@@ -627,16 +627,21 @@ int scatter_windows(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, 
                       [&] { return launch_part_scatter(g, w, t, st, h->num_sms); });
 }
 
+// Room for `need` output records; all of it or, on an error, none.
 int ensure_output(kma_handle* h, u64 need) {
   if (need <= h->out_cap && h->out_keys) return KMA_OK;
-  dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
-  h->out_cap = 0;
+  auto drop = [&] {
+    dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
+    h->out_cap = 0;
+  };
+  drop();
   u64 cap = std::max<u64>(need + need / 8, 1024);
   int rc;
-  if ((rc = dalloc(h, &h->out_keys, 2 * cap))) return rc;
-  if ((rc = dalloc(h, &h->out_counts, cap))) return rc;
-  if ((rc = dalloc(h, &h->out_ext, 8 * cap))) return rc;
-  if ((rc = dalloc(h, &h->out_codes, 2 * cap))) return rc;
+  if ((rc = dalloc(h, &h->out_keys, 2 * cap)) || (rc = dalloc(h, &h->out_counts, cap)) || (rc = dalloc(h, &h->out_ext, 8 * cap)) ||
+      (rc = dalloc(h, &h->out_codes, 2 * cap))) {
+    drop();
+    return rc;
+  }
   h->out_cap = cap;
   return KMA_OK;
 }
@@ -666,7 +671,7 @@ PartOut part_out(kma_handle* h) {
 }
 
 // Partitioned mode: output room before anything is in the table, for as many keys as it was
-// sized for (or as much as there is: more records than fit are classified again afterwards).
+// sized for, if there is memory for them (more records than fit are classified again afterwards).
 int guess_output(kma_handle* h) {
   const double load = h->p.load_factor > 0 ? h->p.load_factor : 0.5;
   const int rc = ensure_output(h, (u64)((double)h->d.plan.table_slots * load));
@@ -716,7 +721,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   PartSplit s;
   std::memset(&s, 0, sizeof(s));
   PartGeom g = part_geom(h);
-  const PartOut o = part_out(h);
+  PartOut o = part_out(h);
   // first slot of the hashes of bucket b (part_of, table_index)
   auto first_slot = [&](unsigned b) -> u64 {
     const u64 top = (u64)b << (32 - h->d.log_b);
@@ -796,7 +801,15 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     if (e == cudaSuccess) break;
     cudaGetLastError();
     if (e != cudaErrorMemoryAllocation) return cuda_fail(e, "split output");
-    if (!may_sync || at_once <= kSplitLeast) return KMA_ENOMEM;
+    if (!may_sync) return KMA_ENOMEM;
+    if (at_once <= kSplitLeast) {  // then without output room: the records are classified when their number is known
+      if (!h->out_keys) return KMA_ENOMEM;
+      cudaFreeAsync(h->out_keys, st); cudaFreeAsync(h->out_counts, st); cudaFreeAsync(h->out_ext, st); cudaFreeAsync(h->out_codes, st);
+      h->out_keys = nullptr, h->out_counts = nullptr, h->out_ext = nullptr, h->out_codes = nullptr;
+      h->out_cap = 0;
+      o = part_out(h);
+      at_once = 2 * kSplitAtOnce, at_most = kSplitGroups / 2;
+    }
     KMA_CUDA(cudaStreamSynchronize(st));  // what has been freed on it is there for the next attempt
   }
   auto run = [&]() -> int {
@@ -1286,7 +1299,7 @@ static int finalize_many(kma_handle* const* hs, uint32_t n, kma_result* out) {
     if (h->d.P > 1 && !(h->host_status->flags & kFlagOutput)) continue;
     cudaStream_t saved = h->stream;
     h->stream = h0->stream;
-    e = ensure_output(h, h->host_status->table_keys);
+    e = ensure_output(h, h->d.P > 1 ? h->host_status->n_out : h->host_status->table_keys);
     h->stream = saved;
     if (e) { h->failed = true; ok[i] = 0; if (!first_err) first_err = e; continue; }
     if (h->d.P > 1) KMA_CUDA(cudaMemsetAsync(&h->status->flags, 0, sizeof(h->status->flags), h0->stream));
@@ -1436,12 +1449,13 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
   const bool parts = h->d.P > 1;
   const u64 S = h->d.plan.table_slots;
   // One table: the keys counted so far bound the records. Partitions: nothing is in the table
-  // yet; room for as many records as the caller has room for (more of them: classified again
-  // below).
+  // yet; room for as many records as the caller has room for, if there is memory for them (more:
+  // classified again below).
   int rc = read_status(h);
   if (rc) return rc;
   if ((rc = flags_to_code(h->host_status->flags))) { h->failed = true; return rc; }
-  if ((rc = ensure_output(h, parts ? std::min<u64>(capacity, S) : h->host_status->table_keys))) { h->failed = true; return rc; }
+  rc = ensure_output(h, parts ? std::min<u64>(capacity, S) : h->host_status->table_keys);
+  if (rc && !(parts && rc == KMA_ENOMEM)) { h->failed = true; return rc; }
   KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
   const unsigned G = (unsigned)std::max<u64>(1, std::min<u64>(kFinalizeGroups, parts ? h->d.P : S / kClassTile));
   unsigned published = 0;  // groups whose records have been appended to the output
@@ -1505,12 +1519,21 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
   KMA_CUDA(cudaStreamSynchronize(h->copy_stream));
   if (h->host_status->n_out > h->out_cap && !(h->host_status->flags & ~kFlagOutput)) {
     // more records than the caller (and so the device output) has room for: all of them into a
-    // larger device output; the host has the first `capacity` of the same set
+    // larger device output; the host has the first `capacity` of the same set. Or there was no memory
+    // for that output before the counting: then the host gets them now
     if ((rc = ensure_output(h, h->host_status->n_out))) { h->failed = true; return rc; }
     KMA_CUDA(cudaMemsetAsync(&h->status->flags, 0, sizeof(h->status->flags), h->stream));
     KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
     published = 0;
     if ((rc = publish(0, S)) || (rc = read_status(h))) { h->failed = true; return rc; }
+    const u64 n = std::min<u64>(capacity, h->host_status->n_out);
+    if (done < n) {
+      if (keys) KMA_CUDA(cudaMemcpyAsync(keys, h->out_keys, n * 16, cudaMemcpyDeviceToHost, h->stream));
+      if (counts) KMA_CUDA(cudaMemcpyAsync(counts, h->out_counts, n * 4, cudaMemcpyDeviceToHost, h->stream));
+      if (ext) KMA_CUDA(cudaMemcpyAsync(ext, h->out_ext, n * 32, cudaMemcpyDeviceToHost, h->stream));
+      if (codes) KMA_CUDA(cudaMemcpyAsync(codes, h->out_codes, n * 2, cudaMemcpyDeviceToHost, h->stream));
+      KMA_CUDA(cudaStreamSynchronize(h->stream));
+    }
   }
   if ((rc = flags_to_code(h->host_status->flags))) {
     h->failed = true;

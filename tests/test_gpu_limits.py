@@ -272,8 +272,9 @@ LITTLE_MEMORY = """
 import sys
 import torch as gpu
 from test_gpu_limits import device_reads, same_result
-from paper_1705_11147_gb300 import BatchGraph, KmerAnalysis, host_result_buffers, make_params
+from paper_1705_11147_gb300 import KmerAnalysis, host_result_buffers, make_params
 k, keys, leave, host = (int(x) for x in sys.argv[1:])
+out = host_result_buffers(4_000_000, pinned=True)
 reads = device_reads(gpu, 600_000, 150, 171, 1_500_000, 5)
 kw = dict(k=k, min_depth=2, max_bases=reads[0].numel(), max_reads=600_000, expected_distinct=4_000_000)
 ka = KmerAnalysis(make_params(**kw, expected_keys=keys, partitions=8))
@@ -285,14 +286,14 @@ gpu.cuda.synchronize()
 gpu.cuda.empty_cache()
 free = gpu.cuda.mem_get_info()[0]
 held = gpu.empty(free - (leave << 20), dtype=gpu.uint8, device="cuda")
-if host:
-    n = ka.finalize_to_host(host_result_buffers(4_000_000, pinned=True))
+if host == 1:
+    n = ka.finalize_to_host(out)
 else:
     n = ka.finalize()
-del held
+held = None
 gpu.cuda.empty_cache()
 same_result(gpu, one, ka)
-if host:
+if host == 1:
     w, g = one.copy_result().sorted(), n.sorted()
     assert (w.keys == g.keys).all() and (w.counts == g.counts).all() and (w.ext == g.ext).all() and (w.codes == g.codes).all()
 print("same")
@@ -313,3 +314,10 @@ def little_memory(*args):
 def test_little_memory_for_the_sorts(gpu, k, leave):
     """Not enough memory for the sorted copy of all records at once: smaller groups of buckets."""
     little_memory(k, 3_000_000, leave, 0)
+
+
+@pytest.mark.parametrize("k,keys,leave,host", [(51, 40_000_000, 1500, 0), (51, 40_000_000, 2470, 0), (51, 3_000_000, 240, 1)])
+def test_little_memory_for_the_records(gpu, k, keys, leave, host):
+    """No memory for the output that the table was sized for (2.4 GB), or none for the sorts beside it:
+    the records are brought out when their number is known."""
+    little_memory(k, keys, leave, host)
