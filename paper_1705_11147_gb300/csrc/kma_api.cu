@@ -875,6 +875,14 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
   return rc;
 }
 
+// Partitioned mode: the figures that count_records adds to start at zero (again, if an earlier
+// finalize ran out of memory for another handle of its batch).
+int reset_counted(kma_handle* h, cudaStream_t st) {
+  static_assert(offsetof(DevStatus, first_sightings) - offsetof(DevStatus, table_keys) == 3 * sizeof(u64), "they are in a row");
+  KMA_CUDA(cudaMemsetAsync(&h->status->table_keys, 0, 4 * sizeof(u64), st));
+  return KMA_OK;
+}
+
 // First pass over the windows [q0, q0 + n_pos) of one packed batch (n_reads reads, n_bases
 // bases) on stream `st`. One table: Bloom test-and-set (or counting) in place. Partitions:
 // scatter into tiles, which finalize counts. Nothing here waits for the GPU.
@@ -1213,8 +1221,7 @@ static int enqueue_recount(kma_handle* const* hs, uint32_t n, bool may_sync) {
   for (uint32_t i = 0; i < n; ++i) {
     kma_handle* h = hs[i];
     if (h->d.P <= 1) continue;
-    KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h0->stream));
-    if ((rc = count_records(h, h0, h0->stream, may_sync, 1, [](unsigned) { return (int)KMA_OK; }))) return rc;
+    if ((rc = reset_counted(h, h0->stream)) || (rc = count_records(h, h0, h0->stream, may_sync, 1, [](unsigned) { return (int)KMA_OK; }))) return rc;
   }
   return KMA_OK;
 }
@@ -1456,7 +1463,11 @@ int kmer_analysis_finalize_to_host(kma_handle* h, uint64_t* keys, uint32_t* coun
   if ((rc = flags_to_code(h->host_status->flags))) { h->failed = true; return rc; }
   rc = ensure_output(h, parts ? std::min<u64>(capacity, S) : h->host_status->table_keys);
   if (rc && !(parts && rc == KMA_ENOMEM)) { h->failed = true; return rc; }
-  KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
+  if (parts) {
+    if ((rc = reset_counted(h, h->stream))) return rc;
+  } else {
+    KMA_CUDA(cudaMemsetAsync(&h->status->n_out, 0, 2 * sizeof(u64), h->stream));
+  }
   const unsigned G = (unsigned)std::max<u64>(1, std::min<u64>(kFinalizeGroups, parts ? h->d.P : S / kClassTile));
   unsigned published = 0;  // groups whose records have been appended to the output
   // Publish the record count so far.

@@ -272,9 +272,16 @@ LITTLE_MEMORY = """
 import sys
 import torch as gpu
 from test_gpu_limits import device_reads, same_result
-from paper_1705_11147_gb300 import KmerAnalysis, host_result_buffers, make_params
+from paper_1705_11147_gb300 import KmerAnalysis, finalize_batch, host_result_buffers, make_params
+from paper_1705_11147_gb300.capi import KMA_ENOMEM, KmaError
 k, keys, leave, host = (int(x) for x in sys.argv[1:])
 out = host_result_buffers(4_000_000, pinned=True)
+few = device_reads(gpu, 2_000, 150, 171, 10_000, 9)
+small, alone = (KmerAnalysis(make_params(k=k, min_depth=2, max_bases=300_000, max_reads=2_000, expected_distinct=100_000, partitions=2))
+                for _ in range(2))
+for h in (small, alone):
+    h.count(*few)
+alone.finalize()
 reads = device_reads(gpu, 600_000, 150, 171, 1_500_000, 5)
 kw = dict(k=k, min_depth=2, max_bases=reads[0].numel(), max_reads=600_000, expected_distinct=4_000_000)
 ka = KmerAnalysis(make_params(**kw, expected_keys=keys, partitions=8))
@@ -288,6 +295,18 @@ free = gpu.cuda.mem_get_info()[0]
 held = gpu.empty(free - (leave << 20), dtype=gpu.uint8, device="cuda")
 if host == 1:
     n = ka.finalize_to_host(out)
+elif host == 2:
+    try:
+        finalize_batch([small, ka])
+        raise AssertionError("there was enough memory")
+    except KmaError as e:
+        assert e.code == KMA_ENOMEM
+    del held
+    gpu.cuda.empty_cache()
+    finalize_batch([small, ka])
+    assert small.result_info.table_keys == alone.result_info.table_keys
+    assert small.timings()["first_sightings"] == alone.timings()["first_sightings"]
+    same_result(gpu, alone, small)
 else:
     n = ka.finalize()
 held = None
@@ -321,3 +340,9 @@ def test_little_memory_for_the_records(gpu, k, keys, leave, host):
     """No memory for the output that the table was sized for (2.4 GB), or none for the sorts beside it:
     the records are brought out when their number is known."""
     little_memory(k, keys, leave, host)
+
+
+def test_finalize_again(gpu):
+    """A batch whose second handle finds no memory can be finalized when there is: the first one's
+    figures are not added up twice."""
+    little_memory(51, 3_000_000, 90, 2)
