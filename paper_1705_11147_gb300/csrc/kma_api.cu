@@ -528,13 +528,15 @@ void set_pack_waits(kma_handle* h, PackBatch& pb) {
   pb.wait_limit = h->p.fault_inject == 1 ? kWaitPollsInjected : kWaitPolls;
 }
 
+// Arena positions of a batch: its bases and a separator behind every read.
+u64 batch_positions(u64 n_reads, u64 n_bases) { return std::max<u64>(1, (n_bases + n_reads + 63) / 64) * 64; }
+
 // Reserve arena positions for a batch of n_reads reads (n_bases bases), packed on stream `st`,
 // and describe it for the pack kernel. The windows of the batch read up to 192 positions past
 // its end; the 256 positions behind it are set invalid here (ordered before the packing on
 // `st`), and the next batch's packing overwrites them.
 int reserve_batch(kma_handle* h, u64 n_reads, u64 n_bases, PackDesc& pd, u64& q0, u64& n_pos, cudaStream_t st) {
-  n_pos = ((n_bases + n_reads + 63) / 64) * 64;
-  if (n_pos == 0) n_pos = 64;
+  n_pos = batch_positions(n_reads, n_bases);
   if (h->q_used + n_pos + kBatchSlack > h->d.plan.arena_positions) return KMA_EFULL;
   if (h->bases_used + n_bases > h->p.max_bases) return KMA_EFULL;
   q0 = h->q_used;
@@ -1138,10 +1140,25 @@ int kmer_analysis_count(kma_handle* h, const char* seq, const char* qual, const 
   // Host input: validate offsets, then stream chunks through two staging buffers; the copy
   // of chunk i+1 overlaps the packing and first pass of chunk i.
   if (!offsets_nondecreasing(offsets, n_reads)) return KMA_EINVAL;
-  if (offsets[n_reads] - offsets[0] + h->bases_used > h->p.max_bases) return KMA_EFULL;
-  if ((rc = setup_staging(h))) return rc;
   const u64 nb_all = offsets[n_reads] - offsets[0];
+  if (nb_all + h->bases_used > h->p.max_bases) return KMA_EFULL;
   const u64 piece = std::min(h->d.staging, std::max(kHostPiece, nb_all / 8));
+  // one past the last read of the piece that starts at read r0: the reads that end inside it
+  // (offsets do not decrease), at least one
+  auto piece_end = [&](u64 r0) -> u64 {
+    const u64 r_max = std::min<u64>(n_reads, r0 + h->stage_offs_cap - 1);
+    const u64 r1 = (u64)(std::upper_bound(offsets + r0 + 1, offsets + r_max + 1, offsets[r0] + piece) - offsets) - 1;
+    return std::max(r1, r0 + 1);
+  };
+  // all of the call or, on an error, none of it
+  u64 q = h->q_used;
+  for (u64 r0 = 0, r1; r0 < n_reads; r0 = r1) {
+    r1 = piece_end(r0);
+    if (offsets[r1] - offsets[r0] > h->d.staging) return KMA_EINVAL;  // a single read longer than the staging buffer
+    q += batch_positions(r1 - r0, offsets[r1] - offsets[r0]);
+    if (q + kBatchSlack > h->d.plan.arena_positions) return KMA_EFULL;
+  }
+  if ((rc = setup_staging(h))) return rc;
   // With partitions, every staged chunk is packed and scattered, so the copy of the next chunk
   // overlaps both.
   const bool parts = h->d.P > 1 && !h->pack_only;
@@ -1153,11 +1170,7 @@ int kmer_analysis_count(kma_handle* h, const char* seq, const char* qual, const 
   }
   u64 r0 = 0;
   while (r0 < n_reads) {
-    // the reads that end inside the piece (offsets do not decrease); at least one, if it can be staged
-    const u64 r_max = std::min<u64>(n_reads, r0 + h->stage_offs_cap - 1);
-    u64 r1 = (u64)(std::upper_bound(offsets + r0 + 1, offsets + r_max + 1, offsets[r0] + piece) - offsets) - 1;
-    if (r1 == r0) r1 = r0 + 1;
-    if (offsets[r1] - offsets[r0] > h->d.staging) return KMA_EINVAL;  // a single read longer than the staging buffer
+    const u64 r1 = piece_end(r0);
     const u64 nb = offsets[r1] - offsets[r0];
     PackDesc pd;
     u64 q0, n_pos;

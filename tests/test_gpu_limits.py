@@ -346,3 +346,26 @@ def test_finalize_again(gpu):
     """A batch whose second handle finds no memory can be finalized when there is: the first one's
     figures are not added up twice."""
     little_memory(51, 3_000_000, 90, 2)
+
+
+@pytest.mark.parametrize("partitions", [1, 4])
+@pytest.mark.parametrize("reason", ["reads", "long"])
+def test_refused_host_reads(gpu, partitions, reason):
+    """A call that does not fit, by its number of reads or by one read longer than the staging buffer
+    behind others, counts none of its reads, also when it is copied in pieces."""
+    from paper_1705_11147_gb300 import KmerAnalysis, capi, make_params
+    rng = np.random.default_rng(4)
+    seq = np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, 30_000_000)]
+    qual = np.full(len(seq), 70, np.uint8)
+    offsets = np.arange(0, len(seq) + 1, 50, dtype=np.uint64)
+    if reason == "long":
+        offsets = np.concatenate([offsets[:400_000], [np.uint64(len(seq))]])
+    kw = dict(k=31, min_depth=1, use_bloom=False, max_bases=30_000_000, max_reads=1000, expected_distinct=200_000, expected_keys=100_000,
+              staging_bytes=9_000_000 if reason == "long" else 0, partitions=partitions)
+    with KmerAnalysis(make_params(**kw)) as ka:
+        with pytest.raises(capi.KmaError) as e:
+            ka.count(seq, qual, offsets)
+        assert e.value.code == (capi.KMA_EINVAL if reason == "long" else capi.KMA_EFULL)
+        ka.count(seq[:500], qual[:500], offsets[:11])
+        info = ka.finalize()
+        assert int(info.valid_windows) == 200 and int(info.n) == 200
