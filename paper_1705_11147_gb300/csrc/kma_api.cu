@@ -114,7 +114,7 @@ constexpr double kSubBucketFill = 0.72;
 // The sorted copy of the records made by the split: as large as all of them below this size, one
 // launch; above it the buckets are split and counted in groups that share a smaller copy. Smaller
 // groups leave the GPU idle at each one's end (2 GiB, 1 GiB, 256 MiB: 250 Mbases, k = 51 5.41,
-// 5.47, 5.98 ms; 140 Mbases, 30 % of them a satellite's, 10.9, 11.7, 17.3 ms; 12 and 24 groups of 3
+// 5.47, 5.98 ms; 430 Mbases, 30 % of them a satellite's, 10.9, 11.7, 17.3 ms; 12 and 24 groups of 3
 // Gbases 78.0 and 78.9 ms), so they are taken only where there is no memory for more. A handle is
 // planned with the second pair.
 constexpr u64 kSplitAtOnce = 2ull << 30;
@@ -629,19 +629,20 @@ int scatter_windows(kma_handle* h, u64 q0, u64 n_pos, u64 n_reads, u64 n_bases, 
                       [&] { return launch_part_scatter(g, w, t, st, h->num_sms); });
 }
 
+void drop_output(kma_handle* h) {
+  dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
+  h->out_cap = 0;
+}
+
 // Room for `need` output records; all of it or, on an error, none.
 int ensure_output(kma_handle* h, u64 need) {
   if (need <= h->out_cap && h->out_keys) return KMA_OK;
-  auto drop = [&] {
-    dfree(h, h->out_keys); dfree(h, h->out_counts); dfree(h, h->out_ext); dfree(h, h->out_codes);
-    h->out_cap = 0;
-  };
-  drop();
+  drop_output(h);
   u64 cap = std::max<u64>(need + need / 8, 1024);
   int rc;
-  if ((rc = dalloc(h, &h->out_keys, 2 * cap)) || (rc = dalloc(h, &h->out_counts, cap)) || (rc = dalloc(h, &h->out_ext, 8 * cap)) ||
-      (rc = dalloc(h, &h->out_codes, 2 * cap))) {
-    drop();
+  if ((rc = dalloc(h, &h->out_keys, 2 * cap)) || (rc = dalloc(h, &h->out_counts, cap)) ||
+      (rc = dalloc(h, &h->out_ext, 8 * cap)) || (rc = dalloc(h, &h->out_codes, 2 * cap))) {
+    drop_output(h);
     return rc;
   }
   h->out_cap = cap;
@@ -806,9 +807,10 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     if (!may_sync) return KMA_ENOMEM;
     if (at_once <= kSplitLeast) {  // then without output room: the records are classified when their number is known
       if (!h->out_keys) return KMA_ENOMEM;
-      cudaFreeAsync(h->out_keys, st); cudaFreeAsync(h->out_counts, st); cudaFreeAsync(h->out_ext, st); cudaFreeAsync(h->out_codes, st);
-      h->out_keys = nullptr, h->out_counts = nullptr, h->out_ext = nullptr, h->out_codes = nullptr;
-      h->out_cap = 0;
+      const cudaStream_t own = h->stream;
+      h->stream = st;
+      drop_output(h);
+      h->stream = own;
       o = part_out(h);
       at_once = 2 * kSplitAtOnce, at_most = kSplitGroups / 2;
     }
@@ -1234,7 +1236,8 @@ static int enqueue_recount(kma_handle* const* hs, uint32_t n, bool may_sync) {
   for (uint32_t i = 0; i < n; ++i) {
     kma_handle* h = hs[i];
     if (h->d.P <= 1) continue;
-    if ((rc = reset_counted(h, h0->stream)) || (rc = count_records(h, h0, h0->stream, may_sync, 1, [](unsigned) { return (int)KMA_OK; }))) return rc;
+    auto nothing = [](unsigned) { return (int)KMA_OK; };
+    if ((rc = reset_counted(h, h0->stream)) || (rc = count_records(h, h0, h0->stream, may_sync, 1, nothing))) return rc;
   }
   return KMA_OK;
 }

@@ -237,8 +237,9 @@ __global__ void cg_cut_kernel(const unsigned* mn, u64 m, unsigned* nbr, unsigned
 
 // Per vertex: the chosen chain (head with the smaller key; forward keys: the forward chain),
 // position in it, and the contig length in bases (heads only) for the offset scan.
-__global__ void cg_place_kernel(const u64* keys, const unsigned* vrec, const u64* link, u64 m, unsigned k, unsigned canonical, unsigned* head, unsigned* pos,
-                                unsigned char* dir, u64* head_flag, u64* head_len) {
+__global__ void cg_place_kernel(const u64* keys, const unsigned* vrec, const u64* link, u64 m, unsigned k,
+                                unsigned canonical, unsigned* head, unsigned* pos, unsigned char* dir, u64* head_flag,
+                                u64* head_len) {
   const u64 u = (u64)blockIdx.x * blockDim.x + threadIdx.x;
   if (u > m) return;
   if (u == m) {  // scan total slots
@@ -399,7 +400,8 @@ int contig_pass(const u64* keys, const unsigned char* codes, u64 n, unsigned k, 
   unsigned *head = nullptr, *pos = nullptr;
   unsigned char* dir = nullptr;
   u64 *hflag = nullptr, *hlen = nullptr;
-  if (!alloc((void**)&head, m * 4) || !alloc((void**)&pos, m * 4) || !alloc((void**)&dir, m) || !alloc((void**)&hflag, (m + 1) * 8) || !alloc((void**)&hlen, (m + 1) * 8))
+  if (!alloc((void**)&head, m * 4) || !alloc((void**)&pos, m * 4) || !alloc((void**)&dir, m) ||
+      !alloc((void**)&hflag, (m + 1) * 8) || !alloc((void**)&hlen, (m + 1) * 8))
     return fail(-2);
   cg_place_kernel<<<blocks_for(m + 1), kCgThreads, 0, st>>>(keys, vrec, link, m, k, canonical, head, pos, dir,
                                                            hflag, hlen);

@@ -121,8 +121,10 @@ __device__ __forceinline__ unsigned newline_mask(const unsigned char* text, u64 
   }
   // one bit per byte: compare, keep bit 0 of each byte, gather the four of a word
   const unsigned nl = 0x0A0A0A0Au;
-  const unsigned m0 = ((__vcmpeq4(v.x, nl) & 0x01010101u) * 0x01020408u) >> 24, m1 = ((__vcmpeq4(v.y, nl) & 0x01010101u) * 0x01020408u) >> 24;
-  const unsigned m2 = ((__vcmpeq4(v.z, nl) & 0x01010101u) * 0x01020408u) >> 24, m3 = ((__vcmpeq4(v.w, nl) & 0x01010101u) * 0x01020408u) >> 24;
+  const unsigned m0 = ((__vcmpeq4(v.x, nl) & 0x01010101u) * 0x01020408u) >> 24;
+  const unsigned m1 = ((__vcmpeq4(v.y, nl) & 0x01010101u) * 0x01020408u) >> 24;
+  const unsigned m2 = ((__vcmpeq4(v.z, nl) & 0x01010101u) * 0x01020408u) >> 24;
+  const unsigned m3 = ((__vcmpeq4(v.w, nl) & 0x01010101u) * 0x01020408u) >> 24;
   unsigned m = (m0 & 15u) | ((m1 & 15u) << 4) | ((m2 & 15u) << 8) | ((m3 & 15u) << 12);
   const long long last = (long long)n - 1 - i;
   if (last < 16) m |= 1u << last;  // the last byte ends a line either way
@@ -215,14 +217,13 @@ __global__ void fastq_record_kernel(const unsigned char* text, const u64* line_e
   if (!ok) atomicMin(bad, (unsigned long long)r);
 }
 
-// Eight text bytes starting at any address, from the two aligned words that hold them (the second
-// one is read only if it does).
-__device__ __forceinline__ u64 load8(const unsigned char* p, unsigned valid) {
+// Eight text bytes starting at any address, from the one or two aligned words that hold them.
+__device__ __forceinline__ u64 load8(const unsigned char* p) {
   const u64 a = reinterpret_cast<u64>(p);
   const u64* w = reinterpret_cast<const u64*>(a & ~7ull);
   const unsigned s = (unsigned)(a & 7) * 8;
   u64 v = __ldg(w) >> s;
-  if (s && valid > 8 - s / 8) v |= __ldg(w + 1) << (64 - s);
+  if (s) v |= __ldg(w + 1) << (64 - s);
   return v;
 }
 
@@ -235,7 +236,7 @@ __device__ __forceinline__ void copy_line(const unsigned char* src, unsigned cha
   if (head > len) head = len;
   if (lane < head) dst[lane] = src[lane];
   const u64 words = (len - head) / 8;
-  for (u64 w = lane; w < words; w += kLineLanes) *reinterpret_cast<u64*>(dst + head + 8 * w) = load8(src + head + 8 * w, 8);
+  for (u64 w = lane; w < words; w += kLineLanes) *reinterpret_cast<u64*>(dst + head + 8 * w) = load8(src + head + 8 * w);
   const u64 done = head + 8 * words;
   if (lane < len - done) dst[done + lane] = src[done + lane];
 }

@@ -172,7 +172,8 @@ __device__ __forceinline__ int find_pack_sample(const PackBatch& B, u64 c) {
   return lo;
 }
 
-// Last read r with start ps_r = offsets[r] - o0 + r <= p, found by a warp: the answer lies in [lo, hi) and offsets[lo] - o0 + lo <= p;
+// Last read r with start ps_r = offsets[r] - o0 + r <= p, found by a warp: the answer lies in
+// [lo, hi) and offsets[lo] - o0 + lo <= p;
 // each round the 32 lanes test 32 evenly spaced reads, so ~log32(hi - lo) dependent loads
 // instead of log2. Called by all lanes of a warp with the same arguments; all return it.
 // With non-decreasing offsets the lanes that qualify are a prefix of the warp; `bad` is set
@@ -288,7 +289,7 @@ __device__ __forceinline__ unsigned complement16(unsigned c) {
 // consecutive threads are consecutive, so the stores coalesce.
 // Bound by the instructions issued: 68 a position when each thread packed its 64 positions four
 // at a time and looked for a read's end in each group (with 16-way bank conflicts between the
-// threads' words, which cost nothing beside that). 214 M positions: 564 us -> 239 us; 3.1 G
+// threads' words, which cost nothing beside that). 252 M positions: 564 us -> 239 us; 3.0 G
 // positions: 5.50 ms -> 2.67 ms, 3.1 TB/s of input and output.
 __global__ void __launch_bounds__(kPackThreads, 4) pack_kernel(const __grid_constant__ PackBatch B) {
   __shared__ __align__(16) unsigned char s_seq[kPackBuf];

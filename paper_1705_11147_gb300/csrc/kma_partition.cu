@@ -20,7 +20,7 @@
 // L2 took 4.6 L2 requests per window, 21 ns per 1000 windows, and a second pass over the first
 // sightings another 8 ns. A sort pass reads and writes 8 or 16 bytes per window in whole lines,
 // and with all occurrences of a k-mer in one shared memory the singletons (error k-mers) are known
-// exactly, so they cost no memory traffic outside the SM. 2.4 G windows, k = 31: 110 ms -> 79 ms
+// exactly, so they cost no memory traffic outside the SM. 2.4 G windows, k = 51: 110 ms -> 78 ms
 // from reads to answers, 166 M windows, k = 51: 8.2 ms -> 5.7 ms.
 #include <mutex>
 #include <utility>
@@ -306,10 +306,11 @@ __global__ void __launch_bounds__(kScatterThreads, 1) part_scatter_kernel(const 
 // buckets in order, so the pieces of one line meet in L2. A sub-bucket has room for G.cap
 // records; what does not fit (very frequent k-mers) goes to an overflow segment of the bucket.
 //
-// Bound by the instructions issued, about 150 a record; a third and a fourth CTA per SM (40 and 32
-// registers) and sub-tiles of 3072, 6144 or 8192 records were slower. 166 M records of 16 bytes:
-// 0.94 ms; 2.4 G of 8 bytes: 25 ms (1.17 and 27 ms when the records were moved to their sorted
-// places, from and to registers).
+// Bound by the waits on shared memory between its steps (134 instructions a record, 46 % of the
+// issue slots used, DRAM at 4.3 TB/s); a third and a fourth CTA per SM (40 and 32 registers) and
+// sub-tiles of 3072, 6144 or 8192 records were slower. 134 M records of 16 bytes: 0.94 ms; 2.4 G
+// of them: 25 ms (1.17 and 27 ms when the records were moved to their sorted places, from and to
+// registers).
 
 constexpr int kSplitThreads = 512;
 constexpr int kSplitItems = kPartSubTile / kSplitThreads;
@@ -355,7 +356,7 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
   extern __shared__ __align__(128) unsigned char s_raw[];
   __shared__ u64 s_over;
   u64* s_rec = reinterpret_cast<u64*>(s_raw);                                  // [sub-tile * KW]
-  unsigned short* s_ord = reinterpret_cast<unsigned short*>(s_rec + kPartSubTile * KW);  // [sub-tile] the record at a sorted position
+  unsigned short* s_ord = reinterpret_cast<unsigned short*>(s_rec + kPartSubTile * KW);  // [sub-tile] record at a sorted place
   unsigned* s_bin = reinterpret_cast<unsigned*>(s_ord + kPartSubTile);         // [sub_max] counts, then offsets
   unsigned* s_to = s_bin + G.sub_max;                                          // [sub_max] place minus sorted position
   unsigned* s_wsum = s_to + G.sub_max;                                         // [32]
@@ -384,8 +385,10 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
       const uint4 v = __ldg(reinterpret_cast<const uint4*>(row));
       const unsigned next = __ldg(row + kSplitBuckets);  // inside the row's padding for the last buckets
       unsigned short* o = s_off + i * (kSplitBuckets + 1);
-      o[0] = (unsigned short)v.x, o[1] = (unsigned short)(v.x >> 16), o[2] = (unsigned short)v.y, o[3] = (unsigned short)(v.y >> 16);
-      o[4] = (unsigned short)v.z, o[5] = (unsigned short)(v.z >> 16), o[6] = (unsigned short)v.w, o[7] = (unsigned short)(v.w >> 16);
+      o[0] = (unsigned short)v.x, o[1] = (unsigned short)(v.x >> 16);
+      o[2] = (unsigned short)v.y, o[3] = (unsigned short)(v.y >> 16);
+      o[4] = (unsigned short)v.z, o[5] = (unsigned short)(v.z >> 16);
+      o[6] = (unsigned short)v.w, o[7] = (unsigned short)(v.w >> 16);
       o[8] = (unsigned short)next;
     }
     __syncthreads();
@@ -524,20 +527,20 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
             else *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(v0, v1);
           }
         } else {
-        for (unsigned i = tid; i < n; i += kSplitThreads) {
-          u64 v0, v1 = 0;
-          if (KW == 1) {
-            v0 = s_rec[s_ord[i]];
-          } else {
-            const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[s_ord[i]];
-            v0 = v.x;
-            v1 = v.y;
+          for (unsigned i = tid; i < n; i += kSplitThreads) {
+            u64 v0, v1 = 0;
+            if (KW == 1) {
+              v0 = s_rec[s_ord[i]];
+            } else {
+              const ulonglong2 v = reinterpret_cast<const ulonglong2*>(s_rec)[s_ord[i]];
+              v0 = v.x;
+              v1 = v.y;
+            }
+            const unsigned p = sub_of(v0, G.log_b, n_sub);
+            u64* to = i < s_lim[p] ? out + (u64)(s_to[p] + i) * KW : S.over + (s_over + (s_bin[p] + i)) * KW;
+            if (KW == 1) *to = v0;
+            else *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(v0, v1);
           }
-          const unsigned p = sub_of(v0, G.log_b, n_sub);
-          u64* to = i < s_lim[p] ? out + (u64)(s_to[p] + i) * KW : S.over + (s_over + (s_bin[p] + i)) * KW;
-          if (KW == 1) *to = v0;
-          else *reinterpret_cast<ulonglong2*>(to) = make_ulonglong2(v0, v1);
-        }
         }
         __syncthreads();  // s_bin, s_rec and s_wsum are rewritten
       }
@@ -563,10 +566,11 @@ __global__ void __launch_bounds__(kSplitThreads, 2) part_split_kernel(const __gr
 // Sub-buckets that overflowed (very frequent k-mers) and those with more keys than the second
 // table holds are listed for part_large_kernel.
 //
-// Bound by instruction issue and, between the steps, by the barriers. 166 M records of 16 bytes:
-// 1.65 ms; 2.4 G of 8 bytes: 23.0 ms. Rejected: a table with the keys and counters themselves that
-// records are added to from registers (a probe of a 16-byte key behind a 64-bit compare-and-swap
-// takes 70 instructions for 32 records, 12 in all per record and warp instead of 6).
+// Bound by the barriers between the steps and by shared memory (207 instructions a record, 56 % of
+// the issue slots used). 166 M records of 16 bytes: 1.65 ms; 2.4 G of them: 23.0 ms. Rejected: a
+// table with the keys and counters themselves that records are added to from registers (a probe of
+// a 16-byte key behind a 64-bit compare-and-swap takes 70 instructions for 32 records, 12 in all
+// per record and warp instead of 6).
 
 constexpr int kCountThreads = 640;  // 512 and 768: 1 % and 6 % slower
 constexpr int kCountCtas = 2;                // per SM
@@ -1310,7 +1314,8 @@ __global__ void __launch_bounds__(kInsertThreads) part_insert_kernel(const __gri
     __syncthreads();  // all of the block have read base
     if (threadIdx.x == 0) {
       __threadfence();
-      if (atomicAdd(reinterpret_cast<unsigned*>(S.inserted), 1u) == gridDim.x - 1 && n) atomicAdd(&G.status->n_out, n);  // everyone has
+      const bool last = atomicAdd(reinterpret_cast<unsigned*>(S.inserted), 1u) == gridDim.x - 1;  // everyone has read it
+      if (last && n) atomicAdd(&G.status->n_out, n);
     }
   } else {
     for (u64 t = blockIdx.x; t * kInsertTile < n; t += gridDim.x) {
