@@ -245,7 +245,8 @@ def roofline(timing: dict, res_info, positions: int, peak_gbs: float, plan_used,
     partitions (part_scatter_kernel + part_split_kernel, the two sorts, over all launches of one
       step): 0.75 B per arena position read, and per record (one per valid window, 8 B for
       k <= 32, else 16) one write by the scatter and a read and a write by the split. A second
-      figure is the counting (part_count_kernel), which reads every record once."""
+      figure is the counting (part_count_kernel, and part_large_kernel for what does not fit its
+      shared memory), which reads every record once."""
     W = int(res_info.valid_windows)
     F = int(timing["first_sightings"])
     ms = timing["ms_pass"] / max(timing["n_pass"], 1)
@@ -254,7 +255,7 @@ def roofline(timing: dict, res_info, positions: int, peak_gbs: float, plan_used,
         rec = 16 if k > 32 else 8
         steps = max(timing["n_pack"], 1)
         counted = timing["ms_pass"] / steps
-        extra["count"] = {"kernel": "part_count_kernel", "ms_per_step": round(counted, 3),
+        extra["count"] = {"kernel": "part_count_kernel + part_large_kernel", "ms_per_step": round(counted, 3),
                           "algo_bytes_per_step": W * rec,
                           "achieved": round(W * rec / (counted * 1e-3) / 1e9, 1),
                           "frac": round(W * rec / (counted * 1e-3) / 1e9 / peak_gbs, 4)}
@@ -267,7 +268,9 @@ def roofline(timing: dict, res_info, positions: int, peak_gbs: float, plan_used,
         kernel, files, summary = ("pass_kernel (Bloom mode)", ["kma_kernels.cu", "kma_device.cuh"],
                                   "pass_kernel_large_200m.md")
     achieved = algo / (ms * 1e-3) / 1e9
-    prof = profiled_values(summary, kernel_source_digest(files))
+    # the capture of the sorts is of two-word keys (16-byte records)
+    two_words = plan_used.partitions <= 1 or k > 32
+    prof = profiled_values(summary, kernel_source_digest(files)) if two_words else {}
     out = {"bound": "hbm", "achieved": round(achieved, 1), "peak": peak_gbs, "unit": "GB/s",
            "frac": round(achieved / peak_gbs, 4),
            "traffic": int(prof["dram_bytes_per_unit"] * W) if "dram_bytes_per_unit" in prof else None,

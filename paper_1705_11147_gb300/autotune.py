@@ -38,15 +38,14 @@ DEFAULT_CANDIDATES = [
     dict(partitions=-1, warp_aggregate=True),  # automatic count, warp aggregation
 ]
 
-# on-chip partitions: partition count around the automatic one, sub-table load factor, records
-# per thread of the record passes
+# on-chip partitions: partition count around the automatic one, table load factor (the sorts'
+# launch shapes are the library's)
 PARTITIONED_CANDIDATES = [
     dict(),
     dict(partition_scale=0.5),
     dict(partition_scale=2.0),
     dict(load_factor=0.6),
     dict(load_factor=0.7),
-    dict(windows_per_thread=4),
     dict(partition_scale=0.5, load_factor=0.7),
 ]
 

@@ -312,8 +312,8 @@ class BatchGraph:
     """Many samples in one CUDA graph. Samples counted in one table are packed and counted
     together (one packing launch and one persistent counting launch), then recounted and
     classified together (kmer_analysis_finalize_batch_async). Samples large enough to be
-    partitioned run their scatter/record passes one after another inside the same graph, each
-    finalized before the next starts, so only one sample's record buckets exist at a time.
+    partitioned are sorted and counted one after another inside the same graph, each
+    finalized before the next starts, so only one sample's records exist at a time.
     Captured once, replayed per step. `reads[i]` = (seq, qual, offsets) CUDA tensors of
     handle i; all handles are moved to the capture stream."""
 
