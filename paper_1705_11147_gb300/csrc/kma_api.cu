@@ -692,8 +692,10 @@ unsigned lanes_for(double len) {
 // below `end` have been enqueued. The groups share the sorted copy of the split: all records at once when
 // they are few, otherwise from the bucket totals, a twelfth of the records or the largest bucket;
 // smaller ones when there is no memory for that. When the call may not wait for the GPU (may_sync
-// = false, capture) the groups are a twelfth of the buckets, and only the room for records without
-// a place in their sub-bucket is for all (any bucket may hold them).
+// = false, capture) the groups are of equal numbers of buckets, as many as there are 2 GiB of
+// records (twelve at most), and only the room for records without a place in their sub-bucket is
+// for all (any bucket may hold them): a graph of 64 samples of up to 1.3 Gbases takes 281 ms (299
+// with twelve groups for each sample above 2 GiB, 276 in one with twice the memory).
 template <typename F>
 int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sync, unsigned parts, F&& after) {
   const unsigned B = 1u << h->d.log_b;
@@ -718,7 +720,7 @@ int count_records(kma_handle* h, kma_handle* timed, cudaStream_t st, bool may_sy
     return rc ? rc : after(B);
   }
   constexpr unsigned kStep = kSplitBuckets;  // groups are whole work items of the split
-  if (!may_sync && bound * h->d.rec_bytes > kSplitAtOnce) parts = std::max<unsigned>(parts, kSplitGroups);
+  if (!may_sync) parts = std::max(parts, (unsigned)std::min<u64>(kSplitGroups, bound * h->d.rec_bytes / kSplitAtOnce + 1));
   parts = std::min(parts, B / kStep);
   double counted = bases / std::max(1u, h->p.n_parts);  // windows there may be
   PartSplit s;
